@@ -30,14 +30,14 @@ from paper_2605_05607_b200 import synth  # noqa: E402
 
 METRIC = "fused MoE layer tokens/sec"
 UNIT = "tokens/s"
-KERNELS_PER_STEP = 10  # gate split, gate, topk, masks, scan, offsets, fill, gemm1, gemm2, combine
+KERNELS_PER_STEP = 9  # gate, topk, masks, scan, offsets, fill, gemm1, gemm2, combine
 
 
 def kernels_per_step(cfg, flags: int, fp8: bool) -> int:
     """Launches of one moe_layer call, following the library's own choice of forms (see MOE_FLAG_* in tcmoe.h)."""
     from paper_2605_05607_b200 import binding as B
     if flags & B.MOE_FLAG_FUSED_FFN:
-        return 7 + 2                                   # ... layout, then the task-table kernel and the tracker-paced kernel
+        return 6 + 2                                   # ... layout, then the task-table kernel and the tracker-paced kernel
     n = KERNELS_PER_STEP + (2 if fp8 else 0)           # FP8: + quantisation of x and of h
     if flags & B.MOE_FLAG_COMBINE_IN_EPILOGUE:
         return n                                       # no combine kernel, one rounding pass instead

@@ -2,19 +2,25 @@
 //     logits[T, E] = x[T, d] (bf16) * w_gate[d, E] (fp32), fp32 result.
 //
 // x is bf16, so every product x * w is exact once w is written as hi + mid + lo with three bf16
-// terms (8 + 8 + 8 mantissa bits cover fp32's 24).  The kernel therefore runs ONE bf16 UMMA
-// accumulation over K' = 3 d: iteration j multiplies k-block j / 3 of x with k-block j / 3 of
-// split j % 3, all into the same fp32 accumulator in TMEM.  The fp32 ALUs would need 2 T d E flop
-// (120 GFLOP, 3.7 ms for the DeepSeek-V3-shaped layer); the tensor pipe does 3x that in ~0.3 ms.
+// terms (8 + 8 + 8 mantissa bits cover fp32's 24): three bf16 UMMAs per k-step into fp32
+// accumulators in TMEM (the fp32 ALUs would need 2 T d E flop: 120 GFLOP, 3.7 ms for the
+// DeepSeek-V3-shaped layer).
 //
-// One CTA per (128-token tile, 256-expert tile); warps 0-3 epilogue (TMEM -> fp32 stores), warp 4
-// TMA producer, warp 5 UMMA issuer and TMEM owner.  Two schedules:
-//  - E <= 128 ("side by side"): the hi / mid / lo slabs of a k-block sit next to each other as
-//    columns of one B tile (3 x ceil(E/64) slabs <= 6), x is loaded once per k-block, one or two
-//    UMMAs fill separate accumulator column groups and the epilogue adds the three groups;
-//    d/64 iterations of (A 16 KB + B <= 48 KB), 3 stages.
-//  - larger E: the three terms are accumulated in place, 3 d/64 iterations of (A 16 KB + B 32 KB),
-//    4 stages (the accumulators of 3 x 256 columns would not fit the 512 TMEM columns).
+// A task is a 128-token x GN-expert tile and the whole of K.  Sixteen warps (groups that take turns)
+// read the fp32 block of w_gate, split it and write the three terms straight into the swizzled
+// MN-major operand tiles: no split copy of the weight in memory and no launch for it.  x comes by TMA.
+// What bounds it: for few tokens the walk along K, one k-block of 64 after the other, so tiles are
+// narrow (a short k-block, and E / GN thread blocks share the work); for many tokens shared-memory
+// bandwidth (the UMMAs read the rows of x once per 256 columns), so tiles are wide and two row tiles share
+// a split weight block.  Up to 128 experts the three terms are summed apart, as one wide B of 3 GN columns: an
+// UMMA takes about 70 cycles for any N up to 128.  More experts keep one running sum (TMEM columns).
+// Measured, us, against the form with a split kernel and one tile width (T, d, E): 64, 4096, 128: 41 -> 24.5;
+// 128, 7168, 256: 157 -> 66; 1777, 2880, 128: 34 -> 20.5; 8192, 4096, 128: 49 -> 37-41; 16384, 4096, 128: 55 -> 54;
+// 32768, 7168, 256: 350-420 -> 308-322.
+// K is never divided over thread blocks, although that would be faster still for a decode batch (9 us
+// at T = 64, d = 4096, E = 128): a logit is the same sum in the same order whatever the tile, and a
+// different order moves it by up to 1e-4, enough to change the selection of a token whose k-th and next
+// key nearly tie.
 #include "ffn_common.cuh"
 
 #include <atomic>
@@ -24,44 +30,32 @@ namespace {
 
 using namespace ffn;
 
-constexpr int A_BYTES = BM * BK * 2;
-constexpr int MAX_STAGES = 4;
+constexpr int A_BYTES = BM * BK * 2;            // 16 KiB of x
+constexpr int RING_BYTES = 192 * 1024;
+constexpr int MAX_STAGES = 8;
 constexpr int NUM_BARS = 2 * MAX_STAGES + 1;
-constexpr int RING_BYTES = 4 * (A_BYTES + 4 * 8192);   // = 3 * (A_BYTES + 6 * 8192) = 192 KiB
-constexpr int SMEM_BYTES = 1024 + RING_BYTES + NUM_BARS * 8 + 64;
-constexpr int THREADS = 192;
-
-// w_gate fp32 [d, E] -> bf16 [3, d, Epad]: hi, mid, lo terms, zero in the padding columns
-__global__ void __launch_bounds__(256) split_gate_kernel(const float* __restrict__ wg, __nv_bfloat16* __restrict__ out,
-                                                         int d, int E, int Epad) {
-  grid_dependency_sync();
-  const size_t n = (size_t)d * Epad;
-  for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x) {
-    const int row = (int)(i / Epad), col = (int)(i % Epad);
-    float w = (col < E) ? __ldg(wg + (size_t)row * E + col) : 0.f;
-    const __nv_bfloat16 hi = __float2bfloat16_rn(w);
-    w = __fsub_rn(w, __bfloat162float(hi));          // exact
-    const __nv_bfloat16 mid = __float2bfloat16_rn(w);
-    w = __fsub_rn(w, __bfloat162float(mid));         // exact
-    out[i] = hi;
-    out[n + i] = mid;
-    out[2 * n + i] = __float2bfloat16_rn(w);
-  }
-}
+constexpr int SMEM_BYTES = 1024 + RING_BYTES + A_BYTES + NUM_BARS * 8 + 64;   // + A_BYTES: see a_bytes
+constexpr int SPLIT_WARPS = 16;
+constexpr int TMA_WARP = SPLIT_WARPS, MMA_WARP = SPLIT_WARPS + 1;
+constexpr int THREADS = (SPLIT_WARPS + 2) * 32;
 
 struct GateParams {
-  float* logits;
-  int T, E, KB, n_tiles;
-  int side_by_side;   // 1: hi | mid | lo as column groups of one B tile (E <= 128)
+  const float* w;     // [d, E]
+  float* logits;      // [T, E]
+  int T, d, E, KB, n_tiles;
+  int m_sub;          // 128-row tiles per task, 1 or 2: they share the split weight block
+  int a_bytes;        // bytes of x per row tile and stage: fewer than 128 rows are loaded when T is small (the UMMA then
+                      // reads whatever follows; only rows >= T depend on it)
+  int apart;          // 1: hi, mid and lo sums in accumulators of their own, added at the end; 0: one running sum
   int32_t* status;
 };
 
+template <int GN, int GROUPS>
 __global__ void __launch_bounds__(THREADS, 1)
-gate_umma_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant__ CUtensorMap map_w,
-                 const GateParams p) {
+gate_umma_kernel(const __grid_constant__ CUtensorMap map_x, const GateParams p) {
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
-  uint64_t* bars = reinterpret_cast<uint64_t*>(smem + RING_BYTES);
+  uint64_t* bars = reinterpret_cast<uint64_t*>(smem + RING_BYTES + A_BYTES);
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + NUM_BARS);
   int* abort_s = reinterpret_cast<int*>(tmem_slot + 1);
 
@@ -72,29 +66,27 @@ gate_umma_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constan
   const uint32_t done_bar = bar_base + 8u * (2 * MAX_STAGES);
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int mt = blockIdx.x / p.n_tiles, nt = blockIdx.x % p.n_tiles;
-  const int row0 = mt * BM, n0 = nt * UMMA_N;
-  const int ncols = min(UMMA_N, ((p.E - n0) + 63) & ~63);   // expert columns of this tile, in 64-column slabs
-  const int nslab = ncols >> 6;
-  const bool sbs = p.side_by_side != 0;
-  const int bslabs = sbs ? 3 * nslab : nslab;            // B slabs per stage
-  const int NSTAGE = sbs ? 3 : 4;
-  const int STAGE_BYTES = A_BYTES + (sbs ? 6 : 4) * 8192;
-  const int iters = sbs ? p.KB : 3 * p.KB;
+  const int row0 = (blockIdx.x / p.n_tiles) * p.m_sub * BM, n0 = (blockIdx.x % p.n_tiles) * GN;
+  const int n_sub = p.m_sub > 1 && row0 + BM < p.T ? 2 : 1;           // row tiles of this task that have rows
+  // a stage: hi | mid | lo columns of the weight block side by side in 64-column slabs of 8 KiB, then the x tiles
+  constexpr int GROUP_WARPS = SPLIT_WARPS / GROUPS;
+  constexpr int B_BYTES = (3 * GN + 63) / 64 * 8192;
+  // A group that has filled block i knows that block i - n_stages was consumed.  Its next one, i + GROUPS, needs
+  // i + GROUPS - 2 n_stages consumed for its parity wait to mean the right phase: no more groups than stages.
+  static_assert(GROUPS <= RING_BYTES / (B_BYTES + 2 * A_BYTES) && GROUPS <= MAX_STAGES, "more groups than stages");
+  const int stage_bytes = B_BYTES + p.m_sub * p.a_bytes, n_stages = min(MAX_STAGES, RING_BYTES / stage_bytes);
+  const int ncols = min(GN, (p.E - n0 + 31) & ~31);                   // expert columns of this tile, zero beyond E
 
   if (threadIdx.x == 0) {
     for (int s = 0; s < MAX_STAGES; ++s) {
-      ptx::mbar_init(full_bar(s), 1);
+      ptx::mbar_init(full_bar(s), GROUP_WARPS + 1);   // one group of split warps + the TMA thread (expect_tx)
       ptx::mbar_init(empty_bar(s), 1);
     }
     ptx::mbar_init(done_bar, 1);
     ptx::fence_mbar_init();
   }
-  if (warp == 4 && lane == 0) {
-    ptx::prefetch_tensormap(&map_x);
-    ptx::prefetch_tensormap(&map_w);
-  }
-  if (warp == 5) {
+  if (warp == TMA_WARP && lane == 0) ptx::prefetch_tensormap(&map_x);
+  if (warp == MMA_WARP) {
     ptx::tmem_alloc(ptx::smem_u32(tmem_slot), 512);
     ptx::tmem_relinquish();
   }
@@ -112,98 +104,181 @@ gate_umma_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constan
     *abort_flag = 1;
   };
 
-  if (warp < 4) {
+  if (warp < SPLIT_WARPS) {
+    // ================================ weight block -> three bf16 terms ================================
+    // Thread: 8 columns (one 16-byte piece of a swizzle row) of CHUNKS rows of K.  Group g takes every GROUPS-th
+    // k-block and keeps DEPTH of its blocks on the way in registers.
+    constexpr int PIECES = GN / 8, ROWS = GROUP_WARPS * 32 / PIECES, CHUNKS = BK / ROWS;
+    constexpr int DEPTH = CHUNKS >= 4 ? 1 : 4 / CHUNKS;
+    static_assert(CHUNKS * ROWS == BK, "whole passes");
+    const int group = warp / GROUP_WARPS, tid = threadIdx.x % (GROUP_WARPS * 32);
+    const int piece = tid % PIECES, krow = tid / PIECES;
+    const int col = n0 + piece * 8;
+    const bool vec = (p.E & 3) == 0;
+    const bool plain = vec && col + 8 <= p.E;                             // whole vectors inside the row
+    float w[DEPTH][CHUNKS][8];
+    auto load = [&](int kb, float (&v)[CHUNKS][8]) {
+      const float* src = p.w + (size_t)(kb * BK + krow) * p.E + col;
+      if (plain && kb * BK + BK <= p.d) {
+#pragma unroll
+        for (int c = 0; c < CHUNKS; ++c) {
+          const float4* q = reinterpret_cast<const float4*>(src + (size_t)(c * ROWS) * p.E);
+          const float4 a = __ldg(q), b = __ldg(q + 1);
+          v[c][0] = a.x; v[c][1] = a.y; v[c][2] = a.z; v[c][3] = a.w;
+          v[c][4] = b.x; v[c][5] = b.y; v[c][6] = b.z; v[c][7] = b.w;
+        }
+      } else {
+#pragma unroll
+        for (int c = 0; c < CHUNKS; ++c)
+#pragma unroll
+          for (int i = 0; i < 8; ++i)
+            v[c][i] = (kb * BK + c * ROWS + krow < p.d && col + i < p.E) ? __ldg(src + (size_t)(c * ROWS) * p.E + i) : 0.f;
+      }
+    };
+    int s = 0, ph = 1;
+    auto advance = [&](int n) {
+      for (s += n; s >= n_stages; s -= n_stages) ph ^= 1;
+    };
+    advance(group);
+    auto block = [&](int kb, float (&v)[CHUNKS][8]) {
+      if (!ptx::mbar_wait_warp(empty_bar(s), ph, abort_flag, global_abort)) { timeout(2); return false; }
+      const uint32_t dst0 = smem_base + s * stage_bytes;
+#pragma unroll
+      for (int c = 0; c < CHUNKS; ++c) {
+        const int k = c * ROWS + krow;
+        uint32_t q[3][4];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+          float a = v[c][2 * i], b = v[c][2 * i + 1];
+#pragma unroll
+          for (int t = 0; t < 3; ++t) {   // the remainders are exact
+            const __nv_bfloat162 r = __floats2bfloat162_rn(a, b);
+            const uint32_t u = *reinterpret_cast<const uint32_t*>(&r);
+            q[t][i] = u;
+            a = __fsub_rn(a, __uint_as_float(u << 16));
+            b = __fsub_rn(b, __uint_as_float(u & 0xFFFF0000u));
+          }
+        }
+#pragma unroll
+        for (int t = 0; t < 3; ++t) {
+          const int at = t * PIECES + piece;   // 16-byte piece of the 3 GN columns
+          ptx::st_shared_v4(dst0 + (at >> 3) * 8192 + k * 128 + (((at & 7) ^ (k & 7)) << 4), q[t][0], q[t][1], q[t][2], q[t][3]);
+        }
+      }
+      ptx::fence_proxy_async_smem();
+      __syncwarp();
+      if (lane == 0) ptx::mbar_arrive(full_bar(s));
+      if (kb + GROUPS * DEPTH < p.KB) load(kb + GROUPS * DEPTH, v);
+      advance(GROUPS);
+      return true;
+    };
+    bool ok = !*abort_flag;
+#pragma unroll
+    for (int i = 0; i < DEPTH; ++i)
+      if (ok && group + GROUPS * i < p.KB) load(group + GROUPS * i, w[i]);
+    for (int kb = group; ok && kb < p.KB; kb += GROUPS * DEPTH) {
+#pragma unroll
+      for (int i = 0; i < DEPTH; ++i)
+        if (ok && kb + GROUPS * i < p.KB) ok = block(kb + GROUPS * i, w[i]);
+    }
     // ================================ epilogue ================================
     if (!*abort_flag) {
       if (!ptx::mbar_wait_warp<true>(done_bar, 0, abort_flag, global_abort)) {
         timeout(1);
       } else {
         ptx::tc_fence_after();
-        const int row = row0 + warp * 32 + lane;
-        const bool valid = row < p.T;
-        const uint32_t taddr = tmem_base + ((uint32_t)(warp * 32) << 16);
-        float* out = p.logits + (size_t)(valid ? row : 0) * p.E + n0;
-        const bool vec = (p.E & 3) == 0;
-        for (int c = 0; c < ncols; c += 32) {
+        // warp w: rows 32 (w % 4) .. + 31, every fourth 32-column block from w / 4 on
+        for (int u = warp >> 2; u < n_sub * (GN / 32); u += SPLIT_WARPS / 4) {
+          const int i = u / (GN / 32), c = (u % (GN / 32)) * 32;
+          const int row = row0 + i * BM + (warp & 3) * 32 + lane;
+          if (c >= ncols) continue;
+          const uint32_t taddr = tmem_base + ((uint32_t)((warp & 3) * 32) << 16) + c;
           uint32_t acc[32];
-          ptx::tmem_ld32(taddr + c, acc);
-          if (sbs) {   // logits = (hi + mid) + lo: the three column groups are ncols apart
-            uint32_t mid[32], lo[32];
-            ptx::tmem_ld32(taddr + ncols + c, mid);
-            ptx::tmem_ld32(taddr + 2 * ncols + c, lo);
-            ptx::tmem_ld_wait();
+          if (p.apart) {   // logits = (hi + mid) + lo
+            uint32_t other[32];
+            ptx::tmem_ld32(taddr + (i * 3) * GN, acc);
 #pragma unroll
-            for (int v = 0; v < 32; ++v)
-              acc[v] = __float_as_uint(__fadd_rn(__fadd_rn(__uint_as_float(acc[v]), __uint_as_float(mid[v])),
-                                                 __uint_as_float(lo[v])));
-          }
-          ptx::tmem_ld_wait();
-          if (valid) {
-            if (vec) {
-#pragma unroll
-              for (int v = 0; v < 8; ++v)
-                if (n0 + c + v * 4 < p.E)
-                  *reinterpret_cast<uint4*>(out + c + v * 4) =
-                      make_uint4(acc[v * 4], acc[v * 4 + 1], acc[v * 4 + 2], acc[v * 4 + 3]);
-            } else {
+            for (int t = 1; t < 3; ++t) {
+              ptx::tmem_ld32(taddr + (i * 3 + t) * GN, other);
+              ptx::tmem_ld_wait_on(acc);
+              ptx::tmem_ld_wait_on(other);
 #pragma unroll
               for (int v = 0; v < 32; ++v)
-                if (n0 + c + v < p.E) out[c + v] = __uint_as_float(acc[v]);
+                acc[v] = __float_as_uint(__fadd_rn(__uint_as_float(acc[v]), __uint_as_float(other[v])));
             }
+          } else {
+            ptx::tmem_ld32(taddr + i * GN, acc);
+            ptx::tmem_ld_wait_on(acc);
+          }
+          if (row >= p.T) continue;
+          float* out = p.logits + (size_t)row * p.E + n0 + c;
+          if (vec) {
+#pragma unroll
+            for (int v = 0; v < 8; ++v)
+              if (n0 + c + v * 4 < p.E)
+                *reinterpret_cast<uint4*>(out + v * 4) = make_uint4(acc[v * 4], acc[v * 4 + 1], acc[v * 4 + 2], acc[v * 4 + 3]);
+          } else {
+#pragma unroll
+            for (int v = 0; v < 32; ++v)
+              if (n0 + c + v < p.E) out[v] = __uint_as_float(acc[v]);
           }
         }
         ptx::tc_fence_before();
       }
     }
-  } else if (warp == 4) {
-    // ================================ TMA producer ================================
+  } else if (warp == TMA_WARP) {
+    // ================================ TMA producer (rows of x) ================================
     if (lane == 0 && !*abort_flag) {
-      int slab_col[6], slab_split[6];   // slab c = (split c / nslab, 64-column slab c % nslab), hoisted out of the loop
-#pragma unroll
-      for (int c = 0; c < 6; ++c) {
-        slab_col[c] = n0 + (c % nslab) * 64;
-        slab_split[c] = c / nslab;
-      }
       int s = 0, ph = 1;
-      for (int it = 0; it < iters; ++it) {
-        if (!ptx::mbar_wait(empty_bar(s), ph, abort_flag, global_abort)) { timeout(2); break; }
-        const uint32_t sa = smem_base + s * STAGE_BYTES, sb = sa + A_BYTES;
-        const int kb = sbs ? it : it / 3, split0 = sbs ? 0 : it - kb * 3;
-        ptx::mbar_arrive_expect_tx(full_bar(s), A_BYTES + bslabs * 8192);
-        ptx::tma_load_2d(sa, &map_x, full_bar(s), kb * BK, row0);
-#pragma unroll
-        for (int c = 0; c < 6; ++c)
-          if (c < bslabs) ptx::tma_load_3d(sb + c * 8192, &map_w, full_bar(s), slab_col[c], kb * BK, split0 + slab_split[c]);
-        if (++s == NSTAGE) { s = 0; ph ^= 1; }
+      for (int kb = 0; kb < p.KB; ++kb) {
+        if (!ptx::mbar_wait(empty_bar(s), ph, abort_flag, global_abort)) { timeout(3); break; }
+        ptx::mbar_arrive_expect_tx(full_bar(s), n_sub * p.a_bytes);
+        for (int i = 0; i < n_sub; ++i)
+          ptx::tma_load_2d(smem_base + s * stage_bytes + B_BYTES + i * p.a_bytes, &map_x, full_bar(s), kb * BK, row0 + i * BM);
+        if (++s == n_stages) { s = 0; ph ^= 1; }
       }
     }
   } else {
     // ================================ UMMA issuer ================================
-    if (lane == 0 && !*abort_flag) {
-      const uint64_t a_base = desc_base(16, 1024);
-      const uint64_t b_base = desc_base(BK * 128, 1024);
-      auto idesc_n = [](int n) {
+    if (!*abort_flag) {
+      const bool elected = ptx::elect_one();
+      const uint32_t base = __shfl_sync(0xFFFFFFFFu, smem_base, 0), tmem = __shfl_sync(0xFFFFFFFFu, tmem_base, 0);
+      const uint64_t a_desc = desc_at(desc_base(16, 1024), base + B_BYTES), b_desc = desc_at(desc_base(BK * 128, 1024), base);
+      auto idesc = [](int n) {
         return (1u << 4) | (1u << 7) | (1u << 10) | (1u << 16) | ((uint32_t)(n >> 3) << 17) | ((uint32_t)(BM >> 4) << 24);
       };
-      const int n_first = min(bslabs, 4) * 64, n_second = (bslabs - min(bslabs, 4)) * 64;   // columns per UMMA
+      const uint32_t stage16 = stage_bytes >> 4, a16 = p.a_bytes >> 4;
       bool ok = true;
       int s = 0, ph = 0;
-      for (int it = 0; it < iters; ++it) {
-        if (!ptx::mbar_wait(full_bar(s), ph, abort_flag, global_abort)) { timeout(3); ok = false; break; }
+      for (int kb = 0; kb < p.KB; ++kb) {
+        if (!ptx::mbar_wait(full_bar(s), ph, abort_flag, global_abort)) { timeout(4); ok = false; break; }
         ptx::tc_fence_after();
-        const uint32_t sa = smem_base + s * STAGE_BYTES, sb = sa + A_BYTES;
-        const uint64_t ad = desc_at(a_base, sa), bd = desc_at(b_base, sb);
+        if (elected) {
+          for (int i = 0; i < n_sub; ++i) {
+            const uint64_t ad = a_desc + (s * stage16 + i * a16), bd = b_desc + s * stage16;
+            if (p.apart) {   // the terms as one wide B
+              constexpr int N1 = 3 * GN < 256 ? 3 * GN : 256, N2 = 3 * GN - N1;
 #pragma unroll
-        for (int k = 0; k < BK / 16; ++k) {
-          ptx::umma_bf16(tmem_base, ad + (uint64_t)(k * 2), bd + (uint64_t)(k * 128), idesc_n(n_first), (it | k) != 0);
-          if (n_second > 0)   // slabs 4, 5 start 4 * 8 KiB into the B tile and 256 columns into the accumulator
-            ptx::umma_bf16(tmem_base + 256, ad + (uint64_t)(k * 2), bd + (uint64_t)(2048 + k * 128), idesc_n(n_second),
-                           (it | k) != 0);
+              for (int k = 0; k < BK / 16; ++k) {
+                const uint32_t d = tmem + i * 3 * GN;
+                ptx::umma_bf16(d, ad + (uint64_t)(k * 2), bd + (uint64_t)(k * 128), idesc(N1), (kb | k) > 0);
+                if (N2 > 0)
+                  ptx::umma_bf16(d + N1, ad + (uint64_t)(k * 2), bd + (uint64_t)(N1 / 64 * 512 + k * 128), idesc(N2), (kb | k) > 0);
+              }
+            } else if (GN >= 64) {
+#pragma unroll
+              for (int t = 0; t < 3; ++t)
+#pragma unroll
+                for (int k = 0; k < BK / 16; ++k)
+                  ptx::umma_bf16(tmem + i * GN, ad + (uint64_t)(k * 2), bd + (uint64_t)(t * (GN / 64) * 512 + k * 128), idesc(GN),
+                                 (kb | k | t) > 0);
+            }
+          }
+          ptx::umma_commit(empty_bar(s));
         }
-        ptx::umma_commit(empty_bar(s));
-        if (++s == NSTAGE) { s = 0; ph ^= 1; }
+        if (++s == n_stages) { s = 0; ph ^= 1; }
       }
-      if (ok) ptx::umma_commit(done_bar);
+      if (ok && elected) ptx::umma_commit(done_bar);
     }
   }
 
@@ -213,58 +288,73 @@ gate_umma_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constan
     for (int i = 0; i < 64; ++i) __nanosleep(1000);   // abort path: let bulk copies in flight land
   }
   __syncthreads();
-  if (warp == 5) {
+  if (warp == MMA_WARP) {
     ptx::tc_fence_after();
     ptx::tmem_dealloc(tmem_base, 512);
   }
 }
 
-}  // namespace
+// Tile width and row tiles per task: the cheapest by a model in microseconds, fitted to this kernel: time of a k-block by
+// width and row tiles, 148 thread blocks at a time.  (32: apart only, a running sum needs whole slabs per term.)
+struct GatePlan { int gn, m_sub; };
+GatePlan plan_gate(int T, int E, bool apart) {
+  static const struct { int gn, m_sub; double kb_us[2]; } forms[] = {   // running sum, apart
+      {32, 1, {1e9, 0.3}}, {64, 1, {0.5, 0.4}}, {64, 2, {0.85, 0.6}}, {128, 1, {0.8, 0.8}}, {128, 2, {1.4, 1e9}}};
+  GatePlan best{};
+  double best_us = 1e30;
+  for (const auto& f : forms) {
+    const long long tiles = (long long)((T + f.m_sub * BM - 1) / (f.m_sub * BM)) * ((E + f.gn - 1) / f.gn);
+    const double us = (double)((tiles + 147) / 148) * f.kb_us[apart ? 1 : 0];
+    if (us < best_us) { best_us = us; best = GatePlan{f.gn, f.m_sub}; }
+  }
+  return best;
+}
 
-size_t gate_split_bytes(int d, int E) { return (size_t)3 * d * ((E + 63) & ~63) * 2; }
-
-cudaError_t launch_gate_logits(const Shape& s, const void* x, const float* w_gate, float* logits, void* wsplit,
-                               int32_t* status, cudaStream_t st) {
-  if (s.T == 0) return cudaSuccess;
+template <int GN, int GROUPS>
+cudaError_t launch_width(const GateParams& p, int grid, const CUtensorMap& m_x, cudaStream_t st) {
   // per device; several host threads may get here at once: setting the attribute twice is harmless
   static std::atomic<bool> attr_set[MAX_DEVICES];
   const int dev = current_device();
   if (!attr_set[dev].load(std::memory_order_acquire)) {
-    cudaError_t e = cudaFuncSetAttribute(gate_umma_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_BYTES);
+    cudaError_t e = cudaFuncSetAttribute(gate_umma_kernel<GN, GROUPS>, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_BYTES);
     if (e != cudaSuccess) return e;
     attr_set[dev].store(true, std::memory_order_release);
   }
-  const int Epad = (s.E + 63) & ~63;
-  CUtensorMap m_x, m_w;
+  return launch_pdl(gate_umma_kernel<GN, GROUPS>, grid, THREADS, SMEM_BYTES, st, m_x, p);
+}
+
+}  // namespace
+
+cudaError_t launch_gate_logits(const Shape& s, const void* x, const float* w_gate, float* logits, int32_t* status,
+                               cudaStream_t st) {
+  if (s.T == 0) return cudaSuccess;
+  const bool apart = s.E <= 128;
+  const GatePlan plan = plan_gate(s.T, s.E, apart);
+  const int a_rows = s.T < BM ? (s.T + 7) & ~7 : BM;
+  CUtensorMap m_x;
   {
     cuuint64_t dims[2] = {(cuuint64_t)s.d, (cuuint64_t)s.T};
     cuuint64_t strides[1] = {(cuuint64_t)s.d * 2};
-    cuuint32_t box[2] = {BK, BM};
+    cuuint32_t box[2] = {BK, (cuuint32_t)a_rows};
     if (!ffn::encode_tiled(&m_x, false, 2, x, dims, strides, box)) return cudaErrorInvalidValue;
   }
-  {
-    cuuint64_t dims[3] = {(cuuint64_t)Epad, (cuuint64_t)s.d, 3};
-    cuuint64_t strides[2] = {(cuuint64_t)Epad * 2, (cuuint64_t)Epad * s.d * 2};
-    cuuint32_t box[3] = {64, BK, 1};
-    if (!ffn::encode_tiled(&m_w, false, 3, wsplit, dims, strides, box)) return cudaErrorInvalidValue;
-  }
   ProfileScope prof(KID_GATE, st);
-  const size_t n = (size_t)s.d * Epad;
-  int sb = (int)((n + 255) / 256);
-  if (sb > sm_count() * 8) sb = sm_count() * 8;
-  cudaError_t err = launch_pdl(split_gate_kernel, sb, 256, 0, st, w_gate, static_cast<__nv_bfloat16*>(wsplit), s.d, s.E,
-                               Epad);
-  if (err != cudaSuccess) return err;
   GateParams p;
+  p.w = w_gate;
   p.logits = logits;
   p.T = s.T;
+  p.d = s.d;
   p.E = s.E;
   p.KB = (s.d + BK - 1) / BK;
-  p.n_tiles = (s.E + UMMA_N - 1) / UMMA_N;
-  p.side_by_side = s.E <= 128 ? 1 : 0;
+  p.n_tiles = (s.E + plan.gn - 1) / plan.gn;
+  p.m_sub = plan.m_sub;
+  p.a_bytes = a_rows * BK * 2;
+  p.apart = apart ? 1 : 0;
   p.status = status;
-  const int grid = ((s.T + BM - 1) / BM) * p.n_tiles;
-  return launch_pdl(gate_umma_kernel, grid, THREADS, SMEM_BYTES, st, m_x, m_w, p);
+  const int grid = ((s.T + p.m_sub * BM - 1) / (p.m_sub * BM)) * p.n_tiles;
+  if (plan.gn == 32) return launch_width<32, 4>(p, grid, m_x, st);
+  if (plan.gn == 64) return launch_width<64, 2>(p, grid, m_x, st);
+  return launch_width<128, 2>(p, grid, m_x, st);
 }
 
 }  // namespace tcmoe
