@@ -588,10 +588,12 @@ int moe_gate_backward(const moe_shape_t* shape, const float* logits, const float
   a.dx = dx;
   a.dw_gate = dw_gate;
   a.poff = at<int32_t>(ws, p.poff);
+  a.mt_prefix = at<int32_t>(ws, p.mt_prefix);
   a.pair_prow = at<int32_t>(ws, p.pair_prow);
   a.xs = at<void>(ws, p.xs);
   a.h = at<void>(ws, p.h);
   a.dh = at<void>(ws, p.dh);
+  a.part = at<float>(ws, p.dos);   // dO is not needed any more: (P / 128 + E) d floats fit its (P + 64 E) d bf16
   a.g_row = at<float>(ws, p.g_row);
   a.dkey = at<float>(ws, p.dkey);
   a.wgt = at<float>(ws, p.wgt);

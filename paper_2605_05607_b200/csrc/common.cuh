@@ -132,10 +132,11 @@ struct GateBwdArgs {
   void* dx;                         // [T, d] bf16, in / out: the gate path is added
   float* dw_gate;                   // [d, E] fp32 out
   // left behind by launch_layer_backward
-  const int32_t *poff, *pair_prow;
+  const int32_t *poff, *mt_prefix, *pair_prow;
   const void *xs, *h, *dh;
   // scratch
   float *g_row, *dkey, *wgt;        // [bwd_row_capacity], [T * k], [E, d]
+  float* part;                      // [128-row tiles, d]: partial sums of dw_gate
 };
 cudaError_t launch_gate_backward(const Shape& s, const GateBwdArgs& a, cudaStream_t st);
 // ffn.cu

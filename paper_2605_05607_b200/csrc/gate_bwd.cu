@@ -14,8 +14,8 @@
 // so dL/dw costs one pass over two [rows, f] buffers and no GEMM.  dw_gate is a weighted sum of each expert's rows of
 // xs (also still in the workspace), dx gets k rows of the transposed gate weight per token.
 //
-// Sequence (one stream): row dots -> per-token key gradients -> dw_gate (one block per expert and column slab, rows in
-// ascending order: deterministic) -> transpose of w_gate -> dx update.
+// Sequence (one stream): row dots -> per-token key gradients -> partial sums of dw_gate per 128-row tile -> dw_gate (tiles in
+// ascending order: deterministic, no atomics) and the transpose of w_gate -> dx update.
 #include "common.cuh"
 
 #include <cuda_bf16.h>
@@ -47,6 +47,7 @@ __global__ void __launch_bounds__(256) gate_rowdot_kernel(const uint4* __restric
     const uint4* hr = h + (size_t)r * vec_per_row;
     const uint4* dr = dh + (size_t)r * vec_per_row;
     float s = 0.f;
+#pragma unroll 4
     for (int v = lane; v < vec_per_row; v += 32) s += dot8(__ldcs(hr + v), __ldcs(dr + v));
 #pragma unroll
     for (int off = 16; off > 0; off >>= 1) s += __shfl_xor_sync(0xFFFFFFFFu, s, off);
@@ -89,53 +90,75 @@ __global__ void __launch_bounds__(256) gate_route_bwd_kernel(const int32_t* __re
   }
 }
 
-// dw_gate[c, e] = sum over the rows r of expert e (ascending) of dkey_row[r] * xs[r, c].  Block: 256 threads x 8
-// columns; grid (column slabs, experts).
-__global__ void __launch_bounds__(256) gate_dw_kernel(const uint4* __restrict__ xs, const float* __restrict__ dkey_row,
-                                                      const int32_t* __restrict__ poff,
-                                                      const int32_t* __restrict__ expert_counts,
-                                                      float* __restrict__ dw_gate, int E, int d) {
+// part[m, c] = sum over the rows r of 128-row tile m (ascending) of dkey_row[r] * xs[r, c]; tiles are those of the forward's
+// row prefix, so a tile belongs to one expert.  Block: 128 threads x 8 columns.  Bound by the read of xs; one block per expert
+// and column slab, as this was first, left a popular expert's thousands of rows to a single serial loop (skewed 128-expert
+// layer, T = 3001: 721 us, now 42; T = 8192, d = 4096, top-8 without skew: 174, now 108; d = 2048, 64 experts: 290, now 50).
+constexpr int DW_THREADS = 128, DW_ROWS = 128;
+__global__ void __launch_bounds__(DW_THREADS) gate_dw_kernel(const uint4* __restrict__ xs, const float* __restrict__ dkey_row,
+                                                             const int32_t* __restrict__ poff,
+                                                             const int32_t* __restrict__ expert_counts,
+                                                             const int32_t* __restrict__ mt_prefix, float* __restrict__ part,
+                                                             int E, int d) {
   grid_dependency_sync();
-  const int e = blockIdx.y;
-  const int v = blockIdx.x * blockDim.x + threadIdx.x;   // uint4 index inside the row
+  const int v = blockIdx.x * DW_THREADS + threadIdx.x;   // uint4 index inside the row
   const int vec_per_row = d >> 3;
   if (v >= vec_per_row) return;
-  const int r0 = __ldg(poff + e), n = __ldg(expert_counts + e);
-  float acc[8];
-#pragma unroll
-  for (int q = 0; q < 8; ++q) acc[q] = 0.f;
-  const uint4* col = xs + (size_t)r0 * vec_per_row + v;
-#pragma unroll 4
-  for (int i = 0; i < n; ++i) {
-    const float g = __ldg(dkey_row + r0 + i);
-    const uint4 xv = __ldcs(col + (size_t)i * vec_per_row);
-    const __nv_bfloat162* px = reinterpret_cast<const __nv_bfloat162*>(&xv);
-#pragma unroll
-    for (int q = 0; q < 4; ++q) {
-      const float2 f = __bfloat1622float2(px[q]);
-      acc[2 * q] = fmaf(g, f.x, acc[2 * q]);
-      acc[2 * q + 1] = fmaf(g, f.y, acc[2 * q + 1]);
+  const int tiles = __ldg(mt_prefix + E);
+  for (int m = blockIdx.y; m < tiles; m += gridDim.y) {
+    int lo = 0, hi = E;   // mt_prefix[lo] <= m < mt_prefix[hi]
+    while (hi - lo > 1) {
+      const int mid = (lo + hi) >> 1;
+      if (__ldg(mt_prefix + mid) <= m) lo = mid; else hi = mid;
     }
-  }
+    const int first = (m - __ldg(mt_prefix + lo)) * DW_ROWS;
+    const int r0 = __ldg(poff + lo) + first, n = min(DW_ROWS, __ldg(expert_counts + lo) - first);
+    float acc[8];
 #pragma unroll
-  for (int q = 0; q < 8; ++q) dw_gate[(size_t)(v * 8 + q) * E + e] = acc[q];
+    for (int q = 0; q < 8; ++q) acc[q] = 0.f;
+    const uint4* col = xs + (size_t)r0 * vec_per_row + v;
+#pragma unroll 8
+    for (int i = 0; i < n; ++i) {
+      const float g = __ldg(dkey_row + r0 + i);
+      const uint4 xv = __ldcs(col + (size_t)i * vec_per_row);
+      const __nv_bfloat162* px = reinterpret_cast<const __nv_bfloat162*>(&xv);
+#pragma unroll
+      for (int q = 0; q < 4; ++q) {
+        const float2 f = __bfloat1622float2(px[q]);
+        acc[2 * q] = fmaf(g, f.x, acc[2 * q]);
+        acc[2 * q + 1] = fmaf(g, f.y, acc[2 * q + 1]);
+      }
+    }
+    float4* out = reinterpret_cast<float4*>(part + (size_t)m * d + v * 8);
+    out[0] = make_float4(acc[0], acc[1], acc[2], acc[3]);
+    out[1] = make_float4(acc[4], acc[5], acc[6], acc[7]);
+  }
 }
 
-// wgt[e, c] = w_gate[c, e]: 32 x 32 tiles through shared memory
-__global__ void __launch_bounds__(256) gate_transpose_kernel(const float* __restrict__ w_gate, float* __restrict__ wgt,
-                                                             int d, int E) {
+// dw_gate[c, e] = sum over the tiles of expert e (ascending) of part[m, c]; wgt[e, c] = w_gate[c, e].  Both are transposes
+// between [., d] and [d, E], 32 x 32 through shared memory.
+__global__ void __launch_bounds__(256) gate_finish_kernel(const float* __restrict__ part, const int32_t* __restrict__ mt_prefix,
+                                                          float* __restrict__ dw_gate, const float* __restrict__ w_gate,
+                                                          float* __restrict__ wgt, int d, int E) {
   grid_dependency_sync();
-  __shared__ float tile[32][33];
+  __shared__ float tile[2][32][33];
   const int c0 = blockIdx.x * 32, e0 = blockIdx.y * 32;
   const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;   // 8 rows per pass
   for (int i = ty; i < 32; i += 8) {
     const int c = c0 + i, e = e0 + tx;
-    tile[i][tx] = (c < d && e < E) ? __ldg(w_gate + (size_t)c * E + e) : 0.f;
+    tile[0][i][tx] = (c < d && e < E) ? __ldg(w_gate + (size_t)c * E + e) : 0.f;
+    float sum = 0.f;
+    if (e0 + i < E && c0 + tx < d) {
+      const int m1 = __ldg(mt_prefix + e0 + i + 1);
+#pragma unroll 8
+      for (int m = __ldg(mt_prefix + e0 + i); m < m1; ++m) sum += __ldcs(part + (size_t)m * d + c0 + tx);
+    }
+    tile[1][i][tx] = sum;
   }
   __syncthreads();
   for (int i = ty; i < 32; i += 8) {
-    const int e = e0 + i, c = c0 + tx;
-    if (e < E && c < d) wgt[(size_t)e * d + c] = tile[tx][i];
+    if (e0 + i < E && c0 + tx < d) wgt[(size_t)(e0 + i) * d + c0 + tx] = tile[0][tx][i];
+    if (c0 + i < d && e0 + tx < E) dw_gate[(size_t)(c0 + i) * E + e0 + tx] = tile[1][tx][i];
   }
 }
 
@@ -194,11 +217,14 @@ cudaError_t launch_gate_backward(const Shape& s, const GateBwdArgs& a, cudaStrea
                         a.logits, a.bias, (long long)a.bias_stride, a.g_row, a.dkey, s.T, s.E, s.k,
                         s.score_fn == 1 ? 1 : 0, n_rows)) != cudaSuccess)
     return err;
-  if ((err = launch_pdl(gate_dw_kernel, dim3((s.d / 8 + 255) / 256, s.E), 256, 0, st, static_cast<const uint4*>(a.xs),
-                        static_cast<const float*>(a.g_row), a.poff, a.expert_counts, a.dw_gate, s.E, s.d)) != cudaSuccess)
+  long long tiles = (long long)s.T * s.k / DW_ROWS + s.E;   // at most; the count is on the device
+  if (tiles > 16384) tiles = 16384;
+  if ((err = launch_pdl(gate_dw_kernel, dim3((s.d / 8 + DW_THREADS - 1) / DW_THREADS, (unsigned)tiles), DW_THREADS, 0, st,
+                        static_cast<const uint4*>(a.xs), static_cast<const float*>(a.g_row), a.poff, a.expert_counts,
+                        a.mt_prefix, a.part, s.E, s.d)) != cudaSuccess)
     return err;
-  if ((err = launch_pdl(gate_transpose_kernel, dim3((s.d + 31) / 32, (s.E + 31) / 32), 256, 0, st, a.w_gate, a.wgt, s.d,
-                        s.E)) != cudaSuccess)
+  if ((err = launch_pdl(gate_finish_kernel, dim3((s.d + 31) / 32, (s.E + 31) / 32), 256, 0, st,
+                        static_cast<const float*>(a.part), a.mt_prefix, a.dw_gate, a.w_gate, a.wgt, s.d, s.E)) != cudaSuccess)
     return err;
   blocks = (s.T + 7) / 8;
   if (blocks > cap) blocks = cap;

@@ -281,3 +281,26 @@ def test_backward_on_a_sparse_routing_table():
         for e, gr in grads.items():
             ref[e] = gr[pos]
         close(O.bf16_to_f64(H.bf16_host(dw[n])), ref, f"sparse d{n}")
+
+
+@pytest.mark.parametrize("rows", [127, 128, 129, 385])
+def test_gate_weight_gradient_tiles(rows):
+    """dw_gate is summed per 128-row tile of an expert: one expert with `rows` rows, one with none, one with the rest."""
+    cfg = synth.MoEConfig("tiles", T=512, d=1032, f=64, E=4, k=2, G=2, seed=rows)
+    bw = Backward(cfg)
+    bias = torch.zeros(cfg.T, cfg.E, device="cuda")
+    bias[:, 0] = 20.0                   # every token takes expert 0
+    bias[:rows, 1] = 20.0               # `rows` tokens take expert 1, the others expert 3; nobody expert 2
+    bias[rows:, 3] = 20.0
+    bw.run.t["bias"] = bias
+    bw.run.route()
+    bw.run.dispatch()
+    bw()
+    dwg = _gate_backward(bw).cpu().numpy().astype(np.float64)
+    run = bw.run
+    ref, _, _, _ = O.gate_backward(H.bf16_host(run.t["x"]), run.t["w_gate"].cpu().numpy(), run.host_bias(), run.host_idx(),
+                                   cfg.score_fn, *(H.bf16_host(run.t[n]) for n in ("w1", "w3", "w2")),
+                                   O.bf16_to_f64(H.bf16_host(bw.dy))[: cfg.T])
+    assert np.array_equal(np.bincount(run.host_idx().reshape(-1), minlength=4), [512, rows, 0, 512 - rows])
+    assert not dwg[:, 2].any()
+    close(dwg, ref, "dw_gate")
