@@ -100,6 +100,7 @@ cudaError_t launch_dispatch(const Shape& s, const void* x, const Layout& L, void
 cudaError_t launch_permute_rows(const Shape& s, const void* src, int src_rows, const int32_t* gather_idx,
                                 int gather_div, const int32_t* expert_offsets, void* xs, int32_t* status,
                                 cudaStream_t st);
+int row_parts(int T, int vec_per_row);   // warps that share a token's row in the row kernels, by the number of tokens
 cudaError_t launch_round_rows(const Shape& s, const float* acc, void* y, cudaStream_t st);
 cudaError_t launch_combine(const Shape& s, const void* o, const Layout& L, const int32_t* topk_idx,
                            const float* topk_w, void* pg, void* y, int32_t* status, cudaStream_t st);

@@ -17,61 +17,97 @@
 namespace tcmoe {
 namespace {
 
-// thread per token: walk the k slots, append each to the list of its (token, group) row
+// Thread per (token, group): the row n = (t, g) takes the token's slots that live in the group, in slot order, then -1 / 0.
+// The rows behind the last dispatched one are filled as unused too.
 __global__ void __launch_bounds__(256) ep_pack_kernel(const int32_t* __restrict__ topk_idx,
                                                       const float* __restrict__ topk_w,
                                                       const int32_t* __restrict__ al,
                                                       const int32_t* __restrict__ group_offsets,
                                                       int32_t* __restrict__ send_idx, float* __restrict__ send_w, int T,
-                                                      int E, int k, int m, int kk) {
+                                                      int E, int k, int G, int m, int kk, int cap_rows) {
   grid_dependency_sync();
-  const int t = blockIdx.x * blockDim.x + threadIdx.x;
-  if (t >= T) return;
-  for (int j = 0; j < k; ++j) {
-    const int e = __ldg(topk_idx + (size_t)t * k + j);
-    if (e < 0 || e >= E) continue;
-    const int g = e / m;
-    int pos = 0;   // slots of this token before j that live in the same group
-    for (int i = 0; i < j; ++i) {
-      const int ei = __ldg(topk_idx + (size_t)t * k + i);
-      if (ei >= 0 && ei < E && ei / m == g) ++pos;
+  const long long first = (long long)blockIdx.x * blockDim.x + threadIdx.x, stride = (long long)gridDim.x * blockDim.x;
+  for (long long i = first; i < (long long)T * G; i += stride) {
+    const int g = (int)(i / T), t = (int)(i % T);   // consecutive threads: consecutive tokens, consecutive rows of the group
+    const int a = __ldg(al + (size_t)g * T + t);
+    if (a < 0) continue;
+    const size_t n = (size_t)__ldg(group_offsets + g) + a;
+    int pos = 0;
+    for (int j = 0; j < k; ++j) {
+      const int e = __ldg(topk_idx + (size_t)t * k + j);
+      if (e < 0 || e >= E || e / m != g) continue;
+      send_idx[n * kk + pos] = e - g * m;
+      send_w[n * kk + pos] = __ldg(topk_w + (size_t)t * k + j);
+      ++pos;
     }
-    const size_t n = (size_t)__ldg(group_offsets + g) + __ldg(al + (size_t)g * T + t);
-    send_idx[n * kk + pos] = e - g * m;
-    send_w[n * kk + pos] = __ldg(topk_w + (size_t)t * k + j);
+    for (; pos < kk; ++pos) {
+      send_idx[n * kk + pos] = -1;
+      send_w[n * kk + pos] = 0.f;
+    }
+  }
+  for (long long i = (long long)__ldg(group_offsets + G) * kk + first; i < (long long)cap_rows * kk; i += stride) {
+    send_idx[i] = -1;
+    send_w[i] = 0.f;
   }
 }
 
-// warp per token: fp32 sum over the groups, ascending g, 8 bf16 per lane per step
+// Warp per (token, column part): fp32 sum over the groups, ascending g.  Lane g finds the row of group g once (32 groups at a
+// time); four rows are in flight per lane.  Bound by the read of the returned rows; one warp per token that looked up every
+// group for every 16-byte column ran at a fifth of the copy bandwidth (2050 tokens of d = 4096, 8 groups: 75 us).
 __global__ void __launch_bounds__(256) ep_finish_kernel(const uint4* __restrict__ back, uint4* __restrict__ y,
                                                         const int32_t* __restrict__ al,
                                                         const int32_t* __restrict__ group_offsets, int T, int G,
-                                                        int vec_per_row) {
+                                                        int vec_per_row, int parts, int vec_per_part) {
   grid_dependency_sync();
   const int lane = threadIdx.x & 31;
   const int wpb = blockDim.x >> 5;
-  for (int t = blockIdx.x * wpb + (threadIdx.x >> 5); t < T; t += gridDim.x * wpb) {
-    for (int v = lane; v < vec_per_row; v += 32) {
+  const long long units = (long long)T * parts;
+  for (long long w = (long long)blockIdx.x * wpb + (threadIdx.x >> 5); w < units; w += (long long)gridDim.x * wpb) {
+    const int t = (int)(w / parts), part = (int)(w % parts);
+    const int v_end = min(vec_per_row, (part + 1) * vec_per_part);
+    for (int v0 = part * vec_per_part; v0 < v_end; v0 += 32) {   // whole warps: the row numbers are shuffled
+      const int v = v0 + lane;
       float acc[8];
 #pragma unroll
       for (int q = 0; q < 8; ++q) acc[q] = 0.f;
-      for (int g = 0; g < G; ++g) {
-        const int a = __ldg(al + (size_t)g * T + t);
-        if (a < 0) continue;
-        const uint4 raw = __ldcs(back + ((size_t)__ldg(group_offsets + g) + a) * vec_per_row + v);
-        const __nv_bfloat162* p = reinterpret_cast<const __nv_bfloat162*>(&raw);
+      for (int g0 = 0; g0 < G; g0 += 32) {
+        int row = -1;
+        if (g0 + lane < G) {
+          const int a = __ldg(al + (size_t)(g0 + lane) * T + t);
+          if (a >= 0) row = __ldg(group_offsets + g0 + lane) + a;
+        }
+        unsigned live = __ballot_sync(0xFFFFFFFFu, row >= 0);
+        while (live) {
+          uint4 buf[4];
+          int n = 0;
 #pragma unroll
-        for (int q = 0; q < 4; ++q) {
-          const float2 f = __bfloat1622float2(p[q]);
-          acc[2 * q] += f.x;
-          acc[2 * q + 1] += f.y;
+          for (int q = 0; q < 4; ++q)
+            if (live) {
+              const int r = __shfl_sync(0xFFFFFFFFu, row, __ffs(live) - 1);
+              live &= live - 1;
+              n = q + 1;
+              if (v < v_end) buf[q] = __ldcs(back + (size_t)r * vec_per_row + v);
+            }
+#pragma unroll
+          for (int q = 0; q < 4; ++q)
+            if (q < n && v < v_end) {
+              const __nv_bfloat162* p = reinterpret_cast<const __nv_bfloat162*>(&buf[q]);
+#pragma unroll
+              for (int i = 0; i < 4; ++i) {
+                const float2 f = __bfloat1622float2(p[i]);
+                acc[2 * i] += f.x;
+                acc[2 * i + 1] += f.y;
+              }
+            }
         }
       }
-      uint4 out;
-      __nv_bfloat162* o = reinterpret_cast<__nv_bfloat162*>(&out);
+      if (v < v_end) {
+        uint4 out;
+        __nv_bfloat162* o = reinterpret_cast<__nv_bfloat162*>(&out);
 #pragma unroll
-      for (int q = 0; q < 4; ++q) o[q] = __floats2bfloat162_rn(acc[2 * q], acc[2 * q + 1]);
-      y[(size_t)t * vec_per_row + v] = out;
+        for (int q = 0; q < 4; ++q) o[q] = __floats2bfloat162_rn(acc[2 * q], acc[2 * q + 1]);
+        y[(size_t)t * vec_per_row + v] = out;
+      }
     }
   }
 }
@@ -82,21 +118,22 @@ cudaError_t launch_ep_pack(const Shape& s, const int32_t* topk_idx, const float*
                            int32_t* send_idx, float* send_w, cudaStream_t st) {
   if (s.T == 0) return cudaSuccess;
   const int m = s.E / s.G, kk = s.k < m ? s.k : m;
-  const size_t cap = (size_t)s.T * (s.k < s.G ? s.k : s.G) * kk;   // dispatched-row capacity x list length
-  cudaError_t err;
-  if ((err = cudaMemsetAsync(send_idx, 0xFF, cap * sizeof(int32_t), st)) != cudaSuccess) return err;   // -1: unused slot
-  if ((err = cudaMemsetAsync(send_w, 0, cap * sizeof(float), st)) != cudaSuccess) return err;
-  return launch_pdl(ep_pack_kernel, (s.T + 255) / 256, 256, 0, st, topk_idx, topk_w, L.al, L.group_offsets, send_idx,
-                    send_w, s.T, s.E, s.k, m, kk);
+  const int cap_rows = s.T * (s.k < s.G ? s.k : s.G);   // dispatched-row capacity
+  long long blocks = ((long long)s.T * s.G + 255) / 256;
+  if (blocks > 4096) blocks = 4096;
+  return launch_pdl(ep_pack_kernel, (unsigned)blocks, 256, 0, st, topk_idx, topk_w, L.al, L.group_offsets, send_idx,
+                    send_w, s.T, s.E, s.k, s.G, m, kk, cap_rows);
 }
 
 cudaError_t launch_ep_finish(const Shape& s, const void* back, const Layout& L, void* y, cudaStream_t st) {
   if (s.T == 0) return cudaSuccess;
-  int blocks = (s.T + 7) / 8;
-  const int cap = sm_count() * 8;
+  const int vec = s.d / 8, parts = row_parts(s.T, vec);
+  const int vec_per_part = ((vec + parts - 1) / parts + 31) & ~31;   // whole warp-strides per part
+  long long blocks = ((long long)s.T * parts + 7) / 8;
+  const long long cap = (long long)sm_count() * 8;
   if (blocks > cap) blocks = cap;
-  return launch_pdl(ep_finish_kernel, blocks, 256, 0, st, static_cast<const uint4*>(back), static_cast<uint4*>(y), L.al,
-                    L.group_offsets, s.T, s.G, s.d / 8);
+  return launch_pdl(ep_finish_kernel, (unsigned)blocks, 256, 0, st, static_cast<const uint4*>(back), static_cast<uint4*>(y),
+                    L.al, L.group_offsets, s.T, s.G, vec, parts, vec_per_part);
 }
 
 }  // namespace tcmoe

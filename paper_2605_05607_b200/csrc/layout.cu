@@ -228,8 +228,6 @@ __global__ void __launch_bounds__(256) dispatch_kernel(const uint4* __restrict__
   }
 }
 
-static int row_parts(int T, int vec_per_row);
-
 cudaError_t launch_dispatch(const Shape& s, const void* x, const Layout& L, void* xg, cudaStream_t st) {
   if (s.T == 0) return cudaSuccess;
   const int vec = s.d / 8;
@@ -315,7 +313,7 @@ __global__ void __launch_bounds__(256, 3) combine_kernel(const CombineArgs c, in
 }
 
 // parts of a row so that about 32 warps per SM exist even for small batches (at most 8, at least 4 vectors per lane)
-static int row_parts(int T, int vec_per_row) {
+int row_parts(int T, int vec_per_row) {
   int parts = 1;
   while (parts < 8 && (long long)T * parts < 32ll * sm_count() * 2 && vec_per_row / (parts * 2) >= 128) parts *= 2;
   return parts;

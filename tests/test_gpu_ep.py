@@ -102,3 +102,38 @@ def test_forward_over_nccl_with_one_rank():
         assert mx <= 1e-2 and mean <= 3e-3, (mx, mean)
     finally:
         dist.destroy_process_group()
+
+
+@pytest.mark.parametrize("T,d,E,k,G", [(1, 8, 4, 1, 4), (33, 264, 80, 6, 40), (300, 1032, 64, 16, 64), (2051, 2056, 8, 2, 2)])
+def test_pack_and_finish_edges(T, d, E, k, G):
+    """Target lists (unused entries and the rows behind the last dispatched one included) and the final reduction, for more
+    than 32 groups, rows that no warp stride divides and rows shared by several warps, against plain tensor operations."""
+    g = torch.Generator(device="cuda").manual_seed(T)
+    shape = B.MoEShape(T, d, 64, E, k, G, 0, 0)
+    idx = torch.rand(T, E, generator=g, device="cuda").topk(k, dim=1).indices.to(torch.int32).contiguous()
+    w = torch.rand(T, k, generator=g, device="cuda")
+    lay, ws = B.alloc_layout(shape), B.alloc_workspace(shape)
+    B.moe_dispatch(shape, None, idx, lay, None, ws)
+    m, cap = E // G, T * min(k, G)
+    kk = min(k, m)
+    send_idx = torch.full((cap, kk), 99, dtype=torch.int32, device="cuda")
+    send_w = torch.full((cap, kk), 99.0, device="cuda")
+    B.moe_ep_pack(shape, idx, w, lay, send_idx, send_w)
+    n = int(lay.group_offsets[G])
+    al, off = lay.al[: G * T].view(G, T).cpu(), lay.group_offsets.cpu()
+    ref_idx, ref_w = torch.full((cap, kk), -1, dtype=torch.int32), torch.zeros(cap, kk)
+    for t in range(T):
+        used = {}
+        for j, e in enumerate(idx[t].tolist()):
+            row, pos = int(off[e // m] + al[e // m, t]), used.get(e // m, 0)
+            ref_idx[row, pos], ref_w[row, pos] = e % m, w[t, j]
+            used[e // m] = pos + 1
+    assert torch.equal(send_idx.cpu(), ref_idx) and torch.equal(send_w.cpu(), ref_w)
+    back = torch.randn(n, d, generator=g, device="cuda").to(torch.bfloat16)
+    y = torch.full((T, d), 7.0, dtype=torch.bfloat16, device="cuda")
+    B.moe_ep_finish(shape, back, lay, y)
+    acc = torch.zeros(T, d, device="cuda")                      # the same fp32 additions in the same order
+    for gi in range(G):
+        a = lay.al[gi * T:(gi + 1) * T]
+        acc[a >= 0] += back[(off[gi] + a[a >= 0]).long()].float()
+    assert torch.equal(y, acc.to(torch.bfloat16))
