@@ -36,9 +36,10 @@ KERNELS_PER_STEP = 9  # gate, topk, masks, scan, offsets, fill, gemm1, gemm2, co
 def kernels_per_step(cfg, flags: int, fp8: bool) -> int:
     """Launches of one moe_layer call, following the library's own choice of forms (see MOE_FLAG_* in tcmoe.h)."""
     from paper_2605_05607_b200 import binding as B
+    layout = 3 if cfg.P <= 32768 else 0                # up to 32768 pairs one kernel instead of four builds the layout
     if flags & B.MOE_FLAG_FUSED_FFN:
-        return 6 + 2                                   # ... layout, then the task-table kernel and the tracker-paced kernel
-    n = KERNELS_PER_STEP + (2 if fp8 else 0)           # FP8: + quantisation of x and of h
+        return 6 - layout + 2                          # ... layout, then the task-table kernel and the tracker-paced kernel
+    n = KERNELS_PER_STEP - layout + (2 if fp8 else 0)  # FP8: + quantisation of x and of h
     if flags & B.MOE_FLAG_COMBINE_IN_EPILOGUE:
         return n                                       # no combine kernel, one rounding pass instead
     wide = cfg.f >= 8192 and cfg.T * cfg.k >= 512 * cfg.E

@@ -35,18 +35,27 @@ __device__ __forceinline__ void grid_dependency_sync() {
 }
 
 template <typename... KArgs, typename... Args>
-cudaError_t launch_pdl(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, Args&&... args) {
+cudaError_t launch_pdl_cluster(unsigned cluster, void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t st,
+                               Args&&... args) {
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = grid;
   cfg.blockDim = block;
   cfg.dynamicSmemBytes = smem;
   cfg.stream = st;
-  cudaLaunchAttribute attr[1];
+  cudaLaunchAttribute attr[2];
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   attr[0].val.programmaticStreamSerializationAllowed = 1;
+  attr[1].id = cudaLaunchAttributeClusterDimension;
+  attr[1].val.clusterDim.x = cluster;
+  attr[1].val.clusterDim.y = 1;
+  attr[1].val.clusterDim.z = 1;
   cfg.attrs = attr;
-  cfg.numAttrs = 1;
+  cfg.numAttrs = cluster > 0 ? 2 : 1;
   return cudaLaunchKernelEx(&cfg, kernel, KArgs(std::forward<Args>(args))...);
+}
+template <typename... KArgs, typename... Args>
+cudaError_t launch_pdl(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, Args&&... args) {
+  return launch_pdl_cluster(0, kernel, grid, block, smem, st, std::forward<Args>(args)...);   // 0: as the kernel declares
 }
 
 // ---- problem description passed to the launchers ---------------------------------------------
@@ -91,7 +100,8 @@ cudaError_t launch_gate_logits(const Shape& s, const void* x, const float* w_gat
 cudaError_t launch_topk(const Shape& s, const float* logits, const float* bias, int64_t bias_stride,
                         int32_t* topk_idx, float* topk_w, int32_t* status, cudaStream_t st,
                         uint32_t* clear = nullptr, size_t clear_words = 0);   // clear: words zeroed on the side
-// layout.cu
+// layout.cu.  layout_in_one(s): the builder is one kernel that keeps the masks in shared memory, nothing to clear before it
+bool layout_in_one(const Shape& s);
 cudaError_t launch_layout(const Shape& s, const int32_t* topk_idx, const Layout& L, const LayoutScratch& sc,
                           int32_t* status, cudaStream_t st, bool masks_cleared = false);
 cudaError_t launch_tile_prefix(const Shape& s, const int32_t* expert_counts, int32_t* mt_prefix, int32_t* mp_prefix,

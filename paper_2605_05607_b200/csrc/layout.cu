@@ -8,6 +8,9 @@
 // an exclusive popcount scan along each mask row gives every token its rank, and a fill pass
 // turns ranks into the row tables.  No atomics touch the result arrays.
 #include "combine.cuh"
+#include "ptx.cuh"
+
+#include <atomic>
 
 namespace tcmoe {
 
@@ -135,6 +138,153 @@ __global__ void __launch_bounds__(256) fill_layout_kernel(const int32_t* __restr
   }
 }
 
+// ---- K2 in one kernel ----------------------------------------------------------------------------
+// The four passes above as one kernel of at most 8 thread blocks (a cluster), for up to 32768 pairs (a sparse table: 131072 slots): every block owns a
+// contiguous range of tokens, builds its masks and their prefixes in shared memory, reads the other blocks' row totals through
+// distributed shared memory and fills its tokens' entries.  The four launches are latency, not work: 16 us of device time and
+// three launch gaps for 256 tokens of top-2, 21 us for 3001 of top-4; in one kernel 6.2 and 9.5 us.  With more pairs the
+// scattered table stores of the fill pass want more than 8 SMs (16384 tokens of top-8: 29 us as four kernels); the slots of a
+// sparse table are mostly unused and cost a read only, so its limit is four times as high.
+constexpr int ONE_THREADS = 1024, ONE_MAX_BLOCKS = 8, ONE_MAX_PAIRS = 32768;
+struct OneShape { int blocks, tokens, words; size_t smem; };   // tokens per block (a multiple of 32) and their mask words
+OneShape one_shape(const Shape& s) {
+  OneShape o;
+  o.blocks = 1;
+  while (o.blocks < ONE_MAX_BLOCKS && o.blocks * 256 < s.T) o.blocks *= 2;
+  o.tokens = ((s.T + o.blocks - 1) / o.blocks + 31) & ~31;
+  o.words = o.tokens / 32;
+  const size_t rows = (size_t)s.E + s.G;
+  o.smem = rows * (o.words + 1) * 4 + rows * (o.words + 1) * 2 + rows * 4 * 2 + 16;
+  return o;
+}
+
+__global__ void __launch_bounds__(ONE_THREADS) layout_one_kernel(const int32_t* __restrict__ topk_idx, Layout L,
+                                                                 int32_t* mt_prefix, int32_t* mp_prefix, int T, int E, int k,
+                                                                 int G, int m, int TL, int W, int32_t* status, int sparse) {
+  extern __shared__ uint32_t one_s[];
+  __shared__ int warp_sum[4][32];
+  const int rows = E + G, ld = W + 1;   // row e < E: expert e, row E + g: group g; a pad word against bank conflicts
+  uint32_t* mask = one_s;                                                  // [rows][ld]
+  int* total = reinterpret_cast<int*>(mask + (size_t)rows * ld);           // [rows] members among this block's tokens
+  int* base = total + rows;                                                // [rows] table entry of the block's first member
+  uint16_t* prefix = reinterpret_cast<uint16_t*>(base + rows);             // [rows][ld] members before the word
+  const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
+  const int rank = blockIdx.x, blocks = gridDim.x;                         // the grid is one cluster
+  const int t0 = rank * TL, tn = max(0, min(TL, T - t0));
+  for (int i = tid; i < rows * ld; i += ONE_THREADS) mask[i] = 0u;
+  grid_dependency_sync();
+  __syncthreads();
+  for (int i = tid; i < tn * k; i += ONE_THREADS) {
+    const int tl = i / k;
+    const int e = __ldg(topk_idx + (size_t)t0 * k + i);
+    if (e < 0 || e >= E) {
+      if (!(sparse && e == -1)) report_error(status, DEV_INDEX_OUT_OF_RANGE, KID_MASKS, t0 + tl, e);   // -1: unused slot
+      continue;
+    }
+    atomicOr(&mask[e * ld + (tl >> 5)], 1u << (tl & 31));
+    atomicOr(&mask[(E + e / m) * ld + (tl >> 5)], 1u << (tl & 31));
+  }
+  __syncthreads();
+  for (int r = tid; r < rows; r += ONE_THREADS) {
+    int n = 0;
+    for (int w = 0; w < W; ++w) {
+      prefix[r * ld + w] = (uint16_t)n;
+      n += __popc(mask[r * ld + w]);
+    }
+    total[r] = n;
+  }
+  ptx::cluster_sync();
+  // thread i: expert i and group i.  Members in the blocks before this one, and in all.
+  int before[2] = {0, 0}, all[2] = {0, 0};
+#pragma unroll
+  for (int j = 0; j < 2; ++j) {
+    if (tid >= (j ? G : E)) continue;
+    const uint32_t at = ptx::smem_u32(total + (j ? E + tid : tid));
+    for (int b = 0; b < blocks; ++b) {
+      const int n = ptx::ld_shared_cluster(ptx::mapa(at, b));
+      if (b < rank) before[j] += n;
+      all[j] += n;
+    }
+  }
+  // exclusive scans over the experts / groups: rows, dispatched rows, 128-row tiles, 256-row tiles
+  int v[4] = {all[0], all[1], (all[0] + 127) >> 7, (all[0] + 255) >> 8}, incl[4];
+#pragma unroll
+  for (int q = 0; q < 4; ++q) {
+    incl[q] = v[q];
+#pragma unroll
+    for (int off = 1; off < 32; off <<= 1) {
+      const int n = __shfl_up_sync(0xFFFFFFFFu, incl[q], off);
+      if (lane >= off) incl[q] += n;
+    }
+    if (lane == 31) warp_sum[q][wid] = incl[q];
+  }
+  __syncthreads();
+  if (wid < 4) {
+    int n = warp_sum[wid][lane];
+#pragma unroll
+    for (int off = 1; off < 32; off <<= 1) {
+      const int u = __shfl_up_sync(0xFFFFFFFFu, n, off);
+      if (lane >= off) n += u;
+    }
+    warp_sum[wid][lane] = n;
+  }
+  __syncthreads();
+#pragma unroll
+  for (int q = 0; q < 4; ++q)
+    if (wid > 0) incl[q] += warp_sum[q][wid - 1];
+  if (tid < E) base[tid] = incl[0] - v[0] + before[0];
+  if (tid < G) base[E + tid] = incl[1] - v[1] + before[1];
+  __shared__ int goff_s[1024];                                             // first dispatched row of a group
+  if (tid < G) goff_s[tid] = incl[1] - v[1];
+  if (rank == 0) {
+    if (tid < E) {
+      L.expert_counts[tid] = all[0];
+      L.expert_offsets[tid + 1] = incl[0];
+      mt_prefix[tid + 1] = incl[2];
+      mp_prefix[tid + 1] = incl[3];
+    }
+    if (tid < G) {
+      L.group_counts[tid] = all[1];
+      L.group_offsets[tid + 1] = incl[1];
+    }
+    if (tid == 0) { L.expert_offsets[0] = 0; L.group_offsets[0] = 0; mt_prefix[0] = 0; mp_prefix[0] = 0; }
+  }
+  __syncthreads();
+  ptx::cluster_arrive();   // this block has read the others' totals
+  auto rank_of = [&](int r, int tl) {
+    return (int)prefix[r * ld + (tl >> 5)] + __popc(mask[r * ld + (tl >> 5)] & ((1u << (tl & 31)) - 1u));
+  };
+  for (int i = tid; i < G * TL; i += ONE_THREADS) {
+    const int g = i / TL, tl = i - g * TL;
+    if (tl >= tn) continue;
+    int a = -1;
+    if (mask[(E + g) * ld + (tl >> 5)] >> (tl & 31) & 1u) {
+      const int row = base[E + g] + rank_of(E + g, tl);
+      a = row - goff_s[g];
+      L.disp_token[row] = t0 + tl;   // TID table entry of the allocated row
+    }
+    L.al[(size_t)g * T + t0 + tl] = a;
+  }
+  for (int i = tid; i < tn * k; i += ONE_THREADS) {
+    const int tl = i / k, p = t0 * k + i;
+    const int e = __ldg(topk_idx + p);
+    if (e < 0 || e >= E) {           // unused slot (sparse top-k), or an index reported above
+      L.pair_row[p] = -1;
+      continue;
+    }
+    const int r = base[e] + rank_of(e, tl), g = E + e / m;
+    L.pair_row[p] = r;
+    L.row_pair[r] = p;
+    L.row_src[r] = base[g] + rank_of(g, tl);
+  }
+  __syncwarp();
+  ptx::cluster_wait();     // no block leaves while another may still read its totals
+}
+
+bool layout_in_one(const Shape& s) {
+  return s.T > 0 && (long long)s.T * s.k <= ((s.flags & 4) ? 4 : 1) * ONE_MAX_PAIRS && one_shape(s).smem <= 160 * 1024;
+}
+
 // exclusive prefixes of 128-row tiles and 256-row pair tiles per expert, from the counts alone
 __global__ void __launch_bounds__(1024) tile_prefix_kernel(const int32_t* __restrict__ expert_counts,
                                                            int32_t* mt_prefix, int32_t* mp_prefix, int E) {
@@ -165,6 +315,18 @@ cudaError_t launch_layout(const Shape& s, const int32_t* topk_idx, const Layout&
                           int32_t* status, cudaStream_t st, bool masks_cleared) {
   const int m = s.E / s.G;
   cudaError_t err;
+  if (layout_in_one(s)) {
+    static std::atomic<bool> attr_set[MAX_DEVICES];   // per device; setting the attribute twice is harmless
+    const int dev = current_device();
+    if (!attr_set[dev].load(std::memory_order_acquire)) {
+      if ((err = cudaFuncSetAttribute(layout_one_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 160 * 1024)) != cudaSuccess)
+        return err;
+      attr_set[dev].store(true, std::memory_order_release);
+    }
+    const OneShape o = one_shape(s);
+    return launch_pdl_cluster(o.blocks, layout_one_kernel, o.blocks, ONE_THREADS, o.smem, st, topk_idx, L, sc.mt_prefix,
+                              sc.mp_prefix, s.T, s.E, s.k, s.G, m, o.tokens, o.words, status, (s.flags & 4) ? 1 : 0);
+  }
   if (!masks_cleared &&
       (err = cudaMemsetAsync(sc.emask, 0, sizeof(uint32_t) * (size_t)(s.E + s.G) * sc.W, st)) != cudaSuccess)
     return err;  // emask and gmask are adjacent

@@ -1,0 +1,59 @@
+"""Dispatch layout at the edges of its two builders: one kernel of 1, 2, 4 or 8 thread blocks up to 32768 pairs, four kernels
+beyond; mask words of 32 tokens, blocks without tokens, 1024 experts, unused slots.  Bit-exact against the oracle."""
+import numpy as np
+import pytest
+import torch
+
+from oracle import moe_oracle as O
+from paper_2605_05607_b200 import binding as B
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("T,E,k,G", [(1, 8, 2, 8), (31, 1024, 32, 1024), (256, 8, 8, 1), (257, 12, 3, 4), (513, 6, 1, 3),
+                                     (1025, 256, 8, 8), (1100, 64, 4, 32), (4096, 64, 8, 32), (4097, 64, 8, 32),
+                                     (16384, 8, 2, 4), (32768, 16, 1, 16)])
+def test_layout_builders(T, E, k, G):
+    rng = np.random.default_rng(T + E)
+    skew = -1.5 * np.log(1 + rng.permutation(E))                      # popular and empty experts
+    idx = np.argsort(-(rng.gumbel(size=(T, E)) + skew), axis=1)[:, :k].astype(np.int32)
+    shape = B.MoEShape(T, 64, 64, E, k, G, 0, 0)
+    lay, ws = B.alloc_layout(shape), B.alloc_workspace(shape)
+    d_idx = torch.from_numpy(np.ascontiguousarray(idx)).cuda().view(-1)
+    for _ in range(2):                                                # the second call finds the first one's scratch
+        B.moe_dispatch(shape, None, d_idx, lay, None, ws)
+    ref = O.layout(idx, E, G)
+    for name in ("expert_counts", "expert_offsets", "group_counts", "group_offsets", "pair_row", "row_pair", "row_src"):
+        assert np.array_equal(getattr(lay, name).cpu().numpy()[: ref[name].size], ref[name]), name
+    assert np.array_equal(lay.al.cpu().numpy()[: G * T].reshape(G, T), ref["al"])
+    assert np.array_equal(lay.disp_token.cpu().numpy()[: ref["n_disp"]], ref["disp_token"])
+    pre = B.moe_workspace_layout(shape)["mt_prefix"]
+    tiles = np.concatenate([[0], np.cumsum((ref["expert_counts"] + 127) // 128)])
+    assert np.array_equal(ws[pre: pre + 4 * (E + 1)].view(torch.int32).cpu().numpy(), tiles)
+    assert B.moe_status(ws)[0] == 0
+
+
+@pytest.mark.parametrize("T", [8192, 16384, 16385])
+def test_layout_of_a_sparse_table(T):
+    """Unused slots (-1): one kernel up to 131072 slots, four beyond; both against the same layout built slot by slot."""
+    E, k = 16, 8
+    rng = np.random.default_rng(T)
+    idx = np.argsort(rng.random((T, E)), axis=1)[:, :k].astype(np.int32)
+    idx[rng.random((T, k)) < 0.8] = -1
+    shape = B.MoEShape(T, 64, 64, E, k, 1, 0, B.MOE_FLAG_SPARSE_TOPK)
+    lay, ws = B.alloc_layout(shape), B.alloc_workspace(shape)
+    B.moe_dispatch(shape, None, torch.from_numpy(idx).cuda().view(-1), lay, None, ws)
+    counts = np.bincount(idx[idx >= 0], minlength=E)
+    offsets = np.concatenate([[0], np.cumsum(counts)])
+    pair_row = np.full(T * k, -1, np.int64)
+    flat = idx.reshape(-1)
+    for e in range(E):
+        pair_row[np.nonzero(flat == e)[0]] = offsets[e] + np.arange(counts[e])      # ascending token
+    used = np.nonzero(flat >= 0)[0]
+    assert np.array_equal(lay.expert_offsets.cpu().numpy()[: E + 1], offsets)
+    assert np.array_equal(lay.pair_row.cpu().numpy()[: T * k], pair_row)
+    assert np.array_equal(lay.row_pair.cpu().numpy()[pair_row[used]], used)
+    seen = (idx >= 0).any(axis=1)
+    assert np.array_equal(lay.al.cpu().numpy()[:T], np.where(seen, np.cumsum(seen) - 1, -1))
+    assert np.array_equal(lay.row_src.cpu().numpy()[pair_row[used]], (np.cumsum(seen) - 1)[used // k])
+    assert B.moe_status(ws)[0] == 0
