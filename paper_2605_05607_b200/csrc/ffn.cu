@@ -103,11 +103,11 @@ bool make_act_map(CUtensorMap* map, const void* base, long long rows, int K) {
   return encode_tiled(map, false, 2, base, dims, strides, box);
 }
 
-// E4M3 weights [E, N, K] (K contiguous): box = 128 bytes of K x 128 output columns x 1, 128-byte swizzle
-bool make_weight_map_fp8(CUtensorMap* map, const void* base, int E, int N, int K) {
+// E4M3 weights [E, N, K] (K contiguous): box = 128 bytes of K x box_cols output columns x 1, 128-byte swizzle
+bool make_weight_map_fp8(CUtensorMap* map, const void* base, int E, int N, int K, int box_cols) {
   cuuint64_t dims[3] = {(cuuint64_t)K, (cuuint64_t)N, (cuuint64_t)E};
   cuuint64_t strides[2] = {(cuuint64_t)K, (cuuint64_t)N * K};
-  cuuint32_t box[3] = {128, 128, 1};
+  cuuint32_t box[3] = {128, (cuuint32_t)box_cols, 1};
   return encode_tiled(map, true, 3, base, dims, strides, box);
 }
 
@@ -176,6 +176,15 @@ static bool small_experts(const Shape& s) {
   return (long long)s.T * s.k < 512ll * s.E;
 }
 
+// Fewer full-width tiles than SMs (an upper bound from the shape: every expert that can be reached has one 128-row tile, and one
+// more per 128 pairs): GEMM tiles of 64 output columns.  Wider ones leave SMs idle and the rest waiting on one SM's share of the
+// memory bandwidth: one token of top-2 on d = 4096, f = 14336 (32 tiles of GEMM-2) 87 us, narrow 58; 256 tokens of d = 512, f = 1024:
+// GEMM-1 13.2 -> 10.6, GEMM-2 12.4 -> 9.7.
+static bool narrow_tiles(const Shape& s, int n_tiles) {
+  const long long P = (long long)s.T * s.k;
+  return ((s.E < P ? s.E : P) + P / 128) * n_tiles < 148;
+}
+
 size_t fused_table_blocks(const Shape& s) { return ffn::fused_max_blocks(s.T, s.k, s.E); }
 size_t fused_tracker_bytes(const Shape& s) { return ffn::fused_tracker_words(s.T, s.k, s.E) * sizeof(int32_t); }
 
@@ -239,7 +248,7 @@ cudaError_t launch_expert_ffn(const Shape& s, const FfnArgs& a, cudaStream_t st)
   g1.E = s.E;
   g1.K = s.d;
   g1.N = s.f;
-  g1.n_tiles = (s.f + 127) / 128;
+  g1.n_tiles = (s.f + 127) / 128;   // (the single-CTA launchers set their own)
   g1.status = a.status;
   cudaError_t err;
   if (a.pair_gemm1 && a.xs != nullptr) {
@@ -252,7 +261,7 @@ cudaError_t launch_expert_ffn(const Shape& s, const FfnArgs& a, cudaStream_t st)
     g1.tile_prefix = a.mp_prefix;
     err = ffn::launch_gemm1_pair(g1, m_w1, m_w3, m_xs, st);
   } else {
-    err = ffn::launch_gemm1(g1, m_w1, m_w3, false, st);
+    err = ffn::launch_gemm1(g1, m_w1, m_w3, false, narrow_tiles(s, (s.f + 127) / 128), st);
   }
   if (err != cudaSuccess) return err;
 
@@ -274,7 +283,7 @@ cudaError_t launch_expert_ffn(const Shape& s, const FfnArgs& a, cudaStream_t st)
     g2.a_src = a.h;
     g2.a_ld = s.f;
     g2.tile_prefix = a.mt_prefix;
-    return ffn::launch_gemm2_single(g2, m_w2, false, st);
+    return ffn::launch_gemm2_single(g2, m_w2, false, narrow_tiles(s, (s.d + 255) / 256), st);
   }
   return ffn::launch_gemm2(g2, m_w2, m_h, false, st);
 }
@@ -284,8 +293,11 @@ cudaError_t launch_expert_ffn_fp8(const Shape& s, const FfnArgs& a, const Fp8Arg
   if (s.T == 0) return cudaSuccess;
   const int P = s.T * s.k;
   CUtensorMap m_w1, m_w3, m_w2, m_h;
-  if (!make_weight_map_fp8(&m_w1, a.w1, s.E, s.f, s.d) || !make_weight_map_fp8(&m_w3, a.w3, s.E, s.f, s.d) ||
-      !make_weight_map_fp8(&m_w2, a.w2, s.E, s.d, s.f) || !make_act_map_fp8(&m_h, q.hq, P, s.f))
+  const bool single2 = small_experts(s) && a.y_acc == nullptr;
+  const bool narrow1 = narrow_tiles(s, (s.f + 127) / 128), narrow2 = single2 && narrow_tiles(s, (s.d + 255) / 256);
+  if (!make_weight_map_fp8(&m_w1, a.w1, s.E, s.f, s.d, narrow1 ? 64 : 128) ||
+      !make_weight_map_fp8(&m_w3, a.w3, s.E, s.f, s.d, narrow1 ? 64 : 128) ||
+      !make_weight_map_fp8(&m_w2, a.w2, s.E, s.d, s.f, narrow2 ? 64 : 128) || !make_act_map_fp8(&m_h, q.hq, P, s.f))
     return cudaErrorInvalidValue;
 
   ffn::GemmParams g1{};
@@ -301,12 +313,12 @@ cudaError_t launch_expert_ffn_fp8(const Shape& s, const FfnArgs& a, const Fp8Arg
   g1.E = s.E;
   g1.K = s.d;
   g1.N = s.f;
-  g1.n_tiles = (s.f + 127) / 128;
+  g1.n_tiles = (s.f + 127) / 128;   // (the single-CTA launchers set their own)
   g1.status = a.status;
   g1.a_scale = q.sx;
   g1.b_scale = q.s1;
   g1.b_scale2 = q.s3;
-  cudaError_t err = ffn::launch_gemm1(g1, m_w1, m_w3, true, st);
+  cudaError_t err = ffn::launch_gemm1(g1, m_w1, m_w3, true, narrow1, st);
   if (err != cudaSuccess) return err;
   if ((err = launch_quantize_rows(a.h, P, s.f, q.hq, q.sh, st)) != cudaSuccess) return err;
 
@@ -326,11 +338,11 @@ cudaError_t launch_expert_ffn_fp8(const Shape& s, const FfnArgs& a, const Fp8Arg
   g2.y_div = s.k;
   g2.a_scale = q.sh;
   g2.b_scale = q.s2;
-  if (small_experts(s) && a.y_acc == nullptr) {
+  if (single2) {
     g2.a_src = q.hq;
     g2.a_ld = s.f;
     g2.tile_prefix = a.mt_prefix;
-    return ffn::launch_gemm2_single(g2, m_w2, true, st);
+    return ffn::launch_gemm2_single(g2, m_w2, true, narrow2, st);
   }
   return ffn::launch_gemm2(g2, m_w2, m_h, true, st);
 }

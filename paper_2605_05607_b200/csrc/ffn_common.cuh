@@ -94,15 +94,15 @@ __device__ __forceinline__ uint64_t desc_at(uint64_t base, uint32_t smem_addr) {
   return base | (uint64_t)((smem_addr & 0x3FFFF) >> 4);
 }
 
-// instruction descriptor of the FP8 form: D fp32, A/B E4M3 (format code 0), both K-major, N = 256, M = m
-__host__ __device__ constexpr uint32_t idesc_e4m3(int m) {
-  return (1u << 4) | (0u << 7) | (0u << 10) | (0u << 15) | (0u << 16) | ((uint32_t)(UMMA_N >> 3) << 17) |
+// instruction descriptor of the FP8 form: D fp32, A/B E4M3 (format code 0), both K-major, N = n, M = m
+__host__ __device__ constexpr uint32_t idesc_e4m3(int m, int n = UMMA_N) {
+  return (1u << 4) | (0u << 7) | (0u << 10) | (0u << 15) | (0u << 16) | ((uint32_t)(n >> 3) << 17) |
          ((uint32_t)(m >> 4) << 24);
 }
 
-// instruction descriptor: D fp32, A/B bf16, A K-major, B MN-major, N = 256, M = m
-__host__ __device__ constexpr uint32_t idesc_bf16(int m) {
-  return (1u << 4) | (1u << 7) | (1u << 10) | (0u << 15) | (1u << 16) | ((uint32_t)(UMMA_N >> 3) << 17) |
+// instruction descriptor: D fp32, A/B bf16, A K-major, B MN-major, N = n, M = m
+__host__ __device__ constexpr uint32_t idesc_bf16(int m, int n = UMMA_N) {
+  return (1u << 4) | (1u << 7) | (1u << 10) | (0u << 15) | (1u << 16) | ((uint32_t)(n >> 3) << 17) |
          ((uint32_t)(m >> 4) << 24);
 }
 
@@ -157,7 +157,7 @@ bool encode_tiled(CUtensorMap* map, bool bytes, int rank, const void* base, cons
 void clear_map_cache();
 bool make_weight_map(CUtensorMap* map, const void* base, int E, int K, int N);
 bool make_act_map(CUtensorMap* map, const void* base, long long rows, int K);
-bool make_weight_map_fp8(CUtensorMap* map, const void* base, int E, int N, int K);
+bool make_weight_map_fp8(CUtensorMap* map, const void* base, int E, int N, int K, int box_cols = 128);
 bool make_act_map_fp8(CUtensorMap* map, const void* base, int rows, int K);
 bool make_weight_map_kmajor(CUtensorMap* map, const void* base, int E, int rows, int cols);
 bool make_rows_map_mn(CUtensorMap* map, const void* base, long long rows, int cols);
@@ -166,7 +166,7 @@ cudaError_t launch_wgrad_pair(const CUtensorMap& m_a, const CUtensorMap& m_b, co
 
 // fp8 = false: bf16 operands, weights [E, K, N] (B MN-major).  fp8 = true: E4M3 operands, weights
 // [E, N, K] (B K-major), 128 elements of K per pipeline stage, scales applied in the epilogue.
-cudaError_t launch_gemm1(const GemmParams& p, const CUtensorMap& m_w1, const CUtensorMap& m_w3, bool fp8,
+cudaError_t launch_gemm1(GemmParams p, const CUtensorMap& m_w1, const CUtensorMap& m_w3, bool fp8, bool narrow,
                          cudaStream_t st);
 cudaError_t launch_gemm2(const GemmParams& p, const CUtensorMap& m_w2, const CUtensorMap& m_h, bool fp8,
                          cudaStream_t st);
@@ -183,7 +183,7 @@ cudaError_t launch_ffn_fused(FusedParams p, const int32_t* expert_counts, int32_
                              int32_t* n_blocks, int32_t* tracker, const CUtensorMap& m_w1, const CUtensorMap& m_w3,
                              const CUtensorMap& m_w2, cudaStream_t st);
 // GEMM-2 on 128-row single-CTA tiles (small experts): p.a_src / p.a_ld = h rows, no Combine-in-epilogue form
-cudaError_t launch_gemm2_single(const GemmParams& p, const CUtensorMap& m_w2, bool fp8, cudaStream_t st);
+cudaError_t launch_gemm2_single(GemmParams p, const CUtensorMap& m_w2, bool fp8, bool narrow, cudaStream_t st);
 
 }  // namespace ffn
 }  // namespace tcmoe

@@ -37,27 +37,23 @@ namespace tcmoe {
 namespace ffn {
 namespace {
 
-constexpr int NSTAGE = 4;
 constexpr int A_BYTES = BM * BK * 2;         // 16 KiB
-constexpr int B_BYTES = UMMA_N * BK * 2;     // 32 KiB = four 64-column slabs of 8 KiB
-constexpr int STAGE_BYTES = A_BYTES + B_BYTES;
-constexpr int NUM_BARS = 2 * NSTAGE + 4;
+constexpr int RING_BYTES = 192 * 1024;       // 4 stages of A + a 256-column B, more of narrower ones
+constexpr int MAX_STAGES = 8;
+constexpr int NUM_BARS = 2 * MAX_STAGES + 4;
 constexpr int STAGE_OUT_WARP = 32 * 144;     // epilogue transpose buffer of one warp: 32 rows x (128 + 16) bytes
 constexpr int TABLE_BYTES = (2 * (MAX_E + 1) * 4 + 15) & ~15;
 constexpr int COLSCALE_WARP = UMMA_N * 4;     // FP8: one warp's copy of the tile's 128 + 128 output-column scales
 constexpr int SMEM_BYTES =
-    1024 + NSTAGE * STAGE_BYTES + NUM_BARS * 8 + 64 + TABLE_BYTES + 4 * STAGE_OUT_WARP + 4 * COLSCALE_WARP;
+    1024 + RING_BYTES + NUM_BARS * 8 + 64 + TABLE_BYTES + 4 * STAGE_OUT_WARP + 4 * COLSCALE_WARP;
 constexpr int THREADS = 320;
 constexpr int GATHER_THREADS = 128;
-constexpr int BN_OUT = 128;
-constexpr uint32_t IDESC = idesc_bf16(BM);
 // The producers (TMA thread, 128 gather threads) wait for a free stage with a suspend-time hint: parked in hardware
 // instead of polling.  At the board's power limit the layer's time follows energy: GEMM-1 alone in a loop on the
 // DeepSeek-V3 shape 15.78 -> 15.50 ms with the hint (two alternations, same box), a single cold launch 13.41 -> 13.48.
 // The UMMA thread's wait for a full stage is on the critical path and keeps the plain form (hinting it too gives the
 // gain back).
 constexpr uint32_t FEED_HINT = 1000;
-constexpr uint32_t IDESC_F8 = idesc_e4m3(BM);
 
 // FP8 = true: A rows and weights are E4M3 codes, a stage holds 128 elements of K (the same 128
 // bytes per row), W1 / W3 come K-major from [E, N, K] as two 128-row boxes, and the epilogue applies
@@ -68,13 +64,23 @@ constexpr uint32_t IDESC_F8 = idesc_e4m3(BM);
 // the 256-column B tile come from the one weight map (map_w1), the epilogue writes
 // o[r, n] = w_r * acc[r, n] for 256 columns.  Used instead of the CTA-pair kernel when experts are small
 // (128-row tiles pad far less than 256-row pair tiles when most experts hold fewer than 128 rows).
-template <bool FP8, bool PLAIN>
+//
+// NARROW = true: tiles of a quarter (PLAIN: 64 columns) or half the width (64 columns of W1 and of W3), for layers with fewer
+// full-width tiles than SMs: one decoded token reads two wide experts' weights through 32 full-width tiles of GEMM-2.  The
+// sums are the same, element by element.
+template <bool FP8, bool PLAIN, bool NARROW>
 __global__ void __launch_bounds__(THREADS, 1)
 ffn_gemm1_kernel(const __grid_constant__ CUtensorMap map_w1, const __grid_constant__ CUtensorMap map_w3,
                  const GemmParams p) {
+  constexpr int BN = !NARROW ? UMMA_N : PLAIN ? 64 : 128;   // accumulator columns of a tile
+  constexpr int BN_OUT = PLAIN ? BN : BN / 2;               // output columns
+  constexpr int HALF = BN > 64 ? BN / 2 : BN;               // columns from each of the two weight maps (BN = 64: one)
+  constexpr int B_BYTES = BN * BK * 2, STAGE_BYTES = A_BYTES + B_BYTES;   // B: 64-column slabs of 8 KiB
+  constexpr int NSTAGE = RING_BYTES / STAGE_BYTES;
+  static_assert(NSTAGE <= MAX_STAGES, "barriers");
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
-  uint64_t* bars = reinterpret_cast<uint64_t*>(smem + NSTAGE * STAGE_BYTES);
+  uint64_t* bars = reinterpret_cast<uint64_t*>(smem + RING_BYTES);
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + NUM_BARS);
   int* abort_s = reinterpret_cast<int*>(tmem_slot + 1);
   int* tp_s = reinterpret_cast<int*>(tmem_slot + 16);
@@ -85,9 +91,9 @@ ffn_gemm1_kernel(const __grid_constant__ CUtensorMap map_w1, const __grid_consta
   const uint32_t smem_base = ptx::smem_u32(smem);
   const uint32_t bar_base = ptx::smem_u32(bars);
   auto full_bar = [&](int s) { return bar_base + 8u * s; };
-  auto empty_bar = [&](int s) { return bar_base + 8u * (NSTAGE + s); };
-  auto tfull_bar = [&](int b) { return bar_base + 8u * (2 * NSTAGE + b); };
-  auto tempty_bar = [&](int b) { return bar_base + 8u * (2 * NSTAGE + 2 + b); };
+  auto empty_bar = [&](int s) { return bar_base + 8u * (MAX_STAGES + s); };
+  auto tfull_bar = [&](int b) { return bar_base + 8u * (2 * MAX_STAGES + b); };
+  auto tempty_bar = [&](int b) { return bar_base + 8u * (2 * MAX_STAGES + 2 + b); };
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
 
@@ -131,7 +137,7 @@ ffn_gemm1_kernel(const __grid_constant__ CUtensorMap map_w1, const __grid_consta
     p.status[ST_ABORT] = 1;
     *abort_flag = 1;
   };
-  auto tile_of = [&](int w) { return decode_tile(w, tp_s, eoff_s, p.E, p.n_tiles, PLAIN ? 2 * BN_OUT : BN_OUT, BM, 0); };
+  auto tile_of = [&](int w) { return decode_tile(w, tp_s, eoff_s, p.E, p.n_tiles, BN_OUT, BM, 0); };
 
   if (warp < 4) {
     // ================================ epilogue ================================
@@ -141,7 +147,7 @@ ffn_gemm1_kernel(const __grid_constant__ CUtensorMap map_w1, const __grid_consta
       const int buf = tl & 1;
       if (!ptx::mbar_wait_warp<true>(tfull_bar(buf), (tl >> 1) & 1, abort_flag, global_abort)) { timeout(1); break; }
       ptx::tc_fence_after();
-      const uint32_t taddr = tmem_base + ((uint32_t)(warp * 32) << 16) + (uint32_t)(buf * UMMA_N);
+      const uint32_t taddr = tmem_base + ((uint32_t)(warp * 32) << 16) + (uint32_t)(buf * BN);
       // A thread owns one accumulator row; 32 threads storing 16 bytes each to 32 different rows
       // would cost 32 memory transactions per instruction.  The warp transposes 64 output columns
       // at a time through shared memory (rows padded to 144 bytes: conflict-free both ways) and
@@ -161,14 +167,14 @@ ffn_gemm1_kernel(const __grid_constant__ CUtensorMap map_w1, const __grid_consta
         if (FP8) {
           const float* g = p.b_scale + (size_t)t.e * p.N + t.n0;
 #pragma unroll
-          for (int i = 0; i < UMMA_N / 32; ++i) {
+          for (int i = 0; i < BN / 32; ++i) {
             const int n = lane + 32 * i;
             sb_col[n] = (t.n0 + n < p.N) ? __ldg(g + n) : 0.f;
           }
           __syncwarp();
         }
 #pragma unroll 1
-        for (int cc = 0; cc < 4; ++cc) {
+        for (int cc = 0; cc < BN / 64; ++cc) {
           uint32_t acc0[32], acc1[32];
           ptx::tmem_ld32(taddr + cc * 64, acc0);
           ptx::tmem_ld32(taddr + cc * 64 + 32, acc1);
@@ -213,7 +219,7 @@ ffn_gemm1_kernel(const __grid_constant__ CUtensorMap map_w1, const __grid_consta
         // ---- GEMM-1 form: SwiGLU of the W1 / W3 halves, 128 output columns
       float sa = 1.f;   // FP8: scale of this thread's row (the gather source row)
       float* s1 = colscale_base + warp * UMMA_N;   // this warp's copy of the W1 / W3 column scales (0 beyond N)
-      float* s3 = s1 + 128;
+      float* s3 = s1 + BN_OUT;
       if (FP8) {
         const int lrow = warp * 32 + lane;
         if (lrow < t.rows) {
@@ -223,7 +229,7 @@ ffn_gemm1_kernel(const __grid_constant__ CUtensorMap map_w1, const __grid_consta
         }
         const size_t g = (size_t)t.e * p.N + t.n0;
 #pragma unroll
-        for (int i = 0; i < 4; ++i) {
+        for (int i = 0; i < BN_OUT / 32; ++i) {
           const int n = lane + 32 * i;
           const bool in = t.n0 + n < p.N;
           s1[n] = in ? (__ldg(p.b_scale + g + n)) : 0.f;
@@ -232,10 +238,10 @@ ffn_gemm1_kernel(const __grid_constant__ CUtensorMap map_w1, const __grid_consta
         __syncwarp();
       }
 #pragma unroll 1
-      for (int c = 0; c < 4; ++c) {
+      for (int c = 0; c < BN_OUT / 32; ++c) {
         uint32_t a1[32], a3[32];
         ptx::tmem_ld32(taddr + c * 32, a1);
-        ptx::tmem_ld32(taddr + 128 + c * 32, a3);
+        ptx::tmem_ld32(taddr + BN_OUT + c * 32, a3);
         ptx::tmem_ld_wait();
 #pragma unroll
         for (int v = 0; v < 4; ++v) {
@@ -292,16 +298,17 @@ ffn_gemm1_kernel(const __grid_constant__ CUtensorMap map_w1, const __grid_consta
           const uint32_t sb = smem_base + s * STAGE_BYTES + A_BYTES;
           ptx::mbar_arrive_expect_tx(full_bar(s), B_BYTES);
           const int k0 = kb * BK_ELEMS;
-          const CUtensorMap* hi_map = PLAIN ? &map_w1 : &map_w3;   // second 128 accumulator columns
-          const int hi_n = PLAIN ? t.n0 + 128 : t.n0;
-          if (FP8) {   // K-major boxes of 128 output columns x 128 bytes of K
+          const CUtensorMap* hi_map = PLAIN ? &map_w1 : &map_w3;   // second half of the accumulator columns
+          const int hi_n = PLAIN ? t.n0 + HALF : t.n0;
+          if (FP8) {   // K-major boxes of HALF output columns x 128 bytes of K
             ptx::tma_load_3d(sb, &map_w1, full_bar(s), k0, t.n0, t.e);
-            ptx::tma_load_3d(sb + 16384, hi_map, full_bar(s), k0, hi_n, t.e);
+            if (BN > HALF) ptx::tma_load_3d(sb + HALF * 128, hi_map, full_bar(s), k0, hi_n, t.e);
           } else {     // MN-major slabs of 64 output columns x 64 rows of K
-            ptx::tma_load_3d(sb, &map_w1, full_bar(s), t.n0, k0, t.e);
-            ptx::tma_load_3d(sb + 8192, &map_w1, full_bar(s), t.n0 + 64, k0, t.e);
-            ptx::tma_load_3d(sb + 16384, hi_map, full_bar(s), hi_n, k0, t.e);
-            ptx::tma_load_3d(sb + 24576, hi_map, full_bar(s), hi_n + 64, k0, t.e);
+#pragma unroll
+            for (int c = 0; c < BN / 64; ++c) {
+              const bool hi = c * 64 >= HALF;
+              ptx::tma_load_3d(sb + c * 8192, hi ? hi_map : &map_w1, full_bar(s), (hi ? hi_n - HALF : t.n0) + c * 64, k0, t.e);
+            }
           }
         }
         if (!ok) break;
@@ -309,35 +316,36 @@ ffn_gemm1_kernel(const __grid_constant__ CUtensorMap map_w1, const __grid_consta
     }
   } else if (warp == 5) {
     // ================================ UMMA issuer ================================
-    if (lane == 0) {
-      const uint64_t a_base = desc_base(16, 1024);
-      const uint64_t b_base = FP8 ? desc_base(16, 1024) : desc_base(BK * 128, 1024);   // K-major : MN-major
-      uint32_t it = 0;
-      int tl = 0;
-      for (int w = blockIdx.x; w < total && !*abort_flag; w += gridDim.x, ++tl) {
-        const int buf = tl & 1;
-        if (!ptx::mbar_wait(tempty_bar(buf), ((tl >> 1) & 1) ^ 1, abort_flag, global_abort)) { timeout(3); break; }
+    // the warp walks the loop, one elected lane issues (see ptx::elect_one)
+    const bool elected = ptx::elect_one();
+    const uint32_t base = __shfl_sync(0xFFFFFFFFu, smem_base, 0), tmem = __shfl_sync(0xFFFFFFFFu, tmem_base, 0);
+    const uint64_t a_desc = desc_at(desc_base(16, 1024), base);
+    const uint64_t b_desc = desc_at(FP8 ? desc_base(16, 1024) : desc_base(BK * 128, 1024), base + A_BYTES);   // K-major : MN-major
+    constexpr uint32_t IDESC = FP8 ? idesc_e4m3(BM, BN) : idesc_bf16(BM, BN);
+    constexpr int B_STEP = FP8 ? 2 : 128;   // 32 bytes of K per UMMA (16 bf16 / 32 E4M3): +32 B inside the swizzle row, or +2 atoms
+    int s = 0, tl = 0;
+    uint32_t ph = 0;
+    bool ok = true;
+    for (int w = blockIdx.x; ok && w < total && !*abort_flag; w += gridDim.x, ++tl) {
+      const int buf = tl & 1;
+      if (!ptx::mbar_wait(tempty_bar(buf), ((tl >> 1) & 1) ^ 1, abort_flag, global_abort)) { timeout(3); break; }
+      ptx::tc_fence_after();
+      const uint32_t d_tmem = tmem + (uint32_t)(buf * BN);
+      for (int kb = 0; kb < KB; ++kb) {
+        if (!ptx::mbar_wait(full_bar(s), ph, abort_flag, global_abort)) { timeout(4); ok = false; break; }
         ptx::tc_fence_after();
-        const uint32_t d_tmem = tmem_base + (uint32_t)(buf * UMMA_N);
-        bool ok = true;
-        for (int kb = 0; kb < KB; ++kb, ++it) {
-          const int s = it % NSTAGE;
-          if (!ptx::mbar_wait(full_bar(s), (it / NSTAGE) & 1, abort_flag, global_abort)) {
-            timeout(4); ok = false; break;
-          }
-          ptx::tc_fence_after();
-          const uint32_t sa = smem_base + s * STAGE_BYTES, sb = sa + A_BYTES;
-          const uint64_t ad = desc_at(a_base, sa), bd = desc_at(b_base, sb);
+        if (elected) {
+          const uint64_t ad = a_desc + (uint64_t)(s * (STAGE_BYTES >> 4)), bd = b_desc + (uint64_t)(s * (STAGE_BYTES >> 4));
 #pragma unroll
-          for (int k = 0; k < 4; ++k) {   // 32 bytes of K per UMMA (16 bf16 / 32 E4M3): +32 B inside the swizzle row
-            if (FP8) ptx::umma_f8(d_tmem, ad + (uint64_t)(k * 2), bd + (uint64_t)(k * 2), IDESC_F8, (kb | k) != 0);
-            else ptx::umma_bf16(d_tmem, ad + (uint64_t)(k * 2), bd + (uint64_t)(k * 128), IDESC, (kb | k) != 0);   // B: +2 atoms
+          for (int k = 0; k < 4; ++k) {
+            if (FP8) ptx::umma_f8(d_tmem, ad + (uint64_t)(k * 2), bd + (uint64_t)(k * B_STEP), IDESC, (kb | k) != 0);
+            else ptx::umma_bf16(d_tmem, ad + (uint64_t)(k * 2), bd + (uint64_t)(k * B_STEP), IDESC, (kb | k) != 0);
           }
           ptx::umma_commit(empty_bar(s));   // free the stage when these UMMAs have read it
         }
-        if (!ok) break;
-        ptx::umma_commit(tfull_bar(buf));   // accumulator complete
+        if (++s == NSTAGE) { s = 0; ph ^= 1u; }
       }
+      if (ok && elected) ptx::umma_commit(tfull_bar(buf));   // accumulator complete
     }
   } else {
     // ================================ A gather producers ================================
@@ -410,31 +418,37 @@ ffn_gemm1_kernel(const __grid_constant__ CUtensorMap map_w1, const __grid_consta
 }  // namespace
 
 namespace {
-template <bool FP8, bool PLAIN>
+template <bool FP8, bool PLAIN, bool NARROW>
 cudaError_t launch_form(const GemmParams& p, const CUtensorMap& m_a, const CUtensorMap& m_b, cudaStream_t st) {
   // per device; several host threads may get here at once: setting the attribute twice is harmless
   static std::atomic<bool> attr_set[MAX_DEVICES];
   const int dev = current_device();
   if (!attr_set[dev].load(std::memory_order_acquire)) {
-    cudaError_t e = cudaFuncSetAttribute(ffn_gemm1_kernel<FP8, PLAIN>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+    cudaError_t e = cudaFuncSetAttribute(ffn_gemm1_kernel<FP8, PLAIN, NARROW>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                          SMEM_BYTES);
     if (e != cudaSuccess) return e;
     attr_set[dev].store(true, std::memory_order_release);
   }
   ProfileScope prof(PLAIN ? KID_GEMM2 : KID_GEMM1, st);
-  return launch_pdl(ffn_gemm1_kernel<FP8, PLAIN>, sm_count(), THREADS, SMEM_BYTES, st, m_a, m_b, p);
+  return launch_pdl(ffn_gemm1_kernel<FP8, PLAIN, NARROW>, sm_count(), THREADS, SMEM_BYTES, st, m_a, m_b, p);
 }
 }  // namespace
 
-cudaError_t launch_gemm1(const GemmParams& p, const CUtensorMap& m_w1, const CUtensorMap& m_w3, bool fp8,
+// narrow: 64 output columns per tile instead of 128 (GEMM-1) or 256 (GEMM-2); p.n_tiles is set here.  The FP8 weight maps then
+// have boxes of 64 columns (make_weight_map_fp8).
+cudaError_t launch_gemm1(GemmParams p, const CUtensorMap& m_w1, const CUtensorMap& m_w3, bool fp8, bool narrow,
                          cudaStream_t st) {
-  return fp8 ? launch_form<true, false>(p, m_w1, m_w3, st) : launch_form<false, false>(p, m_w1, m_w3, st);
+  p.n_tiles = narrow ? (p.N + 63) / 64 : (p.N + 127) / 128;
+  if (fp8) return narrow ? launch_form<true, false, true>(p, m_w1, m_w3, st) : launch_form<true, false, false>(p, m_w1, m_w3, st);
+  return narrow ? launch_form<false, false, true>(p, m_w1, m_w3, st) : launch_form<false, false, false>(p, m_w1, m_w3, st);
 }
 
 // GEMM-2 through the single-CTA kernel (128-row tiles): p.a_src = h (or its E4M3 copy), p.a_ld = f,
-// p.tile_prefix = the 128-row tile prefix, p.n_tiles = ceil(N / 256); m_w2 is the weight map.
-cudaError_t launch_gemm2_single(const GemmParams& p, const CUtensorMap& m_w2, bool fp8, cudaStream_t st) {
-  return fp8 ? launch_form<true, true>(p, m_w2, m_w2, st) : launch_form<false, true>(p, m_w2, m_w2, st);
+// p.tile_prefix = the 128-row tile prefix; m_w2 is the weight map.
+cudaError_t launch_gemm2_single(GemmParams p, const CUtensorMap& m_w2, bool fp8, bool narrow, cudaStream_t st) {
+  p.n_tiles = narrow ? (p.N + 63) / 64 : (p.N + 255) / 256;
+  if (fp8) return narrow ? launch_form<true, true, true>(p, m_w2, m_w2, st) : launch_form<true, true, false>(p, m_w2, m_w2, st);
+  return narrow ? launch_form<false, true, true>(p, m_w2, m_w2, st) : launch_form<false, true, false>(p, m_w2, m_w2, st);
 }
 
 }  // namespace ffn

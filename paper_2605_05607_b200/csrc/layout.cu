@@ -139,12 +139,12 @@ __global__ void __launch_bounds__(256) fill_layout_kernel(const int32_t* __restr
 }
 
 // ---- K2 in one kernel ----------------------------------------------------------------------------
-// The four passes above as one kernel of at most 8 thread blocks (a cluster), for up to 32768 pairs (a sparse table: 131072 slots): every block owns a
+// The four passes above as one kernel of at most 8 thread blocks (a cluster), for up to 32768 pairs: every block owns a
 // contiguous range of tokens, builds its masks and their prefixes in shared memory, reads the other blocks' row totals through
 // distributed shared memory and fills its tokens' entries.  The four launches are latency, not work: 16 us of device time and
 // three launch gaps for 256 tokens of top-2, 21 us for 3001 of top-4; in one kernel 6.2 and 9.5 us.  With more pairs the
-// scattered table stores of the fill pass want more than 8 SMs (16384 tokens of top-8: 29 us as four kernels); the slots of a
-// sparse table are mostly unused and cost a read only, so its limit is four times as high.
+// scattered table stores of the fill pass want more than 8 SMs (16384 tokens of top-8: 29 us as four kernels; 10880 tokens of a sparse
+// top-8 table: 19 us either way).
 constexpr int ONE_THREADS = 1024, ONE_MAX_BLOCKS = 8, ONE_MAX_PAIRS = 32768;
 struct OneShape { int blocks, tokens, words; size_t smem; };   // tokens per block (a multiple of 32) and their mask words
 OneShape one_shape(const Shape& s) {
@@ -282,7 +282,7 @@ __global__ void __launch_bounds__(ONE_THREADS) layout_one_kernel(const int32_t* 
 }
 
 bool layout_in_one(const Shape& s) {
-  return s.T > 0 && (long long)s.T * s.k <= ((s.flags & 4) ? 4 : 1) * ONE_MAX_PAIRS && one_shape(s).smem <= 160 * 1024;
+  return s.T > 0 && (long long)s.T * s.k <= ONE_MAX_PAIRS && one_shape(s).smem <= 160 * 1024;
 }
 
 // exclusive prefixes of 128-row tiles and 256-row pair tiles per expert, from the counts alone

@@ -33,9 +33,9 @@ def test_layout_builders(T, E, k, G):
     assert B.moe_status(ws)[0] == 0
 
 
-@pytest.mark.parametrize("T", [8192, 16384, 16385])
+@pytest.mark.parametrize("T", [4096, 4097])
 def test_layout_of_a_sparse_table(T):
-    """Unused slots (-1): one kernel up to 131072 slots, four beyond; both against the same layout built slot by slot."""
+    """Unused slots (-1): one kernel up to 32768 slots, four beyond; both against the same layout built slot by slot."""
     E, k = 16, 8
     rng = np.random.default_rng(T)
     idx = np.argsort(rng.random((T, E)), axis=1)[:, :k].astype(np.int32)

@@ -571,3 +571,31 @@ def test_tensor_map_cache_is_transparent():
                              H.bf16_host(r2.t["w3"]), H.bf16_host(r2.t["w2"]), cfg2.k, cfg2.score_fn)
     H.assert_close_out(O.bf16_to_f64(H.bf16_host(r2.y)[: cfg2.T]), y_def, "layer after cache churn")
     assert r2.status()[0] == 0
+
+
+@pytest.mark.parametrize("fp8", [False, True], ids=["bf16", "fp8"])
+@pytest.mark.parametrize("T", [1, 33, 300])
+def test_narrow_gemm_tiles_give_the_same_bits(T, fp8):
+    """With few tiles the GEMMs run on tiles of 64 output columns.  A token's output depends on nothing but the token, so the
+    first rows of a batch that is large enough for full-width tiles are the same bits (ragged K and N, two row tiles)."""
+    big = synth.MoEConfig("wide", T=1020, d=2064, f=1008, E=4, k=2, G=2, seed=31)
+    t = synth.make_inputs(big, "cuda")
+    if fp8:
+        q = {}
+        for n in ("w1", "w3", "w2"):
+            q[n] = torch.empty(big.E, t[n].shape[2], t[n].shape[1], dtype=torch.uint8, device="cuda")
+            q["s" + n] = torch.empty(big.E, t[n].shape[2], dtype=torch.float32, device="cuda")
+            B.moe_quantize_weights(t[n], q[n], q["s" + n])
+
+    def layer(n):
+        shape = B.make_shape(big.with_(T=n))
+        ws, y = B.alloc_workspace(shape), torch.empty(n, big.d, dtype=torch.bfloat16, device="cuda")
+        x = t["x"][:n].contiguous()
+        if fp8:
+            B.moe_layer_fp8(shape, x, t["w_gate"], None, q["w1"], q["sw1"], q["w3"], q["sw3"], q["w2"], q["sw2"], y, ws)
+        else:
+            B.moe_layer(shape, x, t["w_gate"], None, t["w1"], t["w3"], t["w2"], y, ws)
+        assert B.moe_status(ws)[0] == 0
+        return y
+
+    assert torch.equal(layer(T), layer(big.T)[:T])
