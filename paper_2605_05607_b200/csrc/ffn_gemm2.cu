@@ -17,7 +17,7 @@
 // Barrier ownership in a pair:
 //   full[s]    leader's copy: the leader announces the bytes of both CTAs, both CTAs' TMA loads
 //              credit it
-//   empty[s]   each CTA's own copy, signalled by the leader's tcgen05.commit (one commit per CTA)
+//   empty[s]   each CTA's own copy, signalled by the leader's tcgen05.commit
 //   tfull[b]   each CTA's own copy (accumulator buffer b complete), same
 //   tempty[b]  leader's copy: the 4 epilogue warps of each CTA arrive when buffer b is drained
 //
@@ -409,43 +409,42 @@ ffn_gemm2_kernel(const __grid_constant__ CUtensorMap map_b0, const __grid_consta
     }
   } else if (warp == 5) {
     // ================================ UMMA issuer (leader CTA only) ================================
-    if (rank == 0 && lane == 0) {
-      const uint64_t a_base = desc_base(16, 1024);
-      const uint64_t b_base = KMAJ ? desc_base(16, 1024) : desc_base(BK * 128, 1024);   // K-major : MN-major
-      uint32_t it = 0;
-      int tl = 0;
-      for (int w = cluster_id; w < total && !*abort_flag; w += num_clusters, ++tl) {
+    // the warp walks the loop, one elected lane issues (see ptx::elect_one)
+    if (rank == 0) {
+      const bool elected = ptx::elect_one();
+      const uint32_t base = __shfl_sync(0xFFFFFFFFu, smem_base, 0), tmem = __shfl_sync(0xFFFFFFFFu, tmem_base, 0);
+      const uint64_t mn = desc_base(BK * 128, 1024), km = desc_base(16, 1024);   // MN-major, K-major
+      const uint64_t a_desc = desc_at(WGRAD ? mn : km, base), b_desc = desc_at(KMAJ ? km : mn, base + A_BYTES);
+      constexpr int A_STEP = WGRAD ? 128 : 2, B_STEP = KMAJ ? 2 : 128;            // 32 bytes of K: 16 bf16 / 32 E4M3
+      constexpr uint32_t ID = FP8 ? IDESC_F8 : WGRAD ? IDESC_WG : BKMAJ ? IDESC_BK : IDESC;
+      int s = 0, tl = 0;
+      uint32_t ph = 0;
+      bool ok = true;
+      for (int w = cluster_id; ok && w < total && !*abort_flag; w += num_clusters, ++tl) {
         const int buf = tl & 1;
         if (!ptx::mbar_wait_cluster<HINT>(tempty_bar(buf), ((tl >> 1) & 1) ^ 1, abort_flag, global_abort)) {
           timeout(3); break;
         }
         ptx::tc_fence_after();
-        const uint32_t d_tmem = tmem_base + (uint32_t)(buf * UMMA_N);
-        bool ok = true;
+        const uint32_t d_tmem = tmem + (uint32_t)(buf * UMMA_N);
         const int KBt = WGRAD ? tile_of(w).kb : KB;
-        for (int kb = 0; kb < KBt; ++kb, ++it) {
-          const int s = it % NSTAGE;
-          if (!ptx::mbar_wait_cluster<HINT>(full_bar(s), (it / NSTAGE) & 1, abort_flag, global_abort)) {
+        for (int kb = 0; kb < KBt; ++kb) {
+          if (!ptx::mbar_wait_cluster<HINT>(full_bar(s), ph, abort_flag, global_abort)) {
             timeout(4); ok = false; break;
           }
           ptx::tc_fence_after();
-          const uint32_t sa = smem_base + s * STAGE_BYTES, sb = sa + A_BYTES;
-          const uint64_t ad = desc_at(WGRAD ? b_base : a_base, sa), bd = desc_at(b_base, sb);   // WGRAD: A is MN-major too
-          auto bd_a = [](uint64_t d, int k) { return d + (uint64_t)(k * 128); };               // 16 rows of K = 2 KiB
+          if (elected) {
+            const uint64_t ad = a_desc + (uint64_t)(s * (STAGE_BYTES >> 4)), bd = b_desc + (uint64_t)(s * (STAGE_BYTES >> 4));
 #pragma unroll
-          for (int k = 0; k < 4; ++k) {   // 32 bytes of K per UMMA (16 bf16 / 32 E4M3): +32 B inside the swizzle row
-            if (FP8) ptx::umma_f8_pair(d_tmem, ad + (uint64_t)(k * 2), bd + (uint64_t)(k * 2), IDESC_F8, (kb | k) != 0);
-            else if (WGRAD) ptx::umma_bf16_pair(d_tmem, bd_a(ad, k), bd + (uint64_t)(k * 128), IDESC_WG, (kb | k) != 0);
-            else if (BKMAJ) ptx::umma_bf16_pair(d_tmem, ad + (uint64_t)(k * 2), bd + (uint64_t)(k * 2), IDESC_BK, (kb | k) != 0);
-            else ptx::umma_bf16_pair(d_tmem, ad + (uint64_t)(k * 2), bd + (uint64_t)(k * 128), IDESC, (kb | k) != 0);   // B: +2 atoms
+            for (int k = 0; k < 4; ++k) {
+              if (FP8) ptx::umma_f8_pair(d_tmem, ad + (uint64_t)(k * A_STEP), bd + (uint64_t)(k * B_STEP), ID, (kb | k) != 0);
+              else ptx::umma_bf16_pair(d_tmem, ad + (uint64_t)(k * A_STEP), bd + (uint64_t)(k * B_STEP), ID, (kb | k) != 0);
+            }
+            ptx::umma_commit_both(empty_bar(s));   // free the stage in both CTAs once these UMMAs have read it
           }
-          // free the stage in both CTAs once these UMMAs have read it
-          ptx::umma_commit_pair(ptx::mapa(empty_bar(s), 0));
-          ptx::umma_commit_pair(ptx::mapa(empty_bar(s), 1));
+          if (++s == NSTAGE) { s = 0; ph ^= 1u; }
         }
-        if (!ok) break;
-        ptx::umma_commit_pair(ptx::mapa(tfull_bar(buf), 0));   // accumulator complete, both halves
-        ptx::umma_commit_pair(ptx::mapa(tfull_bar(buf), 1));
+        if (ok && elected) ptx::umma_commit_both(tfull_bar(buf));   // accumulator complete, both halves
       }
     }
   }
