@@ -19,9 +19,11 @@
 //              credit it
 //   empty[s]   each CTA's own copy, signalled by the leader's tcgen05.commit
 //   tfull[b]   each CTA's own copy (accumulator buffer b complete), same
-//   tempty[b]  leader's copy: the 4 epilogue warps of each CTA arrive when buffer b is drained
+//   tempty[b]  leader's copy: the 8 epilogue warps of each CTA arrive when buffer b is drained
 //
-// Warp roles: 0-3 epilogue, 4 TMA producer, 5 UMMA issuer (leader only) and TMEM owner.
+// Warp roles: 0-7 epilogue, 8 TMA producer, 9 UMMA issuer (leader only) and TMEM owner.  Eight epilogue warps (two per row
+// quarter, half of the columns each): with four, a tile's epilogue took 4500-6400 cycles and bound every short K walk
+// (weight gradients of experts with a hundred rows; FP8 with K = 1536, whose main loop is 6100 cycles).
 // Accumulators are double-buffered in TMEM; every wait is bounded; neither CTA retires before its
 // peer has stopped touching its shared memory and TMEM (cluster barrier at the end).
 #include "ffn_common.cuh"
@@ -37,12 +39,13 @@ constexpr int A_BYTES = BM * BK * 2;            // 16 KiB: this CTA's 128 rows
 constexpr int B_BYTES = (UMMA_N / 2) * BK * 2;  // 16 KiB: this CTA's half of the B tile (two 64-column slabs)
 constexpr int STAGE_BYTES = A_BYTES + B_BYTES;
 constexpr int NUM_BARS = 2 * NSTAGE + 4;
-constexpr int STAGE_OUT_WARP = 32 * 144;          // epilogue transpose buffer of one warp: 32 rows x (128 + 16) bytes
+constexpr int EPI_WARPS = 8, TMA_WARP = EPI_WARPS, MMA_WARP = EPI_WARPS + 1;
+constexpr int STAGE_OUT_WARP = 32 * 64;           // epilogue transpose buffer of one warp: 32 rows x 32 columns, swizzled
 constexpr int TABLE_BYTES = (2 * (MAX_E + 1) * 4 + 15) & ~15;
-constexpr int COLSCALE_WARP = UMMA_N * 4;          // FP8: one warp's copy of the tile's 256 output-column scales
+constexpr int COLSCALE_WARP = UMMA_N / 2 * 4;      // FP8: the scales of the 128 output columns that a warp owns
 constexpr int SMEM_BYTES =
-    1024 + NSTAGE * STAGE_BYTES + NUM_BARS * 8 + 64 + TABLE_BYTES + 4 * STAGE_OUT_WARP + 4 * COLSCALE_WARP;
-constexpr int THREADS = 192;
+    1024 + NSTAGE * STAGE_BYTES + NUM_BARS * 8 + 64 + TABLE_BYTES + EPI_WARPS * (STAGE_OUT_WARP + COLSCALE_WARP);
+constexpr int THREADS = (EPI_WARPS + 2) * 32;
 constexpr uint32_t IDESC = idesc_bf16(2 * BM);
 constexpr uint32_t IDESC_F8 = idesc_e4m3(2 * BM);
 constexpr uint32_t IDESC_BK = idesc_bf16(2 * BM) & ~(1u << 16);   // bf16 with a K-major B operand
@@ -90,7 +93,7 @@ ffn_gemm2_kernel(const __grid_constant__ CUtensorMap map_b0, const __grid_consta
   int* tp_s = reinterpret_cast<int*>(tmem_slot + 16);
   int* eoff_s = tp_s + (MAX_E + 1);
   const uint32_t stage_base = ptx::smem_u32(tp_s) + TABLE_BYTES;   // 16-byte aligned
-  float* colscale_base = reinterpret_cast<float*>(reinterpret_cast<uint8_t*>(tp_s) + TABLE_BYTES + 4 * STAGE_OUT_WARP);
+  float* colscale_base = reinterpret_cast<float*>(reinterpret_cast<uint8_t*>(tp_s) + TABLE_BYTES + EPI_WARPS * STAGE_OUT_WARP);
 
   const uint32_t smem_base = ptx::smem_u32(smem);
   const uint32_t bar_base = ptx::smem_u32(bars);
@@ -110,17 +113,17 @@ ffn_gemm2_kernel(const __grid_constant__ CUtensorMap map_b0, const __grid_consta
     }
     for (int b = 0; b < 2; ++b) {
       ptx::mbar_init(tfull_bar(b), 1);      // tcgen05.commit
-      ptx::mbar_init(tempty_bar(b), 8);     // one lane per epilogue warp, both CTAs
+      ptx::mbar_init(tempty_bar(b), 2 * EPI_WARPS);   // one lane per epilogue warp, both CTAs
     }
     ptx::fence_mbar_init();
   }
-  if (warp == 4 && lane == 0) {
+  if (warp == TMA_WARP && lane == 0) {
     ptx::prefetch_tensormap(&map_b0);
     ptx::prefetch_tensormap(&map_b1);
     ptx::prefetch_tensormap(&map_h);
     if (MODE == PAIR_KSPLIT) ptx::prefetch_tensormap(&map_a1);
   }
-  if (warp == 5) {
+  if (warp == MMA_WARP) {
     ptx::tmem_alloc_pair(ptx::smem_u32(tmem_slot), 512);
     ptx::tmem_relinquish_pair();
   }
@@ -164,44 +167,70 @@ ffn_gemm2_kernel(const __grid_constant__ CUtensorMap map_b0, const __grid_consta
     return decode_tile(w, tp_s, eoff_s, p.E, p.n_tiles, BN_OUT, 2 * BM, rank);
   };
 
-  if (warp < 4) {
+  if (warp < EPI_WARPS) {
     // ================================ epilogue (both CTAs) ================================
+    const int quarter = warp & 3, half = warp >> 2;   // rows (TMEM lanes) and half of the columns this warp owns
+    constexpr int COLS = BN_OUT / 2;                  // output columns of a warp
+    // A thread owns one accumulator row, but 32 threads storing 16 bytes each to 32 different rows cost 32 memory
+    // transactions per instruction.  The warp transposes 32 columns at a time through shared memory (64-byte rows, pieces
+    // swizzled by row pair: conflict-free both ways) and stores 64-byte row segments, 8 rows per instruction.
+    const uint32_t stage = stage_base + (uint32_t)(warp * STAGE_OUT_WARP);
+    const int srow = lane >> 2, piece = lane & 3;
+    auto put = [&](int v, uint32_t q0, uint32_t q1, uint32_t q2, uint32_t q3) {   // columns 8 v .. + 7 of this thread's row
+      ptx::st_shared_v4(stage + lane * 64 + ((v ^ ((lane >> 1) & 3)) << 4), q0, q1, q2, q3);
+    };
     int tl = 0;
     for (int w = cluster_id; w < total && !*abort_flag; w += num_clusters, ++tl) {
       const Tile t = tile_of(w);
       const int buf = tl & 1;
       if (!ptx::mbar_wait_warp<false, HINT>(tfull_bar(buf), (tl >> 1) & 1, abort_flag, global_abort)) { timeout(1); break; }
       ptx::tc_fence_after();
-      const int lrow = warp * 32 + lane;
+      const int lrow = quarter * 32 + lane;
       const bool valid = lrow < t.rows;
       const size_t grow = (size_t)(valid ? t.row0 + lrow : 0);
-      const uint32_t taddr = tmem_base + ((uint32_t)(warp * 32) << 16) + (uint32_t)(buf * UMMA_N);
+      const int col0 = t.n0 + half * COLS;            // first output column of this warp
+      const uint32_t taddr = tmem_base + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(buf * UMMA_N + half * COLS);
+      auto send = [&](int c) {                        // 32 staged columns -> rows of out
+        __syncwarp();
+        const int col = col0 + c * 32 + piece * 8;
+        if (col < p.N) {
+#pragma unroll
+          for (int i = 0; i < 4; ++i) {
+            const int r = i * 8 + srow;               // row of this warp's 32
+            if (quarter * 32 + r < t.rows) {
+              const uint4 q = ptx::ld_shared_v4(stage + r * 64 + ((piece ^ ((r >> 1) & 3)) << 4));
+              *reinterpret_cast<uint4*>(p.out + (size_t)(t.out_row0 + quarter * 32 + r) * (size_t)p.out_ld + col) = q;
+            }
+          }
+        }
+        __syncwarp();
+      };
       float* yrow = nullptr;
       float wr = 1.f;
       if (valid && !GLU && !WGRAD && (RED || p.topk_w != nullptr)) {
         const int pair = __ldg(p.row_pair + grow);
         if (p.topk_w != nullptr) wr = __ldg(p.topk_w + pair);
         if (FP8) wr *= __ldg(p.a_scale + grow);   // row scale of h joins the gate weight
-        if (RED) yrow = p.y_acc + (size_t)(pair / p.y_div) * (size_t)p.N + t.n0;
+        if (RED) yrow = p.y_acc + (size_t)(pair / p.y_div) * (size_t)p.N + col0;
       }
       // FP8: the tile's output-column scales, one copy per warp (0 beyond N), staged while the
       // main loop of this tile may still be running
-      float* sb_col = colscale_base + warp * UMMA_N;
+      float* sb_col = colscale_base + warp * (UMMA_N / 2);
       if (FP8) {
-        const float* g = p.b_scale + (size_t)t.e * p.N + t.n0;
+        const float* g = p.b_scale + (size_t)t.e * p.N + col0;
 #pragma unroll
-        for (int i = 0; i < UMMA_N / 32; ++i) {
+        for (int i = 0; i < COLS / 32; ++i) {
           const int n = lane + 32 * i;
-          sb_col[n] = (t.n0 + n < p.N) ? __ldg(g + n) : 0.f;
+          sb_col[n] = (col0 + n < p.N) ? __ldg(g + n) : 0.f;
         }
         __syncwarp();
       }
       if (MODE == PAIR_GLU_BWD) {
-        // backward of SwiGLU on the recomputed pre-activations: a thread owns one row and walks its 128 columns 32 at
+        // backward of SwiGLU on the recomputed pre-activations: a thread owns one row and walks its 64 columns 32 at
         // a time; dh comes from global memory (64 bytes of the row per step), h / da1 / da3 go straight back
-        const size_t rowoff = grow * (size_t)p.out_ld + t.n0;
+        const size_t rowoff = grow * (size_t)p.out_ld + col0;
 #pragma unroll 1
-        for (int c = 0; c < 4; ++c) {
+        for (int c = 0; c < 2; ++c) {
           uint32_t a1[32], a3[32];
           ptx::tmem_ld32(taddr + c * 32, a1);
           ptx::tmem_ld32(taddr + 128 + c * 32, a3);
@@ -209,7 +238,7 @@ ffn_gemm2_kernel(const __grid_constant__ CUtensorMap map_b0, const __grid_consta
           if (valid) {
 #pragma unroll
             for (int v = 0; v < 4; ++v) {
-              const int col = t.n0 + c * 32 + v * 8;
+              const int col = col0 + c * 32 + v * 8;
               if (col < p.N) {
                 const size_t at = rowoff + c * 32 + v * 8;
                 const uint4 dq = *reinterpret_cast<const uint4*>(p.dh + at);
@@ -242,12 +271,9 @@ ffn_gemm2_kernel(const __grid_constant__ CUtensorMap map_b0, const __grid_consta
           }
         }
       } else if (GLU) {
-        // SwiGLU of the W1 half (columns 0..127) and the W3 half (128..255): 128 columns of h, transposed
-        // through shared memory 64 columns at a time and stored as whole 128-byte row segments
-        const uint32_t stage = stage_base + (uint32_t)(warp * STAGE_OUT_WARP);
-        const int srow = lane >> 3, piece = lane & 7;
+        // SwiGLU of the W1 half (accumulator columns 0..127) and the W3 half (128..255)
 #pragma unroll 1
-        for (int c = 0; c < 4; ++c) {
+        for (int c = 0; c < 2; ++c) {
           uint32_t a1[32], a3[32];
           ptx::tmem_ld32(taddr + c * 32, a1);
           ptx::tmem_ld32(taddr + 128 + c * 32, a3);
@@ -261,27 +287,13 @@ ffn_gemm2_kernel(const __grid_constant__ CUtensorMap map_b0, const __grid_consta
               q[i] = pack2(silu_mul(__uint_as_float(a1[j]), __uint_as_float(a3[j])),
                            silu_mul(__uint_as_float(a1[j + 1]), __uint_as_float(a3[j + 1])));
             }
-            ptx::st_shared_v4(stage + lane * 144 + (c & 1) * 64 + v * 16, q[0], q[1], q[2], q[3]);
+            put(v, q[0], q[1], q[2], q[3]);
           }
-          if (c & 1) {
-            __syncwarp();
-            const int col = t.n0 + (c - 1) * 32 + piece * 8;
-            if (col < p.N) {
-#pragma unroll
-              for (int i = 0; i < 8; ++i) {
-                const int r = i * 4 + srow;
-                if (warp * 32 + r < t.rows) {
-                  const uint4 q = ptx::ld_shared_v4(stage + r * 144 + piece * 16);
-                  *reinterpret_cast<uint4*>(p.out + (size_t)(t.row0 + warp * 32 + r) * (size_t)p.out_ld + col) = q;
-                }
-              }
-            }
-            __syncwarp();
-          }
+          send(c);
         }
       } else if (RED) {
 #pragma unroll 1
-        for (int c = 0; c < 8; ++c) {
+        for (int c = 0; c < 4; ++c) {
           uint32_t acc[32];
           ptx::tmem_ld32(taddr + c * 32, acc);
           ptx::tmem_ld_wait();
@@ -295,7 +307,7 @@ ffn_gemm2_kernel(const __grid_constant__ CUtensorMap map_b0, const __grid_consta
           if (valid) {
 #pragma unroll
             for (int v = 0; v < 4; ++v) {
-              if (t.n0 + c * 32 + v * 8 < p.N) {
+              if (col0 + c * 32 + v * 8 < p.N) {
                 float* dst = yrow + c * 32 + v * 8;
                 ptx::red_add_v4(dst, wr * __uint_as_float(acc[v * 8]), wr * __uint_as_float(acc[v * 8 + 1]),
                                 wr * __uint_as_float(acc[v * 8 + 2]), wr * __uint_as_float(acc[v * 8 + 3]));
@@ -306,57 +318,26 @@ ffn_gemm2_kernel(const __grid_constant__ CUtensorMap map_b0, const __grid_consta
           }
         }
       } else {
-        // A thread owns one accumulator row, but 32 threads storing 16 bytes each to 32 different
-        // rows cost 32 memory transactions per instruction.  The warp therefore transposes 64
-        // columns at a time through shared memory (rows padded to 144 bytes: conflict-free both
-        // ways) and stores whole 128-byte row segments, 8 lanes per row, 4 rows per instruction.
-        const uint32_t stage = stage_base + (uint32_t)(warp * STAGE_OUT_WARP);
-        const int srow = lane >> 3, piece = lane & 7;
 #pragma unroll 1
-        for (int cc = 0; cc < 4; ++cc) {
-          uint32_t acc0[32], acc1[32];
-          ptx::tmem_ld32(taddr + cc * 64, acc0);
-          ptx::tmem_ld32(taddr + cc * 64 + 32, acc1);
-          ptx::tmem_ld_wait_on(acc0);
-          ptx::tmem_ld_wait_on(acc1);
+        for (int c = 0; c < 4; ++c) {
+          uint32_t acc[32];
+          ptx::tmem_ld32(taddr + c * 32, acc);
+          ptx::tmem_ld_wait_on(acc);
           if (WGRAD && t.kb == 0) {   // an expert without rows: the accumulator was never written
 #pragma unroll
-            for (int j = 0; j < 32; ++j) { acc0[j] = 0u; acc1[j] = 0u; }
+            for (int j = 0; j < 32; ++j) acc[j] = 0u;
           }
           if (FP8) {   // per-output-column weight scales
 #pragma unroll
-            for (int j = 0; j < 32; ++j) {
-              const int n = cc * 64 + j;
-              acc0[j] = __float_as_uint(__uint_as_float(acc0[j]) * sb_col[n]);
-              acc1[j] = __float_as_uint(__uint_as_float(acc1[j]) * sb_col[n + 32]);
-            }
+            for (int j = 0; j < 32; ++j) acc[j] = __float_as_uint(__uint_as_float(acc[j]) * sb_col[c * 32 + j]);
           }
 #pragma unroll
-          for (int v = 0; v < 4; ++v) {
-            ptx::st_shared_v4(stage + lane * 144 + v * 16,
-                              pack2(wr * __uint_as_float(acc0[v * 8]), wr * __uint_as_float(acc0[v * 8 + 1])),
-                              pack2(wr * __uint_as_float(acc0[v * 8 + 2]), wr * __uint_as_float(acc0[v * 8 + 3])),
-                              pack2(wr * __uint_as_float(acc0[v * 8 + 4]), wr * __uint_as_float(acc0[v * 8 + 5])),
-                              pack2(wr * __uint_as_float(acc0[v * 8 + 6]), wr * __uint_as_float(acc0[v * 8 + 7])));
-            ptx::st_shared_v4(stage + lane * 144 + 64 + v * 16,
-                              pack2(wr * __uint_as_float(acc1[v * 8]), wr * __uint_as_float(acc1[v * 8 + 1])),
-                              pack2(wr * __uint_as_float(acc1[v * 8 + 2]), wr * __uint_as_float(acc1[v * 8 + 3])),
-                              pack2(wr * __uint_as_float(acc1[v * 8 + 4]), wr * __uint_as_float(acc1[v * 8 + 5])),
-                              pack2(wr * __uint_as_float(acc1[v * 8 + 6]), wr * __uint_as_float(acc1[v * 8 + 7])));
-          }
-          __syncwarp();
-          const int col = t.n0 + cc * 64 + piece * 8;
-          if (col < p.N) {
-#pragma unroll
-            for (int i = 0; i < 8; ++i) {
-              const int r = i * 4 + srow;           // row of this warp's 32
-              if (warp * 32 + r < t.rows) {
-                const uint4 q = ptx::ld_shared_v4(stage + r * 144 + piece * 16);
-                *reinterpret_cast<uint4*>(p.out + (size_t)(t.out_row0 + warp * 32 + r) * (size_t)p.out_ld + col) = q;
-              }
-            }
-          }
-          __syncwarp();
+          for (int v = 0; v < 4; ++v)
+            put(v, pack2(wr * __uint_as_float(acc[v * 8]), wr * __uint_as_float(acc[v * 8 + 1])),
+                pack2(wr * __uint_as_float(acc[v * 8 + 2]), wr * __uint_as_float(acc[v * 8 + 3])),
+                pack2(wr * __uint_as_float(acc[v * 8 + 4]), wr * __uint_as_float(acc[v * 8 + 5])),
+                pack2(wr * __uint_as_float(acc[v * 8 + 6]), wr * __uint_as_float(acc[v * 8 + 7])));
+          send(c);
         }
       }
       ptx::tc_fence_before();
@@ -367,7 +348,7 @@ ffn_gemm2_kernel(const __grid_constant__ CUtensorMap map_b0, const __grid_consta
       // (K = 512: 860 -> 1049 TFLOP/s with the relaxed form)
       if (lane == 0) ptx::mbar_arrive_cluster_relaxed(ptx::mapa(tempty_bar(buf), 0));
     }
-  } else if (warp == 4) {
+  } else if (warp == TMA_WARP) {
     // ================================ TMA producer (both CTAs) ================================
     if (lane == 0) {
       uint32_t it = 0;
@@ -407,7 +388,7 @@ ffn_gemm2_kernel(const __grid_constant__ CUtensorMap map_b0, const __grid_consta
         if (!ok) break;
       }
     }
-  } else if (warp == 5) {
+  } else if (warp == MMA_WARP) {
     // ================================ UMMA issuer (leader CTA only) ================================
     // the warp walks the loop, one elected lane issues (see ptx::elect_one)
     if (rank == 0) {
@@ -456,7 +437,7 @@ ffn_gemm2_kernel(const __grid_constant__ CUtensorMap map_b0, const __grid_consta
     for (int i = 0; i < 64; ++i) __nanosleep(1000);
   }
   ptx::cluster_sync();   // neither CTA leaves while its peer may still touch its shared memory / TMEM
-  if (warp == 5) {
+  if (warp == MMA_WARP) {
     ptx::tc_fence_after();
     ptx::tmem_dealloc_pair(tmem_base, 512);
   }
