@@ -17,41 +17,96 @@ __device__ __forceinline__ uint8_t to_e4m3(float v, float scale) {
 }
 __device__ __forceinline__ float scale_of(float amax) { return amax == 0.f ? 1.f : __fdiv_rn(amax, 448.f); }
 
-// One warp per row: pass 1 takes max|v| (16-byte loads), pass 2 re-reads the row (L1 / L2) and
-// writes 8 codes per lane per step.  cols % 8 == 0.
-__global__ void __launch_bounds__(256) quantize_rows_kernel(const uint4* __restrict__ src, uint2* __restrict__ dst,
+// Two codes at once, the low byte that of `a`.  fl32(v / scale) comes from the reciprocal, which the whole row shares, by
+// Markstein's correction (P. Markstein, "Computation of elementary functions on the IBM RISC System/6000 processor", IBM J. Res.
+// Dev. 34, 1990): with inv = RN(1 / s) and q within an ulp of v / s, RN(q + (v - q s) * inv), the residual exact, is RN(v / s) as long
+// as nothing leaves the normal range.  Values so small that the residual does round to code 0 either way.  (Taking the code
+// where both ends of an error interval around v * inv agree was no faster than dividing: quotients of 8-bit significands
+// tie exactly too often, and one lane's division stops its warp.)
+__device__ __forceinline__ uint32_t to_e4m3_pair(float a, float b, float inv, float scale) {
+  float qa = a * inv, qb = b * inv;
+#pragma unroll
+  for (int i = 0; i < 2; ++i) {   // the first step makes q faithful, the second is the one that rounds correctly
+    qa = fmaf(fmaf(-qa, scale, a), inv, qa);
+    qb = fmaf(fmaf(-qb, scale, b), inv, qb);
+  }
+  return __nv_cvt_float2_to_fp8x2(make_float2(copysignf(qa, a), copysignf(qb, b)),   // -0 stays -0
+                                  __NV_SATFINITE, __NV_E4M3);
+}
+// WARPS warps per row (1, or the whole block of 4 for long rows).  The row stays in registers between the maximum and the codes
+// when it has at most KEEP vectors per lane; a longer one is read again.  cols % 8 == 0.  Bound by memory now, by the divisions
+// before: 131072 rows of 1536 columns 159 -> 104 us (5.8 TB/s), 16384 of 4096 65 -> 50, 32768 of 7168 201 -> 132 (5.3 TB/s).
+template <int KEEP, int WARPS>
+__global__ void __launch_bounds__(WARPS == 1 ? 256 : WARPS * 32) quantize_rows_kernel(const uint4* __restrict__ src, uint2* __restrict__ dst,
                                                             float* __restrict__ scale, long long rows, int vec_per_row) {
   grid_dependency_sync();
-  const int lane = threadIdx.x & 31;
-  const long long wpb = blockDim.x >> 5;
-  for (long long r = blockIdx.x * wpb + (threadIdx.x >> 5); r < rows; r += (long long)gridDim.x * wpb) {
-    const uint4* row = src + r * vec_per_row;
-    float amax = 0.f;
-    for (int v = lane; v < vec_per_row; v += 32) {
-      const uint4 raw = __ldg(row + v);
-      const __nv_bfloat162* p = reinterpret_cast<const __nv_bfloat162*>(&raw);
+  __shared__ float amax_s[WARPS];
+  constexpr int LANES = WARPS * 32;
+  const int lane = WARPS == 1 ? threadIdx.x & 31 : threadIdx.x;   // of the row's threads
+  const long long rpb = blockDim.x / LANES;
+  auto amax_of = [](const uint4& raw, float amax) {
+    const __nv_bfloat162* p = reinterpret_cast<const __nv_bfloat162*>(&raw);
 #pragma unroll
-      for (int q = 0; q < 4; ++q) {
-        const float2 f = __bfloat1622float2(p[q]);
-        amax = fmaxf(amax, fmaxf(fabsf(f.x), fabsf(f.y)));
-      }
+    for (int q = 0; q < 4; ++q) {
+      const float2 f = __bfloat1622float2(p[q]);
+      amax = fmaxf(amax, fmaxf(fabsf(f.x), fabsf(f.y)));
     }
+    return amax;
+  };
+  for (long long r = blockIdx.x * rpb + (WARPS == 1 ? threadIdx.x >> 5 : 0); r < rows; r += (long long)gridDim.x * rpb) {
+    const uint4* row = src + r * vec_per_row;
+    uint4 keep[KEEP];
+    float amax = 0.f;
+#pragma unroll
+    for (int i = 0; i < KEEP; ++i)
+      keep[i] = lane + LANES * i < vec_per_row ? __ldg(row + lane + LANES * i) : make_uint4(0u, 0u, 0u, 0u);
+#pragma unroll
+    for (int i = 0; i < KEEP; ++i) amax = amax_of(keep[i], amax);
+#pragma unroll 1
+    for (int v = lane + LANES * KEEP; v < vec_per_row; v += LANES) amax = amax_of(__ldg(row + v), amax);
 #pragma unroll
     for (int off = 16; off > 0; off >>= 1) amax = fmaxf(amax, __shfl_xor_sync(0xFFFFFFFFu, amax, off));
+    if (WARPS > 1) {
+      __syncthreads();   // the last row's maxima have been read
+      if ((lane & 31) == 0) amax_s[lane >> 5] = amax;
+      __syncthreads();
+#pragma unroll
+      for (int i = 0; i < WARPS; ++i) amax = fmaxf(amax, amax_s[i]);
+    }
     const float sc = scale_of(amax);
     if (lane == 0) scale[r] = sc;
     uint2* out = dst + r * vec_per_row;
-    for (int v = lane; v < vec_per_row; v += 32) {
-      const uint4 raw = __ldg(row + v);
+    if (!(sc >= 0x1p-80f && sc < 0x1p100f)) {   // the reciprocal or a residual could leave the normal range: divide
+#pragma unroll 1
+      for (int v = lane; v < vec_per_row; v += LANES) {
+        const uint4 raw = __ldg(row + v);
+        const __nv_bfloat162* p = reinterpret_cast<const __nv_bfloat162*>(&raw);
+        uint32_t w[2] = {0u, 0u};
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+          const float2 f = __bfloat1622float2(p[q]);
+          w[q >> 1] |= ((uint32_t)to_e4m3(f.x, sc) | ((uint32_t)to_e4m3(f.y, sc) << 8)) << (16 * (q & 1));
+        }
+        out[v] = make_uint2(w[0], w[1]);
+      }
+      continue;
+    }
+    const float inv = __frcp_rn(sc);
+    auto codes = [&](const uint4& raw) {
       const __nv_bfloat162* p = reinterpret_cast<const __nv_bfloat162*>(&raw);
-      uint32_t w[2] = {0u, 0u};
+      uint32_t c[4];
 #pragma unroll
       for (int q = 0; q < 4; ++q) {
         const float2 f = __bfloat1622float2(p[q]);
-        w[q >> 1] |= ((uint32_t)to_e4m3(f.x, sc) | ((uint32_t)to_e4m3(f.y, sc) << 8)) << (16 * (q & 1));
+        c[q] = to_e4m3_pair(f.x, f.y, inv, sc);
       }
-      out[v] = make_uint2(w[0], w[1]);
-    }
+      return make_uint2(__byte_perm(c[0], c[1], 0x5410), __byte_perm(c[2], c[3], 0x5410));
+    };
+#pragma unroll
+    for (int i = 0; i < KEEP; ++i)
+      if (lane + LANES * i < vec_per_row) out[lane + LANES * i] = codes(keep[i]);
+#pragma unroll 1
+    for (int v = lane + LANES * KEEP; v < vec_per_row; v += LANES) out[v] = codes(__ldg(row + v));
   }
 }
 
@@ -102,11 +157,14 @@ __global__ void __launch_bounds__(256) quantize_weights_kernel(const __nv_bfloat
 
 cudaError_t launch_quantize_rows(const void* src, long long rows, int cols, void* dst, float* scale, cudaStream_t st) {
   if (rows <= 0 || cols <= 0) return cudaSuccess;
-  long long blocks = (rows + 7) / 8;
-  const long long cap = (long long)sm_count() * 8;
-  if (blocks > cap) blocks = cap;
-  return launch_pdl(quantize_rows_kernel, (unsigned)blocks, 256, 0, st, static_cast<const uint4*>(src),
-                    static_cast<uint2*>(dst), scale, rows, cols / 8);
+  const long long cap = (long long)sm_count() * 16;
+  const uint4* in = static_cast<const uint4*>(src);
+  uint2* out = static_cast<uint2*>(dst);
+  auto grid = [&](long long n) { return (unsigned)(n > cap ? cap : n); };
+  if (cols <= 512) return launch_pdl(quantize_rows_kernel<2, 1>, grid((rows + 7) / 8), 256, 0, st, in, out, scale, rows, cols / 8);
+  if (cols <= 1536) return launch_pdl(quantize_rows_kernel<6, 1>, grid((rows + 7) / 8), 256, 0, st, in, out, scale, rows, cols / 8);
+  if (cols <= 4096) return launch_pdl(quantize_rows_kernel<4, 4>, grid(rows), 128, 0, st, in, out, scale, rows, cols / 8);
+  return launch_pdl(quantize_rows_kernel<8, 4>, grid(rows), 128, 0, st, in, out, scale, rows, cols / 8);   // registers: 8192 columns
 }
 
 cudaError_t launch_quantize_weights(const void* w, int E, int K, int N, void* wq, float* scale, cudaStream_t st) {

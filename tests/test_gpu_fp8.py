@@ -167,3 +167,22 @@ def test_fp8_random_shape_sweep():
         _, _, y_ref = O.combine(o_ref, lay, idx_ref, run.host_w() if in_combine else None, cfg.E, cfg.G)
         y_gpu = O.bf16_to_f64(H.bf16_host(run.y)[: cfg.T])
         H.assert_close_out(y_gpu, y_ref, f"{cfg}")
+
+
+@pytest.mark.parametrize("cols", [8, 512, 520, 1536, 1544, 4096, 4104, 8200, 14336])
+def test_quantize_rows_bit_exact_by_row_length(cols):
+    """Rows that fit the registers of each form and rows that do not; every exponent from the row's largest value down to
+    where codes vanish, largest values of every magnitude (subnormal scales included), so that quotients fall on and beside
+    every rounding boundary."""
+    rows = 1 + 2_000_000 // cols
+    g = torch.Generator(device="cuda").manual_seed(cols)
+    r = lambda *shape: torch.rand(*shape, generator=g, device="cuda", dtype=torch.float64)
+    top = torch.exp2(r(rows, 1) * 250 - 125)
+    x = (top * torch.exp2(-18 * r(rows, cols)) * torch.where(r(rows, cols) < 0.5, -1.0, 1.0)).to(torch.bfloat16)
+    x[0, 0] = -0.0
+    q = torch.zeros(rows, cols, dtype=torch.uint8, device="cuda")
+    s = torch.zeros(rows, dtype=torch.float32, device="cuda")
+    B.moe_quantize_rows(x, q, s)
+    q_ref, s_ref = F.quantize_rows(O.bf16_to_f64(H.bf16_host(x)))
+    assert np.array_equal(s.cpu().numpy(), s_ref)
+    assert np.array_equal(q.cpu().numpy(), q_ref)
