@@ -246,7 +246,7 @@ int moe_layer_backward(const moe_shape_t* shape, const void* x, const void* dy, 
  *     dw_gate[:, e] = sum over the pairs (t, j) with e_j = e of dkey[t, j] * x[t, :]        fp32 [d, E], written whole,
  *     dx[t, :]     += sum_j dkey[t, j] * w_gate[:, e_j]                                     bf16 [T, d], in / out.
  * MUST follow moe_layer_backward for the same shape, routing and backward workspace on the same stream: it reads
- * what that call leaves in `ws` (the recomputed h, dH, the per-expert rows of x and the padded row numbers) and the
+ * what that call leaves in `ws` (row sums of h * dH, the per-expert rows of x, the padded row numbers) and the
  * dx it wrote.  `logits` are the forward's fp32 router logits [T, E] (moe_layer's optional output); required for
  * sigmoid scores, ignored (may be NULL) for softmax.  logit_bias / bias_row_stride as in moe_route.  `layout` is the
  * forward's layout (only expert_counts is read).  shape->flags: 0 or MOE_FLAG_SPARSE_TOPK.

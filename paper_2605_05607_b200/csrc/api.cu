@@ -472,7 +472,7 @@ namespace tcmoe {
 namespace {
 // Regions of the backward workspace, in order, each on a 1 KiB boundary.
 struct BwdPlan {
-  size_t status, poff, mt_prefix, mp_prefix, pair_prow, xs, dos, dh, h, da1, da3, dxs, g_row, dkey, wgt, total;
+  size_t status, poff, mt_prefix, mp_prefix, pair_prow, xs, dos, dh, h, da1, da3, dxs, row_dots, g_row, dkey, wgt, total;
 };
 BwdPlan bwd_plan(const moe_shape_t& s) {
   BwdPlan p{};
@@ -496,6 +496,7 @@ BwdPlan bwd_plan(const moe_shape_t& s) {
   p.da1 = take(R * (size_t)s.f * 2);
   p.da3 = take(R * (size_t)s.f * 2);
   p.dxs = take(R * (size_t)s.d * 2);
+  p.row_dots = take((size_t)bwd_dot_parts(to_shape(s)) * R * 4);   // for moe_gate_backward
   p.g_row = take(R * 4);                       // moe_gate_backward: row dots, then key gradients per padded row
   p.dkey = take(P * 4);                        //   key gradients per pair
   p.wgt = take(E * (size_t)s.d * 4);           //   the gate weight transposed
@@ -554,6 +555,7 @@ int moe_layer_backward(const moe_shape_t* shape, const void* x, const void* dy, 
   a.da1 = at<void>(ws, p.da1);
   a.da3 = at<void>(ws, p.da3);
   a.dxs = at<void>(ws, p.dxs);
+  a.row_dots = at<float>(ws, p.row_dots);
   a.status = at<int32_t>(ws, p.status);
   TCMOE_CUDA(launch_layer_backward(to_shape(*shape), a, static_cast<cudaStream_t>(stream)));
   return MOE_OK;
@@ -591,8 +593,7 @@ int moe_gate_backward(const moe_shape_t* shape, const float* logits, const float
   a.mt_prefix = at<int32_t>(ws, p.mt_prefix);
   a.pair_prow = at<int32_t>(ws, p.pair_prow);
   a.xs = at<void>(ws, p.xs);
-  a.h = at<void>(ws, p.h);
-  a.dh = at<void>(ws, p.dh);
+  a.row_dots = at<float>(ws, p.row_dots);
   a.part = at<float>(ws, p.dos);   // dO is not needed any more: (P / 128 + E) d floats fit its (P + 64 E) d bf16
   a.g_row = at<float>(ws, p.g_row);
   a.dkey = at<float>(ws, p.dkey);

@@ -117,6 +117,7 @@ __global__ void __launch_bounds__(256) bwd_zero_pads_kernel(const int32_t* __res
 
 // rows of every padded row buffer for a shape: all pairs plus at most 63 pad rows per expert
 size_t bwd_row_capacity(const Shape& s) { return (size_t)s.T * s.k + 64 * (size_t)s.E; }
+int bwd_dot_parts(const Shape& s) { return 2 * ((s.f + 127) / 128); }
 
 cudaError_t launch_layer_backward(const Shape& s, const BwdArgs& a, cudaStream_t st) {
   if (s.T == 0) {   // no rows: every weight gradient is zero
@@ -178,6 +179,8 @@ cudaError_t launch_layer_backward(const Shape& s, const BwdArgs& a, cudaStream_t
   r.out2 = static_cast<__nv_bfloat16*>(a.da1);
   r.out3 = static_cast<__nv_bfloat16*>(a.da3);
   r.dh = static_cast<const __nv_bfloat16*>(a.dh);
+  r.row_dots = a.row_dots;
+  r.dots_ld = R;
   r.out_ld = s.f;
   r.expert_offsets = a.poff;
   r.tile_prefix = a.mp_prefix;

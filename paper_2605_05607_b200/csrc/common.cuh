@@ -127,9 +127,11 @@ struct BwdArgs {
   // scratch (padded row space: bwd_row_capacity() rows each)
   int32_t *poff, *mt_prefix, *mp_prefix, *pair_prow;
   void *xs, *dos, *dh, *h, *da1, *da3, *dxs;
+  float* row_dots;                  // [bwd_dot_parts, bwd_row_capacity]
   int32_t* status;
 };
 size_t bwd_row_capacity(const Shape& s);
+int bwd_dot_parts(const Shape& s);   // partial sums per row of h . dH (64 columns of f each, in whole tiles of 128)
 cudaError_t launch_layer_backward(const Shape& s, const BwdArgs& a, cudaStream_t st);
 // gate_bwd.cu: gradient of the gate network, after launch_layer_backward on the same scratch
 struct GateBwdArgs {
@@ -144,7 +146,8 @@ struct GateBwdArgs {
   float* dw_gate;                   // [d, E] fp32 out
   // left behind by launch_layer_backward
   const int32_t *poff, *mt_prefix, *pair_prow;
-  const void *xs, *h, *dh;
+  const void* xs;
+  const float* row_dots;
   // scratch
   float *g_row, *dkey, *wgt;        // [bwd_row_capacity], [T * k], [E, d]
   float* part;                      // [128-row tiles, d]: partial sums of dw_gate

@@ -42,6 +42,8 @@ struct GemmParams {
   const __nv_bfloat16* dh;      // [rows, N] incoming gradient of h (same leading dimension as out)
   __nv_bfloat16* out2;          // dA1 [rows, N]
   __nv_bfloat16* out3;          // dA3 [rows, N]
+  float* row_dots;              // [2 n_tiles, dots_ld]: sum of h * dh over 64 columns of a row
+  long long dots_ld;
   int k_split;                  // k-blocks taken from each of the two (A, B) pairs
 };
 

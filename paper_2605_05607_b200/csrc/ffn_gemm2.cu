@@ -64,7 +64,7 @@ constexpr uint32_t HINT = 4000;   // try_wait suspend-time hint (ns), see ptx::m
 //   PAIR_GLU      GEMM-1 with the SwiGLU epilogue (see the head of this file): map_b0 = W1, map_b1 = W3, 128 output
 //                 columns per tile
 //   PAIR_GLU_BWD  the same GEMM recomputed in the backward pass: from a1 = a.W1, a3 = a.W3 and the incoming dh tile the
-//                 epilogue writes h, da1 = dh * a3 * silu'(a1) and da3 = dh * silu(a1)
+//                 epilogue writes h, da1 = dh * a3 * silu'(a1) and da3 = dh * silu(a1), and per 64 columns the row sums of h * dh
 //   PAIR_WGRAD    dW[e] = A_e^T . B_e over the rows of expert e in the padded row space (segments start at poff[e], a multiple of 64, pad
 //                 rows zero, so no block of 64 rows mixes experts and an expert without rows gets zeros): a task is a
 //                 256 x 256 tile of one expert's gradient (p.K = its row count M, p.N its columns), the K walk runs over
@@ -183,6 +183,18 @@ ffn_gemm2_kernel(const __grid_constant__ CUtensorMap map_b0, const __grid_consta
     for (int w = cluster_id; w < total && !*abort_flag; w += num_clusters, ++tl) {
       const Tile t = tile_of(w);
       const int buf = tl & 1;
+      uint4 dh[2][4];
+      if (MODE == PAIR_GLU_BWD) {   // the incoming gradient of h, 64 columns of the warp's rows, while the main loop runs
+#pragma unroll
+        for (int c = 0; c < 2; ++c)
+#pragma unroll
+          for (int i = 0; i < 4; ++i) {
+            const int r = quarter * 32 + i * 8 + srow, col = t.n0 + half * COLS + c * 32 + piece * 8;
+            dh[c][i] = r < t.rows && col < p.N
+                           ? __ldg(reinterpret_cast<const uint4*>(p.dh + (size_t)(t.row0 + r) * (size_t)p.out_ld + col))
+                           : make_uint4(0u, 0u, 0u, 0u);
+          }
+      }
       if (!ptx::mbar_wait_warp<false, HINT>(tfull_bar(buf), (tl >> 1) & 1, abort_flag, global_abort)) { timeout(1); break; }
       ptx::tc_fence_after();
       const int lrow = quarter * 32 + lane;
@@ -190,7 +202,7 @@ ffn_gemm2_kernel(const __grid_constant__ CUtensorMap map_b0, const __grid_consta
       const size_t grow = (size_t)(valid ? t.row0 + lrow : 0);
       const int col0 = t.n0 + half * COLS;            // first output column of this warp
       const uint32_t taddr = tmem_base + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(buf * UMMA_N + half * COLS);
-      auto send = [&](int c) {                        // 32 staged columns -> rows of out
+      auto send = [&](__nv_bfloat16* out, int c) {    // 32 staged columns -> rows of out
         __syncwarp();
         const int col = col0 + c * 32 + piece * 8;
         if (col < p.N) {
@@ -199,7 +211,7 @@ ffn_gemm2_kernel(const __grid_constant__ CUtensorMap map_b0, const __grid_consta
             const int r = i * 8 + srow;               // row of this warp's 32
             if (quarter * 32 + r < t.rows) {
               const uint4 q = ptx::ld_shared_v4(stage + r * 64 + ((piece ^ ((r >> 1) & 3)) << 4));
-              *reinterpret_cast<uint4*>(p.out + (size_t)(t.out_row0 + quarter * 32 + r) * (size_t)p.out_ld + col) = q;
+              *reinterpret_cast<uint4*>(out + (size_t)(t.out_row0 + quarter * 32 + r) * (size_t)p.out_ld + col) = q;
             }
           }
         }
@@ -226,50 +238,60 @@ ffn_gemm2_kernel(const __grid_constant__ CUtensorMap map_b0, const __grid_consta
         __syncwarp();
       }
       if (MODE == PAIR_GLU_BWD) {
-        // backward of SwiGLU on the recomputed pre-activations: a thread owns one row and walks its 64 columns 32 at
-        // a time; dh comes from global memory (64 bytes of the row per step), h / da1 / da3 go straight back
-        const size_t rowoff = grow * (size_t)p.out_ld + col0;
-#pragma unroll 1
+        // backward of SwiGLU on the recomputed pre-activations, 32 columns at a time: dh comes to the owner of its row through
+        // the staging buffer, h / dA1 / dA3 leave through it
+        float dot = 0.f;   // h . dh over this warp's columns, of the rounded values (the gate's gradient needs it)
+#pragma unroll
         for (int c = 0; c < 2; ++c) {
+          __syncwarp();
+#pragma unroll
+          for (int i = 0; i < 4; ++i) {
+            const int r = i * 8 + srow;
+            ptx::st_shared_v4(stage + r * 64 + ((piece ^ ((r >> 1) & 3)) << 4), dh[c][i].x, dh[c][i].y, dh[c][i].z, dh[c][i].w);
+          }
           uint32_t a1[32], a3[32];
           ptx::tmem_ld32(taddr + c * 32, a1);
           ptx::tmem_ld32(taddr + 128 + c * 32, a3);
           ptx::tmem_ld_wait();
-          if (valid) {
+          __syncwarp();
+          uint32_t q1[16], q3[16];
 #pragma unroll
-            for (int v = 0; v < 4; ++v) {
-              const int col = col0 + c * 32 + v * 8;
-              if (col < p.N) {
-                const size_t at = rowoff + c * 32 + v * 8;
-                const uint4 dq = *reinterpret_cast<const uint4*>(p.dh + at);
-                const __nv_bfloat162* dp = reinterpret_cast<const __nv_bfloat162*>(&dq);
-                uint32_t qh[4], q1[4], q3[4];
+          for (int v = 0; v < 4; ++v) {
+            const uint4 dq = ptx::ld_shared_v4(stage + lane * 64 + ((v ^ ((lane >> 1) & 3)) << 4));
+            const __nv_bfloat162* dp = reinterpret_cast<const __nv_bfloat162*>(&dq);
+            uint32_t qh[4];
 #pragma unroll
-                for (int i = 0; i < 4; ++i) {
-                  const int j = v * 8 + 2 * i;
-                  const float2 dhv = __bfloat1622float2(dp[i]);
-                  float hh[2], d1[2], d3[2];
+            for (int i = 0; i < 4; ++i) {
+              const int j = v * 8 + 2 * i;
+              const float2 dhv = __bfloat1622float2(dp[i]);
+              float hh[2], d1[2], d3[2];
 #pragma unroll
-                  for (int u = 0; u < 2; ++u) {
-                    const float x1 = __uint_as_float(a1[j + u]), x3 = __uint_as_float(a3[j + u]);
-                    const float dv = u ? dhv.y : dhv.x;
-                    const float sg = __fdividef(1.f, 1.f + __expf(-x1));
-                    const float sl = x1 * sg;
-                    hh[u] = sl * x3;
-                    d3[u] = dv * sl;
-                    d1[u] = dv * x3 * (sg * (1.f + x1 * (1.f - sg)));
-                  }
-                  qh[i] = pack2(hh[0], hh[1]);
-                  q1[i] = pack2(d1[0], d1[1]);
-                  q3[i] = pack2(d3[0], d3[1]);
-                }
-                *reinterpret_cast<uint4*>(p.out + at) = make_uint4(qh[0], qh[1], qh[2], qh[3]);
-                *reinterpret_cast<uint4*>(p.out2 + at) = make_uint4(q1[0], q1[1], q1[2], q1[3]);
-                *reinterpret_cast<uint4*>(p.out3 + at) = make_uint4(q3[0], q3[1], q3[2], q3[3]);
+              for (int u = 0; u < 2; ++u) {
+                const float x1 = __uint_as_float(a1[j + u]), x3 = __uint_as_float(a3[j + u]);
+                const float dv = u ? dhv.y : dhv.x;
+                const float sg = __fdividef(1.f, 1.f + __expf(-x1));
+                const float sl = x1 * sg;
+                hh[u] = sl * x3;
+                d3[u] = dv * sl;
+                d1[u] = dv * x3 * (sg * (1.f + x1 * (1.f - sg)));
               }
+              qh[i] = pack2(hh[0], hh[1]);
+              q1[v * 4 + i] = pack2(d1[0], d1[1]);
+              q3[v * 4 + i] = pack2(d3[0], d3[1]);
+              const float2 hr = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&qh[i]));
+              dot = fmaf(hr.x, dhv.x, fmaf(hr.y, dhv.y, dot));
             }
+            put(v, qh[0], qh[1], qh[2], qh[3]);   // over the piece just read: the same row and place
           }
+          send(p.out, c);
+#pragma unroll
+          for (int v = 0; v < 4; ++v) put(v, q1[v * 4], q1[v * 4 + 1], q1[v * 4 + 2], q1[v * 4 + 3]);
+          send(p.out2, c);
+#pragma unroll
+          for (int v = 0; v < 4; ++v) put(v, q3[v * 4], q3[v * 4 + 1], q3[v * 4 + 2], q3[v * 4 + 3]);
+          send(p.out3, c);
         }
+        if (valid) p.row_dots[(size_t)(t.n0 / BN_OUT * 2 + half) * p.dots_ld + grow] = dot;
       } else if (GLU) {
         // SwiGLU of the W1 half (accumulator columns 0..127) and the W3 half (128..255)
 #pragma unroll 1
@@ -289,7 +311,7 @@ ffn_gemm2_kernel(const __grid_constant__ CUtensorMap map_b0, const __grid_consta
             }
             put(v, q[0], q[1], q[2], q[3]);
           }
-          send(c);
+          send(p.out, c);
         }
       } else if (RED) {
 #pragma unroll 1
@@ -337,7 +359,7 @@ ffn_gemm2_kernel(const __grid_constant__ CUtensorMap map_b0, const __grid_consta
                 pack2(wr * __uint_as_float(acc[v * 8 + 2]), wr * __uint_as_float(acc[v * 8 + 3])),
                 pack2(wr * __uint_as_float(acc[v * 8 + 4]), wr * __uint_as_float(acc[v * 8 + 5])),
                 pack2(wr * __uint_as_float(acc[v * 8 + 6]), wr * __uint_as_float(acc[v * 8 + 7])));
-          send(c);
+          send(p.out, c);
         }
       }
       ptx::tc_fence_before();

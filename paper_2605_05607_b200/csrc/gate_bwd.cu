@@ -11,10 +11,10 @@
 // The expert part of the backward pass (bwd.cu) has just produced, in the padded row space of its workspace,
 // h (the recomputed SwiGLU output of every pair) and dH = (w * dy) . W2^T.  Their row-wise dot product is
 //     h[r] . dH[r] = w_r * (h[r] . W2) . dy[t_r] = g  of the pair in row r,
-// so dL/dw costs one pass over two [rows, f] buffers and no GEMM.  dw_gate is a weighted sum of each expert's rows of
+// so dL/dw costs no GEMM; the backward SwiGLU epilogue, which holds both, leaves its sums over 64 columns each.  dw_gate is a weighted sum of each expert's rows of
 // xs (also still in the workspace), dx gets k rows of the transposed gate weight per token.
 //
-// Sequence (one stream): row dots -> per-token key gradients -> partial sums of dw_gate per 128-row tile -> dw_gate (tiles in
+// Sequence (one stream): sums of the row dots -> per-token key gradients -> partial sums of dw_gate per 128-row tile -> dw_gate (tiles in
 // ascending order: deterministic, no atomics) and the transpose of w_gate -> dx update.
 #include "common.cuh"
 
@@ -23,35 +23,17 @@
 namespace tcmoe {
 namespace {
 
-__device__ __forceinline__ float dot8(const uint4& a, const uint4& b) {
-  const __nv_bfloat162* pa = reinterpret_cast<const __nv_bfloat162*>(&a);
-  const __nv_bfloat162* pb = reinterpret_cast<const __nv_bfloat162*>(&b);
-  float s = 0.f;
-#pragma unroll
-  for (int q = 0; q < 4; ++q) {
-    const float2 fa = __bfloat1622float2(pa[q]), fb = __bfloat1622float2(pb[q]);
-    s = fmaf(fa.x, fb.x, s);
-    s = fmaf(fa.y, fb.y, s);
-  }
-  return s;
-}
-
-// g_row[r] = h[r] . dH[r] for the rows in use (r < poff[E]); a warp per row
-__global__ void __launch_bounds__(256) gate_rowdot_kernel(const uint4* __restrict__ h, const uint4* __restrict__ dh,
-                                                          const int32_t* __restrict__ poff, float* __restrict__ g_row,
-                                                          int E, int vec_per_row) {
+// g_row[r] = h[r] . dH[r] for the rows in use (r < poff[E]): the partial sums that the recomputed GEMM-1 left per 64 columns
+// (a pass over both buffers for it took 79 us on 65536 rows of f = 1536).
+__global__ void __launch_bounds__(256) gate_rowdot_kernel(const float* __restrict__ row_dots, int parts, long long ld,
+                                                          const int32_t* __restrict__ poff, float* __restrict__ g_row, int E) {
   grid_dependency_sync();
-  const int lane = threadIdx.x & 31, wpb = blockDim.x >> 5;
   const int rows = __ldg(poff + E);
-  for (int r = blockIdx.x * wpb + (threadIdx.x >> 5); r < rows; r += gridDim.x * wpb) {
-    const uint4* hr = h + (size_t)r * vec_per_row;
-    const uint4* dr = dh + (size_t)r * vec_per_row;
+  for (int r = blockIdx.x * blockDim.x + threadIdx.x; r < rows; r += gridDim.x * blockDim.x) {
     float s = 0.f;
-#pragma unroll 4
-    for (int v = lane; v < vec_per_row; v += 32) s += dot8(__ldcs(hr + v), __ldcs(dr + v));
-#pragma unroll
-    for (int off = 16; off > 0; off >>= 1) s += __shfl_xor_sync(0xFFFFFFFFu, s, off);
-    if (lane == 0) g_row[r] = s;
+#pragma unroll 8
+    for (int q = 0; q < parts; ++q) s += __ldcs(row_dots + (size_t)q * ld + r);
+    g_row[r] = s;
   }
 }
 
@@ -208,10 +190,10 @@ cudaError_t launch_gate_backward(const Shape& s, const GateBwdArgs& a, cudaStrea
   const int n_rows = (int)bwd_row_capacity(s);
   ProfileScope prof(KID_GATE_BWD, st);
   const int cap = sm_count() * 8;
-  int blocks = (n_rows + 7) / 8;
+  int blocks = (n_rows + 255) / 256;
   if (blocks > cap) blocks = cap;
-  if ((err = launch_pdl(gate_rowdot_kernel, blocks, 256, 0, st, static_cast<const uint4*>(a.h),
-                        static_cast<const uint4*>(a.dh), a.poff, a.g_row, s.E, s.f / 8)) != cudaSuccess)
+  if ((err = launch_pdl(gate_rowdot_kernel, blocks, 256, 0, st, a.row_dots, bwd_dot_parts(s), (long long)n_rows, a.poff, a.g_row,
+                        s.E)) != cudaSuccess)
     return err;
   if ((err = launch_pdl(gate_route_bwd_kernel, (s.T + 255) / 256, 256, 0, st, a.topk_idx, a.topk_w, a.pair_prow,
                         a.logits, a.bias, (long long)a.bias_stride, a.g_row, a.dkey, s.T, s.E, s.k,
