@@ -147,13 +147,11 @@ cudaError_t launch_layer_backward(const Shape& s, const BwdArgs& a, cudaStream_t
                         static_cast<uint4*>(a.dos), vec)) != cudaSuccess)
     return err;
 
-  CUtensorMap m_w1, m_w3, m_w1t, m_w3t, m_w2t, m_xs, m_do, m_da1, m_da3;
+  CUtensorMap m_w1, m_w3, m_w1t, m_w3t, m_w2t;
   CUtensorMap r_xs, r_h, r_do, r_da1, r_da3;
   if (!ffn::make_weight_map(&m_w1, a.w1, s.E, s.d, s.f) || !ffn::make_weight_map(&m_w3, a.w3, s.E, s.d, s.f) ||
       !ffn::make_weight_map_kmajor(&m_w1t, a.w1, s.E, s.d, s.f) || !ffn::make_weight_map_kmajor(&m_w3t, a.w3, s.E, s.d, s.f) ||
-      !ffn::make_weight_map_kmajor(&m_w2t, a.w2, s.E, s.f, s.d) || !ffn::make_act_map(&m_xs, a.xs, R, s.d) ||
-      !ffn::make_act_map(&m_do, a.dos, R, s.d) || !ffn::make_act_map(&m_da1, a.da1, R, s.f) ||
-      !ffn::make_act_map(&m_da3, a.da3, R, s.f) || !ffn::make_rows_map_mn(&r_xs, a.xs, R, s.d) ||
+      !ffn::make_weight_map_kmajor(&m_w2t, a.w2, s.E, s.f, s.d) || !ffn::make_rows_map_mn(&r_xs, a.xs, R, s.d) ||
       !ffn::make_rows_map_mn(&r_h, a.h, R, s.f) || !ffn::make_rows_map_mn(&r_do, a.dos, R, s.d) ||
       !ffn::make_rows_map_mn(&r_da1, a.da1, R, s.f) || !ffn::make_rows_map_mn(&r_da3, a.da3, R, s.f))
     return cudaErrorInvalidValue;
@@ -161,6 +159,8 @@ cudaError_t launch_layer_backward(const Shape& s, const BwdArgs& a, cudaStream_t
   // dH = dO . W2^T : [R, d] x [d, f], the gate weight is already inside dO
   ffn::GemmParams g{};
   g.out = static_cast<__nv_bfloat16*>(a.dh);
+  g.a_src = a.dos;
+  g.a_rows = (int)R;
   g.out_ld = s.f;
   g.expert_offsets = a.poff;
   g.tile_prefix = a.mp_prefix;
@@ -171,7 +171,7 @@ cudaError_t launch_layer_backward(const Shape& s, const BwdArgs& a, cudaStream_t
   g.status = a.status;
   {
     ProfileScope prof(KID_GEMM2, st);
-    if ((err = ffn::launch_bwd_dh(g, m_w2t, m_do, st)) != cudaSuccess) return err;
+    if ((err = ffn::launch_bwd_dh(g, m_w2t, st)) != cudaSuccess) return err;
   }
   // GEMM-1 recomputed, backward SwiGLU epilogue: h, dA1, dA3
   ffn::GemmParams r{};
@@ -181,6 +181,8 @@ cudaError_t launch_layer_backward(const Shape& s, const BwdArgs& a, cudaStream_t
   r.dh = static_cast<const __nv_bfloat16*>(a.dh);
   r.row_dots = a.row_dots;
   r.dots_ld = R;
+  r.a_src = a.xs;
+  r.a_rows = (int)R;
   r.out_ld = s.f;
   r.expert_offsets = a.poff;
   r.tile_prefix = a.mp_prefix;
@@ -191,13 +193,16 @@ cudaError_t launch_layer_backward(const Shape& s, const BwdArgs& a, cudaStream_t
   r.status = a.status;
   {
     ProfileScope prof(KID_GEMM1, st);
-    if ((err = ffn::launch_bwd_glu(r, m_w1, m_w3, m_xs, st)) != cudaSuccess) return err;
+    if ((err = ffn::launch_bwd_glu(r, m_w1, m_w3, st)) != cudaSuccess) return err;
   }
   // dW2[e] = H^T . dO
   if ((err = ffn::launch_wgrad_pair(r_h, r_do, a.poff, a.dw2, s.E, s.f, s.d, a.status, st)) != cudaSuccess) return err;
   // dXs = dA1 . W1^T + dA3 . W3^T : [R, f] x [f, d], twice into one accumulator
   ffn::GemmParams q{};
   q.out = static_cast<__nv_bfloat16*>(a.dxs);
+  q.a_src = a.da1;
+  q.a_src2 = a.da3;
+  q.a_rows = (int)R;
   q.out_ld = s.d;
   q.expert_offsets = a.poff;
   q.tile_prefix = a.mp_prefix;
@@ -209,7 +214,7 @@ cudaError_t launch_layer_backward(const Shape& s, const BwdArgs& a, cudaStream_t
   q.status = a.status;
   {
     ProfileScope prof(KID_GEMM2, st);
-    if ((err = ffn::launch_bwd_dx(q, m_w1t, m_w3t, m_da1, m_da3, st)) != cudaSuccess) return err;
+    if ((err = ffn::launch_bwd_dx(q, m_w1t, m_w3t, st)) != cudaSuccess) return err;
   }
   // dx[t] = sum of the token's rows of dXs: the Combine stage on the padded row numbers, un-weighted
   Layout Lp = a.L;

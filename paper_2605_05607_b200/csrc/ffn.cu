@@ -43,7 +43,7 @@ struct MapEntry {
   MapKey key;
   CUtensorMap map;
 };
-constexpr int MAP_CACHE_ENTRIES = 64;
+constexpr int MAP_CACHE_ENTRIES = 128;   // a training step uses about 45
 std::mutex g_map_mutex;
 MapEntry g_map_cache[MAP_CACHE_ENTRIES];
 int g_map_count = 0, g_map_next = 0;   // entries in use, next slot to overwrite (round robin)
@@ -95,12 +95,12 @@ bool make_weight_map(CUtensorMap* map, const void* base, int E, int K, int N) {
   return encode_tiled(map, false, 3, base, dims, strides, box);
 }
 
-// bf16 activations [rows, K] row-major: box = 64 (K) x 128 rows
-bool make_act_map(CUtensorMap* map, const void* base, long long rows, int K) {
+// activations [rows, K] row-major, bf16 or E4M3: box = 128 bytes of K x box_rows rows
+bool make_act_map(CUtensorMap* map, const void* base, long long rows, int K, bool fp8, int box_rows) {
   cuuint64_t dims[2] = {(cuuint64_t)K, (cuuint64_t)rows};
-  cuuint64_t strides[1] = {(cuuint64_t)K * 2};
-  cuuint32_t box[2] = {BK, BM};
-  return encode_tiled(map, false, 2, base, dims, strides, box);
+  cuuint64_t strides[1] = {(cuuint64_t)K * (fp8 ? 1 : 2)};
+  cuuint32_t box[2] = {fp8 ? 128u : (cuuint32_t)BK, (cuuint32_t)box_rows};
+  return encode_tiled(map, fp8, 2, base, dims, strides, box);
 }
 
 // E4M3 weights [E, N, K] (K contiguous): box = 128 bytes of K x box_cols output columns x 1, 128-byte swizzle
@@ -109,14 +109,6 @@ bool make_weight_map_fp8(CUtensorMap* map, const void* base, int E, int N, int K
   cuuint64_t strides[2] = {(cuuint64_t)K, (cuuint64_t)N * K};
   cuuint32_t box[3] = {128, (cuuint32_t)box_cols, 1};
   return encode_tiled(map, true, 3, base, dims, strides, box);
-}
-
-// E4M3 activations [rows, K]: box = 128 bytes of K x 128 rows
-bool make_act_map_fp8(CUtensorMap* map, const void* base, int rows, int K) {
-  cuuint64_t dims[2] = {(cuuint64_t)K, (cuuint64_t)rows};
-  cuuint64_t strides[1] = {(cuuint64_t)K};
-  cuuint32_t box[2] = {128, BM};
-  return encode_tiled(map, true, 2, base, dims, strides, box);
 }
 
 // bf16 weights [E, K, N] read as the TRANSPOSED operand of a backward GEMM: the same memory seen as [E, N' = K, K' = N]
@@ -139,9 +131,7 @@ bool make_rows_map_mn(CUtensorMap* map, const void* base, long long rows, int co
 }  // namespace ffn
 
 using ffn::make_weight_map;
-using ffn::make_act_map;
 using ffn::make_weight_map_fp8;
-using ffn::make_act_map_fp8;
 
 int current_device() {
   int dev = 0;
@@ -230,9 +220,9 @@ cudaError_t launch_expert_ffn(const Shape& s, const FfnArgs& a, cudaStream_t st)
   if (s.T == 0) return cudaSuccess;
   if ((s.flags & 8) && a.y_acc == nullptr && a.blk_start != nullptr) return launch_expert_ffn_fused(s, a, st);
   const int P = s.T * s.k;
-  CUtensorMap m_w1, m_w3, m_w2, m_h;
+  CUtensorMap m_w1, m_w3, m_w2;
   if (!make_weight_map(&m_w1, a.w1, s.E, s.d, s.f) || !make_weight_map(&m_w3, a.w3, s.E, s.d, s.f) ||
-      !make_weight_map(&m_w2, a.w2, s.E, s.f, s.d) || !make_act_map(&m_h, a.h, P, s.f))
+      !make_weight_map(&m_w2, a.w2, s.E, s.f, s.d))
     return cudaErrorInvalidValue;
 
   ffn::GemmParams g1{};
@@ -253,13 +243,13 @@ cudaError_t launch_expert_ffn(const Shape& s, const FfnArgs& a, cudaStream_t st)
   cudaError_t err;
   if (a.pair_gemm1 && a.xs != nullptr) {
     // Dispatch writes the per-expert layout tensors, GEMM-1 runs on CTA pairs (MOE_FLAG_GEMM1_PAIR, or the shape rule)
-    CUtensorMap m_xs;
-    if (!make_act_map(&m_xs, a.xs, P, s.d)) return cudaErrorInvalidValue;
     if ((err = launch_permute_rows(s, a.a_src, a.a_rows, a.gather_idx, a.gather_div, a.expert_offsets, a.xs, a.status,
                                    st)) != cudaSuccess)
       return err;
+    g1.a_src = a.xs;
+    g1.a_rows = P;
     g1.tile_prefix = a.mp_prefix;
-    err = ffn::launch_gemm1_pair(g1, m_w1, m_w3, m_xs, st);
+    err = ffn::launch_gemm1_pair(g1, m_w1, m_w3, st);
   } else {
     err = ffn::launch_gemm1(g1, m_w1, m_w3, false, narrow_tiles(s, (s.f + 127) / 128), st);
   }
@@ -285,19 +275,21 @@ cudaError_t launch_expert_ffn(const Shape& s, const FfnArgs& a, cudaStream_t st)
     g2.tile_prefix = a.mt_prefix;
     return ffn::launch_gemm2_single(g2, m_w2, false, narrow_tiles(s, (s.d + 255) / 256), st);
   }
-  return ffn::launch_gemm2(g2, m_w2, m_h, false, st);
+  g2.a_src = a.h;
+  g2.a_rows = P;
+  return ffn::launch_gemm2(g2, m_w2, false, st);
 }
 
 // FP8 form: GEMM-1 on E4M3 rows and weights -> h (bf16) -> per-row quantisation of h -> GEMM-2 on E4M3.
 cudaError_t launch_expert_ffn_fp8(const Shape& s, const FfnArgs& a, const Fp8Args& q, cudaStream_t st) {
   if (s.T == 0) return cudaSuccess;
   const int P = s.T * s.k;
-  CUtensorMap m_w1, m_w3, m_w2, m_h;
+  CUtensorMap m_w1, m_w3, m_w2;
   const bool single2 = small_experts(s) && a.y_acc == nullptr;
   const bool narrow1 = narrow_tiles(s, (s.f + 127) / 128), narrow2 = single2 && narrow_tiles(s, (s.d + 255) / 256);
   if (!make_weight_map_fp8(&m_w1, a.w1, s.E, s.f, s.d, narrow1 ? 64 : 128) ||
       !make_weight_map_fp8(&m_w3, a.w3, s.E, s.f, s.d, narrow1 ? 64 : 128) ||
-      !make_weight_map_fp8(&m_w2, a.w2, s.E, s.d, s.f, narrow2 ? 64 : 128) || !make_act_map_fp8(&m_h, q.hq, P, s.f))
+      !make_weight_map_fp8(&m_w2, a.w2, s.E, s.d, s.f, narrow2 ? 64 : 128))
     return cudaErrorInvalidValue;
 
   ffn::GemmParams g1{};
@@ -344,7 +336,9 @@ cudaError_t launch_expert_ffn_fp8(const Shape& s, const FfnArgs& a, const Fp8Arg
     g2.tile_prefix = a.mt_prefix;
     return ffn::launch_gemm2_single(g2, m_w2, true, narrow2, st);
   }
-  return ffn::launch_gemm2(g2, m_w2, m_h, true, st);
+  g2.a_src = q.hq;
+  g2.a_rows = P;
+  return ffn::launch_gemm2(g2, m_w2, true, st);
 }
 
 }  // namespace tcmoe

@@ -17,9 +17,10 @@ constexpr int UMMA_N = 256;   // accumulator columns per tile
 constexpr int MAX_E = 1024;
 
 struct GemmParams {
-  const void* a_src;            // GEMM-1 gather source (xg or x): bf16, or E4M3 codes in the FP8 form
+  const void* a_src;            // single-CTA kernel: gather source (xg or x); pair kernel: rows [a_rows, K]; bf16 or E4M3
+  const void* a_src2;           // PAIR_KSPLIT: rows of the second K part
   int a_ld;                     // elements per source row
-  int a_rows;                   // rows of the gather source: indices outside [0, a_rows) are reported, not read
+  int a_rows;                   // rows of a_src; of the gather source: indices outside [0, a_rows) are reported, not read
   const int32_t* gather_idx;    // row_src, or row_pair with gather_div = k (token = row_pair / k)
   int gather_div;
   __nv_bfloat16* out;
@@ -49,6 +50,7 @@ struct GemmParams {
 
 struct Tile {
   int e, n0, row0, rows;
+  int left;           // rows of the expert from the (pair) tile's first row on
   int out_row0, kb;   // weight-gradient tiles of the pair kernel: first output row of this CTA, k-blocks of the task
 };
 
@@ -78,7 +80,8 @@ __device__ __forceinline__ Tile decode_tile(int w, const int* tp, const int* eof
   t.e = lo;
   t.n0 = (local / gsize) * bn_out;
   t.row0 = eoff[lo] + (g * mg + local % gsize) * rows_per_tile + rank * BM;
-  t.rows = min(BM, eoff[lo + 1] - t.row0);
+  t.left = eoff[lo + 1] - (t.row0 - rank * BM);
+  t.rows = min(BM, t.left - rank * BM);
   t.out_row0 = t.row0;
   t.kb = 0;
   return t;
@@ -158,9 +161,8 @@ bool encode_tiled(CUtensorMap* map, bool bytes, int rank, const void* base, cons
                   const cuuint64_t* strides, const cuuint32_t* box);
 void clear_map_cache();
 bool make_weight_map(CUtensorMap* map, const void* base, int E, int K, int N);
-bool make_act_map(CUtensorMap* map, const void* base, long long rows, int K);
+bool make_act_map(CUtensorMap* map, const void* base, long long rows, int K, bool fp8, int box_rows);
 bool make_weight_map_fp8(CUtensorMap* map, const void* base, int E, int N, int K, int box_cols = 128);
-bool make_act_map_fp8(CUtensorMap* map, const void* base, int rows, int K);
 bool make_weight_map_kmajor(CUtensorMap* map, const void* base, int E, int rows, int cols);
 bool make_rows_map_mn(CUtensorMap* map, const void* base, long long rows, int cols);
 cudaError_t launch_wgrad_pair(const CUtensorMap& m_a, const CUtensorMap& m_b, const int32_t* poff, void* dw, int E, int M,
@@ -170,15 +172,11 @@ cudaError_t launch_wgrad_pair(const CUtensorMap& m_a, const CUtensorMap& m_b, co
 // [E, N, K] (B K-major), 128 elements of K per pipeline stage, scales applied in the epilogue.
 cudaError_t launch_gemm1(GemmParams p, const CUtensorMap& m_w1, const CUtensorMap& m_w3, bool fp8, bool narrow,
                          cudaStream_t st);
-cudaError_t launch_gemm2(const GemmParams& p, const CUtensorMap& m_w2, const CUtensorMap& m_h, bool fp8,
-                         cudaStream_t st);
-cudaError_t launch_gemm1_pair(const GemmParams& p, const CUtensorMap& m_w1, const CUtensorMap& m_w3,
-                              const CUtensorMap& m_xs, cudaStream_t st);
-cudaError_t launch_bwd_dh(const GemmParams& p, const CUtensorMap& m_w2t, const CUtensorMap& m_do, cudaStream_t st);
-cudaError_t launch_bwd_glu(const GemmParams& p, const CUtensorMap& m_w1, const CUtensorMap& m_w3, const CUtensorMap& m_xs,
-                           cudaStream_t st);
-cudaError_t launch_bwd_dx(const GemmParams& p, const CUtensorMap& m_w1t, const CUtensorMap& m_w3t, const CUtensorMap& m_da1,
-                          const CUtensorMap& m_da3, cudaStream_t st);
+cudaError_t launch_gemm2(const GemmParams& p, const CUtensorMap& m_w2, bool fp8, cudaStream_t st);
+cudaError_t launch_gemm1_pair(const GemmParams& p, const CUtensorMap& m_w1, const CUtensorMap& m_w3, cudaStream_t st);
+cudaError_t launch_bwd_dh(const GemmParams& p, const CUtensorMap& m_w2t, cudaStream_t st);
+cudaError_t launch_bwd_glu(const GemmParams& p, const CUtensorMap& m_w1, const CUtensorMap& m_w3, cudaStream_t st);
+cudaError_t launch_bwd_dx(const GemmParams& p, const CUtensorMap& m_w1t, const CUtensorMap& m_w3t, cudaStream_t st);
 size_t fused_max_blocks(int T, int k, int E);   // capacity of blk_start (+1) / blk_info for a shape
 size_t fused_tracker_words(int T, int k, int E);   // int32 words of the tracker region (dacc | done | tbcnt2 | nready | queue)
 cudaError_t launch_ffn_fused(FusedParams p, const int32_t* expert_counts, int32_t* blk_start, int4* blk_info,

@@ -71,16 +71,21 @@ constexpr uint32_t HINT = 4000;   // try_wait suspend-time hint (ns), see ptx::m
 //                 the expert's rows in blocks of 64, both operands are MN-major boxes of 64 columns x 64 rows; CTA `rank`
 //                 holds rows m0 + 128 * rank of the tile and columns n0 + 128 * rank of B
 //   PAIR_KSPLIT   acc = A0 . B0 + A1 . B1 (dX = dA1 . W1^T + dA3 . W3^T): the first p.k_split k-blocks come from
-//                 (map_h, map_b0), the rest from (map_a1, map_b1); plain epilogue
+//                 (rows.a0, map_b0), the rest from (rows.a1, map_b1); plain epilogue
 // BKMAJ: the bf16 weight operand is read K-major (one box of 128 columns x 64 K per CTA and stage), which is how
 // W^T looks when W is stored [K, N] with N contiguous: the backward GEMMs read the forward weights in place.
 enum { PAIR_PLAIN = 0, PAIR_GLU = 1, PAIR_GLU_BWD = 2, PAIR_KSPLIT = 3, PAIR_WGRAD = 4 };
 
+// Maps of the row operand(s): boxes of 32, 64, 96 and 128 rows ([3] alone for PAIR_WGRAD, whose boxes are 64 columns x 64 rows).
+// A CTA loads the rows its tile has, rounded up to 32, in one box; what the stage held before stays behind them and only
+// reaches accumulator rows that are not stored.  Training step of the Small layer 2003 -> 1967 us; no change where weights or
+// the padded UMMAs themselves are the bound.
+struct RowMaps { CUtensorMap a0[4], a1[4]; };
+
 template <bool RED, bool FP8, int MODE, bool BKMAJ>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(THREADS, 1)
 ffn_gemm2_kernel(const __grid_constant__ CUtensorMap map_b0, const __grid_constant__ CUtensorMap map_b1,
-                 const __grid_constant__ CUtensorMap map_h, const __grid_constant__ CUtensorMap map_a1,
-                 const GemmParams p) {
+                 const __grid_constant__ RowMaps rows, const GemmParams p) {
   constexpr bool GLU = MODE == PAIR_GLU || MODE == PAIR_GLU_BWD;
   constexpr bool KMAJ = FP8 || BKMAJ;   // the weight operand is K-major in shared memory
   static_assert(!(MODE != PAIR_PLAIN && (RED || FP8)), "only the plain form has the reducing / FP8 variants");
@@ -120,8 +125,8 @@ ffn_gemm2_kernel(const __grid_constant__ CUtensorMap map_b0, const __grid_consta
   if (warp == TMA_WARP && lane == 0) {
     ptx::prefetch_tensormap(&map_b0);
     ptx::prefetch_tensormap(&map_b1);
-    ptx::prefetch_tensormap(&map_h);
-    if (MODE == PAIR_KSPLIT) ptx::prefetch_tensormap(&map_a1);
+    ptx::prefetch_tensormap(&rows.a0[3]);
+    if (MODE == PAIR_KSPLIT) ptx::prefetch_tensormap(&rows.a1[3]);
   }
   if (warp == MMA_WARP) {
     ptx::tmem_alloc_pair(ptx::smem_u32(tmem_slot), 512);
@@ -161,6 +166,7 @@ ffn_gemm2_kernel(const __grid_constant__ CUtensorMap map_b0, const __grid_consta
       t.row0 = eoff_s[t.e];                                  // first (padded) row of the expert: start of the K walk
       t.kb = (eoff_s[t.e + 1] - t.row0) / BK;
       t.rows = min(BM, p.K - m0);                            // rows of dW[e] this CTA owns (<= 0: none)
+      t.left = 0;
       t.out_row0 = t.e * p.K + m0;
       return t;
     }
@@ -378,6 +384,10 @@ ffn_gemm2_kernel(const __grid_constant__ CUtensorMap map_b0, const __grid_consta
         const Tile t = tile_of(w);
         bool ok = true;
         const int KBt = WGRAD ? t.kb : KB;
+        // 32-row blocks of the tile in this CTA and in both (the expert's rows from the pair's first row on: t.left)
+        auto blocks32 = [](int left) { return min(max(left + 31, 0) >> 5, BM / 32); };
+        const int mine = WGRAD ? 4 : blocks32(t.left - rank * BM);
+        const uint32_t bytes = 2 * B_BYTES + (WGRAD ? 8 : blocks32(t.left) + blocks32(t.left - BM)) * (A_BYTES / 4);
         for (int kb = 0; kb < KBt; ++kb, ++it) {
           const int s = it % NSTAGE;
           if (!ptx::mbar_wait<false, HINT>(empty_bar(s), ((it / NSTAGE) & 1) ^ 1, abort_flag, global_abort)) {
@@ -386,18 +396,18 @@ ffn_gemm2_kernel(const __grid_constant__ CUtensorMap map_b0, const __grid_consta
           const uint32_t sa = smem_base + s * STAGE_BYTES, sb = sa + A_BYTES;
           const uint32_t lead_full = ptx::mapa(full_bar(s), 0);
           // the leader announces the bytes of both CTAs; the peer's copies only complete them
-          if (rank == 0) ptx::mbar_arrive_expect_tx(full_bar(s), 2 * STAGE_BYTES);
+          if (rank == 0) ptx::mbar_arrive_expect_tx(full_bar(s), bytes);
           if (WGRAD) {   // four MN-major boxes of 64 columns x 64 rows: this CTA's 128 rows of A^T and 128 columns of B
             const int r0 = t.row0 + kb * BK, ma = t.out_row0 - t.e * p.K;
-            ptx::tma_load_2d_pair(sa, &map_h, lead_full, ma, r0);
-            ptx::tma_load_2d_pair(sa + 8192, &map_h, lead_full, ma + 64, r0);
+            ptx::tma_load_2d_pair(sa, &rows.a0[3], lead_full, ma, r0);
+            ptx::tma_load_2d_pair(sa + 8192, &rows.a0[3], lead_full, ma + 64, r0);
             ptx::tma_load_2d_pair(sb, &map_b0, lead_full, t.n0 + rank * 128, r0);
             ptx::tma_load_2d_pair(sb + 8192, &map_b0, lead_full, t.n0 + rank * 128 + 64, r0);
             continue;
           }
           const bool second = MODE == PAIR_KSPLIT && kb >= p.k_split;     // second (A, B) pair of the K walk
           const int k0 = (second ? kb - p.k_split : kb) * BK_ELEMS;
-          ptx::tma_load_2d_pair(sa, second ? &map_a1 : &map_h, lead_full, k0, t.row0);
+          if (mine > 0) ptx::tma_load_2d_pair(sa, (second ? rows.a1 : rows.a0) + mine - 1, lead_full, k0, t.row0);
           const CUtensorMap* map_b = MODE == PAIR_KSPLIT ? (second ? &map_b1 : &map_b0) : (rank == 0 ? &map_b0 : &map_b1);
           const int nb = GLU ? t.n0 : t.n0 + rank * 128;   // this CTA's 128 columns of the B tile
           if (KMAJ) {   // one K-major box: this CTA's 128 output columns x 128 bytes of K
@@ -518,55 +528,66 @@ cudaError_t set_pair_attributes() {
 }
 }  // namespace
 
-cudaError_t launch_gemm2(const GemmParams& p, const CUtensorMap& m_w2, const CUtensorMap& m_h, bool fp8,
-                         cudaStream_t st) {
+// every row operand: p.a_src [p.a_rows, K] (PAIR_KSPLIT: p.a_src2 too)
+static bool make_row_maps(RowMaps* m, const GemmParams& p, bool fp8) {
+  for (int i = 0; i < 4; ++i) {
+    if (!make_act_map(&m->a0[i], p.a_src, p.a_rows, p.K, fp8, 32 * (i + 1))) return false;
+    if (p.a_src2 != nullptr && !make_act_map(&m->a1[i], p.a_src2, p.a_rows, p.K, fp8, 32 * (i + 1))) return false;
+  }
+  return true;
+}
+
+cudaError_t launch_gemm2(const GemmParams& p, const CUtensorMap& m_w2, bool fp8, cudaStream_t st) {
   cudaError_t e = set_pair_attributes();
   if (e != cudaSuccess) return e;
+  RowMaps rows{};
+  if (!make_row_maps(&rows, p, fp8)) return cudaErrorInvalidValue;
   ProfileScope prof(KID_GEMM2, st);
   const bool red = p.y_acc != nullptr;
   const int g = pair_grid();
   if (fp8) {
-    if (red) return launch_pdl(ffn_gemm2_kernel<true, true, PAIR_PLAIN, false>, g, THREADS, SMEM_BYTES, st, m_w2, m_w2, m_h, m_h, p);
-    return launch_pdl(ffn_gemm2_kernel<false, true, PAIR_PLAIN, false>, g, THREADS, SMEM_BYTES, st, m_w2, m_w2, m_h, m_h, p);
+    if (red) return launch_pdl(ffn_gemm2_kernel<true, true, PAIR_PLAIN, false>, g, THREADS, SMEM_BYTES, st, m_w2, m_w2, rows, p);
+    return launch_pdl(ffn_gemm2_kernel<false, true, PAIR_PLAIN, false>, g, THREADS, SMEM_BYTES, st, m_w2, m_w2, rows, p);
   }
-  if (red) return launch_pdl(ffn_gemm2_kernel<true, false, PAIR_PLAIN, false>, g, THREADS, SMEM_BYTES, st, m_w2, m_w2, m_h, m_h, p);
-  return launch_pdl(ffn_gemm2_kernel<false, false, PAIR_PLAIN, false>, g, THREADS, SMEM_BYTES, st, m_w2, m_w2, m_h, m_h, p);
+  if (red) return launch_pdl(ffn_gemm2_kernel<true, false, PAIR_PLAIN, false>, g, THREADS, SMEM_BYTES, st, m_w2, m_w2, rows, p);
+  return launch_pdl(ffn_gemm2_kernel<false, false, PAIR_PLAIN, false>, g, THREADS, SMEM_BYTES, st, m_w2, m_w2, rows, p);
 }
 
-// GEMM-1 on CTA pairs: m_xs maps the expert-sorted activation rows [P, K]; p.tile_prefix = the 256-row pair-tile
+// GEMM-1 on CTA pairs from the expert-sorted activation rows (p.a_src = xs); p.tile_prefix = the 256-row pair-tile
 // prefix, p.n_tiles = ceil(N / 128), p.out = h.
-cudaError_t launch_gemm1_pair(const GemmParams& p, const CUtensorMap& m_w1, const CUtensorMap& m_w3,
-                              const CUtensorMap& m_xs, cudaStream_t st) {
+cudaError_t launch_gemm1_pair(const GemmParams& p, const CUtensorMap& m_w1, const CUtensorMap& m_w3, cudaStream_t st) {
   cudaError_t e = set_pair_attributes();
   if (e != cudaSuccess) return e;
+  RowMaps rows{};
+  if (!make_row_maps(&rows, p, false)) return cudaErrorInvalidValue;
   ProfileScope prof(KID_GEMM1, st);
-  return launch_pdl(ffn_gemm2_kernel<false, false, PAIR_GLU, false>, pair_grid(), THREADS, SMEM_BYTES, st, m_w1, m_w3, m_xs,
-                    m_xs, p);
+  return launch_pdl(ffn_gemm2_kernel<false, false, PAIR_GLU, false>, pair_grid(), THREADS, SMEM_BYTES, st, m_w1, m_w3, rows, p);
 }
 
 // Backward pass, all on CTA pairs (see bwd.cu for the sequence):
-//   launch_bwd_dh    dh = dO . W2^T          A = dO rows (m_do), B = W2 read K-major (m_w2t), N = f, K = d
+//   launch_bwd_dh    dh = dO . W2^T          p.a_src = dO, B = W2 read K-major (m_w2t), N = f, K = d
 //   launch_bwd_glu   GEMM-1 recomputed with the backward SwiGLU epilogue: p.dh in, p.out = h, p.out2 = dA1, p.out3 = dA3
-//   launch_bwd_dx    dXs = dA1 . W1^T + dA3 . W3^T   A = (m_da1, m_da3), B = (m_w1t, m_w3t) K-major, p.k_split k-blocks each
-cudaError_t launch_bwd_dh(const GemmParams& p, const CUtensorMap& m_w2t, const CUtensorMap& m_do, cudaStream_t st) {
+//   launch_bwd_dx    dXs = dA1 . W1^T + dA3 . W3^T   p.a_src = dA1, p.a_src2 = dA3, B = (m_w1t, m_w3t) K-major, p.k_split k-blocks each
+cudaError_t launch_bwd_dh(const GemmParams& p, const CUtensorMap& m_w2t, cudaStream_t st) {
   cudaError_t e = set_pair_attributes();
   if (e != cudaSuccess) return e;
-  return launch_pdl(ffn_gemm2_kernel<false, false, PAIR_PLAIN, true>, pair_grid(), THREADS, SMEM_BYTES, st, m_w2t, m_w2t,
-                    m_do, m_do, p);
+  RowMaps rows{};
+  if (!make_row_maps(&rows, p, false)) return cudaErrorInvalidValue;
+  return launch_pdl(ffn_gemm2_kernel<false, false, PAIR_PLAIN, true>, pair_grid(), THREADS, SMEM_BYTES, st, m_w2t, m_w2t, rows, p);
 }
-cudaError_t launch_bwd_glu(const GemmParams& p, const CUtensorMap& m_w1, const CUtensorMap& m_w3, const CUtensorMap& m_xs,
-                           cudaStream_t st) {
+cudaError_t launch_bwd_glu(const GemmParams& p, const CUtensorMap& m_w1, const CUtensorMap& m_w3, cudaStream_t st) {
   cudaError_t e = set_pair_attributes();
   if (e != cudaSuccess) return e;
-  return launch_pdl(ffn_gemm2_kernel<false, false, PAIR_GLU_BWD, false>, pair_grid(), THREADS, SMEM_BYTES, st, m_w1, m_w3,
-                    m_xs, m_xs, p);
+  RowMaps rows{};
+  if (!make_row_maps(&rows, p, false)) return cudaErrorInvalidValue;
+  return launch_pdl(ffn_gemm2_kernel<false, false, PAIR_GLU_BWD, false>, pair_grid(), THREADS, SMEM_BYTES, st, m_w1, m_w3, rows, p);
 }
-cudaError_t launch_bwd_dx(const GemmParams& p, const CUtensorMap& m_w1t, const CUtensorMap& m_w3t, const CUtensorMap& m_da1,
-                          const CUtensorMap& m_da3, cudaStream_t st) {
+cudaError_t launch_bwd_dx(const GemmParams& p, const CUtensorMap& m_w1t, const CUtensorMap& m_w3t, cudaStream_t st) {
   cudaError_t e = set_pair_attributes();
   if (e != cudaSuccess) return e;
-  return launch_pdl(ffn_gemm2_kernel<false, false, PAIR_KSPLIT, true>, pair_grid(), THREADS, SMEM_BYTES, st, m_w1t, m_w3t,
-                    m_da1, m_da3, p);
+  RowMaps rows{};
+  if (!make_row_maps(&rows, p, false)) return cudaErrorInvalidValue;
+  return launch_pdl(ffn_gemm2_kernel<false, false, PAIR_KSPLIT, true>, pair_grid(), THREADS, SMEM_BYTES, st, m_w1t, m_w3t, rows, p);
 }
 
 // Weight gradient on CTA pairs: dw[e] = A_e^T . B_e, A = [rows, M], B = [rows, N] in the padded row space (maps with
@@ -585,9 +606,10 @@ cudaError_t launch_wgrad_pair(const CUtensorMap& m_a, const CUtensorMap& m_b, co
   p.N = N;
   p.n_tiles = (N + 255) / 256;
   p.status = status;
+  RowMaps rows{};
+  rows.a0[3] = m_a;
   ProfileScope prof(KID_WGRAD, st);
-  return launch_pdl(ffn_gemm2_kernel<false, false, PAIR_WGRAD, false>, pair_grid(), THREADS, SMEM_BYTES, st, m_b, m_b, m_a,
-                    m_a, p);
+  return launch_pdl(ffn_gemm2_kernel<false, false, PAIR_WGRAD, false>, pair_grid(), THREADS, SMEM_BYTES, st, m_b, m_b, rows, p);
 }
 
 }  // namespace ffn
