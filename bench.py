@@ -36,7 +36,8 @@ KERNELS_PER_STEP = 9  # gate, topk, masks, scan, offsets, fill, gemm1, gemm2, co
 def kernels_per_step(cfg, flags: int, fp8: bool) -> int:
     """Launches of one moe_layer call, following the library's own choice of forms (see MOE_FLAG_* in tcmoe.h)."""
     from paper_2605_05607_b200 import binding as B
-    layout = 3 if cfg.P <= 32768 else 0                # up to 32768 pairs one kernel instead of four builds the layout
+    # up to 32768 pairs one kernel instead of four builds the layout, for up to 512 tokens the top-k is in it too
+    layout = 0 if cfg.P > 32768 else 4 if cfg.T <= 512 and cfg.E <= 256 else 3
     if flags & B.MOE_FLAG_FUSED_FFN:
         return 6 - layout + 2                          # ... layout, then the task-table kernel and the tracker-paced kernel
     n = KERNELS_PER_STEP - layout + (2 if fp8 else 0)  # FP8: + quantisation of x and of h

@@ -736,10 +736,14 @@ static int layer_impl(const moe_shape_t* shape, const void* x, const float* w_ga
   TCMOE_CUDA(launch_gate_logits(s, x, w_gate, lg, status, st));
   // the top-k kernel also zeroes the layout builder's bitmasks where it uses them (emask and gmask are adjacent)
   const LayoutScratch sc = scratch(ws, p);
-  TCMOE_CUDA(launch_topk(s, lg, logit_bias, bias_row_stride, idx, tw, status, st, sc.emask,
-                         layout_in_one(s) ? 0 : (size_t)(s.E + s.G) * sc.W));
-  // layout only: the dispatched copy xg is never written, GEMM-1 gathers token rows from x
-  TCMOE_CUDA(launch_layout(s, idx, L, sc, status, st, /*masks_cleared=*/s.T > 0));
+  if (topk_in_layout(s)) {
+    TCMOE_CUDA(launch_topk_layout(s, lg, logit_bias, bias_row_stride, idx, tw, L, sc, status, st));
+  } else {
+    TCMOE_CUDA(launch_topk(s, lg, logit_bias, bias_row_stride, idx, tw, status, st, sc.emask,
+                           layout_in_one(s) ? 0 : (size_t)(s.E + s.G) * sc.W));
+    // layout only: the dispatched copy xg is never written, GEMM-1 gathers token rows from x
+    TCMOE_CUDA(launch_layout(s, idx, L, sc, status, st, /*masks_cleared=*/s.T > 0));
+  }
   FfnArgs a{};
   a.a_src = x;
   Fp8Args q{};

@@ -102,6 +102,10 @@ cudaError_t launch_topk(const Shape& s, const float* logits, const float* bias, 
                         uint32_t* clear = nullptr, size_t clear_words = 0);   // clear: words zeroed on the side
 // layout.cu.  layout_in_one(s): the builder is one kernel that keeps the masks in shared memory, nothing to clear before it
 bool layout_in_one(const Shape& s);
+// topk_in_layout(s): the top-k of the layer can run inside that kernel too
+bool topk_in_layout(const Shape& s);
+cudaError_t launch_topk_layout(const Shape& s, const float* logits, const float* bias, int64_t bias_stride, int32_t* topk_idx,
+                               float* topk_w, const Layout& L, const LayoutScratch& sc, int32_t* status, cudaStream_t st);
 cudaError_t launch_layout(const Shape& s, const int32_t* topk_idx, const Layout& L, const LayoutScratch& sc,
                           int32_t* status, cudaStream_t st, bool masks_cleared = false);
 cudaError_t launch_tile_prefix(const Shape& s, const int32_t* expert_counts, int32_t* mt_prefix, int32_t* mp_prefix,

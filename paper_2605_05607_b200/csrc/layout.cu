@@ -9,6 +9,7 @@
 // turns ranks into the row tables.  No atomics touch the result arrays.
 #include "combine.cuh"
 #include "ptx.cuh"
+#include "route.cuh"
 
 #include <atomic>
 
@@ -145,20 +146,29 @@ __global__ void __launch_bounds__(256) fill_layout_kernel(const int32_t* __restr
 // three launch gaps for 256 tokens of top-2, 21 us for 3001 of top-4; in one kernel 6.2 and 9.5 us.  With more pairs the
 // scattered table stores of the fill pass want more than 8 SMs (16384 tokens of top-8: 29 us as four kernels; 10880 tokens of a sparse
 // top-8 table: 19 us either way).
-constexpr int ONE_THREADS = 1024, ONE_MAX_BLOCKS = 8, ONE_MAX_PAIRS = 32768;
+constexpr int ONE_THREADS = 1024, ONE_MAX_BLOCKS = 8, ONE_MAX_PAIRS = 32768, ONE_MAX_SMEM = 160 * 1024;
 struct OneShape { int blocks, tokens, words; size_t smem; };   // tokens per block (a multiple of 32) and their mask words
-OneShape one_shape(const Shape& s) {
+OneShape one_shape(const Shape& s, bool topk) {
   OneShape o;
   o.blocks = 1;
-  while (o.blocks < ONE_MAX_BLOCKS && o.blocks * 256 < s.T) o.blocks *= 2;
+  while (o.blocks < ONE_MAX_BLOCKS && o.blocks * (topk ? 32 : 256) < s.T) o.blocks *= 2;
   o.tokens = ((s.T + o.blocks - 1) / o.blocks + 31) & ~31;
   o.words = o.tokens / 32;
   const size_t rows = (size_t)s.E + s.G;
-  o.smem = rows * (o.words + 1) * 4 + rows * (o.words + 1) * 2 + rows * 4 * 2 + 16;
+  o.smem = rows * (o.words + 1) * 4 + rows * (o.words + 1) * 2 + rows * 4 * 2 + 16 + (topk ? (size_t)o.tokens * s.k * 4 : 0);
   return o;
 }
 
-__global__ void __launch_bounds__(ONE_THREADS) layout_one_kernel(const int32_t* __restrict__ topk_idx, Layout L,
+// With KPL > 0 the kernel first takes the top-k of its tokens (a warp each, E <= 32 KPL) and writes topk_idx / topk_w: for a batch
+// of up to 512 tokens the top-k kernel is a launch's latency as well.
+struct TopkArgs {
+  const float *logits, *bias;
+  long long bias_stride;
+  float* topk_w;
+  int score_fn;
+};
+template <int KPL>
+__global__ void __launch_bounds__(ONE_THREADS) layout_one_kernel(int32_t* topk_idx, const TopkArgs tk, Layout L,
                                                                  int32_t* mt_prefix, int32_t* mp_prefix, int T, int E, int k,
                                                                  int G, int m, int TL, int W, int32_t* status, int sparse) {
   extern __shared__ uint32_t one_s[];
@@ -167,16 +177,31 @@ __global__ void __launch_bounds__(ONE_THREADS) layout_one_kernel(const int32_t* 
   uint32_t* mask = one_s;                                                  // [rows][ld]
   int* total = reinterpret_cast<int*>(mask + (size_t)rows * ld);           // [rows] members among this block's tokens
   int* base = total + rows;                                                // [rows] table entry of the block's first member
-  uint16_t* prefix = reinterpret_cast<uint16_t*>(base + rows);             // [rows][ld] members before the word
+  int* idx_s = base + rows;                                                // [TL][k] (KPL > 0): the selection of the block's tokens
+  uint16_t* prefix = reinterpret_cast<uint16_t*>(idx_s + (KPL > 0 ? TL * k : 0));   // [rows][ld] members before the word
   const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
   const int rank = blockIdx.x, blocks = gridDim.x;                         // the grid is one cluster
   const int t0 = rank * TL, tn = max(0, min(TL, T - t0));
   for (int i = tid; i < rows * ld; i += ONE_THREADS) mask[i] = 0u;
   grid_dependency_sync();
+  if (KPL > 0) {
+    bool nonfinite = false;
+    for (int tl = wid; tl < tn; tl += ONE_THREADS / 32) {
+      uint32_t e;
+      float w;
+      topk_token<KPL == 0 ? 1 : KPL>(tk.logits, tk.bias, tk.bias_stride, t0 + tl, E, k, tk.score_fn, lane, nonfinite, e, w);
+      if (lane < k) {
+        idx_s[tl * k + lane] = (int)e;
+        topk_idx[(size_t)(t0 + tl) * k + lane] = (int32_t)e;
+        tk.topk_w[(size_t)(t0 + tl) * k + lane] = w;
+      }
+    }
+    if (__any_sync(0xFFFFFFFFu, nonfinite) && lane == 0) atomicOr(&status[ST_WARN], WARN_NONFINITE_LOGIT);
+  }
   __syncthreads();
   for (int i = tid; i < tn * k; i += ONE_THREADS) {
     const int tl = i / k;
-    const int e = __ldg(topk_idx + (size_t)t0 * k + i);
+    const int e = KPL > 0 ? idx_s[i] : __ldg(topk_idx + (size_t)t0 * k + i);
     if (e < 0 || e >= E) {
       if (!(sparse && e == -1)) report_error(status, DEV_INDEX_OUT_OF_RANGE, KID_MASKS, t0 + tl, e);   // -1: unused slot
       continue;
@@ -267,7 +292,7 @@ __global__ void __launch_bounds__(ONE_THREADS) layout_one_kernel(const int32_t* 
   }
   for (int i = tid; i < tn * k; i += ONE_THREADS) {
     const int tl = i / k, p = t0 * k + i;
-    const int e = __ldg(topk_idx + p);
+    const int e = KPL > 0 ? idx_s[i] : __ldg(topk_idx + p);
     if (e < 0 || e >= E) {           // unused slot (sparse top-k), or an index reported above
       L.pair_row[p] = -1;
       continue;
@@ -282,7 +307,35 @@ __global__ void __launch_bounds__(ONE_THREADS) layout_one_kernel(const int32_t* 
 }
 
 bool layout_in_one(const Shape& s) {
-  return s.T > 0 && (long long)s.T * s.k <= ONE_MAX_PAIRS && one_shape(s).smem <= 160 * 1024;
+  return s.T > 0 && (long long)s.T * s.k <= ONE_MAX_PAIRS && one_shape(s, false).smem <= ONE_MAX_SMEM;
+}
+
+template <int KPL>
+static cudaError_t launch_layout_one(const Shape& s, int32_t* topk_idx, const TopkArgs& tk, const Layout& L,
+                                     const LayoutScratch& sc, int32_t* status, cudaStream_t st) {
+  static std::atomic<bool> attr_set[MAX_DEVICES];   // per device; setting the attribute twice is harmless
+  const int dev = current_device();
+  if (!attr_set[dev].load(std::memory_order_acquire)) {
+    cudaError_t e = cudaFuncSetAttribute(layout_one_kernel<KPL>, cudaFuncAttributeMaxDynamicSharedMemorySize, ONE_MAX_SMEM);
+    if (e != cudaSuccess) return e;
+    attr_set[dev].store(true, std::memory_order_release);
+  }
+  const OneShape o = one_shape(s, KPL > 0);
+  return launch_pdl_cluster(o.blocks, layout_one_kernel<KPL>, o.blocks, ONE_THREADS, o.smem, st, topk_idx, tk, L, sc.mt_prefix,
+                            sc.mp_prefix, s.T, s.E, s.k, s.G, s.E / s.G, o.tokens, o.words, status, (s.flags & 4) ? 1 : 0);
+}
+
+// up to 512 tokens (at most two per warp) of up to 256 experts
+bool topk_in_layout(const Shape& s) { return s.T <= 512 && s.E <= 256 && layout_in_one(s) && one_shape(s, true).smem <= ONE_MAX_SMEM; }
+
+cudaError_t launch_topk_layout(const Shape& s, const float* logits, const float* bias, int64_t bias_stride, int32_t* topk_idx,
+                               float* topk_w, const Layout& L, const LayoutScratch& sc, int32_t* status, cudaStream_t st) {
+  const TopkArgs tk{logits, bias, (long long)bias_stride, topk_w, s.score_fn};
+  ProfileScope prof(KID_TOPK, st);
+  if (s.E <= 32) return launch_layout_one<1>(s, topk_idx, tk, L, sc, status, st);
+  if (s.E <= 64) return launch_layout_one<2>(s, topk_idx, tk, L, sc, status, st);
+  if (s.E <= 128) return launch_layout_one<4>(s, topk_idx, tk, L, sc, status, st);
+  return launch_layout_one<8>(s, topk_idx, tk, L, sc, status, st);
 }
 
 // exclusive prefixes of 128-row tiles and 256-row pair tiles per expert, from the counts alone
@@ -315,18 +368,7 @@ cudaError_t launch_layout(const Shape& s, const int32_t* topk_idx, const Layout&
                           int32_t* status, cudaStream_t st, bool masks_cleared) {
   const int m = s.E / s.G;
   cudaError_t err;
-  if (layout_in_one(s)) {
-    static std::atomic<bool> attr_set[MAX_DEVICES];   // per device; setting the attribute twice is harmless
-    const int dev = current_device();
-    if (!attr_set[dev].load(std::memory_order_acquire)) {
-      if ((err = cudaFuncSetAttribute(layout_one_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 160 * 1024)) != cudaSuccess)
-        return err;
-      attr_set[dev].store(true, std::memory_order_release);
-    }
-    const OneShape o = one_shape(s);
-    return launch_pdl_cluster(o.blocks, layout_one_kernel, o.blocks, ONE_THREADS, o.smem, st, topk_idx, L, sc.mt_prefix,
-                              sc.mp_prefix, s.T, s.E, s.k, s.G, m, o.tokens, o.words, status, (s.flags & 4) ? 1 : 0);
-  }
+  if (layout_in_one(s)) return launch_layout_one<0>(s, const_cast<int32_t*>(topk_idx), TopkArgs{}, L, sc, status, st);
   if (!masks_cleared &&
       (err = cudaMemsetAsync(sc.emask, 0, sizeof(uint32_t) * (size_t)(s.E + s.G) * sc.W, st)) != cudaSuccess)
     return err;  // emask and gmask are adjacent

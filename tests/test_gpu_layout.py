@@ -57,3 +57,30 @@ def test_layout_of_a_sparse_table(T):
     assert np.array_equal(lay.al.cpu().numpy()[:T], np.where(seen, np.cumsum(seen) - 1, -1))
     assert np.array_equal(lay.row_src.cpu().numpy()[pair_row[used]], (np.cumsum(seen) - 1)[used // k])
     assert B.moe_status(ws)[0] == 0
+
+
+@pytest.mark.parametrize("T,E,k,bias", [(1, 8, 2, 0), (32, 32, 32, 0), (33, 33, 5, 33), (256, 64, 4, 0), (257, 128, 8, 128),
+                                        (512, 256, 8, 1), (513, 256, 8, 1), (512, 257, 3, 0)])
+def test_topk_inside_the_layout_kernel(T, E, k, bias):
+    """The layer's routing and layout are those of moe_route and moe_dispatch, whichever kernel takes the top-k."""
+    d = f = 64
+    g = torch.Generator(device="cuda").manual_seed(T * E)
+    x = torch.randn(T, d, generator=g, device="cuda").to(torch.bfloat16)
+    wg = torch.randn(d, E, generator=g, device="cuda") * 0.02
+    b = None if bias == 0 else torch.randn(*((E,) if bias == 1 else (T, E)), generator=g, device="cuda")
+    ws_ = [torch.randn(E, d, f, generator=g, device="cuda").to(torch.bfloat16) for _ in range(3)]
+    shape = B.MoEShape(T, d, f, E, k, 1, T & 1, 0)
+    ws, y = B.alloc_workspace(shape), torch.empty(T, d, dtype=torch.bfloat16, device="cuda")
+    out = []
+    for fused in (False, True):
+        logits, idx = torch.empty(T, E, device="cuda"), torch.full((max(T * k, 4),), -7, dtype=torch.int32, device="cuda")
+        w, lay = torch.full((max(T * k, 4),), -7.0, device="cuda"), B.alloc_layout(shape)
+        if fused:
+            B.moe_layer(shape, x, wg, b, *ws_, y, ws, logits=logits, topk_idx=idx, topk_w=w, layout=lay)
+        else:
+            B.moe_route(shape, x, wg, b, logits, idx, w, ws)
+            B.moe_dispatch(shape, None, idx, lay, None, ws)
+        out.append((logits, idx, w) + tuple(getattr(lay, n) for n, _ in B.MoELayoutC._fields_))
+    for a, c in zip(*out):
+        assert torch.equal(a, c)
+    assert B.moe_status(ws)[0] == 0
