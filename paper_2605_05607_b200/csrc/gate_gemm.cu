@@ -15,7 +15,7 @@
 // a split weight block.  Up to 128 experts the three terms are summed apart, as one wide B of 3 GN columns: an
 // UMMA takes about 70 cycles for any N up to 128.  More experts keep one running sum (TMEM columns).
 // Measured, us, against the form with a split kernel and one tile width (T, d, E): 64, 4096, 128: 41 -> 24.5;
-// 128, 7168, 256: 157 -> 66; 1777, 2880, 128: 34 -> 20.5; 8192, 4096, 128: 49 -> 37-41; 16384, 4096, 128: 55 -> 54;
+// 128, 7168, 256: 157 -> 48; 1777, 2880, 128: 34 -> 20.5; 8192, 4096, 128: 49 -> 37-41; 16384, 4096, 128: 55 -> 54;
 // 32768, 7168, 256: 350-420 -> 308-322.
 // K is never divided over thread blocks, although that would be faster still for a decode batch (9 us
 // at T = 64, d = 4096, E = 128): a logit is the same sum in the same order whatever the tile, and a
@@ -43,14 +43,15 @@ struct GateParams {
   const float* w;     // [d, E]
   float* logits;      // [T, E]
   int T, d, E, KB, n_tiles;
-  int m_sub;          // 128-row tiles per task, 1 or 2: they share the split weight block
-  int a_bytes;        // bytes of x per row tile and stage: fewer than 128 rows are loaded when T is small (the UMMA then
+  int m_sub;          // row tiles per task, 1 or 2: they share the split weight block
+  int a_bytes;        // bytes of x per row tile and stage: fewer rows than the tile has are loaded when T is small (the UMMA then
                       // reads whatever follows; only rows >= T depend on it)
-  int apart;          // 1: hi, mid and lo sums in accumulators of their own, added at the end; 0: one running sum
   int32_t* status;
 };
 
-template <int GN, int GROUPS>
+// ROWS_M: rows of a tile, 64 or 128.  APART: hi, mid and lo sums in accumulators of their own, added at the end; otherwise one
+// running sum.
+template <int GN, int GROUPS, int ROWS_M, bool APART>
 __global__ void __launch_bounds__(THREADS, 1)
 gate_umma_kernel(const __grid_constant__ CUtensorMap map_x, const GateParams p) {
   extern __shared__ uint8_t smem_raw[];
@@ -66,8 +67,8 @@ gate_umma_kernel(const __grid_constant__ CUtensorMap map_x, const GateParams p) 
   const uint32_t done_bar = bar_base + 8u * (2 * MAX_STAGES);
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int row0 = (blockIdx.x / p.n_tiles) * p.m_sub * BM, n0 = (blockIdx.x % p.n_tiles) * GN;
-  const int n_sub = p.m_sub > 1 && row0 + BM < p.T ? 2 : 1;           // row tiles of this task that have rows
+  const int row0 = (blockIdx.x / p.n_tiles) * p.m_sub * ROWS_M, n0 = (blockIdx.x % p.n_tiles) * GN;
+  const int n_sub = p.m_sub > 1 && row0 + ROWS_M < p.T ? 2 : 1;           // row tiles of this task that have rows
   // a stage: hi | mid | lo columns of the weight block side by side in 64-column slabs of 8 KiB, then the x tiles
   constexpr int GROUP_WARPS = SPLIT_WARPS / GROUPS;
   constexpr int B_BYTES = (3 * GN + 63) / 64 * 8192;
@@ -187,14 +188,16 @@ gate_umma_kernel(const __grid_constant__ CUtensorMap map_x, const GateParams p) 
         timeout(1);
       } else {
         ptx::tc_fence_after();
-        // warp w: rows 32 (w % 4) .. + 31, every fourth 32-column block from w / 4 on
+        // warp w: TMEM lanes 32 (w % 4) .. + 31, every fourth 32-column block from w / 4 on.  A 64-row accumulator has row
+        // 16 q + i in lane 32 q + i (i < 16).
+        const int lrow = ROWS_M == 64 ? (lane < 16 ? (warp & 3) * 16 + lane : p.T) : (warp & 3) * 32 + lane;
         for (int u = warp >> 2; u < n_sub * (GN / 32); u += SPLIT_WARPS / 4) {
           const int i = u / (GN / 32), c = (u % (GN / 32)) * 32;
-          const int row = row0 + i * BM + (warp & 3) * 32 + lane;
+          const int row = row0 + i * ROWS_M + lrow;
           if (c >= ncols) continue;
           const uint32_t taddr = tmem_base + ((uint32_t)((warp & 3) * 32) << 16) + c;
           uint32_t acc[32];
-          if (p.apart) {   // logits = (hi + mid) + lo
+          if (APART) {   // logits = (hi + mid) + lo
             uint32_t other[32];
             ptx::tmem_ld32(taddr + (i * 3) * GN, acc);
 #pragma unroll
@@ -234,7 +237,7 @@ gate_umma_kernel(const __grid_constant__ CUtensorMap map_x, const GateParams p) 
         if (!ptx::mbar_wait(empty_bar(s), ph, abort_flag, global_abort)) { timeout(3); break; }
         ptx::mbar_arrive_expect_tx(full_bar(s), n_sub * p.a_bytes);
         for (int i = 0; i < n_sub; ++i)
-          ptx::tma_load_2d(smem_base + s * stage_bytes + B_BYTES + i * p.a_bytes, &map_x, full_bar(s), kb * BK, row0 + i * BM);
+          ptx::tma_load_2d(smem_base + s * stage_bytes + B_BYTES + i * p.a_bytes, &map_x, full_bar(s), kb * BK, row0 + i * ROWS_M);
         if (++s == n_stages) { s = 0; ph ^= 1; }
       }
     }
@@ -245,7 +248,7 @@ gate_umma_kernel(const __grid_constant__ CUtensorMap map_x, const GateParams p) 
       const uint32_t base = __shfl_sync(0xFFFFFFFFu, smem_base, 0), tmem = __shfl_sync(0xFFFFFFFFu, tmem_base, 0);
       const uint64_t a_desc = desc_at(desc_base(16, 1024), base + B_BYTES), b_desc = desc_at(desc_base(BK * 128, 1024), base);
       auto idesc = [](int n) {
-        return (1u << 4) | (1u << 7) | (1u << 10) | (1u << 16) | ((uint32_t)(n >> 3) << 17) | ((uint32_t)(BM >> 4) << 24);
+        return (1u << 4) | (1u << 7) | (1u << 10) | (1u << 16) | ((uint32_t)(n >> 3) << 17) | ((uint32_t)(ROWS_M >> 4) << 24);
       };
       const uint32_t stage16 = stage_bytes >> 4, a16 = p.a_bytes >> 4;
       bool ok = true;
@@ -256,7 +259,7 @@ gate_umma_kernel(const __grid_constant__ CUtensorMap map_x, const GateParams p) 
         if (elected) {
           for (int i = 0; i < n_sub; ++i) {
             const uint64_t ad = a_desc + (s * stage16 + i * a16), bd = b_desc + s * stage16;
-            if (p.apart) {   // the terms as one wide B
+            if (APART) {   // the terms as one wide B
               constexpr int N1 = 3 * GN < 256 ? 3 * GN : 256, N2 = 3 * GN - N1;
 #pragma unroll
               for (int k = 0; k < BK / 16; ++k) {
@@ -265,12 +268,12 @@ gate_umma_kernel(const __grid_constant__ CUtensorMap map_x, const GateParams p) 
                 if (N2 > 0)
                   ptx::umma_bf16(d + N1, ad + (uint64_t)(k * 2), bd + (uint64_t)(N1 / 64 * 512 + k * 128), idesc(N2), (kb | k) > 0);
               }
-            } else if (GN >= 64) {
+            } else {
 #pragma unroll
               for (int t = 0; t < 3; ++t)
 #pragma unroll
                 for (int k = 0; k < BK / 16; ++k)
-                  ptx::umma_bf16(tmem + i * GN, ad + (uint64_t)(k * 2), bd + (uint64_t)(t * (GN / 64) * 512 + k * 128), idesc(GN),
+                  ptx::umma_bf16(tmem + i * GN, ad + (uint64_t)(k * 2), bd + (uint64_t)((t * GN / 64) * 512 + (t * GN % 64) / 8 + k * 128), idesc(GN),
                                  (kb | k | t) > 0);
             }
           }
@@ -294,33 +297,36 @@ gate_umma_kernel(const __grid_constant__ CUtensorMap map_x, const GateParams p) 
   }
 }
 
-// Tile width and row tiles per task: the cheapest by a model in microseconds, fitted to this kernel: time of a k-block by
-// width and row tiles, 148 thread blocks at a time.  (32: apart only, a running sum needs whole slabs per term.)
-struct GatePlan { int gn, m_sub; };
+// Tile width, rows of a tile and row tiles per task: the cheapest by a model in microseconds, fitted to this kernel: time of a
+// k-block, 148 thread blocks at a time.  Tiles of 64 rows halve what a UMMA reads of x, which counts where twelve of them make a
+// k-block (running sum: 128 tokens of d = 7168, 256 experts 66 -> 48 us); with the terms apart they change nothing.
+struct GatePlan { int gn, bm, m_sub; };
 GatePlan plan_gate(int T, int E, bool apart) {
-  static const struct { int gn, m_sub; double kb_us[2]; } forms[] = {   // running sum, apart
-      {32, 1, {1e9, 0.3}}, {64, 1, {0.5, 0.4}}, {64, 2, {0.85, 0.6}}, {128, 1, {0.8, 0.8}}, {128, 2, {1.4, 1e9}}};
+  static const struct { int gn, bm, m_sub; double kb_us[2]; } forms[] = {   // running sum, apart
+      {32, 64, 1, {0.45, 1e9}}, {64, 64, 1, {0.5, 1e9}}, {32, 128, 1, {0.5, 0.3}}, {64, 128, 1, {0.58, 0.4}},
+      {64, 128, 2, {0.85, 0.6}}, {128, 128, 1, {0.8, 0.8}}, {128, 128, 2, {1.4, 1e9}}};
   GatePlan best{};
   double best_us = 1e30;
   for (const auto& f : forms) {
-    const long long tiles = (long long)((T + f.m_sub * BM - 1) / (f.m_sub * BM)) * ((E + f.gn - 1) / f.gn);
+    const int rows = f.m_sub * f.bm;
+    const long long tiles = (long long)((T + rows - 1) / rows) * ((E + f.gn - 1) / f.gn);
     const double us = (double)((tiles + 147) / 148) * f.kb_us[apart ? 1 : 0];
-    if (us < best_us) { best_us = us; best = GatePlan{f.gn, f.m_sub}; }
+    if (us < best_us) { best_us = us; best = GatePlan{f.gn, f.bm, f.m_sub}; }
   }
   return best;
 }
 
-template <int GN, int GROUPS>
+template <int GN, int GROUPS, int ROWS_M, bool APART>
 cudaError_t launch_width(const GateParams& p, int grid, const CUtensorMap& m_x, cudaStream_t st) {
   // per device; several host threads may get here at once: setting the attribute twice is harmless
   static std::atomic<bool> attr_set[MAX_DEVICES];
   const int dev = current_device();
   if (!attr_set[dev].load(std::memory_order_acquire)) {
-    cudaError_t e = cudaFuncSetAttribute(gate_umma_kernel<GN, GROUPS>, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_BYTES);
+    cudaError_t e = cudaFuncSetAttribute(gate_umma_kernel<GN, GROUPS, ROWS_M, APART>, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_BYTES);
     if (e != cudaSuccess) return e;
     attr_set[dev].store(true, std::memory_order_release);
   }
-  return launch_pdl(gate_umma_kernel<GN, GROUPS>, grid, THREADS, SMEM_BYTES, st, m_x, p);
+  return launch_pdl(gate_umma_kernel<GN, GROUPS, ROWS_M, APART>, grid, THREADS, SMEM_BYTES, st, m_x, p);
 }
 
 }  // namespace
@@ -330,7 +336,7 @@ cudaError_t launch_gate_logits(const Shape& s, const void* x, const float* w_gat
   if (s.T == 0) return cudaSuccess;
   const bool apart = s.E <= 128;
   const GatePlan plan = plan_gate(s.T, s.E, apart);
-  const int a_rows = s.T < BM ? (s.T + 7) & ~7 : BM;
+  const int a_rows = s.T < plan.bm ? (s.T + 7) & ~7 : plan.bm;
   CUtensorMap m_x;
   {
     cuuint64_t dims[2] = {(cuuint64_t)s.d, (cuuint64_t)s.T};
@@ -349,12 +355,18 @@ cudaError_t launch_gate_logits(const Shape& s, const void* x, const float* w_gat
   p.n_tiles = (s.E + plan.gn - 1) / plan.gn;
   p.m_sub = plan.m_sub;
   p.a_bytes = a_rows * BK * 2;
-  p.apart = apart ? 1 : 0;
   p.status = status;
-  const int grid = ((s.T + p.m_sub * BM - 1) / (p.m_sub * BM)) * p.n_tiles;
-  if (plan.gn == 32) return launch_width<32, 4>(p, grid, m_x, st);
-  if (plan.gn == 64) return launch_width<64, 2>(p, grid, m_x, st);
-  return launch_width<128, 2>(p, grid, m_x, st);
+  const int grid = ((s.T + p.m_sub * plan.bm - 1) / (p.m_sub * plan.bm)) * p.n_tiles;
+  if (apart) {
+    if (plan.gn == 32) return launch_width<32, 4, 128, true>(p, grid, m_x, st);
+    if (plan.gn == 64) return launch_width<64, 2, 128, true>(p, grid, m_x, st);
+    return launch_width<128, 2, 128, true>(p, grid, m_x, st);
+  }
+  if (plan.bm == 64 && plan.gn == 32) return launch_width<32, 4, 64, false>(p, grid, m_x, st);
+  if (plan.bm == 64) return launch_width<64, 2, 64, false>(p, grid, m_x, st);
+  if (plan.gn == 32) return launch_width<32, 4, 128, false>(p, grid, m_x, st);
+  if (plan.gn == 64) return launch_width<64, 2, 128, false>(p, grid, m_x, st);
+  return launch_width<128, 2, 128, false>(p, grid, m_x, st);
 }
 
 }  // namespace tcmoe
