@@ -175,6 +175,12 @@ static bool narrow_tiles(const Shape& s, int n_tiles) {
   return ((s.E < P ? s.E : P) + P / 128) * n_tiles < 148;
 }
 
+// At most 64 pairs in all, so at most 64 rows per expert whatever the routing: narrow tiles of 64 rows.  One token: d = 4096,
+// f = 14336, top-2 160.0 -> 151.5 us, d = 2048, f = 768, top-8 of 128 52.6 -> 50.3; 8 tokens of d = 2048, f = 4096 100 -> 96.  With more
+// than 148 full-width tiles they stay full-width: narrow 64-row ones gave 151 -> 155 us, 201 -> 205, 266 -> 268, and only with
+// few k-blocks a gain (93 -> 91, 84 -> 71).
+static bool few_rows(const Shape& s) { return (long long)s.T * s.k <= 64; }
+
 size_t fused_table_blocks(const Shape& s) { return ffn::fused_max_blocks(s.T, s.k, s.E); }
 size_t fused_tracker_bytes(const Shape& s) { return ffn::fused_tracker_words(s.T, s.k, s.E) * sizeof(int32_t); }
 
@@ -251,7 +257,7 @@ cudaError_t launch_expert_ffn(const Shape& s, const FfnArgs& a, cudaStream_t st)
     g1.tile_prefix = a.mp_prefix;
     err = ffn::launch_gemm1_pair(g1, m_w1, m_w3, st);
   } else {
-    err = ffn::launch_gemm1(g1, m_w1, m_w3, false, narrow_tiles(s, (s.f + 127) / 128), st);
+    err = ffn::launch_gemm1(g1, m_w1, m_w3, false, narrow_tiles(s, (s.f + 127) / 128), few_rows(s), st);
   }
   if (err != cudaSuccess) return err;
 
@@ -273,7 +279,7 @@ cudaError_t launch_expert_ffn(const Shape& s, const FfnArgs& a, cudaStream_t st)
     g2.a_src = a.h;
     g2.a_ld = s.f;
     g2.tile_prefix = a.mt_prefix;
-    return ffn::launch_gemm2_single(g2, m_w2, false, narrow_tiles(s, (s.d + 255) / 256), st);
+    return ffn::launch_gemm2_single(g2, m_w2, false, narrow_tiles(s, (s.d + 255) / 256), few_rows(s), st);
   }
   g2.a_src = a.h;
   g2.a_rows = P;
@@ -310,7 +316,7 @@ cudaError_t launch_expert_ffn_fp8(const Shape& s, const FfnArgs& a, const Fp8Arg
   g1.a_scale = q.sx;
   g1.b_scale = q.s1;
   g1.b_scale2 = q.s3;
-  cudaError_t err = ffn::launch_gemm1(g1, m_w1, m_w3, true, narrow1, st);
+  cudaError_t err = ffn::launch_gemm1(g1, m_w1, m_w3, true, narrow1, few_rows(s), st);
   if (err != cudaSuccess) return err;
   if ((err = launch_quantize_rows(a.h, P, s.f, q.hq, q.sh, st)) != cudaSuccess) return err;
 
@@ -334,7 +340,7 @@ cudaError_t launch_expert_ffn_fp8(const Shape& s, const FfnArgs& a, const Fp8Arg
     g2.a_src = q.hq;
     g2.a_ld = s.f;
     g2.tile_prefix = a.mt_prefix;
-    return ffn::launch_gemm2_single(g2, m_w2, true, narrow2, st);
+    return ffn::launch_gemm2_single(g2, m_w2, true, narrow2, few_rows(s), st);
   }
   g2.a_src = q.hq;
   g2.a_rows = P;

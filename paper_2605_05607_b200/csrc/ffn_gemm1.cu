@@ -37,9 +37,8 @@ namespace tcmoe {
 namespace ffn {
 namespace {
 
-constexpr int A_BYTES = BM * BK * 2;         // 16 KiB
 constexpr int RING_BYTES = 192 * 1024;       // 4 stages of A + a 256-column B, more of narrower ones
-constexpr int MAX_STAGES = 8;
+constexpr int MAX_STAGES = 12;            // 64 rows x 64 columns: 16 KiB
 constexpr int NUM_BARS = 2 * MAX_STAGES + 4;
 constexpr int STAGE_OUT_WARP = 32 * 144;     // epilogue transpose buffer of one warp: 32 rows x (128 + 16) bytes
 constexpr int TABLE_BYTES = (2 * (MAX_E + 1) * 4 + 15) & ~15;
@@ -68,13 +67,21 @@ constexpr uint32_t FEED_HINT = 1000;
 // NARROW = true: tiles of a quarter (PLAIN: 64 columns) or half the width (64 columns of W1 and of W3), for layers with fewer
 // full-width tiles than SMs: one decoded token reads two wide experts' weights through 32 full-width tiles of GEMM-2.  The
 // sums are the same, element by element.
-template <bool FP8, bool PLAIN, bool NARROW>
+//
+// FEW = true (narrow tiles only): tiles of 64 rows, for layers of at most 64 rows in all.  A stage is then a third smaller and
+// the ring holds more of the weights in flight (96 KiB instead of 64 in GEMM-2), which is what bounds a CTA that streams a column
+// slab of one expert: GEMM-2 of one token, top-2 of d = 4096, f = 14336, 58 -> 46 us (4.1 -> 5.1 TB/s).
+template <bool FP8, bool PLAIN, bool NARROW, bool FEW>
 __global__ void __launch_bounds__(THREADS, 1)
 ffn_gemm1_kernel(const __grid_constant__ CUtensorMap map_w1, const __grid_constant__ CUtensorMap map_w3,
                  const GemmParams p) {
   constexpr int BN = !NARROW ? UMMA_N : PLAIN ? 64 : 128;   // accumulator columns of a tile
   constexpr int BN_OUT = PLAIN ? BN : BN / 2;               // output columns
   constexpr int HALF = BN > 64 ? BN / 2 : BN;               // columns from each of the two weight maps (BN = 64: one)
+  constexpr int ROWS = FEW ? 64 : BM;                       // rows of a tile
+  constexpr int WROWS = ROWS / 4;                           // rows of an epilogue warp: TMEM lanes 32 w .. 32 w + WROWS - 1
+  static_assert(NARROW || !FEW, "64-row tiles come with narrow ones");
+  constexpr int A_BYTES = ROWS * BK * 2;
   constexpr int B_BYTES = BN * BK * 2, STAGE_BYTES = A_BYTES + B_BYTES;   // B: 64-column slabs of 8 KiB
   constexpr int NSTAGE = RING_BYTES / STAGE_BYTES;
   static_assert(NSTAGE <= MAX_STAGES, "barriers");
@@ -156,9 +163,9 @@ ffn_gemm1_kernel(const __grid_constant__ CUtensorMap map_w1, const __grid_consta
       const int srow = lane >> 3, piece = lane & 7;
       if (PLAIN) {
         // ---- GEMM-2 form: o = (gate weight x row scale) * acc * column scale, 256 columns
-        const int lrow = warp * 32 + lane;
+        const int lrow = warp * WROWS + lane;
         float wr = 1.f;
-        if (lrow < t.rows) {
+        if (lane < WROWS && lrow < t.rows) {
           const size_t grow = (size_t)t.row0 + lrow;
           if (p.topk_w != nullptr) wr = __ldg(p.topk_w + __ldg(p.row_pair + grow));
           if (FP8) wr *= __ldg(p.a_scale + grow);
@@ -205,11 +212,11 @@ ffn_gemm1_kernel(const __grid_constant__ CUtensorMap map_w1, const __grid_consta
           const int col = t.n0 + cc * 64 + piece * 8;
           if (col < p.N) {
 #pragma unroll
-            for (int i = 0; i < 8; ++i) {
+            for (int i = 0; i < WROWS / 4; ++i) {
               const int r = i * 4 + srow;
-              if (warp * 32 + r < t.rows) {
+              if (warp * WROWS + r < t.rows) {
                 const uint4 q = ptx::ld_shared_v4(stage + r * 144 + piece * 16);
-                *reinterpret_cast<uint4*>(p.out + (size_t)(t.row0 + warp * 32 + r) * (size_t)p.out_ld + col) = q;
+                *reinterpret_cast<uint4*>(p.out + (size_t)(t.row0 + warp * WROWS + r) * (size_t)p.out_ld + col) = q;
               }
             }
           }
@@ -221,8 +228,8 @@ ffn_gemm1_kernel(const __grid_constant__ CUtensorMap map_w1, const __grid_consta
       float* s1 = colscale_base + warp * UMMA_N;   // this warp's copy of the W1 / W3 column scales (0 beyond N)
       float* s3 = s1 + BN_OUT;
       if (FP8) {
-        const int lrow = warp * 32 + lane;
-        if (lrow < t.rows) {
+        const int lrow = warp * WROWS + lane;
+        if (lane < WROWS && lrow < t.rows) {
           int idx = __ldg(p.gather_idx + t.row0 + lrow);
           if (p.gather_div > 1) idx /= p.gather_div;
           sa = (idx >= 0 && idx < p.a_rows) ? __ldg(p.a_scale + idx) : 0.f;
@@ -267,11 +274,11 @@ ffn_gemm1_kernel(const __grid_constant__ CUtensorMap map_w1, const __grid_consta
           const int col = t.n0 + (c - 1) * 32 + piece * 8;
           if (col < p.N) {
 #pragma unroll
-            for (int i = 0; i < 8; ++i) {
-              const int r = i * 4 + srow;           // row of this warp's 32
-              if (warp * 32 + r < t.rows) {
+            for (int i = 0; i < WROWS / 4; ++i) {
+              const int r = i * 4 + srow;           // row of this warp's
+              if (warp * WROWS + r < t.rows) {
                 const uint4 q = ptx::ld_shared_v4(stage + r * 144 + piece * 16);
-                *reinterpret_cast<uint4*>(p.out + (size_t)(t.row0 + warp * 32 + r) * (size_t)p.out_ld + col) = q;
+                *reinterpret_cast<uint4*>(p.out + (size_t)(t.row0 + warp * WROWS + r) * (size_t)p.out_ld + col) = q;
               }
             }
           }
@@ -321,7 +328,7 @@ ffn_gemm1_kernel(const __grid_constant__ CUtensorMap map_w1, const __grid_consta
     const uint32_t base = __shfl_sync(0xFFFFFFFFu, smem_base, 0), tmem = __shfl_sync(0xFFFFFFFFu, tmem_base, 0);
     const uint64_t a_desc = desc_at(desc_base(16, 1024), base);
     const uint64_t b_desc = desc_at(FP8 ? desc_base(16, 1024) : desc_base(BK * 128, 1024), base + A_BYTES);   // K-major : MN-major
-    constexpr uint32_t IDESC = FP8 ? idesc_e4m3(BM, BN) : idesc_bf16(BM, BN);
+    constexpr uint32_t IDESC = FP8 ? idesc_e4m3(ROWS, BN) : idesc_bf16(ROWS, BN);
     constexpr int B_STEP = FP8 ? 2 : 128;   // 32 bytes of K per UMMA (16 bf16 / 32 E4M3): +32 B inside the swizzle row, or +2 atoms
     int s = 0, tl = 0;
     uint32_t ph = 0;
@@ -356,11 +363,11 @@ ffn_gemm1_kernel(const __grid_constant__ CUtensorMap map_w1, const __grid_consta
     for (int w = blockIdx.x; w < total && !*abort_flag; w += gridDim.x) {
       const Tile t = tile_of(w);
       constexpr int ELEM = FP8 ? 1 : 2;   // bytes per element of the source rows
-      const uint8_t* src[8];
+      const uint8_t* src[ROWS / 16];
       const uint8_t* base = static_cast<const uint8_t*>(p.a_src);
       uint32_t live = 0;
 #pragma unroll
-      for (int j = 0; j < 8; ++j) {
+      for (int j = 0; j < ROWS / 16; ++j) {
         const int lr = rbase + 16 * j;
         src[j] = base;
         if (lr < t.rows) {
@@ -387,7 +394,7 @@ ffn_gemm1_kernel(const __grid_constant__ CUtensorMap map_w1, const __grid_consta
         const int col = kb * 128 + chunk * 16;   // byte offset inside the source row
         const bool kin = col < p.K * ELEM;
 #pragma unroll
-        for (int j = 0; j < 8; ++j) {
+        for (int j = 0; j < ROWS / 16; ++j) {
           const int lr = rbase + 16 * j;
           const uint32_t dst = sa + lr * 128 + ((chunk ^ (lr & 7)) << 4);
           const bool on = kin && ((live >> j) & 1u);
@@ -418,37 +425,41 @@ ffn_gemm1_kernel(const __grid_constant__ CUtensorMap map_w1, const __grid_consta
 }  // namespace
 
 namespace {
-template <bool FP8, bool PLAIN, bool NARROW>
+template <bool FP8, bool PLAIN, bool NARROW, bool FEW>
 cudaError_t launch_form(const GemmParams& p, const CUtensorMap& m_a, const CUtensorMap& m_b, cudaStream_t st) {
   // per device; several host threads may get here at once: setting the attribute twice is harmless
   static std::atomic<bool> attr_set[MAX_DEVICES];
   const int dev = current_device();
+  const auto kernel = ffn_gemm1_kernel<FP8, PLAIN, NARROW, FEW>;
   if (!attr_set[dev].load(std::memory_order_acquire)) {
-    cudaError_t e = cudaFuncSetAttribute(ffn_gemm1_kernel<FP8, PLAIN, NARROW>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         SMEM_BYTES);
+    cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_BYTES);
     if (e != cudaSuccess) return e;
     attr_set[dev].store(true, std::memory_order_release);
   }
   ProfileScope prof(PLAIN ? KID_GEMM2 : KID_GEMM1, st);
-  return launch_pdl(ffn_gemm1_kernel<FP8, PLAIN, NARROW>, sm_count(), THREADS, SMEM_BYTES, st, m_a, m_b, p);
+  return launch_pdl(kernel, sm_count(), THREADS, SMEM_BYTES, st, m_a, m_b, p);
+}
+
+template <bool FP8, bool PLAIN>
+cudaError_t launch_width(const GemmParams& p, const CUtensorMap& m_a, const CUtensorMap& m_b, bool narrow, bool few, cudaStream_t st) {
+  if (!narrow) return launch_form<FP8, PLAIN, false, false>(p, m_a, m_b, st);
+  return few ? launch_form<FP8, PLAIN, true, true>(p, m_a, m_b, st) : launch_form<FP8, PLAIN, true, false>(p, m_a, m_b, st);
 }
 }  // namespace
 
 // narrow: 64 output columns per tile instead of 128 (GEMM-1) or 256 (GEMM-2); p.n_tiles is set here.  The FP8 weight maps then
-// have boxes of 64 columns (make_weight_map_fp8).
-cudaError_t launch_gemm1(GemmParams p, const CUtensorMap& m_w1, const CUtensorMap& m_w3, bool fp8, bool narrow,
+// have boxes of 64 columns (make_weight_map_fp8).  few: no expert has more than 64 rows (used by narrow tiles only).
+cudaError_t launch_gemm1(GemmParams p, const CUtensorMap& m_w1, const CUtensorMap& m_w3, bool fp8, bool narrow, bool few,
                          cudaStream_t st) {
   p.n_tiles = narrow ? (p.N + 63) / 64 : (p.N + 127) / 128;
-  if (fp8) return narrow ? launch_form<true, false, true>(p, m_w1, m_w3, st) : launch_form<true, false, false>(p, m_w1, m_w3, st);
-  return narrow ? launch_form<false, false, true>(p, m_w1, m_w3, st) : launch_form<false, false, false>(p, m_w1, m_w3, st);
+  return fp8 ? launch_width<true, false>(p, m_w1, m_w3, narrow, few, st) : launch_width<false, false>(p, m_w1, m_w3, narrow, few, st);
 }
 
 // GEMM-2 through the single-CTA kernel (128-row tiles): p.a_src = h (or its E4M3 copy), p.a_ld = f,
 // p.tile_prefix = the 128-row tile prefix; m_w2 is the weight map.
-cudaError_t launch_gemm2_single(GemmParams p, const CUtensorMap& m_w2, bool fp8, bool narrow, cudaStream_t st) {
+cudaError_t launch_gemm2_single(GemmParams p, const CUtensorMap& m_w2, bool fp8, bool narrow, bool few, cudaStream_t st) {
   p.n_tiles = narrow ? (p.N + 63) / 64 : (p.N + 255) / 256;
-  if (fp8) return narrow ? launch_form<true, true, true>(p, m_w2, m_w2, st) : launch_form<true, true, false>(p, m_w2, m_w2, st);
-  return narrow ? launch_form<false, true, true>(p, m_w2, m_w2, st) : launch_form<false, true, false>(p, m_w2, m_w2, st);
+  return fp8 ? launch_width<true, true>(p, m_w2, m_w2, narrow, few, st) : launch_width<false, true>(p, m_w2, m_w2, narrow, few, st);
 }
 
 }  // namespace ffn

@@ -599,3 +599,32 @@ def test_narrow_gemm_tiles_give_the_same_bits(T, fp8):
         return y
 
     assert torch.equal(layer(T), layer(big.T)[:T])
+
+
+@pytest.mark.parametrize("fp8", [False, True], ids=["bf16", "fp8"])
+@pytest.mark.parametrize("T,k", [(1, 1), (31, 2), (64, 1), (65, 1)])
+def test_narrow_gemm_tiles_of_few_rows(T, k, fp8):
+    """At most 64 pairs: the narrow tiles have 64 rows.  Every token prefers the same experts, so a tile is filled up to its last
+    row; the first rows of a batch that is large enough for full-width tiles are the same bits (ragged K and N)."""
+    big = synth.MoEConfig("few", T=1020, d=1040, f=1008, E=4, k=k, G=2, seed=32)
+    t = synth.make_inputs(big, "cuda")
+    bias = torch.tensor([3.0, 2.0, 0.0, 0.0], device="cuda")
+    if fp8:
+        q = {}
+        for n in ("w1", "w3", "w2"):
+            q[n] = torch.empty(big.E, t[n].shape[2], t[n].shape[1], dtype=torch.uint8, device="cuda")
+            q["s" + n] = torch.empty(big.E, t[n].shape[2], dtype=torch.float32, device="cuda")
+            B.moe_quantize_weights(t[n], q[n], q["s" + n])
+
+    def layer(n):
+        shape = B.make_shape(big.with_(T=n))
+        ws, y = B.alloc_workspace(shape), torch.empty(n, big.d, dtype=torch.bfloat16, device="cuda")
+        x = t["x"][:n].contiguous()
+        if fp8:
+            B.moe_layer_fp8(shape, x, t["w_gate"], bias, q["w1"], q["sw1"], q["w3"], q["sw3"], q["w2"], q["sw2"], y, ws)
+        else:
+            B.moe_layer(shape, x, t["w_gate"], bias, t["w1"], t["w3"], t["w2"], y, ws)
+        assert B.moe_status(ws)[0] == 0
+        return y
+
+    assert torch.equal(layer(T), layer(big.T)[:T])
