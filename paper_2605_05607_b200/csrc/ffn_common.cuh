@@ -51,6 +51,7 @@ struct GemmParams {
 struct Tile {
   int e, n0, row0, rows;
   int left;           // rows of the expert from the (pair) tile's first row on
+  bool half;          // pair tile of at most 128 rows (set by the pair kernel)
   int out_row0, kb;   // weight-gradient tiles of the pair kernel: first output row of this CTA, k-blocks of the task
 };
 
@@ -82,6 +83,7 @@ __device__ __forceinline__ Tile decode_tile(int w, const int* tp, const int* eof
   t.row0 = eoff[lo] + (g * mg + local % gsize) * rows_per_tile + rank * BM;
   t.left = eoff[lo + 1] - (t.row0 - rank * BM);
   t.rows = min(BM, t.left - rank * BM);
+  t.half = false;
   t.out_row0 = t.row0;
   t.kb = 0;
   return t;

@@ -6,13 +6,19 @@
 // The same kernel, with GLU = true, is the CTA-pair form of GEMM-1 (Sec. II-A "GEMM-1") on rows that Dispatch
 // has already placed in expert-sorted order (the per-expert layout tensors of Sec. III-D):
 //     h[r, n] = silu(a_r . W1[e][:, n]) * (a_r . W3[e][:, n])
-// CTA 0 of the pair then holds the 128-column tile of W1 and CTA 1 the same tile of W3, so the pair's 256
-// accumulator columns are [a.W1 | a.W3] for every row and the epilogue applies SwiGLU to column c and c + 128.
+// Each CTA of the pair then holds 64 columns of W1 and the same 64 of W3, so the pair's 256 accumulator columns are
+// [a.W1 | a.W3 | a.W1 | a.W3], 64 each, for every row and the epilogue applies SwiGLU to columns c and c + 64.
 //
 // Both operands come by TMA (h rows are contiguous in expert-sorted order).  CTAs work in pairs
 // (cluster of 2, tcgen05 cta_group::2): each CTA holds 128 rows of h and one half of the
 // 256-column W2 tile; one UMMA of M = 256 spans the pair, so every weight byte is fetched and read
 // from shared memory once per 256 rows.  Rank 0 of the pair (the leader) issues every UMMA.
+//
+// A row tile of at most 128 rows (most tiles of small experts, half of the last ones of large experts) takes UMMAs of M = 128
+// instead, 64 rows in each CTA, which need half the tensor-pipe time; B is the same.  The accumulator of a CTA is then 64 rows
+// in 128 TMEM columns: lanes 0-63 hold the tile's first 128 accumulator columns, lanes 64-127 the others.
+// Weight-streaming layers (12004 pairs on 128 experts of 2880 x 2880, mostly below 128 rows) were bound by the padded UMMAs:
+// dH 395 -> 352 us, GEMM-1 recomputed 797 -> 693, dX 790 -> 681, against 325 / 645 / 645 for reading the weights.
 //
 // Barrier ownership in a pair:
 //   full[s]    leader's copy: the leader announces the bytes of both CTAs, both CTAs' TMA loads
@@ -146,6 +152,10 @@ ffn_gemm2_kernel(const __grid_constant__ CUtensorMap map_b0, const __grid_consta
   constexpr bool WGRAD = MODE == PAIR_WGRAD;
   const int wg_mt = (p.K + 2 * BM - 1) / (2 * BM), wg_per_expert = wg_mt * p.n_tiles;   // weight-gradient tiles per expert
   const int total = WGRAD ? p.E * wg_per_expert : tp_s[p.E] * p.n_tiles;
+  // 128-row tiles where they are most of the tiles, or where a pair has enough tiles to even out the two lengths.  With a handful
+  // of mixed tiles the longest chain is as long as before, and pairs that read the same weights no longer do so at the same time:
+  // GEMM-2 of 4096 x 14336 experts with 1024 rows (8 tiles per pair) 705 -> 724 us, its GEMM-1 (54 per pair) 1443 -> 1397.
+  const bool halves = total >= 12 * num_clusters || eoff_s[p.E] < 160 * tp_s[p.E];
   constexpr int BK_ELEMS = FP8 ? 2 * BK : BK;   // K elements per stage: 128 bytes per row either way
   const int KB = MODE == PAIR_KSPLIT ? 2 * p.k_split : (p.K + BK_ELEMS - 1) / BK_ELEMS;
   volatile int* abort_flag = abort_s;
@@ -156,7 +166,7 @@ ffn_gemm2_kernel(const __grid_constant__ CUtensorMap map_b0, const __grid_consta
     p.status[ST_ABORT] = 1;
     *abort_flag = 1;
   };
-  auto tile_of = [&](int w) {
+  auto tile_of = [&](int w) {   // .half: a tile of at most 128 rows, 64 in each CTA
     if (WGRAD) {   // (expert, m-tile of 256, n-tile of 256), m-tile fastest: neighbours share the B rows in L2
       Tile t;
       t.e = w / wg_per_expert;
@@ -167,16 +177,24 @@ ffn_gemm2_kernel(const __grid_constant__ CUtensorMap map_b0, const __grid_consta
       t.kb = (eoff_s[t.e + 1] - t.row0) / BK;
       t.rows = min(BM, p.K - m0);                            // rows of dW[e] this CTA owns (<= 0: none)
       t.left = 0;
+      t.half = false;
       t.out_row0 = t.e * p.K + m0;
       return t;
     }
-    return decode_tile(w, tp_s, eoff_s, p.E, p.n_tiles, BN_OUT, 2 * BM, rank);
+    Tile t = decode_tile(w, tp_s, eoff_s, p.E, p.n_tiles, BN_OUT, 2 * BM, rank);
+    t.half = halves && t.left <= BM;
+    if (t.half) {
+      t.row0 -= rank * (BM / 2);
+      t.rows = min(BM / 2, t.left - rank * (BM / 2));
+      t.out_row0 = t.row0;
+    }
+    return t;
   };
 
   if (warp < EPI_WARPS) {
     // ================================ epilogue (both CTAs) ================================
-    const int quarter = warp & 3, half = warp >> 2;   // rows (TMEM lanes) and half of the columns this warp owns
-    constexpr int COLS = BN_OUT / 2;                  // output columns of a warp
+    const int quarter = warp & 3, half = warp >> 2;   // TMEM lanes and half of their columns this warp owns
+    constexpr int COLS = BN_OUT / 2;                  // output columns of a warp (tiles of at most 128 rows: half of them)
     // A thread owns one accumulator row, but 32 threads storing 16 bytes each to 32 different rows cost 32 memory
     // transactions per instruction.  The warp transposes 32 columns at a time through shared memory (64-byte rows, pieces
     // swizzled by row pair: conflict-free both ways) and stores 64-byte row segments, 8 rows per instruction.
@@ -189,25 +207,31 @@ ffn_gemm2_kernel(const __grid_constant__ CUtensorMap map_b0, const __grid_consta
     for (int w = cluster_id; w < total && !*abort_flag; w += num_clusters, ++tl) {
       const Tile t = tile_of(w);
       const int buf = tl & 1;
+      // 128-row halves: rows 32 quarter + lane, columns `half`.  64-row halves: rows 32 (quarter & 1) + lane, columns quarter >> 1,
+      // which the two warps of a quarter share (the backward SwiGLU leaves them to one, for the sums over 64 columns).
+      const int row_w = (t.half ? quarter & 1 : quarter) * 32, part = t.half ? quarter >> 1 : half;
+      const int sub = t.half && MODE != PAIR_GLU_BWD ? half * (COLS / 2) : 0;
+      const int chunks = t.half ? COLS / 64 : COLS / 32;
+      const bool idle = MODE == PAIR_GLU_BWD && t.half && half != 0;
+      const int col0 = t.n0 + part * COLS + sub;      // first output column of this warp
       uint4 dh[2][4];
       if (MODE == PAIR_GLU_BWD) {   // the incoming gradient of h, 64 columns of the warp's rows, while the main loop runs
 #pragma unroll
         for (int c = 0; c < 2; ++c)
 #pragma unroll
           for (int i = 0; i < 4; ++i) {
-            const int r = quarter * 32 + i * 8 + srow, col = t.n0 + half * COLS + c * 32 + piece * 8;
-            dh[c][i] = r < t.rows && col < p.N
+            const int r = row_w + i * 8 + srow, col = col0 + c * 32 + piece * 8;
+            dh[c][i] = r < t.rows && col < p.N && !idle
                            ? __ldg(reinterpret_cast<const uint4*>(p.dh + (size_t)(t.row0 + r) * (size_t)p.out_ld + col))
                            : make_uint4(0u, 0u, 0u, 0u);
           }
       }
       if (!ptx::mbar_wait_warp<false, HINT>(tfull_bar(buf), (tl >> 1) & 1, abort_flag, global_abort)) { timeout(1); break; }
       ptx::tc_fence_after();
-      const int lrow = quarter * 32 + lane;
+      const int lrow = row_w + lane;
       const bool valid = lrow < t.rows;
       const size_t grow = (size_t)(valid ? t.row0 + lrow : 0);
-      const int col0 = t.n0 + half * COLS;            // first output column of this warp
-      const uint32_t taddr = tmem_base + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(buf * UMMA_N + half * COLS);
+      const uint32_t taddr = tmem_base + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(buf * UMMA_N + (t.half ? 0 : half * 128) + sub);
       auto send = [&](__nv_bfloat16* out, int c) {    // 32 staged columns -> rows of out
         __syncwarp();
         const int col = col0 + c * 32 + piece * 8;
@@ -215,9 +239,9 @@ ffn_gemm2_kernel(const __grid_constant__ CUtensorMap map_b0, const __grid_consta
 #pragma unroll
           for (int i = 0; i < 4; ++i) {
             const int r = i * 8 + srow;               // row of this warp's 32
-            if (quarter * 32 + r < t.rows) {
+            if (row_w + r < t.rows) {
               const uint4 q = ptx::ld_shared_v4(stage + r * 64 + ((piece ^ ((r >> 1) & 3)) << 4));
-              *reinterpret_cast<uint4*>(out + (size_t)(t.out_row0 + quarter * 32 + r) * (size_t)p.out_ld + col) = q;
+              *reinterpret_cast<uint4*>(out + (size_t)(t.out_row0 + row_w + r) * (size_t)p.out_ld + col) = q;
             }
           }
         }
@@ -243,7 +267,8 @@ ffn_gemm2_kernel(const __grid_constant__ CUtensorMap map_b0, const __grid_consta
         }
         __syncwarp();
       }
-      if (MODE == PAIR_GLU_BWD) {
+      if (MODE == PAIR_GLU_BWD && idle) {
+      } else if (MODE == PAIR_GLU_BWD) {
         // backward of SwiGLU on the recomputed pre-activations, 32 columns at a time: dh comes to the owner of its row through
         // the staging buffer, h / dA1 / dA3 leave through it
         float dot = 0.f;   // h . dh over this warp's columns, of the rounded values (the gate's gradient needs it)
@@ -257,7 +282,7 @@ ffn_gemm2_kernel(const __grid_constant__ CUtensorMap map_b0, const __grid_consta
           }
           uint32_t a1[32], a3[32];
           ptx::tmem_ld32(taddr + c * 32, a1);
-          ptx::tmem_ld32(taddr + 128 + c * 32, a3);
+          ptx::tmem_ld32(taddr + 64 + c * 32, a3);
           ptx::tmem_ld_wait();
           __syncwarp();
           uint32_t q1[16], q3[16];
@@ -297,14 +322,14 @@ ffn_gemm2_kernel(const __grid_constant__ CUtensorMap map_b0, const __grid_consta
           for (int v = 0; v < 4; ++v) put(v, q3[v * 4], q3[v * 4 + 1], q3[v * 4 + 2], q3[v * 4 + 3]);
           send(p.out3, c);
         }
-        if (valid) p.row_dots[(size_t)(t.n0 / BN_OUT * 2 + half) * p.dots_ld + grow] = dot;
+        if (valid) p.row_dots[(size_t)(t.n0 / BN_OUT * 2 + part) * p.dots_ld + grow] = dot;
       } else if (GLU) {
-        // SwiGLU of the W1 half (accumulator columns 0..127) and the W3 half (128..255)
+        // SwiGLU of 64 columns of W1 and the 64 of W3 behind them
 #pragma unroll 1
-        for (int c = 0; c < 2; ++c) {
+        for (int c = 0; c < chunks; ++c) {
           uint32_t a1[32], a3[32];
           ptx::tmem_ld32(taddr + c * 32, a1);
-          ptx::tmem_ld32(taddr + 128 + c * 32, a3);
+          ptx::tmem_ld32(taddr + 64 + c * 32, a3);
           ptx::tmem_ld_wait();
 #pragma unroll
           for (int v = 0; v < 4; ++v) {
@@ -321,7 +346,7 @@ ffn_gemm2_kernel(const __grid_constant__ CUtensorMap map_b0, const __grid_consta
         }
       } else if (RED) {
 #pragma unroll 1
-        for (int c = 0; c < 4; ++c) {
+        for (int c = 0; c < chunks; ++c) {
           uint32_t acc[32];
           ptx::tmem_ld32(taddr + c * 32, acc);
           ptx::tmem_ld_wait();
@@ -347,7 +372,7 @@ ffn_gemm2_kernel(const __grid_constant__ CUtensorMap map_b0, const __grid_consta
         }
       } else {
 #pragma unroll 1
-        for (int c = 0; c < 4; ++c) {
+        for (int c = 0; c < chunks; ++c) {
           uint32_t acc[32];
           ptx::tmem_ld32(taddr + c * 32, acc);
           ptx::tmem_ld_wait_on(acc);
@@ -385,9 +410,10 @@ ffn_gemm2_kernel(const __grid_constant__ CUtensorMap map_b0, const __grid_consta
         bool ok = true;
         const int KBt = WGRAD ? t.kb : KB;
         // 32-row blocks of the tile in this CTA and in both (the expert's rows from the pair's first row on: t.left)
-        auto blocks32 = [](int left) { return min(max(left + 31, 0) >> 5, BM / 32); };
-        const int mine = WGRAD ? 4 : blocks32(t.left - rank * BM);
-        const uint32_t bytes = 2 * B_BYTES + (WGRAD ? 8 : blocks32(t.left) + blocks32(t.left - BM)) * (A_BYTES / 4);
+        const int cta_rows = t.half ? BM / 2 : BM;
+        auto blocks32 = [&](int left) { return min(max(left + 31, 0), cta_rows) >> 5; };
+        const int mine = WGRAD ? 4 : blocks32(t.left - rank * cta_rows);
+        const uint32_t bytes = 2 * B_BYTES + (WGRAD ? 8 : blocks32(t.left) + blocks32(t.left - cta_rows)) * (A_BYTES / 4);
         for (int kb = 0; kb < KBt; ++kb, ++it) {
           const int s = it % NSTAGE;
           if (!ptx::mbar_wait<false, HINT>(empty_bar(s), ((it / NSTAGE) & 1) ^ 1, abort_flag, global_abort)) {
@@ -408,13 +434,13 @@ ffn_gemm2_kernel(const __grid_constant__ CUtensorMap map_b0, const __grid_consta
           const bool second = MODE == PAIR_KSPLIT && kb >= p.k_split;     // second (A, B) pair of the K walk
           const int k0 = (second ? kb - p.k_split : kb) * BK_ELEMS;
           if (mine > 0) ptx::tma_load_2d_pair(sa, (second ? rows.a1 : rows.a0) + mine - 1, lead_full, k0, t.row0);
-          const CUtensorMap* map_b = MODE == PAIR_KSPLIT ? (second ? &map_b1 : &map_b0) : (rank == 0 ? &map_b0 : &map_b1);
-          const int nb = GLU ? t.n0 : t.n0 + rank * 128;   // this CTA's 128 columns of the B tile
+          const CUtensorMap* map_b = second ? &map_b1 : &map_b0;
+          const int nb = t.n0 + rank * (BN_OUT / 2);   // this CTA's columns of the B tile
           if (KMAJ) {   // one K-major box: this CTA's 128 output columns x 128 bytes of K
             ptx::tma_load_3d_pair(sb, map_b, lead_full, k0, nb, t.e);
-          } else {     // two MN-major slabs of 64 output columns x 64 rows of K
+          } else {     // two MN-major slabs of 64 output columns x 64 rows of K, or one of W1 and the same of W3
             ptx::tma_load_3d_pair(sb, map_b, lead_full, nb, k0, t.e);
-            ptx::tma_load_3d_pair(sb + 8192, map_b, lead_full, nb + 64, k0, t.e);
+            ptx::tma_load_3d_pair(sb + 8192, GLU ? &map_b1 : map_b, lead_full, GLU ? nb : nb + 64, k0, t.e);
           }
         }
         if (!ok) break;
@@ -430,17 +456,20 @@ ffn_gemm2_kernel(const __grid_constant__ CUtensorMap map_b0, const __grid_consta
       const uint64_t a_desc = desc_at(WGRAD ? mn : km, base), b_desc = desc_at(KMAJ ? km : mn, base + A_BYTES);
       constexpr int A_STEP = WGRAD ? 128 : 2, B_STEP = KMAJ ? 2 : 128;            // 32 bytes of K: 16 bf16 / 32 E4M3
       constexpr uint32_t ID = FP8 ? IDESC_F8 : WGRAD ? IDESC_WG : BKMAJ ? IDESC_BK : IDESC;
+      constexpr uint32_t ID_HALF = (ID & ~(0x1Fu << 24)) | ((uint32_t)(BM >> 4) << 24);   // M = 128
       int s = 0, tl = 0;
       uint32_t ph = 0;
       bool ok = true;
       for (int w = cluster_id; ok && w < total && !*abort_flag; w += num_clusters, ++tl) {
         const int buf = tl & 1;
+        const Tile t = tile_of(w);
+        const uint32_t id = t.half ? ID_HALF : ID;
         if (!ptx::mbar_wait_cluster<HINT>(tempty_bar(buf), ((tl >> 1) & 1) ^ 1, abort_flag, global_abort)) {
           timeout(3); break;
         }
         ptx::tc_fence_after();
         const uint32_t d_tmem = tmem + (uint32_t)(buf * UMMA_N);
-        const int KBt = WGRAD ? tile_of(w).kb : KB;
+        const int KBt = WGRAD ? t.kb : KB;
         for (int kb = 0; kb < KBt; ++kb) {
           if (!ptx::mbar_wait_cluster<HINT>(full_bar(s), ph, abort_flag, global_abort)) {
             timeout(4); ok = false; break;
@@ -450,8 +479,8 @@ ffn_gemm2_kernel(const __grid_constant__ CUtensorMap map_b0, const __grid_consta
             const uint64_t ad = a_desc + (uint64_t)(s * (STAGE_BYTES >> 4)), bd = b_desc + (uint64_t)(s * (STAGE_BYTES >> 4));
 #pragma unroll
             for (int k = 0; k < 4; ++k) {
-              if (FP8) ptx::umma_f8_pair(d_tmem, ad + (uint64_t)(k * A_STEP), bd + (uint64_t)(k * B_STEP), ID, (kb | k) != 0);
-              else ptx::umma_bf16_pair(d_tmem, ad + (uint64_t)(k * A_STEP), bd + (uint64_t)(k * B_STEP), ID, (kb | k) != 0);
+              if (FP8) ptx::umma_f8_pair(d_tmem, ad + (uint64_t)(k * A_STEP), bd + (uint64_t)(k * B_STEP), id, (kb | k) != 0);
+              else ptx::umma_bf16_pair(d_tmem, ad + (uint64_t)(k * A_STEP), bd + (uint64_t)(k * B_STEP), id, (kb | k) != 0);
             }
             ptx::umma_commit_both(empty_bar(s));   // free the stage in both CTAs once these UMMAs have read it
           }

@@ -304,3 +304,48 @@ def test_gate_weight_gradient_tiles(rows):
     assert np.array_equal(np.bincount(run.host_idx().reshape(-1), minlength=4), [512, rows, 0, 512 - rows])
     assert not dwg[:, 2].any()
     close(dwg, ref, "dw_gate")
+
+
+@pytest.mark.parametrize("rows", [1, 33, 64, 65, 127, 128, 129])
+def test_pair_tiles_of_at_most_128_rows(rows):
+    """The pair GEMMs split a tile of at most 128 rows 64 + 64 over the two CTAs.  One expert with 192 rows, one with `rows`, one with
+    the rest, one with none: the layer (bf16 and FP8) has the bits of the single-CTA form, the gradients match the oracle."""
+    cfg = synth.MoEConfig("halves", T=192, d=336, f=400, E=4, k=2, G=2, seed=rows)
+    bias = torch.zeros(cfg.T, cfg.E, device="cuda")
+    bias[:, 0] = 20.0
+    bias[:rows, 1] = 20.0
+    bias[rows:, 3] = 20.0
+    inputs = synth.make_inputs(cfg, "cuda")
+    inputs["bias"] = bias
+    q = {}
+    for n in ("w1", "w3", "w2"):
+        E, K, N = inputs[n].shape
+        q[n] = torch.empty(E, N, K, dtype=torch.uint8, device="cuda")
+        q["s" + n] = torch.empty(E, N, dtype=torch.float32, device="cuda")
+        B.moe_quantize_weights(inputs[n], q[n], q["s" + n])
+    out, out8 = [], []
+    for flags, flags8 in ((B.MOE_FLAG_GEMM2_SINGLE,) * 2, (B.MOE_FLAG_GEMM1_PAIR | B.MOE_FLAG_GEMM2_PAIR, B.MOE_FLAG_GEMM2_PAIR)):
+        run = H.Run(cfg, flags, inputs)
+        run.layer()
+        out.append(run.y)
+        shape = B.make_shape(cfg, flags8)
+        ws, y = B.alloc_workspace(shape), torch.empty_like(run.y)
+        B.moe_layer_fp8(shape, inputs["x"], inputs["w_gate"], bias, q["w1"], q["sw1"], q["w3"], q["sw3"], q["w2"], q["sw2"], y, ws)
+        out8.append(y)
+        torch.cuda.synchronize()
+        assert run.status()[0] == 0 and B.moe_status(ws)[0] == 0
+    assert torch.equal(out[0], out[1]) and torch.equal(out8[0], out8[1])
+
+    bw = Backward(cfg)
+    bw.run.t["bias"] = bias
+    bw.run.route()
+    bw.run.dispatch()
+    bw()
+    run = bw.run
+    assert np.array_equal(np.bincount(run.host_idx().reshape(-1), minlength=4), [192, rows, 0, 192 - rows])
+    dx_ref, grads = O.layer_backward(H.bf16_host(run.t["x"]), run.host_idx(), run.host_w(),
+                                     *(H.bf16_host(run.t[n]) for n in ("w1", "w3", "w2")), O.bf16_to_f64(H.bf16_host(bw.dy))[: cfg.T])
+    close(O.bf16_to_f64(H.bf16_host(bw.dx))[: cfg.T], dx_ref, "dx")
+    for e, ref in grads.items():
+        for got, r, n in zip((bw.dw1, bw.dw3, bw.dw2), ref, ("dW1", "dW3", "dW2")):
+            close(O.bf16_to_f64(H.bf16_host(got[e])), r, f"{n} of expert {e}")
