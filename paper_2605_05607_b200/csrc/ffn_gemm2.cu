@@ -252,9 +252,9 @@ ffn_gemm2_kernel(const __grid_constant__ CUtensorMap map_b0, const __grid_consta
       if (valid && !GLU && !WGRAD && (RED || p.topk_w != nullptr)) {
         const int pair = __ldg(p.row_pair + grow);
         if (p.topk_w != nullptr) wr = __ldg(p.topk_w + pair);
-        if (FP8) wr *= __ldg(p.a_scale + grow);   // row scale of h joins the gate weight
         if (RED) yrow = p.y_acc + (size_t)(pair / p.y_div) * (size_t)p.N + col0;
       }
+      if (FP8 && valid) wr *= __ldg(p.a_scale + grow);   // row scale of h joins the gate weight
       // FP8: the tile's output-column scales, one copy per warp (0 beyond N), staged while the
       // main loop of this tile may still be running
       float* sb_col = colscale_base + warp * (UMMA_N / 2);
