@@ -104,7 +104,7 @@ enum { MOE_FLAG_WEIGHT_IN_COMBINE = 1,   /* default (0): gate weight applied in 
        MOE_FLAG_GEMM2_PAIR = 32,         /* GEMM-2 runs on 256-row CTA-pair tiles (cta_group::2) whatever the shape */
        MOE_FLAG_GEMM2_SINGLE = 64,       /* GEMM-2 runs on 128-row single-CTA tiles whatever the shape.  Without either
                                             flag the library picks from the shape: pair tiles unless experts hold
-                                            fewer than 512 rows on average.  The two flags exclude each other; the
+                                            fewer than 192 rows on average.  The two flags exclude each other; the
                                             results of both forms meet the same tolerances.               */
        MOE_FLAG_FUSED_FFN = 8 };         /* moe_expert_ffn / moe_layer (bf16 experts): the stages after the layout run
                                             as ONE persistent kernel paced by the token tracker of Sec. IV-B (tiles of

@@ -156,14 +156,16 @@ int sm_count() {
   return n;
 }
 
-// Experts holding few rows on average: 256-row CTA-pair tiles would be mostly padding (a Zipf-routed
-// 128-expert layer has most experts below 128 rows), so GEMM-2 takes 128-row single-CTA tiles.  Decided from the
-// shape alone (the routing-dependent counts never visit the host); flag bits 32 (MOE_FLAG_GEMM2_PAIR) and 64
-// (MOE_FLAG_GEMM2_SINGLE) force one form.
+// Experts holding few rows on average: a pair spends both its CTAs on what one 128-row tile holds, so GEMM-2 takes 128-row
+// single-CTA tiles.  Decided from the shape alone (the routing-dependent counts never visit the host); flag bits 32
+// (MOE_FLAG_GEMM2_PAIR) and 64 (MOE_FLAG_GEMM2_SINGLE) force one form.  Layer, single / pair, us: 62 rows per expert (128 x 4096 x
+// 1536) 884 / 914, 55 skewed rows (128 x 2880 x 2880) 974 / 1003, 100 (the first in 8 bits) 574 / 588, 181 skewed rows (32 x 2048 x
+// 2048) 273 / 277; 200 rows 1455 / 1420, 200 on 8 experts of 4096 x 8192 464 / 455, 250 in 8 bits 1050 / 1035, 300 skewed rows
+// (64 x 2880 x 2880) 1306 / 1309, 400 rows 2544 / 2498.
 static bool small_experts(const Shape& s) {
   if (s.flags & 32) return false;
   if (s.flags & 64) return true;
-  return (long long)s.T * s.k < 512ll * s.E;
+  return (long long)s.T * s.k < 192ll * s.E;
 }
 
 // Fewer full-width tiles than SMs (an upper bound from the shape: every expert that can be reached has one 128-row tile, and one
