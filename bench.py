@@ -30,24 +30,6 @@ from paper_2605_05607_b200 import synth  # noqa: E402
 
 METRIC = "fused MoE layer tokens/sec"
 UNIT = "tokens/s"
-KERNELS_PER_STEP = 9  # gate, topk, masks, scan, offsets, fill, gemm1, gemm2, combine
-
-
-def kernels_per_step(cfg, flags: int, fp8: bool) -> int:
-    """Launches of one moe_layer call, following the library's own choice of forms (see MOE_FLAG_* in tcmoe.h)."""
-    from paper_2605_05607_b200 import binding as B
-    # up to 32768 pairs one kernel instead of four builds the layout, for up to 512 tokens the top-k is in it too
-    layout = 0 if cfg.P > 32768 else 4 if cfg.T <= 512 and cfg.E <= 256 else 3
-    if flags & B.MOE_FLAG_FUSED_FFN:
-        return 6 - layout + 2                          # ... layout, then the task-table kernel and the tracker-paced kernel
-    n = KERNELS_PER_STEP - layout + (2 if fp8 else 0)  # FP8: + quantisation of x and of h
-    if flags & B.MOE_FLAG_COMBINE_IN_EPILOGUE:
-        return n                                       # no combine kernel, one rounding pass instead
-    wide = cfg.f >= 8192 and cfg.T * cfg.k >= 512 * cfg.E
-    if not fp8 and not flags & B.MOE_FLAG_GEMM1_GATHER and (flags & B.MOE_FLAG_GEMM1_PAIR or wide):
-        n += 1                                         # the layout-tensor pass in front of the CTA-pair GEMM-1
-    return n
-
 NOMINAL_BF16_TFLOPS = 2250.0   # dense bf16 data-sheet figure, for context beside the measured peaks
 BURST_REGION_S = 1.0           # a timed region shorter than this runs before the power cap settles: burst peak
 CPU_SAMPLE_TOKENS = 12         # tokens per oracle pass, the same for the cpu_baseline leg and the reference arm
@@ -641,6 +623,7 @@ def main():
     B.moe_profile_enable(B.KERNEL_IDS["gemm1"])
     ev0, ev1 = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
     barrier()
+    launches0 = B.moe_launch_count()
     wall0 = time.time()
     ev0.record()
     for _ in range(args.steps):
@@ -649,6 +632,7 @@ def main():
     barrier()
     wall1 = time.time()
     elapsed_ms = ev0.elapsed_time(ev1)
+    launches = B.moe_launch_count() - launches0
     g1_ms, g1_launches = B.moe_profile_read()
     B.moe_profile_enable(0)
     elapsed_ms = replicas.max_over_ranks(elapsed_ms, dist, "cuda")
@@ -772,9 +756,7 @@ def main():
                 "pipeline": ("moe_layer_fp8_host" if fp8 else "moe_layer_host") +
                             " on 2 alternating streams (double-buffered staging and workspace)"},
         "value_two_streams": None if two_stream_ms is None else tokens / (two_stream_ms * 1e-3),
-        # FP8: + quantisation of x and of h; ep: route 3, dispatch 5, pack 1, receiver layout 4 + tile prefix 1 + 2 GEMMs +
-        # combine 1, finish 1
-        "gpu_launches": (18 if ep_rank is not None else kernels_per_step(cfg, args.layer_flags, fp8)) * args.steps,
+        "gpu_launches": launches,
         "roofline": {"kernel": "ffn_gemm1_kernel (GEMM-1 + SwiGLU, tcgen05)", "bound": "tensor",
                      "achieved": achieved, "peak": peak, "unit": "TFLOP/s",
                      "frac": (achieved / peak) if achieved else None,

@@ -347,6 +347,10 @@ enum { MOE_KERNEL_TOPK = 1, MOE_KERNEL_MASKS = 2, MOE_KERNEL_FILL = 3, MOE_KERNE
 int moe_profile_enable(int kernel_id);
 int moe_profile_read(float* total_ms, int32_t* launches);
 
+/* Kernels that this library has launched since it was loaded, by all threads (a call made under stream capture counts, replays of
+ * the graph do not): the difference over a region is what a benchmark reports. */
+int moe_launch_count(int64_t* count);
+
 /* ---- expert parallelism across GPUs (group g = GPU g) -------------------------------------------
  * The dispatched buffer xg of moe_dispatch is what travels out (segment g to GPU g: one row per
  * distinct (token, group), Sec. III-D) and one pre-reduced row per (token, group) travels back.

@@ -45,7 +45,8 @@ EXPORTS = ("moe_workspace_bytes", "moe_workspace_layout", "moe_status_reset", "m
            "moe_route", "moe_dispatch", "moe_expert_ffn", "moe_combine", "moe_layer", "moe_layer_host",
            "moe_profile_enable", "moe_profile_read", "moe_dispatch_noalloc", "moe_quantize_rows",
            "moe_quantize_weights", "moe_expert_ffn_fp8", "moe_layer_fp8", "moe_layer_fp8_host", "moe_selftest_wait_timeout", "moe_traffic_stats", "moe_ep_pack", "moe_ep_finish",
-           "moe_payload_efficiency", "moe_backward_workspace_bytes", "moe_layer_backward", "moe_clear_cache", "moe_gate_backward")
+           "moe_payload_efficiency", "moe_backward_workspace_bytes", "moe_layer_backward", "moe_clear_cache", "moe_gate_backward",
+           "moe_launch_count")
 
 
 class MoEShape(ctypes.Structure):
@@ -105,6 +106,7 @@ def lib() -> ctypes.CDLL:
         L.moe_ep_finish.argtypes = [shp, vp, lay, vp, vp]
         L.moe_profile_enable.argtypes = [ctypes.c_int]
         L.moe_profile_read.argtypes = [ctypes.POINTER(ctypes.c_float), ctypes.POINTER(ctypes.c_int32)]
+        L.moe_launch_count.argtypes = [ctypes.POINTER(i64)]
         for name in EXPORTS:
             if name != "moe_strerror":
                 getattr(L, name).restype = ctypes.c_int
@@ -350,6 +352,13 @@ def moe_profile_enable(kernel_id: int) -> None:
 def moe_clear_cache() -> None:
     """Forget the cached TMA tensor maps (host memory only)."""
     _check("moe_clear_cache", lib().moe_clear_cache())
+
+
+def moe_launch_count() -> int:
+    """Kernels launched by the library so far."""
+    n = ctypes.c_int64(0)
+    _check("moe_launch_count", lib().moe_launch_count(ctypes.byref(n)))
+    return n.value
 
 
 def moe_profile_read():

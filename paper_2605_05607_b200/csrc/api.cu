@@ -169,6 +169,9 @@ bool have_device() {
 
 namespace tcmoe {
 namespace {
+}  // namespace
+std::atomic<long long> g_launches{0};
+namespace {
 // State of the timing hook.  One record per process, guarded by a mutex: launches from several host threads
 // may be bracketed while another thread enables, disables or reads the hook.
 constexpr int PROFILE_CAP = 4096;
@@ -305,6 +308,12 @@ int moe_profile_enable(int kernel_id) {
   std::lock_guard<std::mutex> lock(g_profile_mutex);
   g_profile_id.store(kernel_id, std::memory_order_relaxed);
   g_profile_n = 0;
+  return MOE_OK;
+}
+
+int moe_launch_count(int64_t* count) {
+  if (count == nullptr) return MOE_ERR_INVALID_ARG;
+  *count = g_launches.load(std::memory_order_relaxed);
   return MOE_OK;
 }
 

@@ -2,6 +2,7 @@
 #pragma once
 #include <cuda_runtime.h>
 #include <stdint.h>
+#include <atomic>
 #include <utility>
 
 namespace tcmoe {
@@ -34,6 +35,8 @@ __device__ __forceinline__ void grid_dependency_sync() {
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 }
 
+extern std::atomic<long long> g_launches;   // kernels launched since the library was loaded (api.cu)
+
 template <typename... KArgs, typename... Args>
 cudaError_t launch_pdl_cluster(unsigned cluster, void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t st,
                                Args&&... args) {
@@ -51,6 +54,7 @@ cudaError_t launch_pdl_cluster(unsigned cluster, void (*kernel)(KArgs...), dim3 
   attr[1].val.clusterDim.z = 1;
   cfg.attrs = attr;
   cfg.numAttrs = cluster > 0 ? 2 : 1;
+  g_launches.fetch_add(1, std::memory_order_relaxed);
   return cudaLaunchKernelEx(&cfg, kernel, KArgs(std::forward<Args>(args))...);
 }
 template <typename... KArgs, typename... Args>
