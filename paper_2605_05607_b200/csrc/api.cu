@@ -18,7 +18,7 @@ inline size_t round_up(size_t v, size_t a) { return (v + a - 1) / a * a; }
 
 // Regions of the workspace, in order.  Every region starts on a 1 KiB boundary.
 struct WsPlan {
-  size_t status, emask, gmask, eprefix, gprefix, mt_prefix, mp_prefix, blk_start, blk_info, n_blocks, tracker, xs, h, hq, sh, xq, sx, o, logits, topk_idx, topk_w;
+  size_t status, emask, gmask, eprefix, gprefix, mt_prefix, mp_prefix, blk_start, blk_info, n_blocks, tracker, wsplit, xs, h, hq, sh, xq, sx, o, logits, topk_idx, topk_w;
   size_t expert_counts, expert_offsets, group_counts, group_offsets, pair_row, row_pair, al, disp_token, row_src;
   size_t total;
   int W;
@@ -34,6 +34,8 @@ bool pair_gemm1(const moe_shape_t& s) {
   if (s.flags & MOE_FLAG_GEMM1_PAIR) return true;
   return s.f >= 8192 && (long long)s.T * s.k >= 512ll * s.E;
 }
+
+Shape to_shape(const moe_shape_t& s) { return Shape{s.T, s.d, s.f, s.E, s.k, s.G, s.score_fn, s.flags}; }
 
 WsPlan plan(const moe_shape_t& s) {
   WsPlan p{};
@@ -64,6 +66,7 @@ WsPlan plan(const moe_shape_t& s) {
     p.n_blocks = take(3 * 4);
     p.tracker = take(fused_tracker_bytes(Shape{s.T, s.d, s.f, s.E, s.k, s.G, s.score_fn, s.flags}));
   }
+  p.wsplit = take(gate_split_bytes(to_shape(s)));
   // expert-sorted activation rows of the CTA-pair GEMM-1 (only reserved when that form is asked for)
   p.xs = take((pair_gemm1(s) || (s.flags & MOE_FLAG_TRACK_DISPATCH)) ? P * (size_t)s.d * 2 : 0);
   p.h = take(P * (size_t)s.f * 2);
@@ -131,7 +134,6 @@ int check_layout(const moe_layout_t* L) {
   return MOE_OK;
 }
 
-Shape to_shape(const moe_shape_t& s) { return Shape{s.T, s.d, s.f, s.E, s.k, s.G, s.score_fn, s.flags}; }
 Layout to_layout(const moe_layout_t& L) {
   return Layout{L.expert_counts, L.expert_offsets, L.group_counts, L.group_offsets, L.pair_row,
                 L.row_pair,      L.al,             L.disp_token,   L.row_src};
@@ -407,7 +409,7 @@ int moe_route(const moe_shape_t* shape, const void* x, const float* w_gate, cons
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   const Shape s = to_shape(*shape);
   if (w_gate != nullptr)
-    TCMOE_CUDA(launch_gate_logits(s, x, w_gate, logits, at<int32_t>(ws, p.status), st));
+    TCMOE_CUDA(launch_gate_logits(s, x, w_gate, logits, at<void>(ws, p.wsplit), at<int32_t>(ws, p.status), st));
   TCMOE_CUDA(launch_topk(s, logits, logit_bias, bias_row_stride, topk_idx, topk_w, at<int32_t>(ws, p.status), st));
   return MOE_OK;
 }
@@ -742,7 +744,7 @@ static int layer_impl(const moe_shape_t* shape, const void* x, const float* w_ga
                at<int32_t>(ws, p.al),            at<int32_t>(ws, p.disp_token),     at<int32_t>(ws, p.row_src)};
   }
   // gate
-  TCMOE_CUDA(launch_gate_logits(s, x, w_gate, lg, status, st));
+  TCMOE_CUDA(launch_gate_logits(s, x, w_gate, lg, at<void>(ws, p.wsplit), status, st));
   // the top-k kernel also zeroes the layout builder's bitmasks where it uses them (emask and gmask are adjacent)
   const LayoutScratch sc = scratch(ws, p);
   if (topk_in_layout(s)) {

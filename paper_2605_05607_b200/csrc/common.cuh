@@ -97,8 +97,9 @@ struct LayoutScratch {
   int W;
 };
 
-// gate_gemm.cu
-cudaError_t launch_gate_logits(const Shape& s, const void* x, const float* w_gate, float* logits, int32_t* status,
+// gate_gemm.cu: wsplit is scratch of gate_split_bytes(s) bytes for the bf16 terms of w_gate (0: not used for this shape)
+size_t gate_split_bytes(const Shape& s);
+cudaError_t launch_gate_logits(const Shape& s, const void* x, const float* w_gate, float* logits, void* wsplit, int32_t* status,
                                cudaStream_t st);
 // route.cu
 cudaError_t launch_topk(const Shape& s, const float* logits, const float* bias, int64_t bias_stride,

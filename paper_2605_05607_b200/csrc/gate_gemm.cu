@@ -6,17 +6,15 @@
 // accumulators in TMEM (the fp32 ALUs would need 2 T d E flop: 120 GFLOP, 3.7 ms for the
 // DeepSeek-V3-shaped layer).
 //
-// A task is a 128-token x GN-expert tile and the whole of K.  Sixteen warps (groups that take turns)
-// read the fp32 block of w_gate, split it and write the three terms straight into the swizzled
-// MN-major operand tiles: no split copy of the weight in memory and no launch for it.  x comes by TMA.
+// A task is a 128-token x GN-expert tile and the whole of K.  x comes by TMA.  For few tokens sixteen warps (groups that take
+// turns) read the fp32 block of w_gate, split it and write the three terms straight into the swizzled MN-major operand tiles:
+// no split copy of the weight in memory and no launch for it.  For many tokens every task would split the same blocks again,
+// so a kernel before this one writes the terms to the workspace once and they come by TMA too (PRE).
 // What bounds it: for few tokens the walk along K, one k-block of 64 after the other, so tiles are
 // narrow (a short k-block, and E / GN thread blocks share the work); for many tokens shared-memory
-// bandwidth (the UMMAs read the rows of x once per 256 columns), so tiles are wide and two row tiles share
-// a split weight block.  Up to 128 experts the three terms are summed apart, as one wide B of 3 GN columns: an
+// bandwidth (the UMMAs read the rows of x once per 256 columns), so tiles are wide and two row tiles may share
+// a weight block.  Up to 128 experts the three terms are summed apart, as one wide B of 3 GN columns: an
 // UMMA takes about 70 cycles for any N up to 128.  More experts keep one running sum (TMEM columns).
-// Measured, us, against the form with a split kernel and one tile width (T, d, E): 64, 4096, 128: 41 -> 24.5;
-// 128, 7168, 256: 157 -> 48; 1777, 2880, 128: 34 -> 20.5; 8192, 4096, 128: 49 -> 37-41; 16384, 4096, 128: 55 -> 54;
-// 32768, 7168, 256: 350-420 -> 308-322.
 // K is never divided over thread blocks, although that would be faster still for a decode batch (9 us
 // at T = 64, d = 4096, E = 128): a logit is the same sum in the same order whatever the tile, and a
 // different order moves it by up to 1e-4, enough to change the selection of a token whose k-th and next
@@ -35,9 +33,12 @@ constexpr int RING_BYTES = 192 * 1024;
 constexpr int MAX_STAGES = 8;
 constexpr int NUM_BARS = 2 * MAX_STAGES + 1;
 constexpr int SMEM_BYTES = 1024 + RING_BYTES + A_BYTES + NUM_BARS * 8 + 64;   // + A_BYTES: see a_bytes
-constexpr int SPLIT_WARPS = 16;
-constexpr int TMA_WARP = SPLIT_WARPS, MMA_WARP = SPLIT_WARPS + 1;
-constexpr int THREADS = (SPLIT_WARPS + 2) * 32;
+// Warps that split the weight and store the logits; a TMA warp and an UMMA warp follow.  Only stored with PRE: few warps leave
+// room for the next kernel's blocks to start early.
+__host__ __device__ constexpr int work_warps(bool pre) { return pre ? 4 : 16; }
+__host__ __device__ constexpr int threads(bool pre) { return (work_warps(pre) + 2) * 32; }
+constexpr int PRE_MIN_TOKENS = 512;             // fewer tokens never take a split copy of the weight: no workspace for it
+constexpr double PRE_US = 3.0;                  // its launch
 
 struct GateParams {
   const float* w;     // [d, E]
@@ -50,10 +51,10 @@ struct GateParams {
 };
 
 // ROWS_M: rows of a tile, 64 or 128.  APART: hi, mid and lo sums in accumulators of their own, added at the end; otherwise one
-// running sum.
-template <int GN, int GROUPS, int ROWS_M, bool APART>
-__global__ void __launch_bounds__(THREADS, 1)
-gate_umma_kernel(const __grid_constant__ CUtensorMap map_x, const GateParams p) {
+// running sum.  PRE: the three terms come by TMA from the copy that split_gate_kernel made (map_w); the split warps only store.
+template <int GN, int GROUPS, int ROWS_M, bool APART, bool PRE>
+__global__ void __launch_bounds__(threads(PRE), 1)
+gate_umma_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant__ CUtensorMap map_w, const GateParams p) {
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   uint64_t* bars = reinterpret_cast<uint64_t*>(smem + RING_BYTES + A_BYTES);
@@ -70,7 +71,8 @@ gate_umma_kernel(const __grid_constant__ CUtensorMap map_x, const GateParams p) 
   const int row0 = (blockIdx.x / p.n_tiles) * p.m_sub * ROWS_M, n0 = (blockIdx.x % p.n_tiles) * GN;
   const int n_sub = p.m_sub > 1 && row0 + ROWS_M < p.T ? 2 : 1;           // row tiles of this task that have rows
   // a stage: hi | mid | lo columns of the weight block side by side in 64-column slabs of 8 KiB, then the x tiles
-  constexpr int GROUP_WARPS = SPLIT_WARPS / GROUPS;
+  constexpr int WARPS = work_warps(PRE), TMA_WARP = WARPS, MMA_WARP = WARPS + 1;
+  constexpr int GROUP_WARPS = WARPS / GROUPS;
   constexpr int B_BYTES = (3 * GN + 63) / 64 * 8192;
   // A group that has filled block i knows that block i - n_stages was consumed.  Its next one, i + GROUPS, needs
   // i + GROUPS - 2 n_stages consumed for its parity wait to mean the right phase: no more groups than stages.
@@ -80,13 +82,16 @@ gate_umma_kernel(const __grid_constant__ CUtensorMap map_x, const GateParams p) 
 
   if (threadIdx.x == 0) {
     for (int s = 0; s < MAX_STAGES; ++s) {
-      ptx::mbar_init(full_bar(s), GROUP_WARPS + 1);   // one group of split warps + the TMA thread (expect_tx)
+      ptx::mbar_init(full_bar(s), PRE ? 1 : GROUP_WARPS + 1);   // one group of split warps + the TMA thread (expect_tx)
       ptx::mbar_init(empty_bar(s), 1);
     }
     ptx::mbar_init(done_bar, 1);
     ptx::fence_mbar_init();
   }
-  if (warp == TMA_WARP && lane == 0) ptx::prefetch_tensormap(&map_x);
+  if (warp == TMA_WARP && lane == 0) {
+    ptx::prefetch_tensormap(&map_x);
+    if (PRE) ptx::prefetch_tensormap(&map_w);
+  }
   if (warp == MMA_WARP) {
     ptx::tmem_alloc(ptx::smem_u32(tmem_slot), 512);
     ptx::tmem_relinquish();
@@ -105,7 +110,7 @@ gate_umma_kernel(const __grid_constant__ CUtensorMap map_x, const GateParams p) 
     *abort_flag = 1;
   };
 
-  if (warp < SPLIT_WARPS) {
+  if (warp < WARPS) {
     // ================================ weight block -> three bf16 terms ================================
     // Thread: 8 columns (one 16-byte piece of a swizzle row) of CHUNKS rows of K.  Group g takes every GROUPS-th
     // k-block and keeps DEPTH of its blocks on the way in registers.
@@ -115,16 +120,16 @@ gate_umma_kernel(const __grid_constant__ CUtensorMap map_x, const GateParams p) 
     const int group = warp / GROUP_WARPS, tid = threadIdx.x % (GROUP_WARPS * 32);
     const int piece = tid % PIECES, krow = tid / PIECES;
     const int col = n0 + piece * 8;
-    const bool vec = (p.E & 3) == 0;
-    const bool plain = vec && col + 8 <= p.E;                             // whole vectors inside the row
+    const bool vec = (p.E & 3) == 0;                                      // 16-byte vectors, each inside the row or beyond it
     float w[DEPTH][CHUNKS][8];
     auto load = [&](int kb, float (&v)[CHUNKS][8]) {
       const float* src = p.w + (size_t)(kb * BK + krow) * p.E + col;
-      if (plain && kb * BK + BK <= p.d) {
+      if (vec && kb * BK + BK <= p.d) {
 #pragma unroll
         for (int c = 0; c < CHUNKS; ++c) {
           const float4* q = reinterpret_cast<const float4*>(src + (size_t)(c * ROWS) * p.E);
-          const float4 a = __ldg(q), b = __ldg(q + 1);
+          const float4 zero = make_float4(0.f, 0.f, 0.f, 0.f);
+          const float4 a = col < p.E ? __ldg(q) : zero, b = col + 4 < p.E ? __ldg(q + 1) : zero;
           v[c][0] = a.x; v[c][1] = a.y; v[c][2] = a.z; v[c][3] = a.w;
           v[c][4] = b.x; v[c][5] = b.y; v[c][6] = b.z; v[c][7] = b.w;
         }
@@ -176,8 +181,8 @@ gate_umma_kernel(const __grid_constant__ CUtensorMap map_x, const GateParams p) 
     bool ok = !*abort_flag;
 #pragma unroll
     for (int i = 0; i < DEPTH; ++i)
-      if (ok && group + GROUPS * i < p.KB) load(group + GROUPS * i, w[i]);
-    for (int kb = group; ok && kb < p.KB; kb += GROUPS * DEPTH) {
+      if (!PRE && ok && group + GROUPS * i < p.KB) load(group + GROUPS * i, w[i]);
+    for (int kb = group; !PRE && ok && kb < p.KB; kb += GROUPS * DEPTH) {
 #pragma unroll
       for (int i = 0; i < DEPTH; ++i)
         if (ok && kb + GROUPS * i < p.KB) ok = block(kb + GROUPS * i, w[i]);
@@ -188,10 +193,10 @@ gate_umma_kernel(const __grid_constant__ CUtensorMap map_x, const GateParams p) 
         timeout(1);
       } else {
         ptx::tc_fence_after();
-        // warp w: TMEM lanes 32 (w % 4) .. + 31, every fourth 32-column block from w / 4 on.  A 64-row accumulator has row
+        // warp w: TMEM lanes 32 (w % 4) .. + 31, every (warps / 4)-th 32-column block from w / 4 on.  A 64-row accumulator has row
         // 16 q + i in lane 32 q + i (i < 16).
         const int lrow = ROWS_M == 64 ? (lane < 16 ? (warp & 3) * 16 + lane : p.T) : (warp & 3) * 32 + lane;
-        for (int u = warp >> 2; u < n_sub * (GN / 32); u += SPLIT_WARPS / 4) {
+        for (int u = warp >> 2; u < n_sub * (GN / 32); u += WARPS / 4) {
           const int i = u / (GN / 32), c = (u % (GN / 32)) * 32;
           const int row = row0 + i * ROWS_M + lrow;
           if (c >= ncols) continue;
@@ -230,14 +235,20 @@ gate_umma_kernel(const __grid_constant__ CUtensorMap map_x, const GateParams p) 
       }
     }
   } else if (warp == TMA_WARP) {
-    // ================================ TMA producer (rows of x) ================================
+    // ================================ TMA producer (rows of x; PRE: the weight's terms) ================================
     if (lane == 0 && !*abort_flag) {
       int s = 0, ph = 1;
       for (int kb = 0; kb < p.KB; ++kb) {
         if (!ptx::mbar_wait(empty_bar(s), ph, abort_flag, global_abort)) { timeout(3); break; }
-        ptx::mbar_arrive_expect_tx(full_bar(s), n_sub * p.a_bytes);
+        ptx::mbar_arrive_expect_tx(full_bar(s), n_sub * p.a_bytes + (PRE ? B_BYTES : 0));
         for (int i = 0; i < n_sub; ++i)
           ptx::tma_load_2d(smem_base + s * stage_bytes + B_BYTES + i * p.a_bytes, &map_x, full_bar(s), kb * BK, row0 + i * ROWS_M);
+        if (PRE) {
+          static_assert(!PRE || GN % 64 == 0, "a slab of 64 columns holds one term");
+#pragma unroll
+          for (int c = 0; c < B_BYTES / 8192; ++c)
+            ptx::tma_load_3d(smem_base + s * stage_bytes + c * 8192, &map_w, full_bar(s), n0 + c * 64 % GN, kb * BK, c * 64 / GN);
+        }
         if (++s == n_stages) { s = 0; ph ^= 1; }
       }
     }
@@ -297,47 +308,85 @@ gate_umma_kernel(const __grid_constant__ CUtensorMap map_x, const GateParams p) 
   }
 }
 
-// Tile width, rows of a tile and row tiles per task: the cheapest by a model in microseconds, fitted to this kernel: time of a
-// k-block, 148 thread blocks at a time.  Tiles of 64 rows halve what a UMMA reads of x, which counts where twelve of them make a
-// k-block (running sum: 128 tokens of d = 7168, 256 experts 66 -> 48 us); with the terms apart they change nothing.
-struct GatePlan { int gn, bm, m_sub; };
-GatePlan plan_gate(int T, int E, bool apart) {
-  static const struct { int gn, bm, m_sub; double kb_us[2]; } forms[] = {   // running sum, apart
-      {32, 64, 1, {0.45, 1e9}}, {64, 64, 1, {0.5, 1e9}}, {32, 128, 1, {0.5, 0.3}}, {64, 128, 1, {0.58, 0.4}},
-      {64, 128, 2, {0.85, 0.6}}, {128, 128, 1, {0.8, 0.8}}, {128, 128, 2, {1.4, 1e9}}};
+// w_gate fp32 [d, E] -> bf16 [3, d, cols]: hi, mid, lo terms, zero in the padding columns
+__global__ void __launch_bounds__(256) split_gate_kernel(const float* __restrict__ w, __nv_bfloat16* __restrict__ out, int d, int E,
+                                                         int cols) {
+  grid_dependency_sync();
+  const size_t n = (size_t)d * cols;
+  for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x) {
+    const int row = (int)(i / cols), col = (int)(i % cols);
+    float v = col < E ? __ldg(w + (size_t)row * E + col) : 0.f;
+#pragma unroll
+    for (int t = 0; t < 3; ++t) {   // the remainders are exact
+      const __nv_bfloat16 r = __float2bfloat16_rn(v);
+      out[t * n + i] = r;
+      v = __fsub_rn(v, __bfloat162float(r));
+    }
+  }
+}
+
+// Tile width, rows of a tile, row tiles per task and where the terms of the weight come from: the cheapest by a model in
+// microseconds that is fitted to this kernel: tasks go in rounds of one per SM, a round costs `start` and a time per k-block of
+// 64; rows of w_gate whose length is no multiple of 4 are read by the element, which the forms that split inside the GEMM pay in
+// every k-block (16384 tokens, d = 7168: 256 experts 178 us, 250 experts 236).  The split copy costs a launch.
+// Tiles of 64 rows halve what a UMMA reads of x, which counts where twelve of them make a k-block (running sum: 128 tokens
+// of d = 7168, 256 experts 66 -> 48 us); with the terms apart they change nothing.
+// moe_route of (T, d, E), us, without the split copy / with this table: 16384, 2880, 65: 61.4 / 50.4; 16384, 2880, 128: 53.0 / 49.4;
+// 32768, 2880, 96: 102 / 92; 8192, 7168, 256: 115 / 85; 32768, 7168, 250: 459 / 335; 4097, 7168, 258: 194 / 90.
+struct GatePlan { int gn, bm, m_sub; bool pre; };
+GatePlan plan_gate(int T, int d, int E) {
+  struct Cost { double start, kb, kb_ragged; };
+  constexpr Cost NO = {1e9, 0, 0};
+  static const struct { GatePlan form; Cost running, apart; } forms[] = {
+      {{32, 64, 1, false}, {4, 0.37, 0.38}, NO},
+      {{64, 64, 1, false}, {4, 0.43, 0.63}, NO},
+      {{32, 128, 1, false}, {4.3, 0.455, 0.46}, {4.5, 0.318, 0.345}},
+      {{64, 128, 1, false}, {4.8, 0.525, 0.66}, NO},
+      {{64, 128, 2, false}, {7, 0.83, 0.87}, {8, 0.63, 0.68}},
+      {{64, 128, 1, true}, NO, {4.8, 0.33, 0.33}},
+      {{128, 128, 1, true}, {4.8, 0.58, 0.58}, {6, 0.49, 0.49}},
+      {{128, 128, 2, true}, {9, 1.04, 1.04}, NO}};
   GatePlan best{};
   double best_us = 1e30;
   for (const auto& f : forms) {
-    const int rows = f.m_sub * f.bm;
-    const long long tiles = (long long)((T + rows - 1) / rows) * ((E + f.gn - 1) / f.gn);
-    const double us = (double)((tiles + 147) / 148) * f.kb_us[apart ? 1 : 0];
-    if (us < best_us) { best_us = us; best = GatePlan{f.gn, f.bm, f.m_sub}; }
+    if (f.form.pre && T < PRE_MIN_TOKENS) continue;
+    const Cost& c = E <= 128 ? f.apart : f.running;
+    const int rows = f.form.m_sub * f.form.bm, sms = sm_count();
+    const long long tasks = (long long)((T + rows - 1) / rows) * ((E + f.form.gn - 1) / f.form.gn);
+    const double round = c.start + ((d + BK - 1) / BK) * (E % 4 == 0 ? c.kb : c.kb_ragged);
+    const double us = (double)((tasks + sms - 1) / sms) * round + (f.form.pre ? PRE_US : 0.0);
+    if (us < best_us) { best_us = us; best = f.form; }
   }
   return best;
 }
 
-template <int GN, int GROUPS, int ROWS_M, bool APART>
-cudaError_t launch_width(const GateParams& p, int grid, const CUtensorMap& m_x, cudaStream_t st) {
+template <int GN, int GROUPS, int ROWS_M, bool APART, bool PRE = false>
+cudaError_t launch_width(const GateParams& p, int grid, const CUtensorMap& m_x, const CUtensorMap& m_w, cudaStream_t st) {
   // per device; several host threads may get here at once: setting the attribute twice is harmless
   static std::atomic<bool> attr_set[MAX_DEVICES];
   const int dev = current_device();
+  const auto kernel = gate_umma_kernel<GN, GROUPS, ROWS_M, APART, PRE>;
   if (!attr_set[dev].load(std::memory_order_acquire)) {
-    cudaError_t e = cudaFuncSetAttribute(gate_umma_kernel<GN, GROUPS, ROWS_M, APART>, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_BYTES);
+    cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_BYTES);
     if (e != cudaSuccess) return e;
     attr_set[dev].store(true, std::memory_order_release);
   }
-  return launch_pdl(gate_umma_kernel<GN, GROUPS, ROWS_M, APART>, grid, THREADS, SMEM_BYTES, st, m_x, p);
+  return launch_pdl(kernel, grid, threads(PRE), SMEM_BYTES, st, m_x, m_w, p);
 }
 
 }  // namespace
 
-cudaError_t launch_gate_logits(const Shape& s, const void* x, const float* w_gate, float* logits, int32_t* status,
+size_t gate_split_bytes(const Shape& s) {
+  return s.T < PRE_MIN_TOKENS ? 0 : (size_t)3 * s.d * ((s.E + 63) & ~63) * 2;
+}
+
+cudaError_t launch_gate_logits(const Shape& s, const void* x, const float* w_gate, float* logits, void* wsplit, int32_t* status,
                                cudaStream_t st) {
   if (s.T == 0) return cudaSuccess;
   const bool apart = s.E <= 128;
-  const GatePlan plan = plan_gate(s.T, s.E, apart);
+  const GatePlan plan = plan_gate(s.T, s.d, s.E);
   const int a_rows = s.T < plan.bm ? (s.T + 7) & ~7 : plan.bm;
-  CUtensorMap m_x;
+  CUtensorMap m_x, m_w{};
   {
     cuuint64_t dims[2] = {(cuuint64_t)s.d, (cuuint64_t)s.T};
     cuuint64_t strides[1] = {(cuuint64_t)s.d * 2};
@@ -345,6 +394,18 @@ cudaError_t launch_gate_logits(const Shape& s, const void* x, const float* w_gat
     if (!ffn::encode_tiled(&m_x, false, 2, x, dims, strides, box)) return cudaErrorInvalidValue;
   }
   ProfileScope prof(KID_GATE, st);
+  if (plan.pre) {
+    const int cols = (s.E + 63) & ~63;
+    cuuint64_t dims[3] = {(cuuint64_t)cols, (cuuint64_t)s.d, 3};
+    cuuint64_t strides[2] = {(cuuint64_t)cols * 2, (cuuint64_t)cols * s.d * 2};
+    cuuint32_t box[3] = {64, BK, 1};
+    if (!ffn::encode_tiled(&m_w, false, 3, wsplit, dims, strides, box)) return cudaErrorInvalidValue;
+    size_t blocks = ((size_t)s.d * cols + 255) / 256;
+    if (blocks > (size_t)sm_count() * 8) blocks = (size_t)sm_count() * 8;
+    cudaError_t err = launch_pdl(split_gate_kernel, (unsigned)blocks, 256, 0, st, w_gate, static_cast<__nv_bfloat16*>(wsplit), s.d,
+                                 s.E, cols);
+    if (err != cudaSuccess) return err;
+  }
   GateParams p;
   p.w = w_gate;
   p.logits = logits;
@@ -357,16 +418,19 @@ cudaError_t launch_gate_logits(const Shape& s, const void* x, const float* w_gat
   p.a_bytes = a_rows * BK * 2;
   p.status = status;
   const int grid = ((s.T + p.m_sub * plan.bm - 1) / (p.m_sub * plan.bm)) * p.n_tiles;
-  if (apart) {
-    if (plan.gn == 32) return launch_width<32, 4, 128, true>(p, grid, m_x, st);
-    if (plan.gn == 64) return launch_width<64, 2, 128, true>(p, grid, m_x, st);
-    return launch_width<128, 2, 128, true>(p, grid, m_x, st);
+  if (plan.pre) {
+    if (!apart) return launch_width<128, 1, 128, false, true>(p, grid, m_x, m_w, st);
+    if (plan.gn == 64) return launch_width<64, 1, 128, true, true>(p, grid, m_x, m_w, st);
+    return launch_width<128, 1, 128, true, true>(p, grid, m_x, m_w, st);
   }
-  if (plan.bm == 64 && plan.gn == 32) return launch_width<32, 4, 64, false>(p, grid, m_x, st);
-  if (plan.bm == 64) return launch_width<64, 2, 64, false>(p, grid, m_x, st);
-  if (plan.gn == 32) return launch_width<32, 4, 128, false>(p, grid, m_x, st);
-  if (plan.gn == 64) return launch_width<64, 2, 128, false>(p, grid, m_x, st);
-  return launch_width<128, 2, 128, false>(p, grid, m_x, st);
+  if (apart) {
+    if (plan.gn == 32) return launch_width<32, 4, 128, true>(p, grid, m_x, m_x, st);
+    return launch_width<64, 2, 128, true>(p, grid, m_x, m_x, st);
+  }
+  if (plan.bm == 64 && plan.gn == 32) return launch_width<32, 4, 64, false>(p, grid, m_x, m_x, st);
+  if (plan.bm == 64) return launch_width<64, 2, 64, false>(p, grid, m_x, m_x, st);
+  if (plan.gn == 32) return launch_width<32, 4, 128, false>(p, grid, m_x, m_x, st);
+  return launch_width<64, 2, 128, false>(p, grid, m_x, m_x, st);
 }
 
 }  // namespace tcmoe

@@ -113,3 +113,22 @@ def check_layout(run: Run, idx_ref):
     assert np.array_equal(L.al.cpu().numpy()[: cfg.G * cfg.T].reshape(cfg.G, cfg.T), lay["al"]), "al"
     assert np.array_equal(L.disp_token.cpu().numpy()[:n], lay["disp_token"]), "disp_token"
     return lay
+
+
+def device_us(call, n=10, reps=5):
+    """Device time of one call: n of them in a CUDA graph (no host time in between), the quickest of some replays."""
+    call()
+    torch.cuda.synchronize()
+    graph, side = torch.cuda.CUDAGraph(), torch.cuda.Stream()
+    with torch.cuda.graph(graph, stream=side):
+        for _ in range(n):
+            call()
+    e0, e1 = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+    times = []
+    for _ in range(reps):
+        e0.record()
+        graph.replay()
+        e1.record()
+        torch.cuda.synchronize()
+        times.append(e0.elapsed_time(e1) * 1e3 / n)
+    return min(times)
