@@ -140,12 +140,10 @@ __global__ void __launch_bounds__(256) fill_layout_kernel(const int32_t* __restr
 }
 
 // ---- K2 in one kernel ----------------------------------------------------------------------------
-// The four passes above as one kernel of at most 8 thread blocks (a cluster), for up to 32768 pairs: every block owns a
+// The four passes above as one kernel of at most 8 thread blocks (a cluster), for small tables (layout_in_one): every block owns a
 // contiguous range of tokens, builds its masks and their prefixes in shared memory, reads the other blocks' row totals through
 // distributed shared memory and fills its tokens' entries.  The four launches are latency, not work: 16 us of device time and
-// three launch gaps for 256 tokens of top-2, 21 us for 3001 of top-4; in one kernel 6.2 and 9.5 us.  With more pairs the
-// scattered table stores of the fill pass want more than 8 SMs (16384 tokens of top-8: 29 us as four kernels; 10880 tokens of a sparse
-// top-8 table: 19 us either way).
+// three launch gaps for 256 tokens of top-2, 21 us for 3001 of top-4; in one kernel 6.2 and 9.5 us.
 constexpr int ONE_THREADS = 1024, ONE_MAX_BLOCKS = 8, ONE_MAX_PAIRS = 32768, ONE_MAX_SMEM = 160 * 1024;
 struct OneShape { int blocks, tokens, words; size_t smem; };   // tokens per block (a multiple of 32) and their mask words
 OneShape one_shape(const Shape& s, bool topk) {
@@ -306,8 +304,14 @@ __global__ void __launch_bounds__(ONE_THREADS) layout_one_kernel(int32_t* topk_i
   ptx::cluster_wait();     // no block leaves while another may still read its totals
 }
 
+// Eight blocks write the G x T table of allocated rows and the T x k ones, so the one kernel is the better form while there are few
+// entries: microseconds of both, fitted to 1 to 32768 tokens, top-1 to top-32, 1 to 1024 groups.  Four kernels / one, us: 32768 tokens
+// top-1, 1 group 12.3 / 15.1, 8 groups 15.5 / 24.8, 104 groups 40.5 / 143; 16384 tokens top-2, 1 group 12.6 / 14.0, 32 groups 24.5 / 36.6;
+// 8192 tokens top-4, 8 groups 17.7 / 14.6, 64 groups 38.6 / 35.3, 256 groups 81 / 96; 4096 tokens top-8, 256 groups 93 / 57.
 bool layout_in_one(const Shape& s) {
-  return s.T > 0 && (long long)s.T * s.k <= ONE_MAX_PAIRS && one_shape(s, false).smem <= ONE_MAX_SMEM;
+  if (s.T <= 0 || (long long)s.T * s.k > ONE_MAX_PAIRS || one_shape(s, false).smem > ONE_MAX_SMEM) return false;
+  const double one = 5.0 + s.T * (4.2 + 1.7 * s.k + 0.62 * s.G) / 16384, four = 9.5 + 1.2 * s.k + 0.25 * s.G;
+  return one < four;
 }
 
 template <int KPL>

@@ -1,18 +1,20 @@
-"""Dispatch layout at the edges of its two builders: one kernel of 1, 2, 4 or 8 thread blocks up to 32768 pairs, four kernels
-beyond; mask words of 32 tokens, blocks without tokens, 1024 experts, unused slots.  Bit-exact against the oracle."""
+"""Dispatch layout at the edges of its two builders: one kernel of 1, 2, 4 or 8 thread blocks for small tables, four kernels
+for others; mask words of 32 tokens, blocks without tokens, 1024 experts, unused slots.  Bit-exact against the oracle."""
 import numpy as np
 import pytest
 import torch
 
 from oracle import moe_oracle as O
 from paper_2605_05607_b200 import binding as B
+from tests import helpers as H
 
 pytestmark = pytest.mark.gpu
 
 
 @pytest.mark.parametrize("T,E,k,G", [(1, 8, 2, 8), (31, 1024, 32, 1024), (256, 8, 8, 1), (257, 12, 3, 4), (513, 6, 1, 3),
                                      (1025, 256, 8, 8), (1100, 64, 4, 32), (4096, 64, 8, 32), (4097, 64, 8, 32),
-                                     (16384, 8, 2, 4), (32768, 16, 1, 16)])
+                                     (16384, 8, 2, 4), (32768, 16, 1, 16), (8192, 128, 4, 8), (8192, 64, 4, 64),
+                                     (7000, 256, 4, 256), (12001, 64, 1, 8), (14999, 16, 1, 1)])
 def test_layout_builders(T, E, k, G):
     rng = np.random.default_rng(T + E)
     skew = -1.5 * np.log(1 + rng.permutation(E))                      # popular and empty experts
@@ -35,7 +37,7 @@ def test_layout_builders(T, E, k, G):
 
 @pytest.mark.parametrize("T", [4096, 4097])
 def test_layout_of_a_sparse_table(T):
-    """Unused slots (-1): one kernel up to 32768 slots, four beyond; both against the same layout built slot by slot."""
+    """Unused slots (-1): one kernel for 4096 tokens, four for 4097; both against the same layout built slot by slot."""
     E, k = 16, 8
     rng = np.random.default_rng(T)
     idx = np.argsort(rng.random((T, E)), axis=1)[:, :k].astype(np.int32)
@@ -84,3 +86,17 @@ def test_topk_inside_the_layout_kernel(T, E, k, bias):
     for a, c in zip(*out):
         assert torch.equal(a, c)
     assert B.moe_status(ws)[0] == 0
+
+
+@pytest.mark.parametrize("T,E,k,G", [(32768, 104, 1, 104), (32768, 64, 1, 32), (16384, 128, 2, 128)])
+def test_one_token_less_takes_no_longer(T, E, k, G):
+    """Whichever builder a table gets, it takes no longer than that of one token more, which has more than 32768 pairs and so
+    always the four kernels."""
+    def call(T):
+        idx = torch.stack([torch.randperm(E, device="cuda")[:k] for _ in range(64)]).to(torch.int32).repeat(T // 64 + 1, 1)[:T]
+        idx = idx.contiguous().view(-1)
+        shape = B.MoEShape(T, 64, 64, E, k, G, 0, 0)
+        lay, ws = B.alloc_layout(shape), B.alloc_workspace(shape)
+        return lambda: B.moe_dispatch(shape, None, idx, lay, None, ws)
+
+    assert H.device_us(call(T)) <= 1.3 * H.device_us(call(T + 1))      # spread of the clock, of a few microseconds
