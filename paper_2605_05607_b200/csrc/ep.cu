@@ -17,37 +17,54 @@
 namespace tcmoe {
 namespace {
 
-// Thread per (token, group): the row n = (t, g) takes the token's slots that live in the group, in slot order, then -1 / 0.
-// The rows behind the last dispatched one are filled as unused too.
-__global__ void __launch_bounds__(256) ep_pack_kernel(const int32_t* __restrict__ topk_idx,
-                                                      const float* __restrict__ topk_w,
-                                                      const int32_t* __restrict__ al,
-                                                      const int32_t* __restrict__ group_offsets,
-                                                      int32_t* __restrict__ send_idx, float* __restrict__ send_w, int T,
-                                                      int E, int k, int G, int m, int kk, int cap_rows) {
+// Thread per dispatched row n = (t, g): the token's slots that live in the group, in slot order, then -1 / 0.  The rows behind
+// the last dispatched one (and a row whose table entry is no token) are unused.  Lists leave through shared memory, entry by
+// entry, as whole lines.
+constexpr int PACK_ROWS = 128, PACK_LD = PACK_ROWS + 4;   // + 4: eight entries of four rows fall into 32 banks
+__global__ void __launch_bounds__(PACK_ROWS) ep_pack_kernel(const int32_t* __restrict__ topk_idx,
+                                                            const float* __restrict__ topk_w,
+                                                            const int32_t* __restrict__ disp_token,
+                                                            const int32_t* __restrict__ group_offsets,
+                                                            int32_t* __restrict__ send_idx, float* __restrict__ send_w, int T,
+                                                            int k, int G, int m, int kk, int cap_rows) {
+  extern __shared__ int32_t idx_s[];                      // [kk][PACK_LD]
+  float* w_s = reinterpret_cast<float*>(idx_s + kk * PACK_LD);
+  int32_t* goff_s = idx_s + 2 * kk * PACK_LD;             // [G + 1]
   grid_dependency_sync();
-  const long long first = (long long)blockIdx.x * blockDim.x + threadIdx.x, stride = (long long)gridDim.x * blockDim.x;
-  for (long long i = first; i < (long long)T * G; i += stride) {
-    const int g = (int)(i / T), t = (int)(i % T);   // consecutive threads: consecutive tokens, consecutive rows of the group
-    const int a = __ldg(al + (size_t)g * T + t);
-    if (a < 0) continue;
-    const size_t n = (size_t)__ldg(group_offsets + g) + a;
+  const int tid = threadIdx.x;
+  for (int i = tid; i <= G; i += PACK_ROWS) goff_s[i] = __ldg(group_offsets + i);
+  __syncthreads();
+  const int rows = min(goff_s[G], cap_rows);
+  for (long long base = (long long)blockIdx.x * PACK_ROWS; base < cap_rows; base += (long long)gridDim.x * PACK_ROWS) {
+    const long long n = base + tid;
+    const int t = n < rows ? __ldg(disp_token + n) : -1;
     int pos = 0;
-    for (int j = 0; j < k; ++j) {
-      const int e = __ldg(topk_idx + (size_t)t * k + j);
-      if (e < 0 || e >= E || e / m != g) continue;
-      send_idx[n * kk + pos] = e - g * m;
-      send_w[n * kk + pos] = __ldg(topk_w + (size_t)t * k + j);
-      ++pos;
+    if (t >= 0 && t < T) {
+      int g = 0, hi = G;   // goff_s[g] <= n < goff_s[hi]
+      while (hi - g > 1) {
+        const int mid = (g + hi) >> 1;
+        if (goff_s[mid] <= n) g = mid; else hi = mid;
+      }
+      for (int j = 0; j < k && pos < kk; ++j) {
+        const int e = __ldg(topk_idx + (size_t)t * k + j) - g * m;   // m G = E: nothing outside [0, E) passes
+        if (e < 0 || e >= m) continue;
+        idx_s[pos * PACK_LD + tid] = e;
+        w_s[pos * PACK_LD + tid] = __ldg(topk_w + (size_t)t * k + j);
+        ++pos;
+      }
     }
     for (; pos < kk; ++pos) {
-      send_idx[n * kk + pos] = -1;
-      send_w[n * kk + pos] = 0.f;
+      idx_s[pos * PACK_LD + tid] = -1;
+      w_s[pos * PACK_LD + tid] = 0.f;
     }
-  }
-  for (long long i = (long long)__ldg(group_offsets + G) * kk + first; i < (long long)cap_rows * kk; i += stride) {
-    send_idx[i] = -1;
-    send_w[i] = 0.f;
+    __syncthreads();
+    const int entries = (int)min((long long)PACK_ROWS, cap_rows - base) * kk;
+    for (int i = tid; i < entries; i += PACK_ROWS) {
+      const int r = i / kk, q = i - r * kk;
+      send_idx[(size_t)base * kk + i] = idx_s[q * PACK_LD + r];
+      send_w[(size_t)base * kk + i] = w_s[q * PACK_LD + r];
+    }
+    __syncthreads();
   }
 }
 
@@ -119,10 +136,9 @@ cudaError_t launch_ep_pack(const Shape& s, const int32_t* topk_idx, const float*
   if (s.T == 0) return cudaSuccess;
   const int m = s.E / s.G, kk = s.k < m ? s.k : m;
   const int cap_rows = s.T * (s.k < s.G ? s.k : s.G);   // dispatched-row capacity
-  long long blocks = ((long long)s.T * s.G + 255) / 256;
-  if (blocks > 4096) blocks = 4096;
-  return launch_pdl(ep_pack_kernel, (unsigned)blocks, 256, 0, st, topk_idx, topk_w, L.al, L.group_offsets, send_idx,
-                    send_w, s.T, s.E, s.k, s.G, m, kk, cap_rows);
+  const int blocks = min((cap_rows - 1) / PACK_ROWS + 1, sm_count() * 16);
+  return launch_pdl(ep_pack_kernel, blocks, PACK_ROWS, ((size_t)2 * kk * PACK_LD + s.G + 1) * 4, st, topk_idx, topk_w, L.disp_token,
+                    L.group_offsets, send_idx, send_w, s.T, s.k, s.G, m, kk, cap_rows);
 }
 
 cudaError_t launch_ep_finish(const Shape& s, const void* back, const Layout& L, void* y, cudaStream_t st) {

@@ -104,7 +104,8 @@ def test_forward_over_nccl_with_one_rank():
         dist.destroy_process_group()
 
 
-@pytest.mark.parametrize("T,d,E,k,G", [(1, 8, 4, 1, 4), (33, 264, 80, 6, 40), (300, 1032, 64, 16, 64), (2051, 2056, 8, 2, 2)])
+@pytest.mark.parametrize("T,d,E,k,G", [(1, 8, 4, 1, 4), (33, 264, 80, 6, 40), (300, 1032, 64, 16, 64), (2051, 2056, 8, 2, 2),
+                                       (127, 64, 1024, 2, 1024), (129, 72, 64, 32, 2), (130, 520, 12, 3, 4)])
 def test_pack_and_finish_edges(T, d, E, k, G):
     """Target lists (unused entries and the rows behind the last dispatched one included) and the final reduction, for more
     than 32 groups, rows that no warp stride divides and rows shared by several warps, against plain tensor operations."""
@@ -137,3 +138,20 @@ def test_pack_and_finish_edges(T, d, E, k, G):
         a = lay.al[gi * T:(gi + 1) * T]
         acc[a >= 0] += back[(off[gi] + a[a >= 0]).long()].float()
     assert torch.equal(y, acc.to(torch.bfloat16))
+
+
+def test_packing_for_many_groups_takes_no_longer():
+    """Lists are built per dispatched row: 64 groups of one expert cost about what two groups of 32 cost."""
+    T, k, E = 20000, 6, 64
+    idx = torch.stack([torch.randperm(E, device="cuda")[:k] for _ in range(100)]).to(torch.int32).repeat(T // 100, 1).contiguous().view(-1)
+    w = torch.rand(T * k, device="cuda")
+
+    def call(G):
+        shape = B.MoEShape(T, 64, 64, E, k, G, 0, 0)
+        lay, ws = B.alloc_layout(shape), B.alloc_workspace(shape)
+        B.moe_dispatch(shape, None, idx, lay, None, ws)
+        rows, kk = T * min(k, G), min(k, E // G)
+        out = torch.empty(rows, kk, dtype=torch.int32, device="cuda"), torch.empty(rows, kk, device="cuda")
+        return lambda: B.moe_ep_pack(shape, idx, w, lay, *out)
+
+    assert H.device_us(call(64)) <= 1.5 * H.device_us(call(2))
