@@ -68,32 +68,88 @@ __global__ void __launch_bounds__(PACK_ROWS) ep_pack_kernel(const int32_t* __res
   }
 }
 
-// Warp per (token, column part): fp32 sum over the groups, ascending g.  Lane g finds the row of group g once (32 groups at a
-// time); four rows are in flight per lane.  Bound by the read of the returned rows; one warp per token that looked up every
-// group for every 16-byte column ran at a fifth of the copy bandwidth (2050 tokens of d = 4096, 8 groups: 75 us).
-__global__ void __launch_bounds__(256) ep_finish_kernel(const uint4* __restrict__ back, uint4* __restrict__ y,
-                                                        const int32_t* __restrict__ al,
-                                                        const int32_t* __restrict__ group_offsets, int T, int G,
-                                                        int vec_per_row, int parts, int vec_per_part) {
+__device__ __forceinline__ void add_row(float (&acc)[8], const uint4& raw) {
+  const __nv_bfloat162* p = reinterpret_cast<const __nv_bfloat162*>(&raw);
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {
+    const float2 f = __bfloat1622float2(p[i]);
+    acc[2 * i] += f.x;
+    acc[2 * i + 1] += f.y;
+  }
+}
+__device__ __forceinline__ uint4 round_row(const float (&acc)[8]) {
+  uint4 out;
+  __nv_bfloat162* o = reinterpret_cast<__nv_bfloat162*>(&out);
+#pragma unroll
+  for (int q = 0; q < 4; ++q) o[q] = __floats2bfloat162_rn(acc[2 * q], acc[2 * q + 1]);
+  return out;
+}
+
+// Warp per (token, column part): fp32 sum over the groups, ascending g.  Lane g finds the row of group g once; with ROWS > 0 a token
+// touches at most ROWS = min(k, G) groups (2 or 4) and their rows stay in registers, otherwise up to 32 groups' rows stay in the lanes
+// (with more the later ones are looked up per column step).  Four loads are in flight per lane: four rows of a column, or two
+// columns of two.  Bound by the read of the returned rows: 2050 tokens of d = 4096, top-8 of 8 groups 22 us, 8192 tokens of d = 2880, one
+// group 15, two of 8 groups 20 (with the lookup in the column loop and one form for all: 23.5, 28 and 33).
+constexpr int FINISH_BLOCKS = 5;   // resident per SM
+template <int ROWS>
+__global__ void __launch_bounds__(256, FINISH_BLOCKS) ep_finish_kernel(const uint4* __restrict__ back, uint4* __restrict__ y,
+                                                           const int32_t* __restrict__ al,
+                                                           const int32_t* __restrict__ group_offsets, int T, int G,
+                                                           int vec_per_row, int parts, int vec_per_part) {
   grid_dependency_sync();
   const int lane = threadIdx.x & 31;
   const int wpb = blockDim.x >> 5;
-  const long long units = (long long)T * parts;
-  for (long long w = (long long)blockIdx.x * wpb + (threadIdx.x >> 5); w < units; w += (long long)gridDim.x * wpb) {
-    const int t = (int)(w / parts), part = (int)(w % parts);
-    const int v_end = min(vec_per_row, (part + 1) * vec_per_part);
-    for (int v0 = part * vec_per_part; v0 < v_end; v0 += 32) {   // whole warps: the row numbers are shuffled
-      const int v = v0 + lane;
-      float acc[8];
+  const unsigned units = (unsigned)T * parts;   // parts > 1 for a few thousand tokens only
+  for (unsigned w = blockIdx.x * wpb + (threadIdx.x >> 5); w < units; w += gridDim.x * wpb) {
+    const int t = w / parts, part = w % parts;
+    const int v_begin = part * vec_per_part, v_end = min(vec_per_row, v_begin + vec_per_part);
+    auto row_of = [&](int g) {
+      if (g >= G) return -1;
+      const int a = __ldg(al + (size_t)g * T + t);
+      return a >= 0 ? __ldg(group_offsets + g) + a : -1;
+    };
+    uint4* out = y + (size_t)t * vec_per_row;
+    if (ROWS > 0) {
+      constexpr int R = ROWS > 0 ? ROWS : 1, COLS = 4 / R;
+      int r[R];
 #pragma unroll
-      for (int q = 0; q < 8; ++q) acc[q] = 0.f;
+      for (int q = 0; q < R; ++q) r[q] = -1;
+      int n = 0;
       for (int g0 = 0; g0 < G; g0 += 32) {
-        int row = -1;
-        if (g0 + lane < G) {
-          const int a = __ldg(al + (size_t)(g0 + lane) * T + t);
-          if (a >= 0) row = __ldg(group_offsets + g0 + lane) + a;
+        const int row = row_of(g0 + lane);
+        for (unsigned live = __ballot_sync(0xFFFFFFFFu, row >= 0); live; live &= live - 1, ++n) {
+          const int next = __shfl_sync(0xFFFFFFFFu, row, __ffs(live) - 1);
+#pragma unroll
+          for (int q = 0; q < R; ++q)
+            if (q == n) r[q] = next;
         }
-        unsigned live = __ballot_sync(0xFFFFFFFFu, row >= 0);
+      }
+      for (int v = v_begin + lane; v < v_end; v += 32 * COLS) {
+        uint4 buf[R][COLS];
+#pragma unroll
+        for (int q = 0; q < R; ++q)
+#pragma unroll
+          for (int u = 0; u < COLS; ++u)
+            if (q < n && v + 32 * u < v_end) buf[q][u] = __ldcs(back + (size_t)r[q] * vec_per_row + v + 32 * u);
+#pragma unroll
+        for (int u = 0; u < COLS; ++u) {
+          float acc[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+          for (int q = 0; q < R; ++q)
+            if (q < n) add_row(acc, buf[q][u]);
+          if (v + 32 * u < v_end) out[v + 32 * u] = round_row(acc);
+        }
+      }
+      continue;
+    }
+    const int first_row = row_of(lane);
+    const unsigned first = __ballot_sync(0xFFFFFFFFu, first_row >= 0);
+    for (int v0 = v_begin; v0 < v_end; v0 += 32) {   // whole warps: the row numbers are shuffled
+      const int v = v0 + lane;
+      float acc[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+      for (int g0 = 0; g0 < G; g0 += 32) {
+        const int row = g0 == 0 ? first_row : row_of(g0 + lane);
+        unsigned live = g0 == 0 ? first : __ballot_sync(0xFFFFFFFFu, row >= 0);
         while (live) {
           uint4 buf[4];
           int n = 0;
@@ -107,24 +163,10 @@ __global__ void __launch_bounds__(256) ep_finish_kernel(const uint4* __restrict_
             }
 #pragma unroll
           for (int q = 0; q < 4; ++q)
-            if (q < n && v < v_end) {
-              const __nv_bfloat162* p = reinterpret_cast<const __nv_bfloat162*>(&buf[q]);
-#pragma unroll
-              for (int i = 0; i < 4; ++i) {
-                const float2 f = __bfloat1622float2(p[i]);
-                acc[2 * i] += f.x;
-                acc[2 * i + 1] += f.y;
-              }
-            }
+            if (q < n && v < v_end) add_row(acc, buf[q]);
         }
       }
-      if (v < v_end) {
-        uint4 out;
-        __nv_bfloat162* o = reinterpret_cast<__nv_bfloat162*>(&out);
-#pragma unroll
-        for (int q = 0; q < 4; ++q) o[q] = __floats2bfloat162_rn(acc[2 * q], acc[2 * q + 1]);
-        y[(size_t)t * vec_per_row + v] = out;
-      }
+      if (v < v_end) out[v] = round_row(acc);
     }
   }
 }
@@ -146,10 +188,12 @@ cudaError_t launch_ep_finish(const Shape& s, const void* back, const Layout& L, 
   const int vec = s.d / 8, parts = row_parts(s.T, vec);
   const int vec_per_part = ((vec + parts - 1) / parts + 31) & ~31;   // whole warp-strides per part
   long long blocks = ((long long)s.T * parts + 7) / 8;
-  const long long cap = (long long)sm_count() * 8;
+  const long long cap = (long long)sm_count() * 2 * FINISH_BLOCKS;
   if (blocks > cap) blocks = cap;
-  return launch_pdl(ep_finish_kernel, (unsigned)blocks, 256, 0, st, static_cast<const uint4*>(back), static_cast<uint4*>(y),
-                    L.al, L.group_offsets, s.T, s.G, vec, parts, vec_per_part);
+  const int rows = min(s.k, s.G);
+  return launch_pdl(rows <= 2 ? ep_finish_kernel<2> : rows <= 4 ? ep_finish_kernel<4> : ep_finish_kernel<0>, (unsigned)blocks, 256, 0, st,
+                    static_cast<const uint4*>(back), static_cast<uint4*>(y), L.al, L.group_offsets, s.T, s.G, vec, parts,
+                    vec_per_part);
 }
 
 }  // namespace tcmoe

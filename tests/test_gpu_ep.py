@@ -105,7 +105,8 @@ def test_forward_over_nccl_with_one_rank():
 
 
 @pytest.mark.parametrize("T,d,E,k,G", [(1, 8, 4, 1, 4), (33, 264, 80, 6, 40), (300, 1032, 64, 16, 64), (2051, 2056, 8, 2, 2),
-                                       (127, 64, 1024, 2, 1024), (129, 72, 64, 32, 2), (130, 520, 12, 3, 4)])
+                                       (127, 64, 1024, 2, 1024), (129, 72, 64, 32, 2), (130, 520, 12, 3, 4), (9, 1032, 64, 4, 64),
+                                       (9500, 264, 8, 2, 1)])
 def test_pack_and_finish_edges(T, d, E, k, G):
     """Target lists (unused entries and the rows behind the last dispatched one included) and the final reduction, for more
     than 32 groups, rows that no warp stride divides and rows shared by several warps, against plain tensor operations."""
@@ -155,3 +156,17 @@ def test_packing_for_many_groups_takes_no_longer():
         return lambda: B.moe_ep_pack(shape, idx, w, lay, *out)
 
     assert H.device_us(call(64)) <= 1.5 * H.device_us(call(2))
+
+
+@pytest.mark.parametrize("T,d,G", [(8192, 2880, 1), (8192, 4096, 1), (20000, 1032, 1)])
+def test_final_reduction_of_one_row_is_a_copy(T, d, G):
+    """With one group the final reduction moves what a copy of the rows moves."""
+    shape = B.MoEShape(T, d, 64, 8, 2, G, 0, 0)
+    idx = torch.tensor([[0, 1]], dtype=torch.int32, device="cuda").repeat(T, 1).contiguous().view(-1)
+    lay, ws = B.alloc_layout(shape), B.alloc_workspace(shape)
+    B.moe_dispatch(shape, None, idx, lay, None, ws)
+    back = torch.randn(T, d, device="cuda").to(torch.bfloat16)
+    y = torch.empty_like(back)
+    copy_us = H.device_us(lambda: y.copy_(back))
+    assert H.device_us(lambda: B.moe_ep_finish(shape, back, lay, y)) <= 1.5 * copy_us
+    assert torch.equal(y, back)
