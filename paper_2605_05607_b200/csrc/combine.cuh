@@ -69,12 +69,11 @@ __device__ __forceinline__ void combine_rows(const CombineArgs& c, int t, int la
   }
 }
 
-// The same sums for a token with at most two slots in use: the columns of a row are walked four at a time, so eight loads are
-// in flight per lane instead of two (4096 tokens of d = 4096: 23.5 -> 21 us; 256 of d = 512: 4.6 -> 4.0).
-template <bool COHERENT>
+// The same sums for a token with at most two slots in use: the columns of a row are walked COLS at a time, so up to eight loads
+// are in flight per lane instead of two (4096 tokens of d = 4096: 23.5 -> 21 us; 256 of d = 512: 4.6 -> 4.0).
+template <bool COHERENT, int COLS>
 __device__ __forceinline__ void combine_two(const CombineArgs& c, int t, int lane, int kv, const int* s_row, const int* s_dst,
                                             const float* s_w, int v_begin, int v_end) {
-  constexpr int COLS = 4;
   const int vec_per_row = c.vec_per_row;
   v_end = min(v_end, vec_per_row);
   const bool same = kv > 1 && s_dst[0] == s_dst[1];
@@ -120,7 +119,7 @@ __device__ __forceinline__ void combine_two(const CombineArgs& c, int t, int lan
 // with loads that see what other thread blocks of the SAME kernel wrote (the tracker-paced kernel); otherwise
 // streaming loads.  BATCH (2, 4 or 8): rows loaded at a time; 2 is for k <= 2 only, 4 and 8 are correct for any k, the one that matches
 // k wastes no issue slots on absent slots (a top-2 layer through the 8-row form runs at a third of the bandwidth).
-template <bool COHERENT, int BATCH>
+template <bool COHERENT, int BATCH, int COLS = 4>
 __device__ __forceinline__ void combine_token(const CombineArgs& c, int t, int lane, int* s_row, int* s_dst, float* s_w,
                                               int v_begin = 0, int v_end = 0x7FFFFFFF) {
   const int k = c.k;
@@ -156,7 +155,7 @@ __device__ __forceinline__ void combine_token(const CombineArgs& c, int t, int l
   __syncwarp();
   if (lane < k) { s_row[my_pos] = my_row; s_dst[my_pos] = my_dst; s_w[my_pos] = my_w; }
   __syncwarp();
-  if (BATCH == 2) combine_two<COHERENT>(c, t, lane, kv, s_row, s_dst, s_w, v_begin, v_end);
+  if (BATCH == 2) combine_two<COHERENT, COLS>(c, t, lane, kv, s_row, s_dst, s_w, v_begin, v_end);
   else combine_rows<COHERENT, BATCH>(c, t, lane, kv, s_row, s_dst, s_w, v_begin, v_end);
   __syncwarp();
 }

@@ -504,7 +504,7 @@ cudaError_t launch_permute_rows(const Shape& s, const void* src, int src_rows, c
 // One warp per (token, column part); the per-token work is combine_token() (combine.cuh).  With few tokens a row
 // is split over `parts` warps so that enough loads are in flight to reach the memory bandwidth (one warp per token
 // leaves a 4096-token batch at a third of it).
-template <int BATCH>
+template <int BATCH, int COLS = 4>
 __global__ void __launch_bounds__(256, 3) combine_kernel(const CombineArgs c, int parts, int vec_per_part) {
   grid_dependency_sync();
   __shared__ int s_row[8][32];   // per warp: expert-sorted row of the slot at sorted position p
@@ -515,7 +515,7 @@ __global__ void __launch_bounds__(256, 3) combine_kernel(const CombineArgs c, in
   const long long units = (long long)c.T * parts;
   for (long long u = (long long)blockIdx.x * wpb + wid; u < units; u += (long long)gridDim.x * wpb) {
     const int t = (int)(u / parts), part = (int)(u % parts);
-    combine_token<false, BATCH>(c, t, lane, s_row[wid], s_dst[wid], s_w[wid], part * vec_per_part,
+    combine_token<false, BATCH, COLS>(c, t, lane, s_row[wid], s_dst[wid], s_w[wid], part * vec_per_part,
                                 (part + 1) * vec_per_part);
   }
 }
@@ -546,6 +546,10 @@ cudaError_t launch_combine_rows(const Shape& s, const void* o, const Layout& L, 
   CombineArgs c{static_cast<const uint4*>(o), static_cast<uint4*>(y), static_cast<uint4*>(pg), topk_idx, topk_w,
                 L.pair_row, L.al, L.group_offsets, s.T, s.E, s.k, s.E / s.G, vec, (s.flags & 1) ? 1 : 0,
                 n_rows, status};
+  // parts that are no multiple of four warp strides: two columns at a time, so that the last step is not half empty (2050 tokens of
+  // d = 2880 with group sums, 192 columns each: 11.8 -> 10.4 us, 10.7 with single columns)
+  if (s.k <= 2 && vec_per_part % 128 != 0)
+    return launch_pdl(combine_kernel<2, 2>, (unsigned)blocks, 256, 0, st, c, parts, vec_per_part);
   if (s.k <= 2) return launch_pdl(combine_kernel<2>, (unsigned)blocks, 256, 0, st, c, parts, vec_per_part);
   if (s.k <= 4) return launch_pdl(combine_kernel<4>, (unsigned)blocks, 256, 0, st, c, parts, vec_per_part);
   return launch_pdl(combine_kernel<8>, (unsigned)blocks, 256, 0, st, c, parts, vec_per_part);

@@ -628,3 +628,35 @@ def test_narrow_gemm_tiles_of_few_rows(T, k, fp8):
         return y
 
     assert torch.equal(layer(T), layer(big.T)[:T])
+
+
+@pytest.mark.parametrize("T,d", [(1, 8), (300, 264), (300, 4096), (2050, 2880), (2051, 1032)])
+@pytest.mark.parametrize("k", [1, 2])
+def test_combine_of_at_most_two_rows(T, d, k):
+    """Rows that a part's column steps (two or four warp strides) divide and rows they do not, with and without group sums: the same
+    fp32 additions in the same order with tensor operations."""
+    E, G = 8, 4
+    g = torch.Generator(device="cuda").manual_seed(T + d)
+    idx = torch.rand(T, E, generator=g, device="cuda").topk(k, dim=1).indices.to(torch.int32).contiguous()
+    if T * k < 4:
+        idx = torch.cat([idx.view(-1), torch.zeros(4, dtype=torch.int32, device="cuda")])
+    shape = B.MoEShape(T, d, 64, E, k, G, 0, 0)
+    lay, ws = B.alloc_layout(shape), B.alloc_workspace(shape)
+    B.moe_dispatch(shape, None, idx, lay, None, ws)
+    o = torch.randn(T * k, d, generator=g, device="cuda").to(torch.bfloat16)
+    n = int(lay.group_offsets[G])
+    y, pg, y2 = (torch.full((r, d), 7.0, dtype=torch.bfloat16, device="cuda") for r in (T, n, T))
+    B.moe_combine(shape, o, lay, idx, None, pg, y, ws)
+    B.moe_combine(shape, o, lay, idx, None, None, y2, ws)
+    rows = o.float()[lay.pair_row[: T * k].long()].view(T, k, d)
+    group = idx.view(-1)[: T * k].view(T, k).long() // (E // G)
+    part, ref = torch.zeros(G, T, d, device="cuda"), torch.zeros(T, d, device="cuda")
+    for gi in range(G):
+        for j in range(k):
+            part[gi] += torch.where((group[:, j] == gi)[:, None], rows[:, j], 0.0)
+        ref += part[gi]
+    al = lay.al[: G * T].view(G, T)
+    for gi in range(G):
+        seen = al[gi] >= 0
+        assert torch.equal(pg[(lay.group_offsets[gi] + al[gi][seen]).long()], part[gi][seen].to(torch.bfloat16))
+    assert torch.equal(y, ref.to(torch.bfloat16)) and torch.equal(y2, y) and B.moe_status(ws)[0] == 0
