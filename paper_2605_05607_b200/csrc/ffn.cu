@@ -168,20 +168,35 @@ static bool small_experts(const Shape& s) {
   return (long long)s.T * s.k < 192ll * s.E;
 }
 
-// Fewer full-width tiles than SMs (an upper bound from the shape: every expert that can be reached has one 128-row tile, and one
-// more per 128 pairs): GEMM tiles of 64 output columns.  Wider ones leave SMs idle and the rest waiting on one SM's share of the
-// memory bandwidth: one token of top-2 on d = 4096, f = 14336 (32 tiles of GEMM-2) 87 us, narrow 58; 256 tokens of d = 512, f = 1024:
-// GEMM-1 13.2 -> 10.6, GEMM-2 12.4 -> 9.7.
-static bool narrow_tiles(const Shape& s, int n_tiles) {
-  const long long P = (long long)s.T * s.k;
-  return ((s.E < P ? s.E : P) + P / 128) * n_tiles < 148;
+// At most 64 pairs in all, so at most 64 rows per expert whatever the routing: narrow tiles of 64 rows.
+static bool few_rows(const Shape& s) { return (long long)s.T * s.k <= 64; }
+
+// Full-width tiles of a GEMM with `n_tiles` column tiles, balanced routing
+static long long full_tiles(const Shape& s, int n_tiles) {
+  const long long P = (long long)s.T * s.k, e = s.E < P ? s.E : P;
+  return e * ((P + 128 * e - 1) / (128 * e)) * n_tiles;
 }
 
-// At most 64 pairs in all, so at most 64 rows per expert whatever the routing: narrow tiles of 64 rows.  One token: d = 4096,
-// f = 14336, top-2 160.0 -> 151.5 us, d = 2048, f = 768, top-8 of 128 52.6 -> 50.3; 8 tokens of d = 2048, f = 4096 100 -> 96.  With more
-// than 148 full-width tiles they stay full-width: narrow 64-row ones gave 151 -> 155 us, 201 -> 205, 266 -> 268, and only with
-// few k-blocks a gain (93 -> 91, 84 -> 71).
-static bool few_rows(const Shape& s) { return (long long)s.T * s.k <= 64; }
+// Narrow tiles (64 output columns: half of a GEMM-1 tile, a quarter of a GEMM-2 tile) where full-width ones leave SMs idle.  What a
+// CTA has in flight bounds its stream of weights: 128 KiB full-width, 64 KiB narrow (96 with 64-row tiles), so a narrow GEMM-1 tile takes
+// about two thirds of a full one, a narrow GEMM-2 tile half (a third), and what counts is the rounds that all SMs need for them.
+// Layer with full-width / narrow tiles of that GEMM, us, by the number of full-width tiles:
+//   GEMM-1, up to 64 pairs or 8 bits:  96 (44 pairs, 8 experts of 5024 x 1456) 107.8 / 110.3, 120 (40, 8 x 3808 x 1888) 103.8 / 101.7,
+//                       144 (14, 4 x 1920 x 4528) 79.7 / 77.1; 8 bits: 80 (1864, 8 x 2352 x 528) 74.1 / 67.4, 136 (80, 8 x 592 x 2160) 47.9 / 45.1
+//   GEMM-1, more pairs in bf16:  73 (113, 1 x 1760 x 9264) 98.1 / 93.7, 76 (94, 4 x 1168 x 2400) 49.5 / 50.7, 80 (77, 8 x 4496 x 1264) 90.8 / 98.9
+//   GEMM-2, up to 64 pairs:  32 (14, 4 x 1920 x 4528) 79.7 / 67.1, 80 (8, 16 x 2464 x 7552) 156.1 / 150.1, 96 (42, 8 x 2944 x 2944) 109.6 / 111.9,
+//                       128 (8, 8 x 3888 x 9376) 290 / 318
+//   GEMM-2, more pairs:  32 (248, 8 x 1008 x 4160) 79.6 / 68.4, 38 (138, 2 x 4656 x 12240) 199 / 169, 40 (284, 8 x 1264 x 3632) 82.0 / 84.7,
+//                       112 (137, 8 x 3744 x 12608) 373 / 438; short K: 40 (362, 4 x 2368 x 1136) 57.6 / 54.9, 88 (188, 8 x 2624 x 784) 59.6 / 60.9
+static bool narrow_gemm1(const Shape& s, bool fp8) {
+  const long long tiles = full_tiles(s, (s.f + 127) / 128), sms = sm_count();
+  return 2 * tiles <= sms || ((few_rows(s) || fp8) && tiles < sms);
+}
+static bool narrow_gemm2(const Shape& s) {
+  const long long tiles = full_tiles(s, (s.d + 255) / 256), sms = sm_count();
+  if (few_rows(s)) return 5 * tiles <= 3 * sms;
+  return 4 * tiles <= sms + 4 || (s.f <= 1280 && 2 * tiles <= sms);
+}
 
 size_t fused_table_blocks(const Shape& s) { return ffn::fused_max_blocks(s.T, s.k, s.E); }
 size_t fused_tracker_bytes(const Shape& s) { return ffn::fused_tracker_words(s.T, s.k, s.E) * sizeof(int32_t); }
@@ -259,7 +274,7 @@ cudaError_t launch_expert_ffn(const Shape& s, const FfnArgs& a, cudaStream_t st)
     g1.tile_prefix = a.mp_prefix;
     err = ffn::launch_gemm1_pair(g1, m_w1, m_w3, st);
   } else {
-    err = ffn::launch_gemm1(g1, m_w1, m_w3, false, narrow_tiles(s, (s.f + 127) / 128), few_rows(s), st);
+    err = ffn::launch_gemm1(g1, m_w1, m_w3, false, narrow_gemm1(s, false), few_rows(s), st);
   }
   if (err != cudaSuccess) return err;
 
@@ -281,7 +296,7 @@ cudaError_t launch_expert_ffn(const Shape& s, const FfnArgs& a, cudaStream_t st)
     g2.a_src = a.h;
     g2.a_ld = s.f;
     g2.tile_prefix = a.mt_prefix;
-    return ffn::launch_gemm2_single(g2, m_w2, false, narrow_tiles(s, (s.d + 255) / 256), few_rows(s), st);
+    return ffn::launch_gemm2_single(g2, m_w2, false, narrow_gemm2(s), few_rows(s), st);
   }
   g2.a_src = a.h;
   g2.a_rows = P;
@@ -294,7 +309,7 @@ cudaError_t launch_expert_ffn_fp8(const Shape& s, const FfnArgs& a, const Fp8Arg
   const int P = s.T * s.k;
   CUtensorMap m_w1, m_w3, m_w2;
   const bool single2 = small_experts(s) && a.y_acc == nullptr;
-  const bool narrow1 = narrow_tiles(s, (s.f + 127) / 128), narrow2 = single2 && narrow_tiles(s, (s.d + 255) / 256);
+  const bool narrow1 = narrow_gemm1(s, true), narrow2 = single2 && narrow_gemm2(s);
   if (!make_weight_map_fp8(&m_w1, a.w1, s.E, s.f, s.d, narrow1 ? 64 : 128) ||
       !make_weight_map_fp8(&m_w3, a.w3, s.E, s.f, s.d, narrow1 ? 64 : 128) ||
       !make_weight_map_fp8(&m_w2, a.w2, s.E, s.d, s.f, narrow2 ? 64 : 128))
