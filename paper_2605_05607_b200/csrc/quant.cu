@@ -33,7 +33,7 @@ __device__ __forceinline__ uint32_t to_e4m3_pair(float a, float b, float inv, fl
   return __nv_cvt_float2_to_fp8x2(make_float2(copysignf(qa, a), copysignf(qb, b)),   // -0 stays -0
                                   __NV_SATFINITE, __NV_E4M3);
 }
-// WARPS warps per row (1, or the whole block of 4 for long rows).  The row stays in registers between the maximum and the codes
+// WARPS warps per row (1, or the whole block of 4 for long rows; up to 2048 columns many rows take one warp each, few the block).  The row stays in registers between the maximum and the codes
 // when it has at most KEEP vectors per lane; a longer one is read again.  cols % 8 == 0.  Bound by memory now, by the divisions
 // before: 131072 rows of 1536 columns 159 -> 104 us (5.8 TB/s), 16384 of 4096 65 -> 50, 32768 of 7168 201 -> 132 (5.3 TB/s).
 template <int KEEP, int WARPS>
@@ -162,7 +162,11 @@ cudaError_t launch_quantize_rows(const void* src, long long rows, int cols, void
   uint2* out = static_cast<uint2*>(dst);
   auto grid = [&](long long n) { return (unsigned)(n > cap ? cap : n); };
   if (cols <= 512) return launch_pdl(quantize_rows_kernel<2, 1>, grid((rows + 7) / 8), 256, 0, st, in, out, scale, rows, cols / 8);
+  // six vectors per lane where three do: 16384 rows of 768 columns 10.2 us, three 8.0
+  if (cols <= 768) return launch_pdl(quantize_rows_kernel<3, 1>, grid((rows + 7) / 8), 256, 0, st, in, out, scale, rows, cols / 8);
   if (cols <= 1536) return launch_pdl(quantize_rows_kernel<6, 1>, grid((rows + 7) / 8), 256, 0, st, in, out, scale, rows, cols / 8);
+  // us with a block / a warp per row: 16384 of 1544 columns 24.4 / 17.1, 4096 of 1792 6.8 / 5.7, 300 of 2048 2.2 / 2.6
+  if (cols <= 2048 && rows >= 8ll * sm_count()) return launch_pdl(quantize_rows_kernel<8, 1>, grid((rows + 7) / 8), 256, 0, st, in, out, scale, rows, cols / 8);
   if (cols <= 4096) return launch_pdl(quantize_rows_kernel<4, 4>, grid(rows), 128, 0, st, in, out, scale, rows, cols / 8);
   return launch_pdl(quantize_rows_kernel<8, 4>, grid(rows), 128, 0, st, in, out, scale, rows, cols / 8);   // registers: 8192 columns
 }

@@ -169,7 +169,7 @@ def test_fp8_random_shape_sweep():
         H.assert_close_out(y_gpu, y_ref, f"{cfg}")
 
 
-@pytest.mark.parametrize("cols", [8, 512, 520, 1536, 1544, 4096, 4104, 8200, 14336])
+@pytest.mark.parametrize("cols", [8, 512, 520, 768, 776, 1536, 1544, 2048, 2056, 4096, 4104, 8200, 14336])
 def test_quantize_rows_bit_exact_by_row_length(cols):
     """Rows that fit the registers of each form and rows that do not; every exponent from the row's largest value down to
     where codes vanish, largest values of every magnitude (subnormal scales included), so that quotients fall on and beside
@@ -186,3 +186,13 @@ def test_quantize_rows_bit_exact_by_row_length(cols):
     q_ref, s_ref = F.quantize_rows(O.bf16_to_f64(H.bf16_host(x)))
     assert np.array_equal(s.cpu().numpy(), s_ref)
     assert np.array_equal(q.cpu().numpy(), q_ref)
+
+
+def test_one_vector_more_per_row_does_not_double_the_time():
+    """1544 columns are one vector more than 32 lanes keep in six registers each."""
+    def call(cols, rows=131072):
+        x = torch.randn(rows, cols, device="cuda", dtype=torch.bfloat16)
+        q, s = torch.empty(rows, cols, dtype=torch.uint8, device="cuda"), torch.empty(rows, device="cuda")
+        return lambda: B.moe_quantize_rows(x, q, s)
+
+    assert H.device_us(call(1544)) <= 1.6 * H.device_us(call(1536))
