@@ -311,7 +311,7 @@ ffn_fused_kernel(const __grid_constant__ CUtensorMap map_w1, const __grid_consta
           uint32_t a1[32], a3[32];
           ptx::tmem_ld32(taddr + c * 32, a1);
           ptx::tmem_ld32(taddr + 128 + c * 32, a3);
-          ptx::tmem_ld_wait();
+          ptx::tmem_ld_wait_on(a1, a3);
 #pragma unroll
           for (int v = 0; v < 4; ++v) {
             uint32_t q[4];

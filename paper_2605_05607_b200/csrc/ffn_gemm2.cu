@@ -283,7 +283,7 @@ ffn_gemm2_kernel(const __grid_constant__ CUtensorMap map_b0, const __grid_consta
           uint32_t a1[32], a3[32];
           ptx::tmem_ld32(taddr + c * 32, a1);
           ptx::tmem_ld32(taddr + 64 + c * 32, a3);
-          ptx::tmem_ld_wait();
+          ptx::tmem_ld_wait_on(a1, a3);
           __syncwarp();
           uint32_t q1[16], q3[16];
 #pragma unroll
@@ -330,7 +330,7 @@ ffn_gemm2_kernel(const __grid_constant__ CUtensorMap map_b0, const __grid_consta
           uint32_t a1[32], a3[32];
           ptx::tmem_ld32(taddr + c * 32, a1);
           ptx::tmem_ld32(taddr + 64 + c * 32, a3);
-          ptx::tmem_ld_wait();
+          ptx::tmem_ld_wait_on(a1, a3);
 #pragma unroll
           for (int v = 0; v < 4; ++v) {
             uint32_t q[4];
@@ -349,7 +349,7 @@ ffn_gemm2_kernel(const __grid_constant__ CUtensorMap map_b0, const __grid_consta
         for (int c = 0; c < chunks; ++c) {
           uint32_t acc[32];
           ptx::tmem_ld32(taddr + c * 32, acc);
-          ptx::tmem_ld_wait();
+          ptx::tmem_ld_wait_on(acc);
           if (FP8) {
 #pragma unroll
             for (int j = 0; j < 32; ++j) {

@@ -197,6 +197,28 @@ def test_every_kernel_waits_for_its_stream_predecessor():
     assert seen >= 15
 
 
+def test_every_tensor_memory_load_is_waited_for_by_name():
+    """tcgen05.ld fills its registers some time after it was issued.  Only a wait that has the registers as operands keeps their uses
+    below it, so every array that is loaded has to be named by a wait before the next line that is neither load nor wait."""
+    csrc = os.path.join(ROOT, "paper_2605_05607_b200", "csrc")
+    assert not re.search(r"tcgen05\.wait::ld[^;]*;\"\s*:::", open(os.path.join(csrc, "ptx.cuh")).read())
+    seen = 0
+    for fn in sorted(os.listdir(csrc)):
+        if not fn.endswith(".cu"):
+            continue
+        pending = set()
+        for line in open(os.path.join(csrc, fn)):
+            code = line.split("//")[0].strip()
+            load, wait = re.search(r"tmem_ld32\(.*, (\w+)\);", code), re.search(r"tmem_ld_wait_on\(([^)]*)\);", code)
+            if load:
+                pending.add(load.group(1))
+                seen += 1
+            elif wait:
+                pending -= set(wait.group(1).replace(" ", "").split(","))
+            elif code and not code.startswith(("#pragma", "for (int t = 1; t < 3")):
+                assert not pending, f"{fn}: {pending} used before a wait that names them: {code}"
+
+
 def test_product_package_never_imports_the_oracle():
     pkg = os.path.join(ROOT, "paper_2605_05607_b200")
     pat = re.compile(r"^\s*(from|import)\s+oracle\b|oracle[/.]moe_oracle|#include\s+\".*oracle", re.M)
