@@ -198,7 +198,7 @@ def stage_breakdown(cfg, t, reps=5, with_ffn=True):
         "layer_fused": lambda: B.moe_layer(shape, t["x"], t["w_gate"], t["bias"], t["w1"], t["w3"], t["w2"], y, ws),
     }
     kernels = {"route": ["gate", "topk"], "dispatch": ["dispatch"], "expert_ffn": ["gemm1", "gemm2"],
-               "combine": ["combine"], "layer_fused": ["gate", "topk", "gemm1", "gemm2", "combine"]}
+               "combine": ["combine"], "layer_fused": ["gate", "topk", "topk_layout", "gemm1", "gemm2", "combine"]}
     if not with_ffn:
         del calls["expert_ffn"], calls["layer_fused"]
     out = {}
@@ -223,7 +223,8 @@ def stage_breakdown(cfg, t, reps=5, with_ffn=True):
                 fn()
             ms, n = B.moe_profile_read()
             B.moe_profile_enable(0)
-            out[name][kn + "_kernel_ms"] = ms / max(n, 1)
+            if n:
+                out[name][kn + "_kernel_ms"] = ms / n
     n_disp = int(lay.group_offsets[cfg.G].item())
     counts = lay.expert_counts[:E].cpu().numpy()
     pk = peaks()
@@ -291,7 +292,8 @@ def stage_breakdown(cfg, t, reps=5, with_ffn=True):
             calls["layer_fused"]()
         ms, n = B.moe_profile_read()
         B.moe_profile_enable(0)
-        out["layer_fused"][kn + "_in_layer_ms"] = ms / max(n, 1)
+        if n:                                          # top-k: a kernel of its own, or one with the layout (small batches)
+            out["layer_fused"][kn + "_in_layer_ms"] = ms / n
     out["combine"]["in_layer_gbs"] = comb_bytes / out["layer_fused"]["combine_in_layer_ms"] / 1e6
     # FP8 experts (E4M3, per-token and per-output-column scales): the same layer through moe_layer_fp8
     if d % 16 == 0 and f % 16 == 0:

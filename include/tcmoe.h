@@ -336,7 +336,8 @@ int moe_workspace_layout(const moe_shape_t* shape, size_t out[4]);
 /* Kernel ids for moe_profile_enable (also the `where` slot of moe_status). */
 enum { MOE_KERNEL_TOPK = 1, MOE_KERNEL_MASKS = 2, MOE_KERNEL_FILL = 3, MOE_KERNEL_DISPATCH = 4,
        MOE_KERNEL_GEMM1 = 5, MOE_KERNEL_GEMM2 = 6, MOE_KERNEL_COMBINE = 7, MOE_KERNEL_GATE = 8,
-       MOE_KERNEL_WGRAD = 10, MOE_KERNEL_BWD_GATHER = 11, MOE_KERNEL_GATE_BWD = 12 };
+       MOE_KERNEL_WGRAD = 10, MOE_KERNEL_BWD_GATHER = 11, MOE_KERNEL_GATE_BWD = 12,
+       MOE_KERNEL_TOPK_LAYOUT = 13 };   /* top-k and layout of a small batch, which moe_layer takes in one kernel */
 
 /* Per-kernel timing hook for benchmarks (host-side state, one record per process, guarded by a
  * mutex so that launches from several host threads are safe; not part of the method).  After moe_profile_enable(id) every launch of that kernel by any entry point is

@@ -342,7 +342,7 @@ def moe_layer_host(shape, x_host, x_dev, w_gate, logit_bias, w1, w3, w2, y_dev, 
 
 
 KERNEL_IDS = {"topk": 1, "masks": 2, "fill": 3, "dispatch": 4, "gemm1": 5, "gemm2": 6, "combine": 7, "gate": 8,
-              "wgrad": 10, "bwd_gather": 11, "gate_bwd": 12}
+              "wgrad": 10, "bwd_gather": 11, "gate_bwd": 12, "topk_layout": 13}
 
 
 def moe_profile_enable(kernel_id: int) -> None:

@@ -306,7 +306,7 @@ int moe_selftest_wait_timeout(void* ws, uint64_t limit_ns, void* stream) {
 }
 
 int moe_profile_enable(int kernel_id) {
-  if (kernel_id < 0 || kernel_id > 12) return MOE_ERR_INVALID_ARG;
+  if (kernel_id < 0 || kernel_id > 13) return MOE_ERR_INVALID_ARG;
   std::lock_guard<std::mutex> lock(g_profile_mutex);
   g_profile_id.store(kernel_id, std::memory_order_relaxed);
   g_profile_n = 0;

@@ -10,7 +10,7 @@ namespace tcmoe {
 // ---- status block at the start of the workspace (16 x int32) --------------------------------
 enum StatusSlot { ST_CODE = 0, ST_WHERE = 1, ST_DETAIL = 2, ST_AUX = 3, ST_ABORT = 4, ST_WARN = 5 };
 enum KernelId { KID_TOPK = 1, KID_MASKS = 2, KID_FILL = 3, KID_DISPATCH = 4, KID_GEMM1 = 5, KID_GEMM2 = 6,
-                KID_COMBINE = 7, KID_GATE = 8, KID_SELFTEST = 9, KID_WGRAD = 10, KID_BWD = 11, KID_GATE_BWD = 12 };
+                KID_COMBINE = 7, KID_GATE = 8, KID_SELFTEST = 9, KID_WGRAD = 10, KID_BWD = 11, KID_GATE_BWD = 12, KID_TOPK_LAYOUT = 13 };
 constexpr int DEV_TIMEOUT = 1;
 constexpr int DEV_INDEX_OUT_OF_RANGE = 2;
 constexpr int WARN_NONFINITE_LOGIT = 1;

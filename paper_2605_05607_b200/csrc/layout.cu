@@ -335,7 +335,7 @@ bool topk_in_layout(const Shape& s) { return s.T <= 512 && s.E <= 256 && layout_
 cudaError_t launch_topk_layout(const Shape& s, const float* logits, const float* bias, int64_t bias_stride, int32_t* topk_idx,
                                float* topk_w, const Layout& L, const LayoutScratch& sc, int32_t* status, cudaStream_t st) {
   const TopkArgs tk{logits, bias, (long long)bias_stride, topk_w, s.score_fn};
-  ProfileScope prof(KID_TOPK, st);
+  ProfileScope prof(KID_TOPK_LAYOUT, st);
   if (s.E <= 32) return launch_layout_one<1>(s, topk_idx, tk, L, sc, status, st);
   if (s.E <= 64) return launch_layout_one<2>(s, topk_idx, tk, L, sc, status, st);
   if (s.E <= 128) return launch_layout_one<4>(s, topk_idx, tk, L, sc, status, st);
