@@ -171,31 +171,31 @@ static bool small_experts(const Shape& s) {
 // At most 64 pairs in all, so at most 64 rows per expert whatever the routing: narrow tiles of 64 rows.
 static bool few_rows(const Shape& s) { return (long long)s.T * s.k <= 64; }
 
-// Full-width tiles of a GEMM with `n_tiles` column tiles, balanced routing
-static long long full_tiles(const Shape& s, int n_tiles) {
+// 128-row tiles of balanced routing
+static long long row_tiles(const Shape& s) {
   const long long P = (long long)s.T * s.k, e = s.E < P ? s.E : P;
-  return e * ((P + 128 * e - 1) / (128 * e)) * n_tiles;
+  return e * ((P + 128 * e - 1) / (128 * e));
 }
 
 // Narrow tiles (64 output columns: half of a GEMM-1 tile, a quarter of a GEMM-2 tile) where full-width ones leave SMs idle.  What a
 // CTA has in flight bounds its stream of weights: 128 KiB full-width, 64 KiB narrow (96 with 64-row tiles), so a narrow GEMM-1 tile takes
 // about two thirds of a full one, a narrow GEMM-2 tile half (a third), and what counts is the rounds that all SMs need for them.
-// Layer with full-width / narrow tiles of that GEMM, us, by the number of full-width tiles:
-//   GEMM-1, up to 64 pairs or 8 bits:  96 (44 pairs, 8 experts of 5024 x 1456) 107.8 / 110.3, 120 (40, 8 x 3808 x 1888) 103.8 / 101.7,
-//                       144 (14, 4 x 1920 x 4528) 79.7 / 77.1; 8 bits: 80 (1864, 8 x 2352 x 528) 74.1 / 67.4, 136 (80, 8 x 592 x 2160) 47.9 / 45.1
-//   GEMM-1, more pairs in bf16:  73 (113, 1 x 1760 x 9264) 98.1 / 93.7, 76 (94, 4 x 1168 x 2400) 49.5 / 50.7, 80 (77, 8 x 4496 x 1264) 90.8 / 98.9
-//   GEMM-2, up to 64 pairs:  32 (14, 4 x 1920 x 4528) 79.7 / 67.1, 80 (8, 16 x 2464 x 7552) 156.1 / 150.1, 96 (42, 8 x 2944 x 2944) 109.6 / 111.9,
-//                       128 (8, 8 x 3888 x 9376) 290 / 318
-//   GEMM-2, more pairs:  32 (248, 8 x 1008 x 4160) 79.6 / 68.4, 38 (138, 2 x 4656 x 12240) 199 / 169, 40 (284, 8 x 1264 x 3632) 82.0 / 84.7,
-//                       112 (137, 8 x 3744 x 12608) 373 / 438; short K: 40 (362, 4 x 2368 x 1136) 57.6 / 54.9, 88 (188, 8 x 2624 x 784) 59.6 / 60.9
+// Layer with full-width / narrow tiles of that GEMM, us, by the number of narrow tiles:
+//   GEMM-1, up to 64 pairs or 8 bits:  184 (44 pairs, 8 experts of 5024 x 1456) 107.8 / 110.3, 240 (40, 8 x 3808 x 1888) 103.8 / 101.7,
+//                       284 (14, 4 x 1920 x 4528) 79.7 / 77.1; 8 bits: 144 (1864, 8 x 2352 x 528) 74.1 / 67.4, 272 (80, 8 x 592 x 2160) 47.9 / 45.1
+//   GEMM-1, more pairs in bf16:  145 (113, 1 x 1760 x 9264) 98.1 / 93.7, 152 (94, 4 x 1168 x 2400) 49.5 / 50.7, 160 (77, 8 x 4496 x 1264) 90.8 / 98.9
+//   GEMM-2, up to 64 pairs:  120 (14, 4 x 1920 x 4528) 79.7 / 67.1, 312 (8, 16 x 2464 x 7552) 156.1 / 150.1, 368 (42, 8 x 2944 x 2944) 109.6 / 111.9,
+//                       488 (8, 8 x 3888 x 9376) 290 / 318
+//   GEMM-2, more pairs:  128 (248, 8 x 1008 x 4160) 79.6 / 68.4, 144 (72, 16 x 576 x 12128) 110 / 87, 160 (284, 8 x 1264 x 3632) 82.0 / 84.7,
+//                       472 (137, 8 x 3744 x 12608) 373 / 438; short K: 148 (362, 4 x 2368 x 1136) 57.6 / 54.9, 328 (188, 8 x 2624 x 784) 59.6 / 60.9
 static bool narrow_gemm1(const Shape& s, bool fp8) {
-  const long long tiles = full_tiles(s, (s.f + 127) / 128), sms = sm_count();
-  return 2 * tiles <= sms || ((few_rows(s) || fp8) && tiles < sms);
+  const long long rows = row_tiles(s), sms = sm_count();
+  return rows * ((s.f + 63) / 64) <= sms || ((few_rows(s) || fp8) && rows * ((s.f + 127) / 128) < sms);
 }
 static bool narrow_gemm2(const Shape& s) {
-  const long long tiles = full_tiles(s, (s.d + 255) / 256), sms = sm_count();
-  if (few_rows(s)) return 5 * tiles <= 3 * sms;
-  return 4 * tiles <= sms + 4 || (s.f <= 1280 && 2 * tiles <= sms);
+  const long long tiles = row_tiles(s) * ((s.d + 63) / 64), sms = sm_count();
+  if (few_rows(s)) return 5 * tiles <= 12 * sms;
+  return tiles <= sms + 4 || (s.f <= 1280 && tiles <= 2 * sms);
 }
 
 size_t fused_table_blocks(const Shape& s) { return ffn::fused_max_blocks(s.T, s.k, s.E); }
