@@ -25,10 +25,12 @@ struct WsPlan {
 };
 
 // GEMM-1 form.  The CTA-pair form needs the per-expert layout tensors (one more pass over P rows of d) and runs
-// GEMM-1 about 8 % faster; the pass costs about 240 / f of GEMM-1's time, so it pays for wide experts.  Taken when asked
-// for (MOE_FLAG_GEMM1_PAIR), or by itself for f >= 8192 with experts of at least 512 rows on average (measured: the
-// Mixtral-shaped layer gains 3 %, f = 1536 and f = 2048 layers lose 1-6 %); MOE_FLAG_GEMM1_GATHER keeps the gathering
-// form.  bf16 experts outside the tracker-paced kernel only.
+// GEMM-1 faster; the pass costs about 240 / f of GEMM-1's time, so it pays for wide experts.  Taken when asked
+// for (MOE_FLAG_GEMM1_PAIR), or by itself for f >= 8192 with experts of at least 512 rows on average; MOE_FLAG_GEMM1_GATHER
+// keeps the gathering form.  bf16 experts outside the tracker-paced kernel only.  Layer, gathering / pairs, us, by rows per expert:
+// 4096 x 14336: 300 1099 / 1184, 512 1397 / 1286, 1024 2515 / 2311; 4096 x 8192: 300 619 / 658, 512 826 / 760, 1024 1492 / 1401;
+// 7168 x 2048: 512 1486 / 1539, 1024 2552 / 2578; 4096 x 1536: 512 649 / 634, 1500 1772 / 1800.  Between them the line is not tight:
+// 2880 x 2880 gains too from 512 rows on (896 / 848, 1024 1537 / 1436).
 bool pair_gemm1(const moe_shape_t& s) {
   if (s.flags & (MOE_FLAG_FUSED_FFN | MOE_FLAG_GEMM1_GATHER)) return false;
   if (s.flags & MOE_FLAG_GEMM1_PAIR) return true;

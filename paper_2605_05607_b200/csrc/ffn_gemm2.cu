@@ -154,7 +154,11 @@ ffn_gemm2_kernel(const __grid_constant__ CUtensorMap map_b0, const __grid_consta
   const int total = WGRAD ? p.E * wg_per_expert : tp_s[p.E] * p.n_tiles;
   // 128-row tiles where they are most of the tiles, or where a pair has enough tiles to even out the two lengths.  With a handful
   // of mixed tiles the longest chain is as long as before, and pairs that read the same weights no longer do so at the same time:
-  // GEMM-2 of 4096 x 14336 experts with 1024 rows (8 tiles per pair) 705 -> 724 us, its GEMM-1 (54 per pair) 1443 -> 1397.
+  // GEMM-2 of 4096 x 14336 experts with 1024 skewed rows (8 tiles per pair) 705 -> 724 us, its GEMM-1 (54 per pair) 1443 -> 1397.
+  // Layer of both GEMMs on pairs, 128-row tiles on / off, us, even routing, by (rows, tiles per pair of GEMM-1 and GEMM-2): 4096 x 14336
+  // experts (100, 12 and 2) 505 / 584, (300, 24 and 3) 1122 / 1095, (600, 36 and 5) 1572 / 1694; 2880 x 2880 (300, 20 and 10) 670 / 647,
+  // (600, 30 and 16) 984 / 1034; 4096 x 4096 (260, 7 and 3) 281 / 288, (600, 10 and 5) 479 / 509.  So with even routing fewer tiles than
+  // twelve gain as well, and up to 3 % are lost where the tiles left are just over 128 rows; the line follows the skewed layer.
   const bool halves = total >= 12 * num_clusters || eoff_s[p.E] < 160 * tp_s[p.E];
   constexpr int BK_ELEMS = FP8 ? 2 * BK : BK;   // K elements per stage: 128 bytes per row either way
   const int KB = MODE == PAIR_KSPLIT ? 2 * p.k_split : (p.K + BK_ELEMS - 1) / BK_ELEMS;

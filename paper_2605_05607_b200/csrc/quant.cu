@@ -35,7 +35,7 @@ __device__ __forceinline__ uint32_t to_e4m3_pair(float a, float b, float inv, fl
 }
 // WARPS warps per row (1, or the whole block of 4 for long rows; up to 2048 columns many rows take one warp each, few the block).  The row stays in registers between the maximum and the codes
 // when it has at most KEEP vectors per lane; a longer one is read again.  cols % 8 == 0.  Bound by memory now, by the divisions
-// before: 131072 rows of 1536 columns 159 -> 104 us (5.8 TB/s), 16384 of 4096 65 -> 50, 32768 of 7168 201 -> 132 (5.3 TB/s).
+// before: 131072 rows of 1536 columns 152 -> 101 us (6.0 TB/s), 131072 of 4096 370 -> 281 (5.7 TB/s), 16384 of 4096, which stay in L2, 64 -> 37.
 template <int KEEP, int WARPS>
 __global__ void __launch_bounds__(WARPS == 1 ? 256 : WARPS * 32) quantize_rows_kernel(const uint4* __restrict__ src, uint2* __restrict__ dst,
                                                             float* __restrict__ scale, long long rows, int vec_per_row) {
