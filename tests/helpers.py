@@ -115,20 +115,25 @@ def check_layout(run: Run, idx_ref):
     return lay
 
 
-def device_us(call, n=10, reps=5):
-    """Device time of one call: n of them in a CUDA graph (no host time in between), the quickest of some replays."""
-    call()
-    torch.cuda.synchronize()
-    graph, side = torch.cuda.CUDAGraph(), torch.cuda.Stream()
-    with torch.cuda.graph(graph, stream=side):
-        for _ in range(n):
-            call()
-    e0, e1 = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
-    times = []
-    for _ in range(reps):
-        e0.record()
-        graph.replay()
-        e1.record()
+def device_us(*calls, n=10, reps=20):
+    """Device time of each call: n of them in a CUDA graph (no host time in between), the quickest of some replays.  The calls take turns,
+    so that the clock of one stretch of time does not count for one of them alone."""
+    graphs = []
+    for call in calls:
+        call()
         torch.cuda.synchronize()
-        times.append(e0.elapsed_time(e1) * 1e3 / n)
-    return min(times)
+        graph, side = torch.cuda.CUDAGraph(), torch.cuda.Stream()
+        with torch.cuda.graph(graph, stream=side):
+            for _ in range(n):
+                call()
+        graphs.append(graph)
+    e0, e1 = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+    times = [[] for _ in calls]
+    for _ in range(reps):
+        for graph, t in zip(graphs, times):
+            e0.record()
+            graph.replay()
+            e1.record()
+            torch.cuda.synchronize()
+            t.append(e0.elapsed_time(e1) * 1e3 / n)
+    return [min(t) for t in times]

@@ -361,4 +361,6 @@ def test_gradients_of_ragged_rows_take_no_longer():
         return lambda: B.moe_layer_backward(r.shape, t["x"], bw.dy, r.idx, r.w, r.lay, t["w1"], t["w3"], t["w2"], bw.dx, bw.dw1,
                                             bw.dw3, bw.dw2, bw.ws)
 
-    assert H.device_us(call(4104, 1544), n=2) <= 1.2 * H.device_us(call(4112, 1552), n=2)
+    # measured, taking turns: 1.13-1.18; stored sector by sector 1.42-1.44.  The line lies in the middle.
+    us, other = H.device_us(call(4104, 1544), call(4112, 1552), n=2)
+    assert us <= 1.3 * other

@@ -155,7 +155,8 @@ def test_packing_for_many_groups_takes_no_longer():
         out = torch.empty(rows, kk, dtype=torch.int32, device="cuda"), torch.empty(rows, kk, device="cuda")
         return lambda: B.moe_ep_pack(shape, idx, w, lay, *out)
 
-    assert H.device_us(call(64)) <= 1.5 * H.device_us(call(2))
+    us, other = H.device_us(call(64), call(2))
+    assert us <= 1.5 * other
 
 
 @pytest.mark.parametrize("T,d,G", [(8192, 2880, 1), (8192, 4096, 1), (20000, 1032, 1)])
@@ -167,6 +168,6 @@ def test_final_reduction_of_one_row_is_a_copy(T, d, G):
     B.moe_dispatch(shape, None, idx, lay, None, ws)
     back = torch.randn(T, d, device="cuda").to(torch.bfloat16)
     y = torch.empty_like(back)
-    copy_us = H.device_us(lambda: y.copy_(back))
-    assert H.device_us(lambda: B.moe_ep_finish(shape, back, lay, y)) <= 1.5 * copy_us
+    us, copy_us = H.device_us(lambda: B.moe_ep_finish(shape, back, lay, y), lambda: y.copy_(back))
+    assert us <= 1.5 * copy_us
     assert torch.equal(y, back)

@@ -85,7 +85,7 @@ def test_gate_logits(T, d, E):
 @pytest.mark.gpu
 @pytest.mark.parametrize("T,d,E,wider", [(16384, 2880, 129, 192), (8192, 7168, 250, 256), (16384, 7168, 258, 384)])
 def test_fewer_experts_take_no_longer(T, d, E, wider):
-    """A number of experts that is no multiple of the tile's width or of 4 costs at most what the wider gate costs."""
+    """A number of experts that is no multiple of the tile's width or of 4 costs about what the wider gate costs."""
     def call(E):
         x = torch.randn(T, d, device="cuda").to(torch.bfloat16)
         w = torch.randn(d, E, device="cuda") * 0.02
@@ -94,5 +94,7 @@ def test_fewer_experts_take_no_longer(T, d, E, wider):
         out = torch.empty(T, E, device="cuda"), torch.empty(T, dtype=torch.int32, device="cuda"), torch.empty(T, device="cuda")
         return lambda: B.moe_route(shape, x, w, None, *out, ws)
 
-    # 15 % for what the selection of E + 1 more keys and the spread of the clock may take
-    assert H.device_us(call(E)) <= 1.15 * H.device_us(call(wider))
+    # measured, taking turns: 1.12-1.13, 1.08-1.11, 1.00-1.02 (rows of logits that start anywhere); with the split in the GEMM for every
+    # size 1.34, 1.68, 1.41.  The line lies in the middle of the closest two.
+    us, other = H.device_us(call(E), call(wider))
+    assert us <= 1.23 * other
