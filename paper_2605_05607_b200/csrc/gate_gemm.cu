@@ -39,6 +39,8 @@ __host__ __device__ constexpr int work_warps(bool pre) { return pre ? 4 : 16; }
 __host__ __device__ constexpr int threads(bool pre) { return (work_warps(pre) + 2) * 32; }
 constexpr int PRE_MIN_TOKENS = 512;             // fewer tokens never take a split copy of the weight: no workspace for it
 constexpr double PRE_US = 3.0;                  // its launch
+constexpr int STAGE_OUT = 32 * 33;              // floats of a warp's transpose buffer, in the ring
+static_assert(16 * STAGE_OUT * 4 <= RING_BYTES, "buffers of all warps");
 
 struct GateParams {
   const float* w;     // [d, E]
@@ -218,17 +220,28 @@ gate_umma_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constan
             ptx::tmem_ld32(taddr + i * GN, acc);
             ptx::tmem_ld_wait_on(acc);
           }
-          if (row >= p.T) continue;
-          float* out = p.logits + (size_t)row * p.E + n0 + c;
           if (vec) {
+            if (row >= p.T) continue;
+            float* out = p.logits + (size_t)row * p.E + n0 + c;
 #pragma unroll
             for (int v = 0; v < 8; ++v)
               if (n0 + c + v * 4 < p.E)
                 *reinterpret_cast<uint4*>(out + v * 4) = make_uint4(acc[v * 4], acc[v * 4 + 1], acc[v * 4 + 2], acc[v * 4 + 3]);
           } else {
+            // Rows that start anywhere.  A lane that stores its own row by the element makes 32 pieces of each store, which bounds the
+            // kernel for short K; so 32 rows go through the ring, which nothing fills or reads any more, and leave a row per store:
+            // route of 16384 tokens, d = 256, 129 experts 36.0 -> 23.5 us, d = 7168, 250 experts 164 -> 149, 12288, 256, 66: 22.9 -> 15.0.
+            float* st = reinterpret_cast<float*>(smem) + warp * STAGE_OUT;
 #pragma unroll
-            for (int v = 0; v < 32; ++v)
-              if (n0 + c + v < p.E) out[v] = __uint_as_float(acc[v]);
+            for (int v = 0; v < 32; ++v) st[lane * 33 + v] = __uint_as_float(acc[v]);
+            __syncwarp();
+            const int first = row0 + i * ROWS_M + (warp & 3) * (ROWS_M / 4), rows = min(ROWS_M / 4, p.T - first);
+            if (n0 + c + lane < p.E) {
+              float* out = p.logits + (size_t)first * p.E + n0 + c + lane;
+#pragma unroll 8
+              for (int r = 0; r < rows; ++r) out[(size_t)r * p.E] = st[r * 33 + lane];
+            }
+            __syncwarp();
           }
         }
         ptx::tc_fence_before();
@@ -332,7 +345,8 @@ __global__ void __launch_bounds__(256) split_gate_kernel(const float* __restrict
 // Tiles of 64 rows halve what a UMMA reads of x, which counts where twelve of them make a k-block (running sum: 128 tokens
 // of d = 7168, 256 experts 66 -> 48 us); with the terms apart they change nothing.
 // moe_route of (T, d, E), us, without the split copy / with this table: 16384, 2880, 65: 61.4 / 50.4; 16384, 2880, 128: 53.0 / 49.4;
-// 32768, 2880, 96: 102 / 92; 8192, 7168, 256: 115 / 85; 32768, 7168, 250: 459 / 335; 4097, 7168, 258: 194 / 90.
+// 32768, 2880, 96: 102 / 92; 8192, 7168, 256: 115 / 85; 32768, 7168, 250: 459 / 335; 4097, 7168, 258: 194 / 90 (the last two
+// 315 -> 291 and 98 -> 91 in a replayed graph since ragged rows of logits leave whole).
 struct GatePlan { int gn, bm, m_sub; bool pre; };
 GatePlan plan_gate(int T, int d, int E) {
   struct Cost { double start, kb, kb_ragged; };
