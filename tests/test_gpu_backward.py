@@ -351,6 +351,27 @@ def test_pair_tiles_of_at_most_128_rows(rows):
             close(O.bf16_to_f64(H.bf16_host(got[e])), r, f"{n} of expert {e}")
 
 
+@pytest.mark.parametrize("d,f", [(264, 520), (8, 136), (136, 8), (248, 272), (392, 1032)])
+def test_gradients_of_experts_without_rows_are_zero(d, f):
+    """Every element is written, for rows that start at a multiple of 16 bytes (8 columns more than a multiple of 16) as for others."""
+    cfg = synth.MoEConfig("zeros", T=3, d=d, f=f, E=8, k=2, G=1)
+    bw = Backward(cfg)
+    for g in (bw.dw1, bw.dw3, bw.dw2):
+        g.fill_(float("nan"))
+    bw()
+    run = bw.run
+    dx_ref, grads = O.layer_backward(H.bf16_host(run.t["x"]), run.host_idx(), run.host_w(),
+                                     *(H.bf16_host(run.t[n]) for n in ("w1", "w3", "w2")), O.bf16_to_f64(H.bf16_host(bw.dy))[: cfg.T])
+    used = set(run.host_idx().reshape(-1).tolist())
+    assert len(used) < cfg.E
+    for e in range(cfg.E):
+        for i, (got, n) in enumerate(zip((bw.dw1, bw.dw3, bw.dw2), ("dW1", "dW3", "dW2"))):
+            if e in used:
+                close(O.bf16_to_f64(H.bf16_host(got[e])), grads[e][i], f"{n} of expert {e}")
+            else:
+                assert bool((got[e] == 0).all()), (n, e)
+
+
 def test_gradients_of_ragged_rows_take_no_longer():
     """7 tokens of 64 experts: the backward pass writes gradients of mostly empty experts.  Rows of 8 columns more than a multiple of 16
     start inside a 32-byte sector; they cost about what the rows of 8 columns more cost."""
