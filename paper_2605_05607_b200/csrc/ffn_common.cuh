@@ -113,6 +113,11 @@ __host__ __device__ constexpr uint32_t idesc_bf16(int m, int n = UMMA_N) {
          ((uint32_t)(m >> 4) << 24);
 }
 
+// instruction descriptor with the weights as the M operand (128 columns) and n rows of activations as the N operand
+__host__ __device__ constexpr uint32_t idesc_swapped(bool fp8, int n) {
+  return (1u << 4) | (fp8 ? 0u : (1u << 7) | (1u << 10) | (1u << 15)) | ((uint32_t)(n >> 3) << 17) | ((uint32_t)(128 >> 4) << 24);
+}
+
 __device__ __forceinline__ float silu_mul(float a, float b) { return __fdividef(a, 1.f + __expf(-a)) * b; }
 
 __device__ __forceinline__ uint32_t pack2(float lo, float hi) {

@@ -53,6 +53,7 @@ constexpr int GATHER_THREADS = 128;
 // The UMMA thread's wait for a full stage is on the critical path and keeps the plain form (hinting it too gives the
 // gain back).
 constexpr uint32_t FEED_HINT = 1000;
+constexpr int SWAP_ROWS = 96;   // see `swapped`
 
 // FP8 = true: A rows and weights are E4M3 codes, a stage holds 128 elements of K (the same 128
 // bytes per row), W1 / W3 come K-major from [E, N, K] as two 128-row boxes, and the epilogue applies
@@ -144,6 +145,15 @@ ffn_gemm1_kernel(const __grid_constant__ CUtensorMap map_w1, const __grid_consta
     p.status[ST_ABORT] = 1;
     *abort_flag = 1;
   };
+  // An expert of at most 96 rows exchanges the operands: the tile's weight columns are the M side (two UMMAs of 128), its rows, rounded
+  // up to 16, the N side.  A layer of such experts streams weights at the board's power limit, and an UMMA of 128 rows, most of
+  // them padding, over 256 columns costs energy (and copies of zero rows) for the padding too.  Same sums, same bits.
+  // Layers in a loop, us, rows per expert in brackets: 64 tokens, top-8 of 128 x 4096 x 1536 (4) 766 -> 722, 128 tokens, 256 x 7168 x 2048
+  // in 8 bits (4) 1930 -> 1733, 1777 skewed tokens, 128 x 2880 x 2880 946 -> 894, 1200, 128 x 2880 x 2880 in 8 bits (75) 706 -> 686,
+  // 500 top-4 of 32 x 4096 x 1536 (62) 253 -> 249, 800 top-8 of 64 x 2048 x 2048 (100) 343 -> 344; up to 64 rows only: 1200 in 8 bits 703;
+  // up to 128: 800 tokens 350.  The last tile of a larger expert keeps the plain form: a CTA that is done with it earlier leaves the
+  // company of those that read the same weights (32768 tokens, 256 x 7168 x 2048: 23100 -> 25900).
+  auto swapped = [&](const Tile& t) { return !NARROW && t.rows <= SWAP_ROWS && t.row0 == eoff_s[t.e]; };
   auto tile_of = [&](int w) { return decode_tile(w, tp_s, eoff_s, p.E, p.n_tiles, BN_OUT, BM, 0); };
 
   if (warp < 4) {
@@ -161,7 +171,56 @@ ffn_gemm1_kernel(const __grid_constant__ CUtensorMap map_w1, const __grid_consta
       // stores whole 128-byte row segments, 8 lanes per row, 4 rows per instruction.
       const uint32_t stage = stage_base + (uint32_t)(warp * STAGE_OUT_WARP);
       const int srow = lane >> 3, piece = lane & 7;
-      if (PLAIN) {
+      if (swapped(t)) {
+        // lane = output column of a half tile (GEMM-1: the same column of W1 and of W3), TMEM column = row
+        const int c = warp * 32 + lane, odd = lane & 1;
+        const size_t sc = (size_t)t.e * p.N + t.n0 + c;
+        float sa = 1.f, sb = 1.f;   // FP8: column scales
+        if (FP8) {
+          const int hi = PLAIN ? HALF : 0;
+          sa = t.n0 + c < p.N ? __ldg(p.b_scale + sc) : 0.f;
+          sb = t.n0 + hi + c < p.N ? __ldg((PLAIN ? p.b_scale : p.b_scale2) + sc + hi) : 0.f;
+        }
+#pragma unroll 1
+        for (int r0 = 0; r0 < t.rows; r0 += 16) {
+          const int mine = r0 + (lane & 15);
+          float rs = 1.f;   // scale of this lane's row of the 16
+          if (mine < t.rows) {
+            const size_t grow = (size_t)t.row0 + mine;
+            if (PLAIN) {
+              if (p.topk_w != nullptr) rs = __ldg(p.topk_w + __ldg(p.row_pair + grow));
+              if (FP8) rs *= __ldg(p.a_scale + grow);
+            } else if (FP8) {
+              int idx = __ldg(p.gather_idx + grow);
+              if (p.gather_div > 1) idx /= p.gather_div;
+              rs = (idx >= 0 && idx < p.a_rows) ? __ldg(p.a_scale + idx) : 0.f;
+            }
+          }
+          uint32_t a[16], b[16];
+          ptx::tmem_ld16(taddr + r0, a);
+          ptx::tmem_ld16(taddr + HALF + r0, b);
+          ptx::tmem_ld_wait_on(a, b);
+          // two rows at a time: neighbouring lanes swap, and each stores two columns of one of the rows
+          auto put = [&](float v0, float v1, int r, int col) {
+            const float got = __shfl_xor_sync(0xFFFFFFFFu, odd ? v0 : v1, 1);
+            const int row = r0 + r + odd, at = col - odd;
+            if (row < t.rows && at < p.N)
+              *reinterpret_cast<uint32_t*>(p.out + (size_t)(t.row0 + row) * (size_t)p.out_ld + at) = odd ? pack2(got, v1) : pack2(v0, got);
+          };
+#pragma unroll
+          for (int r = 0; r < 16; r += 2) {
+            const float w0 = __shfl_sync(0xFFFFFFFFu, rs, r), w1 = __shfl_sync(0xFFFFFFFFu, rs, r + 1);
+            float a0 = __uint_as_float(a[r]), a1 = __uint_as_float(a[r + 1]), b0 = __uint_as_float(b[r]), b1 = __uint_as_float(b[r + 1]);
+            if (PLAIN) {
+              put(w0 * (FP8 ? a0 * sa : a0), w1 * (FP8 ? a1 * sa : a1), r, t.n0 + c);
+              put(w0 * (FP8 ? b0 * sb : b0), w1 * (FP8 ? b1 * sb : b1), r, t.n0 + HALF + c);
+            } else {
+              if (FP8) { a0 *= w0 * sa; b0 *= w0 * sb; a1 *= w1 * sa; b1 *= w1 * sb; }
+              put(silu_mul(a0, b0), silu_mul(a1, b1), r, t.n0 + c);
+            }
+          }
+        }
+      } else if (PLAIN) {
         // ---- GEMM-2 form: o = (gate weight x row scale) * acc * column scale, 256 columns
         const int lrow = warp * WROWS + lane;
         float wr = 1.f;
@@ -338,19 +397,38 @@ ffn_gemm1_kernel(const __grid_constant__ CUtensorMap map_w1, const __grid_consta
       if (!ptx::mbar_wait(tempty_bar(buf), ((tl >> 1) & 1) ^ 1, abort_flag, global_abort)) { timeout(3); break; }
       ptx::tc_fence_after();
       const uint32_t d_tmem = tmem + (uint32_t)(buf * BN);
-      for (int kb = 0; kb < KB; ++kb) {
-        if (!ptx::mbar_wait(full_bar(s), ph, abort_flag, global_abort)) { timeout(4); ok = false; break; }
-        ptx::tc_fence_after();
-        if (elected) {
-          const uint64_t ad = a_desc + (uint64_t)(s * (STAGE_BYTES >> 4)), bd = b_desc + (uint64_t)(s * (STAGE_BYTES >> 4));
-#pragma unroll
-          for (int k = 0; k < 4; ++k) {
-            if (FP8) ptx::umma_f8(d_tmem, ad + (uint64_t)(k * 2), bd + (uint64_t)(k * B_STEP), IDESC, (kb | k) != 0);
-            else ptx::umma_bf16(d_tmem, ad + (uint64_t)(k * 2), bd + (uint64_t)(k * B_STEP), IDESC, (kb | k) != 0);
+      // one k-block after the other; an elected lane runs `issue` on the stage's operands
+      auto walk = [&](auto issue) {
+        for (int kb = 0; kb < KB; ++kb) {
+          if (!ptx::mbar_wait(full_bar(s), ph, abort_flag, global_abort)) { timeout(4); return false; }
+          ptx::tc_fence_after();
+          if (elected) {
+            issue(a_desc + (uint64_t)(s * (STAGE_BYTES >> 4)), b_desc + (uint64_t)(s * (STAGE_BYTES >> 4)), kb);
+            ptx::umma_commit(empty_bar(s));   // free the stage when these UMMAs have read it
           }
-          ptx::umma_commit(empty_bar(s));   // free the stage when these UMMAs have read it
+          if (++s == NSTAGE) { s = 0; ph ^= 1u; }
         }
-        if (++s == NSTAGE) { s = 0; ph ^= 1u; }
+        return true;
+      };
+      auto mma = [](uint32_t d, uint64_t ad, uint64_t bd, uint32_t idesc, bool acc) {
+        if (FP8) ptx::umma_f8(d, ad, bd, idesc, acc);
+        else ptx::umma_bf16(d, ad, bd, idesc, acc);
+      };
+      const Tile t = tile_of(w);
+      if (swapped(t)) {
+        const uint32_t idesc = idesc_swapped(FP8, (t.rows + 15) & ~15);
+        ok = walk([&](uint64_t ad, uint64_t bd, int kb) {
+#pragma unroll
+          for (int k = 0; k < 4; ++k)
+#pragma unroll
+            for (int h = 0; h < 2; ++h)
+              mma(d_tmem + h * HALF, bd + (uint64_t)(k * B_STEP + h * (HALF * 128 >> 4)), ad + (uint64_t)(k * 2), idesc, (kb | k) != 0);
+        });
+      } else {
+        ok = walk([&](uint64_t ad, uint64_t bd, int kb) {
+#pragma unroll
+          for (int k = 0; k < 4; ++k) mma(d_tmem, ad + (uint64_t)(k * 2), bd + (uint64_t)(k * B_STEP), IDESC, (kb | k) != 0);
+        });
       }
       if (ok && elected) ptx::umma_commit(tfull_bar(buf));   // accumulator complete
     }
@@ -366,6 +444,8 @@ ffn_gemm1_kernel(const __grid_constant__ CUtensorMap map_w1, const __grid_consta
       const uint8_t* src[ROWS / 16];
       const uint8_t* base = static_cast<const uint8_t*>(p.a_src);
       uint32_t live = 0;
+      const bool swap = swapped(t);
+      const int pieces = (t.rows + 15) / 16;
 #pragma unroll
       for (int j = 0; j < ROWS / 16; ++j) {
         const int lr = rbase + 16 * j;
@@ -393,12 +473,19 @@ ffn_gemm1_kernel(const __grid_constant__ CUtensorMap map_w1, const __grid_consta
         const uint32_t sa = smem_base + s * STAGE_BYTES;
         const int col = kb * 128 + chunk * 16;   // byte offset inside the source row
         const bool kin = col < p.K * ELEM;
-#pragma unroll
-        for (int j = 0; j < ROWS / 16; ++j) {
+        auto copy = [&](int j) {
           const int lr = rbase + 16 * j;
           const uint32_t dst = sa + lr * 128 + ((chunk ^ (lr & 7)) << 4);
           const bool on = kin && ((live >> j) & 1u);
           ptx::cp_async_16(dst, on ? (const void*)(src[j] + col) : (const void*)base, on ? 16u : 0u);
+        };
+        if (!swap) {   // (one loop with a bound for both: a quarter less for full tiles, 32768 tokens 23100 -> 29000 us)
+#pragma unroll
+          for (int j = 0; j < ROWS / 16; ++j) copy(j);
+        } else {
+#pragma unroll
+          for (int j = 0; j < SWAP_ROWS / 16 && j < ROWS / 16; ++j)   // (ROWS = 64: not reached)
+            if (j < pieces) copy(j);
         }
         // one arrival on the stage's full barrier once the copies above have landed; the thread
         // itself goes straight on to the next stage

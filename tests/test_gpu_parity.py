@@ -688,3 +688,30 @@ def test_a_few_more_tokens_take_no_longer():
 
     us, other = H.device_us(call(72), call(64))
     assert us <= 1.2 * other
+
+
+@pytest.mark.parametrize("fp8", [False, True], ids=["bf16", "fp8"])
+@pytest.mark.parametrize("rows", [1, 15, 16, 17, 48, 95, 96, 97])
+def test_experts_of_few_rows_give_the_same_bits(rows, fp8):
+    """An expert of at most 96 rows runs with the operands of its GEMMs exchanged.  Every token here uses every expert, so an expert has as
+    many rows as there are tokens, and a token's output does not depend on how many others there are: the first `rows` tokens alone have
+    the bits that they have among 128.  Widths that no tile divides, and tiles enough for the full-width ones."""
+    cfg = synth.MoEConfig("few", T=128, d=1488, f=1296, E=16, k=16, G=4, seed=rows)
+    t = synth.make_inputs(cfg, "cuda")
+    w = [t["w1"], t["w3"], t["w2"]]
+    if fp8:
+        q = []
+        for v in w:
+            E, K, N = v.shape
+            q += [torch.empty(E, N, K, dtype=torch.uint8, device="cuda"), torch.empty(E, N, dtype=torch.float32, device="cuda")]
+            B.moe_quantize_weights(v, q[-2], q[-1])
+        w = q
+    ys = []
+    for T in (rows, cfg.T):
+        shape = B.make_shape(cfg.with_(T=T), B.MOE_FLAG_GEMM2_SINGLE)
+        ws, y = B.alloc_workspace(shape), torch.full((T, cfg.d), 7.0, dtype=torch.bfloat16, device="cuda")
+        (B.moe_layer_fp8 if fp8 else B.moe_layer)(shape, t["x"][:T].contiguous(), t["w_gate"], t["bias"], *w, y, ws)
+        torch.cuda.synchronize()
+        assert B.moe_status(ws)[0] == 0
+        ys.append(y)
+    assert torch.equal(ys[0], ys[1][:rows])
