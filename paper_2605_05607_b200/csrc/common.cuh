@@ -24,7 +24,7 @@ __device__ __forceinline__ void report_error(int32_t* status, int code, int wher
 }
 
 // ---- programmatic dependent launch ------------------------------------------------------------
-// Every kernel of the library is launched with programmatic stream serialisation and starts with
+// Every kernel of the library (but long runs of GEMM-1) is launched with programmatic stream serialisation and starts with
 // grid_dependency_sync(): set-up that touches no global data (barrier init, TMEM allocation,
 // tensor-map prefetch) may run while the previous kernel of the stream drains; nothing is read
 // from or written to global memory before the previous kernel has completed and flushed, so
@@ -37,8 +37,9 @@ __device__ __forceinline__ void grid_dependency_sync() {
 
 extern std::atomic<long long> g_launches;   // kernels launched since the library was loaded (api.cu)
 
+// overlap = false: the kernel starts when the previous one has drained (plain stream order)
 template <typename... KArgs, typename... Args>
-cudaError_t launch_pdl_cluster(unsigned cluster, void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t st,
+cudaError_t launch_kernel(bool overlap, unsigned cluster, void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t st,
                                Args&&... args) {
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = grid;
@@ -47,7 +48,7 @@ cudaError_t launch_pdl_cluster(unsigned cluster, void (*kernel)(KArgs...), dim3 
   cfg.stream = st;
   cudaLaunchAttribute attr[2];
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  attr[0].val.programmaticStreamSerializationAllowed = overlap ? 1 : 0;
   attr[1].id = cudaLaunchAttributeClusterDimension;
   attr[1].val.clusterDim.x = cluster;
   attr[1].val.clusterDim.y = 1;
@@ -56,6 +57,11 @@ cudaError_t launch_pdl_cluster(unsigned cluster, void (*kernel)(KArgs...), dim3 
   cfg.numAttrs = cluster > 0 ? 2 : 1;
   g_launches.fetch_add(1, std::memory_order_relaxed);
   return cudaLaunchKernelEx(&cfg, kernel, KArgs(std::forward<Args>(args))...);
+}
+template <typename... KArgs, typename... Args>
+cudaError_t launch_pdl_cluster(unsigned cluster, void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t st,
+                               Args&&... args) {
+  return launch_kernel(true, cluster, kernel, grid, block, smem, st, std::forward<Args>(args)...);
 }
 template <typename... KArgs, typename... Args>
 cudaError_t launch_pdl(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, Args&&... args) {

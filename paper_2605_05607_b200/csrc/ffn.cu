@@ -274,7 +274,7 @@ cudaError_t launch_expert_ffn(const Shape& s, const FfnArgs& a, cudaStream_t st)
     g1.tile_prefix = a.mp_prefix;
     err = ffn::launch_gemm1_pair(g1, m_w1, m_w3, st);
   } else {
-    err = ffn::launch_gemm1(g1, m_w1, m_w3, false, narrow_gemm1(s, false), few_rows(s), st);
+    err = ffn::launch_gemm1(g1, m_w1, m_w3, P, false, narrow_gemm1(s, false), few_rows(s), st);
   }
   if (err != cudaSuccess) return err;
 
@@ -333,7 +333,7 @@ cudaError_t launch_expert_ffn_fp8(const Shape& s, const FfnArgs& a, const Fp8Arg
   g1.a_scale = q.sx;
   g1.b_scale = q.s1;
   g1.b_scale2 = q.s3;
-  cudaError_t err = ffn::launch_gemm1(g1, m_w1, m_w3, true, narrow1, few_rows(s), st);
+  cudaError_t err = ffn::launch_gemm1(g1, m_w1, m_w3, P, true, narrow1, few_rows(s), st);
   if (err != cudaSuccess) return err;
   if ((err = launch_quantize_rows(a.h, P, s.f, q.hq, q.sh, st)) != cudaSuccess) return err;
 

@@ -177,7 +177,7 @@ cudaError_t launch_wgrad_pair(const CUtensorMap& m_a, const CUtensorMap& m_b, co
 
 // fp8 = false: bf16 operands, weights [E, K, N] (B MN-major).  fp8 = true: E4M3 operands, weights
 // [E, N, K] (B K-major), 128 elements of K per pipeline stage, scales applied in the epilogue.
-cudaError_t launch_gemm1(GemmParams p, const CUtensorMap& m_w1, const CUtensorMap& m_w3, bool fp8, bool narrow, bool few,
+cudaError_t launch_gemm1(GemmParams p, const CUtensorMap& m_w1, const CUtensorMap& m_w3, long long rows, bool fp8, bool narrow, bool few,
                          cudaStream_t st);
 cudaError_t launch_gemm2(const GemmParams& p, const CUtensorMap& m_w2, bool fp8, cudaStream_t st);
 cudaError_t launch_gemm1_pair(const GemmParams& p, const CUtensorMap& m_w1, const CUtensorMap& m_w3, cudaStream_t st);

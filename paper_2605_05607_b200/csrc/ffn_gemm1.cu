@@ -513,7 +513,7 @@ ffn_gemm1_kernel(const __grid_constant__ CUtensorMap map_w1, const __grid_consta
 
 namespace {
 template <bool FP8, bool PLAIN, bool NARROW, bool FEW>
-cudaError_t launch_form(const GemmParams& p, const CUtensorMap& m_a, const CUtensorMap& m_b, cudaStream_t st) {
+cudaError_t launch_form(const GemmParams& p, const CUtensorMap& m_a, const CUtensorMap& m_b, bool overlap, cudaStream_t st) {
   // per device; several host threads may get here at once: setting the attribute twice is harmless
   static std::atomic<bool> attr_set[MAX_DEVICES];
   const int dev = current_device();
@@ -524,29 +524,40 @@ cudaError_t launch_form(const GemmParams& p, const CUtensorMap& m_a, const CUten
     attr_set[dev].store(true, std::memory_order_release);
   }
   ProfileScope prof(PLAIN ? KID_GEMM2 : KID_GEMM1, st);
-  return launch_pdl(kernel, sm_count(), THREADS, SMEM_BYTES, st, m_a, m_b, p);
+  return launch_kernel(overlap, 0, kernel, sm_count(), THREADS, SMEM_BYTES, st, m_a, m_b, p);
 }
 
 template <bool FP8, bool PLAIN>
-cudaError_t launch_width(const GemmParams& p, const CUtensorMap& m_a, const CUtensorMap& m_b, bool narrow, bool few, cudaStream_t st) {
-  if (!narrow) return launch_form<FP8, PLAIN, false, false>(p, m_a, m_b, st);
-  return few ? launch_form<FP8, PLAIN, true, true>(p, m_a, m_b, st) : launch_form<FP8, PLAIN, true, false>(p, m_a, m_b, st);
+cudaError_t launch_width(const GemmParams& p, const CUtensorMap& m_a, const CUtensorMap& m_b, bool narrow, bool few, bool overlap,
+                         cudaStream_t st) {
+  if (!narrow) return launch_form<FP8, PLAIN, false, false>(p, m_a, m_b, overlap, st);
+  return few ? launch_form<FP8, PLAIN, true, true>(p, m_a, m_b, overlap, st) : launch_form<FP8, PLAIN, true, false>(p, m_a, m_b, overlap, st);
 }
 }  // namespace
 
 // narrow: 64 output columns per tile instead of 128 (GEMM-1) or 256 (GEMM-2); p.n_tiles is set here.  The FP8 weight maps then
 // have boxes of 64 columns (make_weight_map_fp8).  few: no expert has more than 64 rows (used by narrow tiles only).
-cudaError_t launch_gemm1(GemmParams p, const CUtensorMap& m_w1, const CUtensorMap& m_w3, bool fp8, bool narrow, bool few,
+//
+// rows: pairs of the layer.  A long GEMM starts when the kernel before it has drained, so that its thread blocks are placed on an
+// empty GPU: neighbours, which share a weight tile, then sit in the same GPC, and the tile reaches it once.  Placed one by one as
+// SMs become free they are scattered, and the GEMM spends more of the board's power on moving operands.  Layers, overlapped / drained, us:
+// 32768 tokens, top-8 of 256 x 7168 x 2048 22750 / 21620; 16384 skewed 12970 / 12570; 8192 top-4 of 64 x 7168 x 4096 in 8 bits
+// 3490 / 3310; 16384 top-4 of 32 x 2048 x 2048 1581 / 1563; 2048 top-4 of 32 x 4096 x 4096 (2^37 products per matrix) 1072 / 1072;
+// 4096 skewed, top-8 of 32 x 2048 x 1024 (2^36) 465 / 467.
+cudaError_t launch_gemm1(GemmParams p, const CUtensorMap& m_w1, const CUtensorMap& m_w3, long long rows, bool fp8, bool narrow, bool few,
                          cudaStream_t st) {
   p.n_tiles = narrow ? (p.N + 63) / 64 : (p.N + 127) / 128;
-  return fp8 ? launch_width<true, false>(p, m_w1, m_w3, narrow, few, st) : launch_width<false, false>(p, m_w1, m_w3, narrow, few, st);
+  const bool overlap = (double)rows * p.K * p.N <= 137438953472.;   // 2^37
+  return fp8 ? launch_width<true, false>(p, m_w1, m_w3, narrow, few, overlap, st)
+             : launch_width<false, false>(p, m_w1, m_w3, narrow, few, overlap, st);
 }
 
 // GEMM-2 through the single-CTA kernel (128-row tiles): p.a_src = h (or its E4M3 copy), p.a_ld = f,
 // p.tile_prefix = the 128-row tile prefix; m_w2 is the weight map.
 cudaError_t launch_gemm2_single(GemmParams p, const CUtensorMap& m_w2, bool fp8, bool narrow, bool few, cudaStream_t st) {
   p.n_tiles = narrow ? (p.N + 63) / 64 : (p.N + 255) / 256;
-  return fp8 ? launch_width<true, true>(p, m_w2, m_w2, narrow, few, st) : launch_width<false, true>(p, m_w2, m_w2, narrow, few, st);
+  return fp8 ? launch_width<true, true>(p, m_w2, m_w2, narrow, few, true, st)
+             : launch_width<false, true>(p, m_w2, m_w2, narrow, few, true, st);
 }
 
 }  // namespace ffn
