@@ -142,7 +142,7 @@ cudaError_t launch_layer_backward(const Shape& s, const BwdArgs& a, cudaStream_t
     if ((err = cudaMemsetAsync(a.dw3, 0, n13, st)) != cudaSuccess) return err;
     return cudaMemsetAsync(a.dw2, 0, n13, st);
   }
-  const long long R = (long long)bwd_row_capacity(s);
+  const long long R = (long long)bwd_row_capacity(s), P = (long long)s.T * s.k;
   const int vec = s.d / 8;
   cudaError_t err;
   if ((err = launch_pdl(bwd_offsets_kernel, 1, 1024, 0, st, a.L.expert_counts, a.poff, a.mt_prefix, a.mp_prefix, s.E)) != cudaSuccess)
@@ -207,7 +207,7 @@ cudaError_t launch_layer_backward(const Shape& s, const BwdArgs& a, cudaStream_t
     if ((err = ffn::launch_bwd_glu(r, m_w1, m_w3, st)) != cudaSuccess) return err;
   }
   // dW2[e] = H^T . dO
-  if ((err = ffn::launch_wgrad_pair(r_h, r_do, a.poff, a.dw2, s.E, s.f, s.d, a.status, st)) != cudaSuccess) return err;
+  if ((err = ffn::launch_wgrad_pair(r_h, r_do, a.poff, P, a.dw2, s.E, s.f, s.d, a.status, st)) != cudaSuccess) return err;
   // dXs = dA1 . W1^T + dA3 . W3^T : [R, f] x [f, d], twice into one accumulator
   ffn::GemmParams q{};
   q.out = static_cast<__nv_bfloat16*>(a.dxs);
@@ -235,8 +235,8 @@ cudaError_t launch_layer_backward(const Shape& s, const BwdArgs& a, cudaStream_t
   if ((err = launch_combine_rows(sc, a.dxs, Lp, a.topk_idx, nullptr, nullptr, a.dx, (int)R, a.status, st)) != cudaSuccess)
     return err;
   // dW1[e] = Xs^T . dA1,  dW3[e] = Xs^T . dA3
-  if ((err = ffn::launch_wgrad_pair(r_xs, r_da1, a.poff, a.dw1, s.E, s.d, s.f, a.status, st)) != cudaSuccess) return err;
-  return ffn::launch_wgrad_pair(r_xs, r_da3, a.poff, a.dw3, s.E, s.d, s.f, a.status, st);
+  if ((err = ffn::launch_wgrad_pair(r_xs, r_da1, a.poff, P, a.dw1, s.E, s.d, s.f, a.status, st)) != cudaSuccess) return err;
+  return ffn::launch_wgrad_pair(r_xs, r_da3, a.poff, P, a.dw3, s.E, s.d, s.f, a.status, st);
 }
 
 }  // namespace tcmoe

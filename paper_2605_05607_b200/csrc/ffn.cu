@@ -128,6 +128,14 @@ bool make_rows_map_mn(CUtensorMap* map, const void* base, long long rows, int co
   return encode_tiled(map, false, 2, base, dims, strides, box);
 }
 
+// bf16 [E, rows, cols] as the target of TMA stores: box = 64 columns x 128 rows x 1
+bool make_store_map(CUtensorMap* map, const void* base, int E, int rows, int cols) {
+  cuuint64_t dims[3] = {(cuuint64_t)cols, (cuuint64_t)rows, (cuuint64_t)E};
+  cuuint64_t strides[2] = {(cuuint64_t)cols * 2, (cuuint64_t)cols * rows * 2};
+  cuuint32_t box[3] = {64, BM, 1};
+  return encode_tiled(map, false, 3, base, dims, strides, box);
+}
+
 }  // namespace ffn
 
 using ffn::make_weight_map;

@@ -172,8 +172,9 @@ bool make_act_map(CUtensorMap* map, const void* base, long long rows, int K, boo
 bool make_weight_map_fp8(CUtensorMap* map, const void* base, int E, int N, int K, int box_cols = 128);
 bool make_weight_map_kmajor(CUtensorMap* map, const void* base, int E, int rows, int cols);
 bool make_rows_map_mn(CUtensorMap* map, const void* base, long long rows, int cols);
-cudaError_t launch_wgrad_pair(const CUtensorMap& m_a, const CUtensorMap& m_b, const int32_t* poff, void* dw, int E, int M,
-                              int N, int32_t* status, cudaStream_t st);
+bool make_store_map(CUtensorMap* map, const void* base, int E, int rows, int cols);
+cudaError_t launch_wgrad_pair(const CUtensorMap& m_a, const CUtensorMap& m_b, const int32_t* poff, long long rows_total, void* dw, int E,
+                              int M, int N, int32_t* status, cudaStream_t st);
 
 // fp8 = false: bf16 operands, weights [E, K, N] (B MN-major).  fp8 = true: E4M3 operands, weights
 // [E, N, K] (B K-major), 128 elements of K per pipeline stage, scales applied in the epilogue.

@@ -45,6 +45,7 @@ constexpr int A_BYTES = BM * BK * 2;            // 16 KiB: this CTA's 128 rows
 constexpr int B_BYTES = (UMMA_N / 2) * BK * 2;  // 16 KiB: this CTA's half of the B tile (two 64-column slabs)
 constexpr int STAGE_BYTES = A_BYTES + B_BYTES;
 constexpr int NUM_BARS = 2 * NSTAGE + 4;
+constexpr int BOX_BYTES = 64 * BM * 2;          // 64 columns x 128 rows of bf16: what a weight gradient stores by TMA at once
 constexpr int EPI_WARPS = 8, TMA_WARP = EPI_WARPS, MMA_WARP = EPI_WARPS + 1;
 constexpr int STAGE_OUT_WARP = 32 * 64;           // epilogue transpose buffer of one warp: 32 rows x 32 columns, swizzled
 constexpr int TABLE_BYTES = (2 * (MAX_E + 1) * 4 + 15) & ~15;
@@ -76,6 +77,7 @@ constexpr uint32_t HINT = 4000;   // try_wait suspend-time hint (ns), see ptx::m
 //                 256 x 256 tile of one expert's gradient (p.K = its row count M, p.N its columns), the K walk runs over
 //                 the expert's rows in blocks of 64, both operands are MN-major boxes of 64 columns x 64 rows; CTA `rank`
 //                 holds rows m0 + 128 * rank of the tile and columns n0 + 128 * rank of B
+//                 TILE_OUT: the tile goes through shared memory and leaves by TMA (map_b1: dW), instead of warp by warp.
 //   PAIR_KSPLIT   acc = A0 . B0 + A1 . B1 (dX = dA1 . W1^T + dA3 . W3^T): the first p.k_split k-blocks come from
 //                 (rows.a0, map_b0), the rest from (rows.a1, map_b1); plain epilogue
 // BKMAJ: the bf16 weight operand is read K-major (one box of 128 columns x 64 K per CTA and stage), which is how
@@ -88,12 +90,15 @@ enum { PAIR_PLAIN = 0, PAIR_GLU = 1, PAIR_GLU_BWD = 2, PAIR_KSPLIT = 3, PAIR_WGR
 // the padded UMMAs themselves are the bound.
 struct RowMaps { CUtensorMap a0[4], a1[4]; };
 
-template <bool RED, bool FP8, int MODE, bool BKMAJ>
+template <bool RED, bool FP8, int MODE, bool BKMAJ, bool TILE_OUT>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(THREADS, 1)
 ffn_gemm2_kernel(const __grid_constant__ CUtensorMap map_b0, const __grid_constant__ CUtensorMap map_b1,
                  const __grid_constant__ RowMaps rows, const GemmParams p) {
   constexpr bool GLU = MODE == PAIR_GLU || MODE == PAIR_GLU_BWD;
   constexpr bool KMAJ = FP8 || BKMAJ;   // the weight operand is K-major in shared memory
+  constexpr int NST = TILE_OUT ? NSTAGE - 2 : NSTAGE;   // the last two stages hold the tile on its way out
+  static_assert(!TILE_OUT || MODE == PAIR_WGRAD, "whole tiles leave by TMA in the weight gradients only");
+  static_assert(4 * BOX_BYTES <= 2 * STAGE_BYTES, "the CTA's part of a tile");
   static_assert(!(MODE != PAIR_PLAIN && (RED || FP8)), "only the plain form has the reducing / FP8 variants");
   constexpr int BN_OUT = GLU ? 128 : 256;
   extern __shared__ uint8_t smem_raw[];
@@ -118,7 +123,7 @@ ffn_gemm2_kernel(const __grid_constant__ CUtensorMap map_b0, const __grid_consta
   const int cluster_id = blockIdx.x >> 1, num_clusters = gridDim.x >> 1;
 
   if (threadIdx.x == 0) {
-    for (int s = 0; s < NSTAGE; ++s) {
+    for (int s = 0; s < NST; ++s) {
       ptx::mbar_init(full_bar(s), 1);       // leader TMA thread (expect_tx for both CTAs)
       ptx::mbar_init(empty_bar(s), 1);      // tcgen05.commit
     }
@@ -374,42 +379,40 @@ ffn_gemm2_kernel(const __grid_constant__ CUtensorMap map_b0, const __grid_consta
             }
           }
         }
-      } else if (WGRAD && (p.N & 15) != 0) {
-        // Rows that start inside a 32-byte sector: a segment's first and last sector are written in two pieces, which costs a gradient
-        // of mostly empty experts more than the stores themselves.  128-byte segments have half as many ends: 64 columns of 16 rows at a
-        // time (backward of 7 tokens top-6 of 64 experts, 4104 x 1544: 1404 -> 1150 us, 2656 x 1608: 810 -> 647).
-#pragma unroll 1
-        for (int c = 0; c < chunks; c += 2) {
+      } else if (TILE_OUT) {
+        // The CTA's 128 x 256 part of the tile through shared memory, four boxes of 64 columns in the layout of a 128-byte swizzle, and
+        // out by TMA, which clips at the edges of dW[e].
+        const uint32_t dst = smem_base + NST * STAGE_BYTES + (quarter * 32 + lane) * 128;
+#pragma unroll
+        for (int c = 0; c < 2; ++c) {
           uint32_t lo[32], hi[32];
-          ptx::tmem_ld32(taddr + c * 32, lo);
-          ptx::tmem_ld32(taddr + c * 32 + 32, hi);
+          ptx::tmem_ld32(taddr + c * 64, lo);
+          ptx::tmem_ld32(taddr + c * 64 + 32, hi);
+          if (c == 0) {   // the stores of the last tile have read theirs
+            if (threadIdx.x == 0) ptx::bulk_wait_read();
+            ptx::named_barrier(1, EPI_WARPS * 32);
+          }
           ptx::tmem_ld_wait_on(lo, hi);
-          uint32_t q[32];   // (an expert without rows: the accumulator was never written)
+          if (t.kb == 0) {   // an expert without rows: the accumulator was never written
 #pragma unroll
-          for (int j = 0; j < 16; ++j) {
-            q[j] = t.kb == 0 ? 0u : pack2(__uint_as_float(lo[2 * j]), __uint_as_float(lo[2 * j + 1]));
-            q[16 + j] = t.kb == 0 ? 0u : pack2(__uint_as_float(hi[2 * j]), __uint_as_float(hi[2 * j + 1]));
+            for (int j = 0; j < 32; ++j) lo[j] = hi[j] = 0u;
           }
-          const int col = col0 + c * 32 + (lane & 7) * 8;
 #pragma unroll
-          for (int h = 0; h < 2; ++h) {
-            if (lane >> 4 == h) {
-#pragma unroll
-              for (int v = 0; v < 8; ++v)
-                ptx::st_shared_v4(stage + (lane & 15) * 128 + ((v ^ (lane & 7)) << 4), q[v * 4], q[v * 4 + 1], q[v * 4 + 2], q[v * 4 + 3]);
-            }
-            __syncwarp();
-            if (col < p.N) {
-#pragma unroll
-              for (int i = 0; i < 4; ++i) {
-                const int r = i * 4 + (lane >> 3), row = row_w + h * 16 + r;
-                if (row < t.rows)
-                  *reinterpret_cast<uint4*>(p.out + (size_t)(t.out_row0 + row) * (size_t)p.out_ld + col) =
-                      ptx::ld_shared_v4(stage + r * 128 + (((lane & 7) ^ (r & 7)) << 4));
-              }
-            }
-            __syncwarp();
+          for (int v = 0; v < 8; ++v) {
+            const uint32_t* q = v < 4 ? lo + v * 8 : hi + (v - 4) * 8;
+            ptx::st_shared_v4(dst + (half * 2 + c) * BOX_BYTES + ((v ^ (lane & 7)) << 4), pack2(__uint_as_float(q[0]), __uint_as_float(q[1])),
+                              pack2(__uint_as_float(q[2]), __uint_as_float(q[3])), pack2(__uint_as_float(q[4]), __uint_as_float(q[5])),
+                              pack2(__uint_as_float(q[6]), __uint_as_float(q[7])));
           }
+        }
+        ptx::fence_proxy_async_smem();
+        ptx::named_barrier(1, EPI_WARPS * 32);
+        if (threadIdx.x == 0 && t.rows > 0) {
+#pragma unroll
+          for (int c = 0; c < 4; ++c)
+            if (t.n0 + c * 64 < p.N)
+              ptx::tma_store_3d(&map_b1, smem_base + NST * STAGE_BYTES + c * BOX_BYTES, t.n0 + c * 64, t.out_row0 - t.e * p.K, t.e);
+          ptx::bulk_commit();
         }
       } else {
 #pragma unroll 1
@@ -442,6 +445,7 @@ ffn_gemm2_kernel(const __grid_constant__ CUtensorMap map_b0, const __grid_consta
       // (K = 512: 860 -> 1049 TFLOP/s with the relaxed form)
       if (lane == 0) ptx::mbar_arrive_cluster_relaxed(ptx::mapa(tempty_bar(buf), 0));
     }
+    if (TILE_OUT && threadIdx.x == 0) ptx::bulk_wait();
   } else if (warp == TMA_WARP) {
     // ================================ TMA producer (both CTAs) ================================
     if (lane == 0) {
@@ -456,8 +460,8 @@ ffn_gemm2_kernel(const __grid_constant__ CUtensorMap map_b0, const __grid_consta
         const int mine = WGRAD ? 4 : blocks32(t.left - rank * cta_rows);
         const uint32_t bytes = 2 * B_BYTES + (WGRAD ? 8 : blocks32(t.left) + blocks32(t.left - cta_rows)) * (A_BYTES / 4);
         for (int kb = 0; kb < KBt; ++kb, ++it) {
-          const int s = it % NSTAGE;
-          if (!ptx::mbar_wait<false, HINT>(empty_bar(s), ((it / NSTAGE) & 1) ^ 1, abort_flag, global_abort)) {
+          const int s = it % NST;
+          if (!ptx::mbar_wait<false, HINT>(empty_bar(s), ((it / NST) & 1) ^ 1, abort_flag, global_abort)) {
             timeout(2); ok = false; break;
           }
           const uint32_t sa = smem_base + s * STAGE_BYTES, sb = sa + A_BYTES;
@@ -525,7 +529,7 @@ ffn_gemm2_kernel(const __grid_constant__ CUtensorMap map_b0, const __grid_consta
             }
             ptx::umma_commit_both(empty_bar(s));   // free the stage in both CTAs once these UMMAs have read it
           }
-          if (++s == NSTAGE) { s = 0; ph ^= 1u; }
+          if (++s == NST) { s = 0; ph ^= 1u; }
         }
         if (ok && elected) ptx::umma_commit_both(tfull_bar(buf));   // accumulator complete, both halves
       }
@@ -563,7 +567,7 @@ int pair_grid() {
     attr.val.clusterDim.z = 1;
     cfg.attrs = &attr;
     cfg.numAttrs = 1;
-    if (cudaOccupancyMaxActiveClusters(&clusters, ffn_gemm2_kernel<false, false, PAIR_PLAIN, false>, &cfg) != cudaSuccess || clusters <= 0) {
+    if (cudaOccupancyMaxActiveClusters(&clusters, ffn_gemm2_kernel<false, false, PAIR_PLAIN, false, false>, &cfg) != cudaSuccess || clusters <= 0) {
       (void)cudaGetLastError();
       clusters = sm_count() / 2;
     }
@@ -582,15 +586,16 @@ cudaError_t set_pair_attributes() {
   const int dev = current_device();
   if (!attr_set[dev].load(std::memory_order_acquire)) {
     const auto attr = cudaFuncAttributeMaxDynamicSharedMemorySize;
-    cudaError_t e = cudaFuncSetAttribute(ffn_gemm2_kernel<false, false, PAIR_PLAIN, false>, attr, SMEM_BYTES);
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(ffn_gemm2_kernel<true, false, PAIR_PLAIN, false>, attr, SMEM_BYTES);
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(ffn_gemm2_kernel<false, true, PAIR_PLAIN, false>, attr, SMEM_BYTES);
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(ffn_gemm2_kernel<true, true, PAIR_PLAIN, false>, attr, SMEM_BYTES);
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(ffn_gemm2_kernel<false, false, PAIR_GLU, false>, attr, SMEM_BYTES);
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(ffn_gemm2_kernel<false, false, PAIR_PLAIN, true>, attr, SMEM_BYTES);
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(ffn_gemm2_kernel<false, false, PAIR_GLU_BWD, false>, attr, SMEM_BYTES);
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(ffn_gemm2_kernel<false, false, PAIR_KSPLIT, true>, attr, SMEM_BYTES);
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(ffn_gemm2_kernel<false, false, PAIR_WGRAD, false>, attr, SMEM_BYTES);
+    cudaError_t e = cudaFuncSetAttribute(ffn_gemm2_kernel<false, false, PAIR_PLAIN, false, false>, attr, SMEM_BYTES);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(ffn_gemm2_kernel<true, false, PAIR_PLAIN, false, false>, attr, SMEM_BYTES);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(ffn_gemm2_kernel<false, true, PAIR_PLAIN, false, false>, attr, SMEM_BYTES);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(ffn_gemm2_kernel<true, true, PAIR_PLAIN, false, false>, attr, SMEM_BYTES);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(ffn_gemm2_kernel<false, false, PAIR_GLU, false, false>, attr, SMEM_BYTES);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(ffn_gemm2_kernel<false, false, PAIR_PLAIN, true, false>, attr, SMEM_BYTES);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(ffn_gemm2_kernel<false, false, PAIR_GLU_BWD, false, false>, attr, SMEM_BYTES);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(ffn_gemm2_kernel<false, false, PAIR_KSPLIT, true, false>, attr, SMEM_BYTES);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(ffn_gemm2_kernel<false, false, PAIR_WGRAD, false, false>, attr, SMEM_BYTES);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(ffn_gemm2_kernel<false, false, PAIR_WGRAD, false, true>, attr, SMEM_BYTES);
     if (e != cudaSuccess) return e;
     attr_set[dev].store(true, std::memory_order_release);
   }
@@ -616,11 +621,11 @@ cudaError_t launch_gemm2(const GemmParams& p, const CUtensorMap& m_w2, bool fp8,
   const bool red = p.y_acc != nullptr;
   const int g = pair_grid();
   if (fp8) {
-    if (red) return launch_pdl(ffn_gemm2_kernel<true, true, PAIR_PLAIN, false>, g, THREADS, SMEM_BYTES, st, m_w2, m_w2, rows, p);
-    return launch_pdl(ffn_gemm2_kernel<false, true, PAIR_PLAIN, false>, g, THREADS, SMEM_BYTES, st, m_w2, m_w2, rows, p);
+    if (red) return launch_pdl(ffn_gemm2_kernel<true, true, PAIR_PLAIN, false, false>, g, THREADS, SMEM_BYTES, st, m_w2, m_w2, rows, p);
+    return launch_pdl(ffn_gemm2_kernel<false, true, PAIR_PLAIN, false, false>, g, THREADS, SMEM_BYTES, st, m_w2, m_w2, rows, p);
   }
-  if (red) return launch_pdl(ffn_gemm2_kernel<true, false, PAIR_PLAIN, false>, g, THREADS, SMEM_BYTES, st, m_w2, m_w2, rows, p);
-  return launch_pdl(ffn_gemm2_kernel<false, false, PAIR_PLAIN, false>, g, THREADS, SMEM_BYTES, st, m_w2, m_w2, rows, p);
+  if (red) return launch_pdl(ffn_gemm2_kernel<true, false, PAIR_PLAIN, false, false>, g, THREADS, SMEM_BYTES, st, m_w2, m_w2, rows, p);
+  return launch_pdl(ffn_gemm2_kernel<false, false, PAIR_PLAIN, false, false>, g, THREADS, SMEM_BYTES, st, m_w2, m_w2, rows, p);
 }
 
 // GEMM-1 on CTA pairs from the expert-sorted activation rows (p.a_src = xs); p.tile_prefix = the 256-row pair-tile
@@ -631,7 +636,7 @@ cudaError_t launch_gemm1_pair(const GemmParams& p, const CUtensorMap& m_w1, cons
   RowMaps rows{};
   if (!make_row_maps(&rows, p, false)) return cudaErrorInvalidValue;
   ProfileScope prof(KID_GEMM1, st);
-  return launch_pdl(ffn_gemm2_kernel<false, false, PAIR_GLU, false>, pair_grid(), THREADS, SMEM_BYTES, st, m_w1, m_w3, rows, p);
+  return launch_pdl(ffn_gemm2_kernel<false, false, PAIR_GLU, false, false>, pair_grid(), THREADS, SMEM_BYTES, st, m_w1, m_w3, rows, p);
 }
 
 // Backward pass, all on CTA pairs (see bwd.cu for the sequence):
@@ -643,27 +648,27 @@ cudaError_t launch_bwd_dh(const GemmParams& p, const CUtensorMap& m_w2t, cudaStr
   if (e != cudaSuccess) return e;
   RowMaps rows{};
   if (!make_row_maps(&rows, p, false)) return cudaErrorInvalidValue;
-  return launch_pdl(ffn_gemm2_kernel<false, false, PAIR_PLAIN, true>, pair_grid(), THREADS, SMEM_BYTES, st, m_w2t, m_w2t, rows, p);
+  return launch_pdl(ffn_gemm2_kernel<false, false, PAIR_PLAIN, true, false>, pair_grid(), THREADS, SMEM_BYTES, st, m_w2t, m_w2t, rows, p);
 }
 cudaError_t launch_bwd_glu(const GemmParams& p, const CUtensorMap& m_w1, const CUtensorMap& m_w3, cudaStream_t st) {
   cudaError_t e = set_pair_attributes();
   if (e != cudaSuccess) return e;
   RowMaps rows{};
   if (!make_row_maps(&rows, p, false)) return cudaErrorInvalidValue;
-  return launch_pdl(ffn_gemm2_kernel<false, false, PAIR_GLU_BWD, false>, pair_grid(), THREADS, SMEM_BYTES, st, m_w1, m_w3, rows, p);
+  return launch_pdl(ffn_gemm2_kernel<false, false, PAIR_GLU_BWD, false, false>, pair_grid(), THREADS, SMEM_BYTES, st, m_w1, m_w3, rows, p);
 }
 cudaError_t launch_bwd_dx(const GemmParams& p, const CUtensorMap& m_w1t, const CUtensorMap& m_w3t, cudaStream_t st) {
   cudaError_t e = set_pair_attributes();
   if (e != cudaSuccess) return e;
   RowMaps rows{};
   if (!make_row_maps(&rows, p, false)) return cudaErrorInvalidValue;
-  return launch_pdl(ffn_gemm2_kernel<false, false, PAIR_KSPLIT, true>, pair_grid(), THREADS, SMEM_BYTES, st, m_w1t, m_w3t, rows, p);
+  return launch_pdl(ffn_gemm2_kernel<false, false, PAIR_KSPLIT, true, false>, pair_grid(), THREADS, SMEM_BYTES, st, m_w1t, m_w3t, rows, p);
 }
 
 // Weight gradient on CTA pairs: dw[e] = A_e^T . B_e, A = [rows, M], B = [rows, N] in the padded row space (maps with
-// boxes of 64 columns x 64 rows), dw [E, M, N] bf16, fully written.
-cudaError_t launch_wgrad_pair(const CUtensorMap& m_a, const CUtensorMap& m_b, const int32_t* poff, void* dw, int E, int M,
-                              int N, int32_t* status, cudaStream_t st) {
+// boxes of 64 columns x 64 rows; rows_total of them without the padding), dw [E, M, N] bf16, fully written.
+cudaError_t launch_wgrad_pair(const CUtensorMap& m_a, const CUtensorMap& m_b, const int32_t* poff, long long rows_total, void* dw, int E,
+                              int M, int N, int32_t* status, cudaStream_t st) {
   cudaError_t e = set_pair_attributes();
   if (e != cudaSuccess) return e;
   GemmParams p{};
@@ -679,7 +684,19 @@ cudaError_t launch_wgrad_pair(const CUtensorMap& m_a, const CUtensorMap& m_b, co
   RowMaps rows{};
   rows.a0[3] = m_a;
   ProfileScope prof(KID_WGRAD, st);
-  return launch_pdl(ffn_gemm2_kernel<false, false, PAIR_WGRAD, false>, pair_grid(), THREADS, SMEM_BYTES, st, m_b, m_b, rows, p);
+  // Experts of few rows: the gradients are bound by their stores, and by what the stores take of the board's power; whole tiles leave by
+  // TMA then.  It takes two of the ring's stages and a barrier of the epilogue warps, which costs more than it gives where the tensor
+  // cores are the bound.  Ragged rows (they start inside a 32-byte sector) leave that way at any size: in pieces of 64 bytes twice as many
+  // sectors are written in two halves.  Training step, us, warps / TMA, by rows per expert: 94 skewed (128 x 2880 x 2880) 5220 / 5074, 125 (64
+  // x 2048 x 1024) 873 / 857, 125 (16 x 4096 x 4096) 1519 / 1469, 187 skewed (128 x 2880 x 2880) 7329 / 7278, 187 (64 x 2048 x 1024) 1119 / 1123,
+  // 250 (64 x 2048 x 1024) 1196 / 1213, 375 (128 x 2048 x 1024) 3011 / 3059; ragged: 19 (64 x 2888 x 2872) 3057 / 2703, 125 (64 x 2056 x 1032)
+  // 1116 / 1085, 1024 (32 x 2056 x 1032) 2411 / 2377.
+  if (rows_total < 192ll * E || (N & 15) != 0) {
+    CUtensorMap m_dw;
+    if (!make_store_map(&m_dw, dw, E, M, N)) return cudaErrorInvalidValue;
+    return launch_pdl(ffn_gemm2_kernel<false, false, PAIR_WGRAD, false, true>, pair_grid(), THREADS, SMEM_BYTES, st, m_b, m_dw, rows, p);
+  }
+  return launch_pdl(ffn_gemm2_kernel<false, false, PAIR_WGRAD, false, false>, pair_grid(), THREADS, SMEM_BYTES, st, m_b, m_b, rows, p);
 }
 
 }  // namespace ffn

@@ -385,3 +385,25 @@ def test_gradients_of_ragged_rows_take_no_longer():
     # measured, taking turns: 1.13-1.18; stored sector by sector 1.42-1.44.  The line lies in the middle.
     us, other = H.device_us(call(4104, 1544), call(4112, 1552), n=2)
     assert us <= 1.3 * other
+
+
+@pytest.mark.parametrize("d,f", [(16, 144), (256, 512), (272, 528), (400, 1040)])
+def test_weight_gradients_leave_alike_by_tma_and_by_the_warps(d, f):
+    """An average of fewer than 192 rows per expert decides how the tiles of the gradients are stored.  One expert with 191 tokens, and with a
+    192nd whose dy is zero: the same sums (the contraction takes 64 rows at a time, padded with zeros), so the same bits."""
+    grads = []
+    for T in (192, 191):
+        bw = Backward(synth.MoEConfig("rows", T=T, d=d, f=f, E=1, k=1, G=1, seed=d))
+        t = bw.run.t
+        if grads:
+            t["x"].copy_(x[:T])
+            bw.dy.copy_(dy[:T])
+            for n in ("w1", "w3", "w2"):
+                t[n].copy_(w[n])
+        else:
+            bw.dy[191] = 0
+            x, dy, w = t["x"], bw.dy, {n: t[n] for n in ("w1", "w3", "w2")}
+        bw()
+        grads.append((bw.dw1, bw.dw3, bw.dw2))
+    assert all(torch.equal(a, b) for a, b in zip(*grads))
+    assert float(grads[0][0].abs().max()) > 0
