@@ -124,10 +124,13 @@ ffn_gemm1_kernel(const __grid_constant__ CUtensorMap map_w1, const __grid_consta
     ptx::tmem_alloc(ptx::smem_u32(tmem_slot), 512);
     ptx::tmem_relinquish();
   }
-  grid_dependency_sync();   // nothing above touches global data
+  // GEMM-2 reads nothing of the kernel before it but the rows (and their scales): its tables and weights were there before that kernel
+  // started, which in turn let this one start only after its own wait.  So the weights of the first stages are fetched while the
+  // other thread blocks of that kernel finish, and only the warps that touch rows wait.
+  if (!PLAIN) grid_dependency_sync();   // nothing above touches global data
   for (int i = threadIdx.x; i <= p.E; i += blockDim.x) {
-    tp_s[i] = p.tile_prefix[i];
-    eoff_s[i] = p.expert_offsets[i];
+    tp_s[i] = __ldcg(p.tile_prefix + i);
+    eoff_s[i] = __ldcg(p.expert_offsets + i);
   }
   if (threadIdx.x == 0) *abort_s = p.status[ST_ABORT];
   ptx::tc_fence_before();
@@ -158,6 +161,7 @@ ffn_gemm1_kernel(const __grid_constant__ CUtensorMap map_w1, const __grid_consta
 
   if (warp < 4) {
     // ================================ epilogue ================================
+    if (PLAIN) grid_dependency_sync();
     int tl = 0;
     for (int w = blockIdx.x; w < total && !*abort_flag; w += gridDim.x, ++tl) {
       const Tile t = tile_of(w);
@@ -434,7 +438,9 @@ ffn_gemm1_kernel(const __grid_constant__ CUtensorMap map_w1, const __grid_consta
     }
   } else {
     // ================================ A gather producers ================================
+    if (PLAIN) grid_dependency_sync();
     const int gt = threadIdx.x - 192;     // 0..127
+    if (PLAIN && gt == 0 && *global_abort) *abort_flag = 1;   // set by the kernel before
     const int chunk = gt & 7;             // 16-byte chunk of the 128-byte K row
     const int rbase = gt >> 3;            // rows rbase + 16 j
     uint32_t it = 0;
