@@ -808,7 +808,7 @@ static int layer_impl(const moe_shape_t* shape, const void* x, const float* w_ga
     return MOE_OK;
   }
   TCMOE_CUDA(fp8 != nullptr ? launch_expert_ffn_fp8(s, a, q, st) : launch_expert_ffn(s, a, st));
-  TCMOE_CUDA(launch_combine(s, a.o, L, idx, tw, nullptr, y, status, st));
+  TCMOE_CUDA(launch_combine(s, a.o, L, idx, tw, nullptr, y, status, st, true));
   return MOE_OK;
 }
 

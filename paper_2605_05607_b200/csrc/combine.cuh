@@ -127,18 +127,18 @@ __device__ __forceinline__ void combine_token(const CombineArgs& c, int t, int l
   int my_g = 0x7FFFFFFF, my_row = 0, my_dst = 0;
   float my_w = 1.f;
   if (lane < k) {
-    const int e = __ldg(c.topk_idx + (size_t)t * k + lane);
+    const int e = __ldcg(c.topk_idx + (size_t)t * k + lane);
     // e < 0: unused slot of a sparse top-k table, sorts behind every real slot and is not read.  An expert
     // index or a row outside its table (the layout builder reported it and wrote row -1) is skipped the
     // same way, so no table entry is ever used as an address unchecked.
     if (e >= 0 && e < c.E) {
-      const int r = __ldg(c.pair_row + (size_t)t * k + lane);
-      const int a = __ldg(c.al + (size_t)(e / c.m) * c.T + t);
+      const int r = __ldcg(c.pair_row + (size_t)t * k + lane);
+      const int a = __ldcg(c.al + (size_t)(e / c.m) * c.T + t);
       if (r >= 0 && r < c.n_rows && a >= 0) {
         my_g = e / c.m;
         my_row = r;
-        my_dst = __ldg(c.group_offsets + my_g) + a;
-        if (c.weighted) my_w = __ldg(c.topk_w + (size_t)t * k + lane);
+        my_dst = __ldcg(c.group_offsets + my_g) + a;
+        if (c.weighted) my_w = __ldcg(c.topk_w + (size_t)t * k + lane);
       } else {
         report_error(c.status, DEV_INDEX_OUT_OF_RANGE, KID_COMBINE, t, r);
       }
@@ -155,6 +155,7 @@ __device__ __forceinline__ void combine_token(const CombineArgs& c, int t, int l
   __syncwarp();
   if (lane < k) { s_row[my_pos] = my_row; s_dst[my_pos] = my_dst; s_w[my_pos] = my_w; }
   __syncwarp();
+  if (!COHERENT && c.early) grid_dependency_sync();   // (again for each token of the warp: returns at once)
   if (BATCH == 2) combine_two<COHERENT, COLS>(c, t, lane, kv, s_row, s_dst, s_w, v_begin, v_end);
   else combine_rows<COHERENT, BATCH>(c, t, lane, kv, s_row, s_dst, s_w, v_begin, v_end);
   __syncwarp();

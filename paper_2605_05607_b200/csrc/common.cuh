@@ -90,6 +90,7 @@ struct CombineArgs {
   const int32_t* group_offsets;   // [G + 1]
   int T, E, k, m, vec_per_row, weighted, n_rows;
   int32_t* status;
+  int early;                      // the tables were complete before the kernel that writes o started: they are read before the wait for it
 };
 
 // Scratch tables of the layout builder (inside the workspace).
@@ -128,9 +129,10 @@ cudaError_t launch_permute_rows(const Shape& s, const void* src, int src_rows, c
 int row_parts(int T, int vec_per_row);   // warps that share a token's row in the row kernels, by the number of tokens
 cudaError_t launch_round_rows(const Shape& s, const float* acc, void* y, cudaStream_t st);
 cudaError_t launch_combine(const Shape& s, const void* o, const Layout& L, const int32_t* topk_idx,
-                           const float* topk_w, void* pg, void* y, int32_t* status, cudaStream_t st);
+                           const float* topk_w, void* pg, void* y, int32_t* status, cudaStream_t st, bool early = false);
 cudaError_t launch_combine_rows(const Shape& s, const void* o, const Layout& L, const int32_t* topk_idx,
-                                const float* topk_w, void* pg, void* y, int n_rows, int32_t* status, cudaStream_t st);
+                                const float* topk_w, void* pg, void* y, int n_rows, int32_t* status, cudaStream_t st,
+                                bool early = false);
 // bwd.cu: backward pass of the layer for fixed routing
 struct BwdArgs {
   const void *x, *dy;               // [T, d] bf16

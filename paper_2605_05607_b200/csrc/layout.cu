@@ -506,7 +506,7 @@ cudaError_t launch_permute_rows(const Shape& s, const void* src, int src_rows, c
 // leaves a 4096-token batch at a third of it).
 template <int BATCH, int COLS = 4>
 __global__ void __launch_bounds__(256, 3) combine_kernel(const CombineArgs c, int parts, int vec_per_part) {
-  grid_dependency_sync();
+  if (!c.early) grid_dependency_sync();
   __shared__ int s_row[8][32];   // per warp: expert-sorted row of the slot at sorted position p
   __shared__ int s_dst[8][32];   // dispatched row (t, g) of that slot's group
   __shared__ float s_w[8][32];
@@ -518,6 +518,7 @@ __global__ void __launch_bounds__(256, 3) combine_kernel(const CombineArgs c, in
     combine_token<false, BATCH, COLS>(c, t, lane, s_row[wid], s_dst[wid], s_w[wid], part * vec_per_part,
                                 (part + 1) * vec_per_part);
   }
+  if (c.early) grid_dependency_sync();   // warps without a token
 }
 
 // parts of a row so that about 32 warps per SM exist even for small batches (at most 8, at least 4 vectors per lane)
@@ -528,13 +529,15 @@ int row_parts(int T, int vec_per_row) {
 }
 
 cudaError_t launch_combine(const Shape& s, const void* o, const Layout& L, const int32_t* topk_idx,
-                           const float* topk_w, void* pg, void* y, int32_t* status, cudaStream_t st) {
-  return launch_combine_rows(s, o, L, topk_idx, topk_w, pg, y, s.T * s.k, status, st);
+                           const float* topk_w, void* pg, void* y, int32_t* status, cudaStream_t st, bool early) {
+  return launch_combine_rows(s, o, L, topk_idx, topk_w, pg, y, s.T * s.k, status, st, early);
 }
 
-// n_rows: rows of `o` (L.pair_row entries outside [0, n_rows) are reported and skipped)
+// n_rows: rows of `o` (L.pair_row entries outside [0, n_rows) are reported and skipped).  early: the kernel before this one is the library's
+// own GEMM that writes o, so the tables are older than it (it waited for the kernel before it and then let this one start): every warp
+// orders its first token's slots before it waits.  Layer of 256 tokens, 8 experts of 512 x 1024 30.5 -> 29.3 us.
 cudaError_t launch_combine_rows(const Shape& s, const void* o, const Layout& L, const int32_t* topk_idx,
-                                const float* topk_w, void* pg, void* y, int n_rows, int32_t* status, cudaStream_t st) {
+                                const float* topk_w, void* pg, void* y, int n_rows, int32_t* status, cudaStream_t st, bool early) {
   if (s.T == 0) return cudaSuccess;
   const int vec = s.d / 8;
   const int parts = row_parts(s.T, vec);
@@ -545,7 +548,7 @@ cudaError_t launch_combine_rows(const Shape& s, const void* o, const Layout& L, 
   ProfileScope prof(KID_COMBINE, st);
   CombineArgs c{static_cast<const uint4*>(o), static_cast<uint4*>(y), static_cast<uint4*>(pg), topk_idx, topk_w,
                 L.pair_row, L.al, L.group_offsets, s.T, s.E, s.k, s.E / s.G, vec, (s.flags & 1) ? 1 : 0,
-                n_rows, status};
+                n_rows, status, early ? 1 : 0};
   // parts that are no multiple of four warp strides: two columns at a time, so that the last step is not half empty (2050 tokens of
   // d = 2880 with group sums, 192 columns each: 11.8 -> 10.4 us, 10.7 with single columns)
   if (s.k <= 2 && vec_per_part % 128 != 0)
