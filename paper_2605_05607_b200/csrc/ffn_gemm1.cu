@@ -8,8 +8,8 @@
 // 128 x 256 x 16 UMMA yields both products (accumulator columns [0,128) = a.W1, [128,256) = a.W3).
 //
 // One persistent CTA per SM (tcgen05 cta_group::1) walks tile tasks decoded from the device-side
-// tile prefix, so no routing-dependent quantity visits the host.  Warp roles: 0-3 epilogue
-// (TMEM -> registers -> SwiGLU -> global), 4 TMA producer, 5 UMMA issuer and TMEM owner, 6-9 gather
+// tile prefix, so no routing-dependent quantity visits the host.  Warp roles: epilogue
+// (TMEM -> registers -> SwiGLU -> global), one TMA producer, one UMMA issuer and TMEM owner, four gather
 // producers.  Accumulators are double-buffered in TMEM (2 x 256 columns): the epilogue of tile i
 // overlaps the main loop of tile i+1.  Every wait is bounded.
 //
@@ -40,13 +40,17 @@ namespace {
 constexpr int RING_BYTES = 192 * 1024;       // 4 stages of A + a 256-column B, more of narrower ones
 constexpr int MAX_STAGES = 12;            // 64 rows x 64 columns: 16 KiB
 constexpr int NUM_BARS = 2 * MAX_STAGES + 4;
-constexpr int STAGE_OUT_WARP = 32 * 144;     // epilogue transpose buffer of one warp: 32 rows x (128 + 16) bytes
+// Four epilogue warps, one per row quarter; eight for short K walks (two per quarter, half of the columns each), where a tile's epilogue
+// takes longer than its main loop (512 cycles per 128 bytes of K) or is most of a layer's last round.
+__host__ __device__ constexpr int epi_warps(bool short_k) { return short_k ? 8 : 4; }
+constexpr int EPI_WARPS_MAX = 8;
+constexpr int STAGE_OUT_WARP = 32 * 64;      // epilogue transpose buffer of one warp: 32 rows x 32 columns, swizzled
 constexpr int TABLE_BYTES = (2 * (MAX_E + 1) * 4 + 15) & ~15;
-constexpr int COLSCALE_WARP = UMMA_N * 4;     // FP8: one warp's copy of the tile's 128 + 128 output-column scales
+constexpr int COLSCALE_WARP = UMMA_N / 2 * 4;   // FP8: one warp's copy of the scales of its columns (half of the accumulator's with eight warps)
 constexpr int SMEM_BYTES =
-    1024 + RING_BYTES + NUM_BARS * 8 + 64 + TABLE_BYTES + 4 * STAGE_OUT_WARP + 4 * COLSCALE_WARP;
-constexpr int THREADS = 320;
+    1024 + RING_BYTES + NUM_BARS * 8 + 64 + TABLE_BYTES + EPI_WARPS_MAX * (STAGE_OUT_WARP + COLSCALE_WARP);
 constexpr int GATHER_THREADS = 128;
+__host__ __device__ constexpr int threads(bool short_k) { return (epi_warps(short_k) + 2) * 32 + GATHER_THREADS; }
 // The producers (TMA thread, 128 gather threads) wait for a free stage with a suspend-time hint: parked in hardware
 // instead of polling.  At the board's power limit the layer's time follows energy: GEMM-1 alone in a loop on the
 // DeepSeek-V3 shape 15.78 -> 15.50 ms with the hint (two alternations, same box), a single cold launch 13.41 -> 13.48.
@@ -72,15 +76,18 @@ constexpr int SWAP_ROWS = 96;   // see `swapped`
 // FEW = true (narrow tiles only): tiles of 64 rows, for layers of at most 64 rows in all.  A stage is then a third smaller and
 // the ring holds more of the weights in flight (96 KiB instead of 64 in GEMM-2), which is what bounds a CTA that streams a column
 // slab of one expert: GEMM-2 of one token, top-2 of d = 4096, f = 14336, 58 -> 46 us (4.1 -> 5.1 TB/s).
-template <bool FP8, bool PLAIN, bool NARROW, bool FEW>
-__global__ void __launch_bounds__(THREADS, 1)
+template <bool FP8, bool PLAIN, bool NARROW, bool FEW, bool SHORT_K>
+__global__ void __launch_bounds__(threads(SHORT_K), 1)
 ffn_gemm1_kernel(const __grid_constant__ CUtensorMap map_w1, const __grid_constant__ CUtensorMap map_w3,
                  const GemmParams p) {
   constexpr int BN = !NARROW ? UMMA_N : PLAIN ? 64 : 128;   // accumulator columns of a tile
   constexpr int BN_OUT = PLAIN ? BN : BN / 2;               // output columns
   constexpr int HALF = BN > 64 ? BN / 2 : BN;               // columns from each of the two weight maps (BN = 64: one)
   constexpr int ROWS = FEW ? 64 : BM;                       // rows of a tile
-  constexpr int WROWS = ROWS / 4;                           // rows of an epilogue warp: TMEM lanes 32 w .. 32 w + WROWS - 1
+  constexpr int WROWS = ROWS / 4;                           // rows of an epilogue warp: TMEM lanes 32 q .. 32 q + WROWS - 1
+  constexpr int EPI_WARPS = epi_warps(SHORT_K), TMA_WARP = EPI_WARPS, MMA_WARP = EPI_WARPS + 1, GATHER_WARP = EPI_WARPS + 2;
+  constexpr int WCOLS = BN_OUT / (EPI_WARPS / 4);           // output columns of an epilogue warp
+  constexpr int SCALES = UMMA_N / (EPI_WARPS / 4);          // FP8: floats of its column scales
   static_assert(NARROW || !FEW, "64-row tiles come with narrow ones");
   constexpr int A_BYTES = ROWS * BK * 2;
   constexpr int B_BYTES = BN * BK * 2, STAGE_BYTES = A_BYTES + B_BYTES;   // B: 64-column slabs of 8 KiB
@@ -94,7 +101,7 @@ ffn_gemm1_kernel(const __grid_constant__ CUtensorMap map_w1, const __grid_consta
   int* tp_s = reinterpret_cast<int*>(tmem_slot + 16);
   int* eoff_s = tp_s + (MAX_E + 1);
   const uint32_t stage_base = ptx::smem_u32(tp_s) + TABLE_BYTES;   // 16-byte aligned
-  float* colscale_base = reinterpret_cast<float*>(reinterpret_cast<uint8_t*>(tp_s) + TABLE_BYTES + 4 * STAGE_OUT_WARP);
+  float* colscale_base = reinterpret_cast<float*>(reinterpret_cast<uint8_t*>(tp_s) + TABLE_BYTES + EPI_WARPS_MAX * STAGE_OUT_WARP);
 
   const uint32_t smem_base = ptx::smem_u32(smem);
   const uint32_t bar_base = ptx::smem_u32(bars);
@@ -112,15 +119,15 @@ ffn_gemm1_kernel(const __grid_constant__ CUtensorMap map_w1, const __grid_consta
     }
     for (int b = 0; b < 2; ++b) {
       ptx::mbar_init(tfull_bar(b), 1);      // tcgen05.commit
-      ptx::mbar_init(tempty_bar(b), 4);     // one lane per epilogue warp
+      ptx::mbar_init(tempty_bar(b), EPI_WARPS);   // one lane per epilogue warp
     }
     ptx::fence_mbar_init();
   }
-  if (warp == 4 && lane == 0) {
+  if (warp == TMA_WARP && lane == 0) {
     ptx::prefetch_tensormap(&map_w1);
     ptx::prefetch_tensormap(&map_w3);
   }
-  if (warp == 5) {
+  if (warp == MMA_WARP) {
     ptx::tmem_alloc(ptx::smem_u32(tmem_slot), 512);
     ptx::tmem_relinquish();
   }
@@ -159,25 +166,42 @@ ffn_gemm1_kernel(const __grid_constant__ CUtensorMap map_w1, const __grid_consta
   auto swapped = [&](const Tile& t) { return !NARROW && t.rows <= SWAP_ROWS && t.row0 == eoff_s[t.e]; };
   auto tile_of = [&](int w) { return decode_tile(w, tp_s, eoff_s, p.E, p.n_tiles, BN_OUT, BM, 0); };
 
-  if (warp < 4) {
+  if (warp < EPI_WARPS) {
     // ================================ epilogue ================================
     if (PLAIN) grid_dependency_sync();
+    const int quarter = warp & 3, half = warp >> 2;   // TMEM lanes this warp owns, and which half of their columns with eight warps
     int tl = 0;
     for (int w = blockIdx.x; w < total && !*abort_flag; w += gridDim.x, ++tl) {
       const Tile t = tile_of(w);
       const int buf = tl & 1;
       if (!ptx::mbar_wait_warp<true>(tfull_bar(buf), (tl >> 1) & 1, abort_flag, global_abort)) { timeout(1); break; }
       ptx::tc_fence_after();
-      const uint32_t taddr = tmem_base + ((uint32_t)(warp * 32) << 16) + (uint32_t)(buf * BN);
-      // A thread owns one accumulator row; 32 threads storing 16 bytes each to 32 different rows
-      // would cost 32 memory transactions per instruction.  The warp transposes 64 output columns
-      // at a time through shared memory (rows padded to 144 bytes: conflict-free both ways) and
-      // stores whole 128-byte row segments, 8 lanes per row, 4 rows per instruction.
+      const uint32_t taddr = tmem_base + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(buf * BN);
+      // A thread owns one accumulator row; 32 threads storing 16 bytes each to 32 different rows would cost 32 memory transactions per
+      // instruction.  The warp transposes 32 output columns at a time through shared memory (64-byte rows, pieces swizzled by row pair:
+      // conflict-free both ways) and stores 64-byte row segments, 8 rows per instruction.
       const uint32_t stage = stage_base + (uint32_t)(warp * STAGE_OUT_WARP);
-      const int srow = lane >> 3, piece = lane & 7;
+      const int srow = lane >> 2, piece = lane & 3;
+      auto put = [&](int v, uint32_t q0, uint32_t q1, uint32_t q2, uint32_t q3) {   // columns 8 v .. + 7 of this thread's row
+        ptx::st_shared_v4(stage + lane * 64 + ((v ^ ((lane >> 1) & 3)) << 4), q0, q1, q2, q3);
+      };
+      auto send = [&](int at) {   // 32 staged columns, from column `at` of the tile on, to the rows of out
+        __syncwarp();
+        const int col = t.n0 + at + piece * 8;
+        if (col < p.N) {
+#pragma unroll
+          for (int i = 0; i < WROWS / 8; ++i) {
+            const int r = i * 8 + srow;   // row of this warp's
+            if (quarter * WROWS + r < t.rows)
+              *reinterpret_cast<uint4*>(p.out + (size_t)(t.row0 + quarter * WROWS + r) * (size_t)p.out_ld + col) =
+                  ptx::ld_shared_v4(stage + r * 64 + ((piece ^ ((r >> 1) & 3)) << 4));
+          }
+        }
+        __syncwarp();
+      };
       if (swapped(t)) {
         // lane = output column of a half tile (GEMM-1: the same column of W1 and of W3), TMEM column = row
-        const int c = warp * 32 + lane, odd = lane & 1;
+        const int c = quarter * 32 + lane, odd = lane & 1;
         const size_t sc = (size_t)t.e * p.N + t.n0 + c;
         float sa = 1.f, sb = 1.f;   // FP8: column scales
         if (FP8) {
@@ -186,7 +210,7 @@ ffn_gemm1_kernel(const __grid_constant__ CUtensorMap map_w1, const __grid_consta
           sb = t.n0 + hi + c < p.N ? __ldg((PLAIN ? p.b_scale : p.b_scale2) + sc + hi) : 0.f;
         }
 #pragma unroll 1
-        for (int r0 = 0; r0 < t.rows; r0 += 16) {
+        for (int r0 = half * 16; r0 < t.rows; r0 += EPI_WARPS * 4) {   // the warps of a quarter take turns
           const int mine = r0 + (lane & 15);
           float rs = 1.f;   // scale of this lane's row of the 16
           if (mine < t.rows) {
@@ -225,135 +249,97 @@ ffn_gemm1_kernel(const __grid_constant__ CUtensorMap map_w1, const __grid_consta
           }
         }
       } else if (PLAIN) {
-        // ---- GEMM-2 form: o = (gate weight x row scale) * acc * column scale, 256 columns
-        const int lrow = warp * WROWS + lane;
+        // ---- GEMM-2 form: o = (gate weight x row scale) * acc * column scale
+        const int lrow = quarter * WROWS + lane;
         float wr = 1.f;
         if (lane < WROWS && lrow < t.rows) {
           const size_t grow = (size_t)t.row0 + lrow;
           if (p.topk_w != nullptr) wr = __ldg(p.topk_w + __ldg(p.row_pair + grow));
           if (FP8) wr *= __ldg(p.a_scale + grow);
         }
-        float* sb_col = colscale_base + warp * UMMA_N;
+        float* sb_col = colscale_base + warp * SCALES;   // scales of this warp's columns (0 beyond N)
         if (FP8) {
-          const float* g = p.b_scale + (size_t)t.e * p.N + t.n0;
+          const int n0 = t.n0 + half * WCOLS;
+          const float* g = p.b_scale + (size_t)t.e * p.N + n0;
 #pragma unroll
-          for (int i = 0; i < BN / 32; ++i) {
+          for (int i = 0; i < WCOLS / 32; ++i) {
             const int n = lane + 32 * i;
-            sb_col[n] = (t.n0 + n < p.N) ? __ldg(g + n) : 0.f;
+            sb_col[n] = (n0 + n < p.N) ? __ldg(g + n) : 0.f;
           }
           __syncwarp();
         }
 #pragma unroll 1
-        for (int cc = 0; cc < BN / 64; ++cc) {
-          uint32_t acc0[32], acc1[32];
-          ptx::tmem_ld32(taddr + cc * 64, acc0);
-          ptx::tmem_ld32(taddr + cc * 64 + 32, acc1);
-          ptx::tmem_ld_wait_on(acc0);
-          ptx::tmem_ld_wait_on(acc1);
+        for (int c = 0; c < WCOLS / 32; ++c) {
+          uint32_t acc[32];
+          ptx::tmem_ld32(taddr + half * WCOLS + c * 32, acc);
+          ptx::tmem_ld_wait_on(acc);
           if (FP8) {
 #pragma unroll
-            for (int j = 0; j < 32; ++j) {
-              const int n = cc * 64 + j;
-              acc0[j] = __float_as_uint(__uint_as_float(acc0[j]) * sb_col[n]);
-              acc1[j] = __float_as_uint(__uint_as_float(acc1[j]) * sb_col[n + 32]);
-            }
+            for (int j = 0; j < 32; ++j) acc[j] = __float_as_uint(__uint_as_float(acc[j]) * sb_col[c * 32 + j]);
           }
 #pragma unroll
-          for (int v = 0; v < 4; ++v) {
-            ptx::st_shared_v4(stage + lane * 144 + v * 16,
-                              pack2(wr * __uint_as_float(acc0[v * 8]), wr * __uint_as_float(acc0[v * 8 + 1])),
-                              pack2(wr * __uint_as_float(acc0[v * 8 + 2]), wr * __uint_as_float(acc0[v * 8 + 3])),
-                              pack2(wr * __uint_as_float(acc0[v * 8 + 4]), wr * __uint_as_float(acc0[v * 8 + 5])),
-                              pack2(wr * __uint_as_float(acc0[v * 8 + 6]), wr * __uint_as_float(acc0[v * 8 + 7])));
-            ptx::st_shared_v4(stage + lane * 144 + 64 + v * 16,
-                              pack2(wr * __uint_as_float(acc1[v * 8]), wr * __uint_as_float(acc1[v * 8 + 1])),
-                              pack2(wr * __uint_as_float(acc1[v * 8 + 2]), wr * __uint_as_float(acc1[v * 8 + 3])),
-                              pack2(wr * __uint_as_float(acc1[v * 8 + 4]), wr * __uint_as_float(acc1[v * 8 + 5])),
-                              pack2(wr * __uint_as_float(acc1[v * 8 + 6]), wr * __uint_as_float(acc1[v * 8 + 7])));
-          }
-          __syncwarp();
-          const int col = t.n0 + cc * 64 + piece * 8;
-          if (col < p.N) {
-#pragma unroll
-            for (int i = 0; i < WROWS / 4; ++i) {
-              const int r = i * 4 + srow;
-              if (warp * WROWS + r < t.rows) {
-                const uint4 q = ptx::ld_shared_v4(stage + r * 144 + piece * 16);
-                *reinterpret_cast<uint4*>(p.out + (size_t)(t.row0 + warp * WROWS + r) * (size_t)p.out_ld + col) = q;
-              }
-            }
-          }
-          __syncwarp();
+          for (int v = 0; v < 4; ++v)
+            put(v, pack2(wr * __uint_as_float(acc[v * 8]), wr * __uint_as_float(acc[v * 8 + 1])),
+                pack2(wr * __uint_as_float(acc[v * 8 + 2]), wr * __uint_as_float(acc[v * 8 + 3])),
+                pack2(wr * __uint_as_float(acc[v * 8 + 4]), wr * __uint_as_float(acc[v * 8 + 5])),
+                pack2(wr * __uint_as_float(acc[v * 8 + 6]), wr * __uint_as_float(acc[v * 8 + 7])));
+          send(half * WCOLS + c * 32);
         }
       } else {
-        // ---- GEMM-1 form: SwiGLU of the W1 / W3 halves, 128 output columns
-      float sa = 1.f;   // FP8: scale of this thread's row (the gather source row)
-      float* s1 = colscale_base + warp * UMMA_N;   // this warp's copy of the W1 / W3 column scales (0 beyond N)
-      float* s3 = s1 + BN_OUT;
-      if (FP8) {
-        const int lrow = warp * WROWS + lane;
-        if (lane < WROWS && lrow < t.rows) {
-          int idx = __ldg(p.gather_idx + t.row0 + lrow);
-          if (p.gather_div > 1) idx /= p.gather_div;
-          sa = (idx >= 0 && idx < p.a_rows) ? __ldg(p.a_scale + idx) : 0.f;
-        }
-        const size_t g = (size_t)t.e * p.N + t.n0;
+        // ---- GEMM-1 form: SwiGLU of the W1 / W3 halves
+        float sa = 1.f;   // FP8: scale of this thread's row (the gather source row)
+        float* s1 = colscale_base + warp * SCALES;   // the W1 / W3 scales of this warp's columns (0 beyond N)
+        float* s3 = s1 + WCOLS;
+        if (FP8) {
+          const int lrow = quarter * WROWS + lane, n0 = t.n0 + half * WCOLS;
+          if (lane < WROWS && lrow < t.rows) {
+            int idx = __ldg(p.gather_idx + t.row0 + lrow);
+            if (p.gather_div > 1) idx /= p.gather_div;
+            sa = (idx >= 0 && idx < p.a_rows) ? __ldg(p.a_scale + idx) : 0.f;
+          }
+          const size_t g = (size_t)t.e * p.N + n0;
 #pragma unroll
-        for (int i = 0; i < BN_OUT / 32; ++i) {
-          const int n = lane + 32 * i;
-          const bool in = t.n0 + n < p.N;
-          s1[n] = in ? (__ldg(p.b_scale + g + n)) : 0.f;
-          s3[n] = in ? (__ldg(p.b_scale2 + g + n)) : 0.f;
+          for (int i = 0; i < WCOLS / 32; ++i) {
+            const int n = lane + 32 * i;
+            const bool in = n0 + n < p.N;
+            s1[n] = in ? (__ldg(p.b_scale + g + n)) : 0.f;
+            s3[n] = in ? (__ldg(p.b_scale2 + g + n)) : 0.f;
+          }
+          __syncwarp();
         }
-        __syncwarp();
-      }
 #pragma unroll 1
-      for (int c = 0; c < BN_OUT / 32; ++c) {
-        uint32_t a1[32], a3[32];
-        ptx::tmem_ld32(taddr + c * 32, a1);
-        ptx::tmem_ld32(taddr + BN_OUT + c * 32, a3);
-        ptx::tmem_ld_wait_on(a1, a3);
+        for (int c = 0; c < WCOLS / 32; ++c) {
+          uint32_t a1[32], a3[32];
+          ptx::tmem_ld32(taddr + half * WCOLS + c * 32, a1);
+          ptx::tmem_ld32(taddr + BN_OUT + half * WCOLS + c * 32, a3);
+          ptx::tmem_ld_wait_on(a1, a3);
 #pragma unroll
-        for (int v = 0; v < 4; ++v) {
-          uint32_t q[4];
+          for (int v = 0; v < 4; ++v) {
+            uint32_t q[4];
 #pragma unroll
-          for (int i = 0; i < 4; ++i) {
-            const int j = v * 8 + 2 * i;
-            float u0 = __uint_as_float(a1[j]), u1 = __uint_as_float(a1[j + 1]);
-            float g0 = __uint_as_float(a3[j]), g1 = __uint_as_float(a3[j + 1]);
-            if (FP8) {
-              const int n = c * 32 + j;
-              u0 *= sa * s1[n];
-              g0 *= sa * s3[n];
-              u1 *= sa * s1[n + 1];
-              g1 *= sa * s3[n + 1];
-            }
-            q[i] = pack2(silu_mul(u0, g0), silu_mul(u1, g1));
-          }
-          ptx::st_shared_v4(stage + lane * 144 + (c & 1) * 64 + v * 16, q[0], q[1], q[2], q[3]);
-        }
-        if (c & 1) {
-          __syncwarp();
-          const int col = t.n0 + (c - 1) * 32 + piece * 8;
-          if (col < p.N) {
-#pragma unroll
-            for (int i = 0; i < WROWS / 4; ++i) {
-              const int r = i * 4 + srow;           // row of this warp's
-              if (warp * WROWS + r < t.rows) {
-                const uint4 q = ptx::ld_shared_v4(stage + r * 144 + piece * 16);
-                *reinterpret_cast<uint4*>(p.out + (size_t)(t.row0 + warp * WROWS + r) * (size_t)p.out_ld + col) = q;
+            for (int i = 0; i < 4; ++i) {
+              const int j = v * 8 + 2 * i;
+              float u0 = __uint_as_float(a1[j]), u1 = __uint_as_float(a1[j + 1]);
+              float g0 = __uint_as_float(a3[j]), g1 = __uint_as_float(a3[j + 1]);
+              if (FP8) {
+                const int n = c * 32 + j;
+                u0 *= sa * s1[n];
+                g0 *= sa * s3[n];
+                u1 *= sa * s1[n + 1];
+                g1 *= sa * s3[n + 1];
               }
+              q[i] = pack2(silu_mul(u0, g0), silu_mul(u1, g1));
             }
+            put(v, q[0], q[1], q[2], q[3]);
           }
-          __syncwarp();
+          send(half * WCOLS + c * 32);
         }
-      }
       }
       ptx::tc_fence_before();
       __syncwarp();
       if (lane == 0) ptx::mbar_arrive(tempty_bar(buf));
     }
-  } else if (warp == 4) {
+  } else if (warp == TMA_WARP) {
     // ================================ TMA producer (weights) ================================
     if (lane == 0) {
       uint32_t it = 0;
@@ -384,7 +370,7 @@ ffn_gemm1_kernel(const __grid_constant__ CUtensorMap map_w1, const __grid_consta
         if (!ok) break;
       }
     }
-  } else if (warp == 5) {
+  } else if (warp == MMA_WARP) {
     // ================================ UMMA issuer ================================
     // the warp walks the loop, one elected lane issues (see ptx::elect_one)
     const bool elected = ptx::elect_one();
@@ -439,7 +425,7 @@ ffn_gemm1_kernel(const __grid_constant__ CUtensorMap map_w1, const __grid_consta
   } else {
     // ================================ A gather producers ================================
     if (PLAIN) grid_dependency_sync();
-    const int gt = threadIdx.x - 192;     // 0..127
+    const int gt = threadIdx.x - GATHER_WARP * 32;   // 0..127
     if (PLAIN && gt == 0 && *global_abort) *abort_flag = 1;   // set by the kernel before
     const int chunk = gt & 7;             // 16-byte chunk of the 128-byte K row
     const int rbase = gt >> 3;            // rows rbase + 16 j
@@ -509,7 +495,7 @@ ffn_gemm1_kernel(const __grid_constant__ CUtensorMap map_w1, const __grid_consta
     for (int i = 0; i < 64; ++i) __nanosleep(1000);
   }
   __syncthreads();
-  if (warp == 5) {
+  if (warp == MMA_WARP) {
     ptx::tc_fence_after();
     ptx::tmem_dealloc(tmem_base, 512);
   }
@@ -518,26 +504,31 @@ ffn_gemm1_kernel(const __grid_constant__ CUtensorMap map_w1, const __grid_consta
 }  // namespace
 
 namespace {
-template <bool FP8, bool PLAIN, bool NARROW, bool FEW>
+template <bool FP8, bool PLAIN, bool NARROW, bool FEW, bool SHORT_K>
 cudaError_t launch_form(const GemmParams& p, const CUtensorMap& m_a, const CUtensorMap& m_b, bool overlap, cudaStream_t st) {
   // per device; several host threads may get here at once: setting the attribute twice is harmless
   static std::atomic<bool> attr_set[MAX_DEVICES];
   const int dev = current_device();
-  const auto kernel = ffn_gemm1_kernel<FP8, PLAIN, NARROW, FEW>;
+  const auto kernel = ffn_gemm1_kernel<FP8, PLAIN, NARROW, FEW, SHORT_K>;
   if (!attr_set[dev].load(std::memory_order_acquire)) {
     cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_BYTES);
     if (e != cudaSuccess) return e;
     attr_set[dev].store(true, std::memory_order_release);
   }
   ProfileScope prof(PLAIN ? KID_GEMM2 : KID_GEMM1, st);
-  return launch_kernel(overlap, 0, kernel, sm_count(), THREADS, SMEM_BYTES, st, m_a, m_b, p);
+  return launch_kernel(overlap, 0, kernel, sm_count(), threads(SHORT_K), SMEM_BYTES, st, m_a, m_b, p);
 }
 
 template <bool FP8, bool PLAIN>
 cudaError_t launch_width(const GemmParams& p, const CUtensorMap& m_a, const CUtensorMap& m_b, bool narrow, bool few, bool overlap,
                          cudaStream_t st) {
-  if (!narrow) return launch_form<FP8, PLAIN, false, false>(p, m_a, m_b, overlap, st);
-  return few ? launch_form<FP8, PLAIN, true, true>(p, m_a, m_b, overlap, st) : launch_form<FP8, PLAIN, true, false>(p, m_a, m_b, overlap, st);
+  // Layers, us, four / eight epilogue warps in the full-width tiles, K walk of GEMM-1 in brackets: 10181 tokens top-1 of 8 x 656 x 4512 in
+  // 8 bits (6) 236 / 230, 529 top-4 of 16 x 608 x 1392 (10; GEMM-2 22) 50.8 / 49.7, 4000 top-4 of 32 x 1504 x 2048 (24) 377.7 / 378.5, of 2048 x
+  // 2048 (32) 461.5 / 463.4, 16384 top-8 of 128 x 4096 x 1536 in 8 bits (32) 3099 / 3106, 32768 top-8 of 256 x 7168 x 2048 (112) 21320 / 21440;
+  // narrow tiles: 256 top-2 of 8 x 512 x 1024 29.3 / 28.6, but of 64 rows (1 token, 8 x 4096 x 14336) 143 / 145.
+  if (!narrow && p.K * (FP8 ? 1 : 2) > 24 * 128) return launch_form<FP8, PLAIN, false, false, false>(p, m_a, m_b, overlap, st);
+  if (!narrow) return launch_form<FP8, PLAIN, false, false, true>(p, m_a, m_b, overlap, st);
+  return few ? launch_form<FP8, PLAIN, true, true, false>(p, m_a, m_b, overlap, st) : launch_form<FP8, PLAIN, true, false, true>(p, m_a, m_b, overlap, st);
 }
 }  // namespace
 

@@ -715,3 +715,19 @@ def test_experts_of_few_rows_give_the_same_bits(rows, fp8):
         assert B.moe_status(ws)[0] == 0
         ys.append(y)
     assert torch.equal(ys[0], ys[1][:rows])
+
+
+@pytest.mark.parametrize("d,f", [(1536, 400), (1544, 400), (400, 1536), (400, 1544)])
+def test_four_and_eight_epilogue_warps_give_the_same_bits(d, f):
+    """A K walk of up to 24 blocks takes eight epilogue warps in the single-CTA GEMMs, a longer one four.  130 rows per expert (a full tile and one
+    of two rows), last column tiles partly filled; the pair kernels' layer has the same sums."""
+    cfg = synth.MoEConfig("epilogue", T=130, d=d, f=f, E=16, k=16, G=4, seed=d)
+    t = synth.make_inputs(cfg, "cuda")
+    ys = []
+    for flags in (B.MOE_FLAG_GEMM1_GATHER | B.MOE_FLAG_GEMM2_SINGLE, B.MOE_FLAG_GEMM1_PAIR | B.MOE_FLAG_GEMM2_PAIR):
+        run = H.Run(cfg, flags, t)
+        run.layer()
+        torch.cuda.synchronize()
+        assert run.status()[0] == 0
+        ys.append(run.y)
+    assert torch.equal(*ys)
