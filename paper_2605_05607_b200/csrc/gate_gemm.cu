@@ -198,8 +198,9 @@ gate_umma_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constan
         // warp w: TMEM lanes 32 (w % 4) .. + 31, every (warps / 4)-th 32-column block from w / 4 on.  A 64-row accumulator has row
         // 16 q + i in lane 32 q + i (i < 16).
         const int lrow = ROWS_M == 64 ? (lane < 16 ? (warp & 3) * 16 + lane : p.T) : (warp & 3) * 32 + lane;
-        for (int u = warp >> 2; u < n_sub * (GN / 32); u += WARPS / 4) {
-          const int i = u / (GN / 32), c = (u % (GN / 32)) * 32;
+        constexpr int PARTS = GN > 32 ? GN / 32 : 1;   // of 32 columns (16-column tiles: the upper half is not used)
+        for (int u = warp >> 2; u < n_sub * PARTS; u += WARPS / 4) {
+          const int i = u / PARTS, c = (u % PARTS) * 32;
           const int row = row0 + i * ROWS_M + lrow;
           if (c >= ncols) continue;
           const uint32_t taddr = tmem_base + ((uint32_t)((warp & 3) * 32) << 16) + c;
@@ -225,7 +226,7 @@ gate_umma_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constan
             float* out = p.logits + (size_t)row * p.E + n0 + c;
 #pragma unroll
             for (int v = 0; v < 8; ++v)
-              if (n0 + c + v * 4 < p.E)
+              if (c + v * 4 < GN && n0 + c + v * 4 < p.E)
                 *reinterpret_cast<uint4*>(out + v * 4) = make_uint4(acc[v * 4], acc[v * 4 + 1], acc[v * 4 + 2], acc[v * 4 + 3]);
           } else {
             // Rows that start anywhere.  A lane that stores its own row by the element makes 32 pieces of each store, which bounds the
@@ -236,7 +237,7 @@ gate_umma_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constan
             for (int v = 0; v < 32; ++v) st[lane * 33 + v] = __uint_as_float(acc[v]);
             __syncwarp();
             const int first = row0 + i * ROWS_M + (warp & 3) * (ROWS_M / 4), rows = min(ROWS_M / 4, p.T - first);
-            if (n0 + c + lane < p.E) {
+            if (c + lane < GN && n0 + c + lane < p.E) {
               float* out = p.logits + (size_t)first * p.E + n0 + c + lane;
 #pragma unroll 8
               for (int r = 0; r < rows; ++r) out[(size_t)r * p.E] = st[r * 33 + lane];
@@ -284,7 +285,7 @@ gate_umma_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constan
         if (__any_sync(0xFFFFFFFFu, !ptx::mbar_wait(full_bar(s), ph, abort_flag, global_abort))) { timeout(4); ok = false; break; }
         ptx::tc_fence_after();
         if (elected) {
-          for (int i = 0; i < (GN == 32 ? 1 : n_sub); ++i) {   // (32 columns: one row tile)
+          for (int i = 0; i < (GN <= 32 ? 1 : n_sub); ++i) {   // (up to 32 columns: one row tile)
             const uint64_t ad = a_desc + (s * stage16 + i * a16), bd = b_desc + s * stage16;
             if (APART) {   // the terms as one wide B
               constexpr int N1 = 3 * GN < 256 ? 3 * GN : 256, N2 = 3 * GN - N1;
@@ -350,6 +351,9 @@ __global__ void __launch_bounds__(256) split_gate_kernel(const float* __restrict
 // moe_route of (T, d, E), us, without the split copy / with this table: 16384, 2880, 65: 61.4 / 50.4; 16384, 2880, 128: 53.0 / 49.4;
 // 32768, 2880, 96: 102 / 92; 8192, 7168, 256: 115 / 85; 32768, 7168, 250: 459 / 335; 4097, 7168, 258: 194 / 90 (the last two
 // 315 -> 291 and 98 -> 91 in a replayed graph since ragged rows of logits leave whole).
+// Up to 128 experts tiles of 16 columns where the SMs take them in as many rounds: a block has half the weight to split and less to
+// move through shared memory per k-block, moe_route of (T, d, E), us, 32 / 16 columns: 64, 4096, 128 23.5 / 20.6; 300, 4096, 65 30.2 / 24.5;
+// 872, 6832, 16 35.8 / 27.8; 1669, 3520, 64 23.9 / 19.4; 200, 256, 64 7.0 / 6.3.
 struct GatePlan { int gn, bm, m_sub; bool pre; };
 GatePlan plan_gate(int T, int d, int E) {
   struct Cost { double start, kb, kb_ragged; };
@@ -357,6 +361,7 @@ GatePlan plan_gate(int T, int d, int E) {
   static const struct { GatePlan form; Cost running, apart; } forms[] = {
       {{32, 64, 1, false}, {4, 0.37, 0.38}, NO},
       {{64, 64, 1, false}, {4, 0.43, 0.63}, NO},
+      {{16, 128, 1, false}, NO, {4.8, 0.24, 0.27}},
       {{32, 128, 1, false}, {4.3, 0.455, 0.46}, {4.5, 0.318, 0.345}},
       {{64, 128, 1, false}, {4.8, 0.525, 0.66}, NO},
       {{64, 128, 2, false}, {7, 0.83, 0.87}, {8, 0.63, 0.68}},
@@ -441,6 +446,7 @@ cudaError_t launch_gate_logits(const Shape& s, const void* x, const float* w_gat
     return launch_width<128, 1, 128, true, true>(p, grid, m_x, m_w, st);
   }
   if (apart) {
+    if (plan.gn == 16) return launch_width<16, 4, 128, true>(p, grid, m_x, m_x, st);
     if (plan.gn == 32) return launch_width<32, 4, 128, true>(p, grid, m_x, m_x, st);
     return launch_width<64, 2, 128, true>(p, grid, m_x, m_x, st);
   }
