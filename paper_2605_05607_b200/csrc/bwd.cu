@@ -28,34 +28,15 @@ namespace {
 __global__ void __launch_bounds__(1024) bwd_offsets_kernel(const int32_t* __restrict__ expert_counts, int32_t* poff,
                                                            int32_t* mt_prefix, int32_t* mp_prefix, int E) {
   grid_dependency_sync();
-  __shared__ int warp_sum[3][32];
-  const int i = threadIdx.x, lane = i & 31, wid = i >> 5;
+  __shared__ int sums[3][32];
+  const int i = threadIdx.x;
   const int n = (i < E) ? expert_counts[i] : 0;
   int v[3] = {(n + 63) & ~63, (n + 127) >> 7, (n + 255) >> 8};
-#pragma unroll
-  for (int q = 0; q < 3; ++q) {
-#pragma unroll
-    for (int off = 1; off < 32; off <<= 1) {
-      const int u = __shfl_up_sync(0xFFFFFFFFu, v[q], off);
-      if (lane >= off) v[q] += u;
-    }
-    if (lane == 31) warp_sum[q][wid] = v[q];
-  }
-  __syncthreads();
-  if (wid < 3) {
-    int u = warp_sum[wid][lane];
-#pragma unroll
-    for (int off = 1; off < 32; off <<= 1) {
-      const int w = __shfl_up_sync(0xFFFFFFFFu, u, off);
-      if (lane >= off) u += w;
-    }
-    warp_sum[wid][lane] = u;
-  }
-  __syncthreads();
+  block_scan(v, sums);
   int32_t* out[3] = {poff, mt_prefix, mp_prefix};
 #pragma unroll
   for (int q = 0; q < 3; ++q) {
-    if (i < E) out[q][i + 1] = v[q] + (wid > 0 ? warp_sum[q][wid - 1] : 0);
+    if (i < E) out[q][i + 1] = v[q];
     if (i == 0) out[q][0] = 0;
   }
 }

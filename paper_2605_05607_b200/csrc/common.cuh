@@ -68,6 +68,35 @@ cudaError_t launch_pdl(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t s
   return launch_pdl_cluster(0, kernel, grid, block, smem, st, std::forward<Args>(args)...);   // 0: as the kernel declares
 }
 
+// Inclusive sums over the 1024 threads of a block, N values each (sums: scratch).
+template <int N>
+__device__ __forceinline__ void block_scan(int (&v)[N], int (&sums)[N][32]) {
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+#pragma unroll
+  for (int q = 0; q < N; ++q) {
+#pragma unroll
+    for (int off = 1; off < 32; off <<= 1) {
+      const int u = __shfl_up_sync(0xFFFFFFFFu, v[q], off);
+      if (lane >= off) v[q] += u;
+    }
+    if (lane == 31) sums[q][wid] = v[q];
+  }
+  __syncthreads();
+  if (wid < N) {
+    int u = sums[wid][lane];
+#pragma unroll
+    for (int off = 1; off < 32; off <<= 1) {
+      const int w = __shfl_up_sync(0xFFFFFFFFu, u, off);
+      if (lane >= off) u += w;
+    }
+    sums[wid][lane] = u;
+  }
+  __syncthreads();
+#pragma unroll
+  for (int q = 0; q < N; ++q)
+    if (wid > 0) v[q] += sums[q][wid - 1];
+}
+
 // ---- problem description passed to the launchers ---------------------------------------------
 struct Shape {
   int T, d, f, E, k, G, score_fn, flags;

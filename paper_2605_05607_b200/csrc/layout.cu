@@ -15,16 +15,19 @@
 
 namespace tcmoe {
 
+// Mask and fill passes: a block takes one mask word of 32 tokens, its eight warps take turns in the slots and groups of these tokens.
+// (With a thread per token a batch of 8192 tokens had 32 blocks, each walking 32 groups and 8 slots one latency after the other:
+// 13 and 33 us; the four kernels of top-8 in 32 groups 37.6 -> 11.5 us.)
+constexpr int WORD_WARPS = 8;
+
 // ---- K2a: membership masks -------------------------------------------------------------------
-__global__ void __launch_bounds__(256) build_masks_kernel(const int32_t* __restrict__ topk_idx, uint32_t* emask,
+__global__ void __launch_bounds__(WORD_WARPS * 32) build_masks_kernel(const int32_t* __restrict__ topk_idx, uint32_t* emask,
                                                           uint32_t* gmask, int T, int E, int k, int m, int W,
                                                           int32_t* status, int sparse) {
   grid_dependency_sync();
-  const int t = blockIdx.x * blockDim.x + threadIdx.x;  // warp w covers tokens 32w .. 32w+31
-  const int lane = threadIdx.x & 31;
-  const int word = t >> 5;
+  const int lane = threadIdx.x & 31, word = blockIdx.x, t = word * 32 + lane;
   const bool live = t < T;
-  for (int j = 0; j < k; ++j) {
+  for (int j = threadIdx.x >> 5; j < k; j += WORD_WARPS) {
     int e = live ? __ldg(topk_idx + (size_t)t * k + j) : -1;
     if (live && (e < 0 || e >= E)) {
       if (!(sparse && e == -1)) report_error(status, DEV_INDEX_OUT_OF_RANGE, KID_MASKS, t, e);   // -1: unused slot
@@ -84,36 +87,25 @@ __global__ void __launch_bounds__(1024) offsets_kernel(const int32_t* __restrict
                                                        int32_t* expert_offsets, int32_t* group_offsets,
                                                        int32_t* mt_prefix, int32_t* mp_prefix, int E, int G) {
   grid_dependency_sync();
-  __shared__ int buf[4][1024];
+  __shared__ int sums[4][32];
   const int i = threadIdx.x;
   const int ce = (i < E) ? expert_counts[i] : 0;
   const int cg = (i < G) ? group_counts[i] : 0;
-  buf[0][i] = ce;
-  buf[1][i] = cg;
-  buf[2][i] = (ce + 127) >> 7;   // 128-row tiles (GEMM-1)
-  buf[3][i] = (ce + 255) >> 8;   // 256-row CTA-pair tiles (GEMM-2)
-  __syncthreads();
-  for (int off = 1; off < 1024; off <<= 1) {  // Hillis-Steele inclusive scan, three lanes at once
-    int a = 0, b = 0, c = 0, d = 0;
-    if (i >= off) { a = buf[0][i - off]; b = buf[1][i - off]; c = buf[2][i - off]; d = buf[3][i - off]; }
-    __syncthreads();
-    buf[0][i] += a; buf[1][i] += b; buf[2][i] += c; buf[3][i] += d;
-    __syncthreads();
-  }
-  if (i < E) { expert_offsets[i + 1] = buf[0][i]; mt_prefix[i + 1] = buf[2][i]; mp_prefix[i + 1] = buf[3][i]; }
-  if (i < G) group_offsets[i + 1] = buf[1][i];
+  int v[4] = {ce, cg, (ce + 127) >> 7, (ce + 255) >> 8};   // 128-row tiles (GEMM-1), 256-row CTA-pair tiles (GEMM-2)
+  block_scan(v, sums);
+  if (i < E) { expert_offsets[i + 1] = v[0]; mt_prefix[i + 1] = v[2]; mp_prefix[i + 1] = v[3]; }
+  if (i < G) group_offsets[i + 1] = v[1];
   if (i == 0) { expert_offsets[0] = 0; group_offsets[0] = 0; mt_prefix[0] = 0; mp_prefix[0] = 0; }
 }
 
 // ---- K2d: ranks -> row tables ----------------------------------------------------------------
-__global__ void __launch_bounds__(256) fill_layout_kernel(const int32_t* __restrict__ topk_idx, Layout L,
+__global__ void __launch_bounds__(WORD_WARPS * 32) fill_layout_kernel(const int32_t* __restrict__ topk_idx, Layout L,
                                                           LayoutScratch sc, int T, int E, int k, int G, int m) {
   grid_dependency_sync();
-  const int t = blockIdx.x * blockDim.x + threadIdx.x;
+  const int word = blockIdx.x, t = word * 32 + (threadIdx.x & 31), warp = threadIdx.x >> 5;
   if (t >= T) return;
-  const int word = t >> 5;
   const uint32_t below = (1u << (t & 31)) - 1u;
-  for (int g = 0; g < G; ++g) {
+  for (int g = warp; g < G; g += WORD_WARPS) {
     const uint32_t bits = sc.gmask[(size_t)g * sc.W + word];
     int a = -1;
     if (bits >> (t & 31) & 1u) {
@@ -122,7 +114,7 @@ __global__ void __launch_bounds__(256) fill_layout_kernel(const int32_t* __restr
     }
     L.al[(size_t)g * T + t] = a;
   }
-  for (int j = 0; j < k; ++j) {
+  for (int j = warp; j < k; j += WORD_WARPS) {
     const int e = __ldg(topk_idx + (size_t)t * k + j);
     if (e < 0 || e >= E) {          // unused slot (sparse top-k), or an index build_masks_kernel reported
       L.pair_row[(size_t)t * k + j] = -1;
@@ -305,12 +297,13 @@ __global__ void __launch_bounds__(ONE_THREADS) layout_one_kernel(int32_t* topk_i
 }
 
 // Eight blocks write the G x T table of allocated rows and the T x k ones, so the one kernel is the better form while there are few
-// entries: microseconds of both, fitted to 1 to 32768 tokens, top-1 to top-32, 1 to 1024 groups.  Four kernels / one, us: 32768 tokens
-// top-1, 1 group 12.3 / 15.1, 8 groups 15.5 / 24.8, 104 groups 40.5 / 143; 16384 tokens top-2, 1 group 12.6 / 14.0, 32 groups 24.5 / 36.6;
-// 8192 tokens top-4, 8 groups 17.7 / 14.6, 64 groups 38.6 / 35.3, 256 groups 81 / 96; 4096 tokens top-8, 256 groups 93 / 57.
+// entries: microseconds of both, fitted to 1 to 32768 tokens, top-1 to top-32, 1 to 1024 groups (a warp of the four kernels walks every
+// eighth slot and group).  Four kernels / one, us: 32768 tokens top-1, 1 group 12.2 / 15.1, 104 groups 16.3 / 143; 12000 top-2, 4 groups
+// 9.0 / 12.6; 4096 top-8, 32 groups 11.0 / 16.5; 5000 top-6, 16 groups 9.8 / 15.2; 3001 top-4, 8 groups 10.7 / 8.2; 2050 top-8, 8 groups
+// 11.1 / 9.3; 1777 top-4, 8 groups 10.3 / 6.5; 600 top-2, 8 groups 12.2 / 4.9.
 bool layout_in_one(const Shape& s) {
   if (s.T <= 0 || (long long)s.T * s.k > ONE_MAX_PAIRS || one_shape(s, false).smem > ONE_MAX_SMEM) return false;
-  const double one = 5.0 + s.T * (4.2 + 1.7 * s.k + 0.62 * s.G) / 16384, four = 9.5 + 1.2 * s.k + 0.25 * s.G;
+  const double one = 5.0 + s.T * (4.2 + 1.7 * s.k + 0.62 * s.G) / 16384, four = 9.0 + (s.k + 7) / 8 + 0.45 * ((s.G + 7) / 8) + 3.2e-5 * s.T * s.k;
   return one < four;
 }
 
@@ -346,20 +339,12 @@ cudaError_t launch_topk_layout(const Shape& s, const float* logits, const float*
 __global__ void __launch_bounds__(1024) tile_prefix_kernel(const int32_t* __restrict__ expert_counts,
                                                            int32_t* mt_prefix, int32_t* mp_prefix, int E) {
   grid_dependency_sync();
-  __shared__ int buf[2][1024];
+  __shared__ int sums[2][32];
   const int i = threadIdx.x;
   const int c = (i < E) ? expert_counts[i] : 0;
-  buf[0][i] = (c + 127) >> 7;
-  buf[1][i] = (c + 255) >> 8;
-  __syncthreads();
-  for (int off = 1; off < 1024; off <<= 1) {
-    int a = 0, b = 0;
-    if (i >= off) { a = buf[0][i - off]; b = buf[1][i - off]; }
-    __syncthreads();
-    buf[0][i] += a; buf[1][i] += b;
-    __syncthreads();
-  }
-  if (i < E) { mt_prefix[i + 1] = buf[0][i]; mp_prefix[i + 1] = buf[1][i]; }
+  int v[2] = {(c + 127) >> 7, (c + 255) >> 8};
+  block_scan(v, sums);
+  if (i < E) { mt_prefix[i + 1] = v[0]; mp_prefix[i + 1] = v[1]; }
   if (i == 0) { mt_prefix[0] = 0; mp_prefix[0] = 0; }
 }
 
@@ -376,8 +361,8 @@ cudaError_t launch_layout(const Shape& s, const int32_t* topk_idx, const Layout&
   if (!masks_cleared &&
       (err = cudaMemsetAsync(sc.emask, 0, sizeof(uint32_t) * (size_t)(s.E + s.G) * sc.W, st)) != cudaSuccess)
     return err;  // emask and gmask are adjacent
-  const int tb = (s.T + 255) / 256;
-  if (s.T > 0 && (err = launch_pdl(build_masks_kernel, tb, 256, 0, st, topk_idx, sc.emask, sc.gmask, s.T, s.E, s.k,
+  const int words = (s.T + 31) / 32;
+  if (s.T > 0 && (err = launch_pdl(build_masks_kernel, words, WORD_WARPS * 32, 0, st, topk_idx, sc.emask, sc.gmask, s.T, s.E, s.k,
                                    m, sc.W, status, (s.flags & 4) ? 1 : 0)) != cudaSuccess)
     return err;
   if ((err = launch_pdl(scan_masks_kernel, s.E + s.G, 256, 0, st, sc.emask, sc.gmask, sc.eprefix, sc.gprefix,
@@ -386,7 +371,7 @@ cudaError_t launch_layout(const Shape& s, const int32_t* topk_idx, const Layout&
   if ((err = launch_pdl(offsets_kernel, 1, 1024, 0, st, L.expert_counts, L.group_counts, L.expert_offsets,
                         L.group_offsets, sc.mt_prefix, sc.mp_prefix, s.E, s.G)) != cudaSuccess)
     return err;
-  if (s.T > 0) return launch_pdl(fill_layout_kernel, tb, 256, 0, st, topk_idx, L, sc, s.T, s.E, s.k, s.G, m);
+  if (s.T > 0) return launch_pdl(fill_layout_kernel, words, WORD_WARPS * 32, 0, st, topk_idx, L, sc, s.T, s.E, s.k, s.G, m);
   return cudaSuccess;
 }
 
