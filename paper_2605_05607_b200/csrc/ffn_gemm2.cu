@@ -385,13 +385,13 @@ ffn_gemm2_kernel(const __grid_constant__ CUtensorMap map_b0, const __grid_consta
         const uint32_t dst = smem_base + NST * STAGE_BYTES + (quarter * 32 + lane) * 128;
 #pragma unroll
         for (int c = 0; c < 2; ++c) {
-          uint32_t lo[32], hi[32];
-          ptx::tmem_ld32(taddr + c * 64, lo);
-          ptx::tmem_ld32(taddr + c * 64 + 32, hi);
           if (c == 0) {   // the stores of the last tile have read theirs
             if (threadIdx.x == 0) ptx::bulk_wait_read();
             ptx::named_barrier(1, EPI_WARPS * 32);
           }
+          uint32_t lo[32], hi[32];
+          ptx::tmem_ld32(taddr + c * 64, lo);
+          ptx::tmem_ld32(taddr + c * 64 + 32, hi);
           ptx::tmem_ld_wait_on(lo, hi);
           if (t.kb == 0) {   // an expert without rows: the accumulator was never written
 #pragma unroll
