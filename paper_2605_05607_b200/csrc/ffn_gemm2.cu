@@ -213,7 +213,8 @@ ffn_gemm2_kernel(const __grid_constant__ CUtensorMap map_b0, const __grid_consta
       ptx::st_shared_v4(stage + lane * 64 + ((v ^ ((lane >> 1) & 3)) << 4), q0, q1, q2, q3);
     };
     int tl = 0;
-    for (int w = cluster_id; w < total && !*abort_flag; w += num_clusters, ++tl) {
+    // (TILE_OUT: the eight warps meet in every tile, so they leave the loop together, by the vote below and not one by one)
+    for (int w = cluster_id; w < total && (TILE_OUT || !*abort_flag); w += num_clusters, ++tl) {
       const Tile t = tile_of(w);
       const int buf = tl & 1;
       // 128-row halves: rows 32 quarter + lane, columns `half`.  64-row halves: rows 32 (quarter & 1) + lane, columns quarter >> 1,
@@ -235,7 +236,15 @@ ffn_gemm2_kernel(const __grid_constant__ CUtensorMap map_b0, const __grid_consta
                            : make_uint4(0u, 0u, 0u, 0u);
           }
       }
-      if (!ptx::mbar_wait_warp<false, HINT>(tfull_bar(buf), (tl >> 1) & 1, abort_flag, global_abort)) { timeout(1); break; }
+      bool go = ptx::mbar_wait_warp<false, HINT>(tfull_bar(buf), (tl >> 1) & 1, abort_flag, global_abort);
+      if (!go) timeout(1);
+      if (TILE_OUT) {
+        // Whether a warp's wait ended with the tile or with an abort is a race, and the barriers of the tile want all eight: one vote.
+        // Each of them gets here in bounded time, and those that go on leave the tile's second barrier together.
+        if (threadIdx.x == 0) ptx::bulk_wait_read();   // the stores of the last tile have read theirs
+        go = ptx::named_barrier_all(1, EPI_WARPS * 32, go && !*abort_flag);
+      }
+      if (!go) break;
       ptx::tc_fence_after();
       const int lrow = row_w + lane;
       const bool valid = lrow < t.rows;
@@ -385,10 +394,6 @@ ffn_gemm2_kernel(const __grid_constant__ CUtensorMap map_b0, const __grid_consta
         const uint32_t dst = smem_base + NST * STAGE_BYTES + (quarter * 32 + lane) * 128;
 #pragma unroll
         for (int c = 0; c < 2; ++c) {
-          if (c == 0) {   // the stores of the last tile have read theirs
-            if (threadIdx.x == 0) ptx::bulk_wait_read();
-            ptx::named_barrier(1, EPI_WARPS * 32);
-          }
           uint32_t lo[32], hi[32];
           ptx::tmem_ld32(taddr + c * 64, lo);
           ptx::tmem_ld32(taddr + c * 64 + 32, hi);
