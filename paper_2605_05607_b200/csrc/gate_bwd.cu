@@ -37,8 +37,8 @@ __global__ void __launch_bounds__(256) gate_rowdot_kernel(const float* __restric
   }
 }
 
-// Key gradients of a token's k pairs, one lane each (`width` lanes per token, k rounded up to a power of two); written per pair (dkey) and in
-// place per padded row (g_row).  Latency of two dependent reads; a thread per token walked its slots one after the other (8192 tokens
+// Key gradients of a token's k pairs, one lane each (1 << shift lanes per token, k rounded up to a power of two, so that their number can pass
+// 2^31 where that of the pairs does not); written per pair (dkey) and in place per padded row (g_row).  Latency of two dependent reads; a thread per token walked its slots one after the other (8192 tokens
 // top-8 22 -> 5 us; the sums have the same order).
 __global__ void __launch_bounds__(256) gate_route_bwd_kernel(const int32_t* __restrict__ topk_idx,
                                                              const float* __restrict__ topk_w,
@@ -46,9 +46,10 @@ __global__ void __launch_bounds__(256) gate_route_bwd_kernel(const int32_t* __re
                                                              const float* __restrict__ logits,
                                                              const float* __restrict__ bias, long long bias_stride,
                                                              float* g_row, float* __restrict__ dkey, int T, int E, int k,
-                                                             int sigmoid, int n_rows, int width) {
+                                                             int sigmoid, int n_rows, int shift) {
   grid_dependency_sync();
-  const int at = blockIdx.x * blockDim.x + threadIdx.x, t = at / width, j = at % width;
+  const long long at = (long long)blockIdx.x * blockDim.x + threadIdx.x, t = at >> shift;
+  const int width = 1 << shift, j = (int)at & (width - 1);
   const bool slot = t < T && j < k;
   const size_t pair = (size_t)t * k + j;
   const int r = slot ? __ldg(pair_prow + pair) : -1;
@@ -195,11 +196,11 @@ cudaError_t launch_gate_backward(const Shape& s, const GateBwdArgs& a, cudaStrea
   if ((err = launch_pdl(gate_rowdot_kernel, blocks, 256, 0, st, a.row_dots, bwd_dot_parts(s), (long long)n_rows, a.poff, a.g_row,
                         s.E)) != cudaSuccess)
     return err;
-  int width = 1;
-  while (width < s.k) width *= 2;
-  if ((err = launch_pdl(gate_route_bwd_kernel, (unsigned)(((long long)s.T * width + 255) / 256), 256, 0, st, a.topk_idx, a.topk_w, a.pair_prow,
+  int shift = 0;
+  while (1 << shift < s.k) ++shift;
+  if ((err = launch_pdl(gate_route_bwd_kernel, (unsigned)((((long long)s.T << shift) + 255) / 256), 256, 0, st, a.topk_idx, a.topk_w, a.pair_prow,
                         a.logits, a.bias, (long long)a.bias_stride, a.g_row, a.dkey, s.T, s.E, s.k,
-                        s.score_fn == 1 ? 1 : 0, n_rows, width)) != cudaSuccess)
+                        s.score_fn == 1 ? 1 : 0, n_rows, shift)) != cudaSuccess)
     return err;
   long long tiles = (long long)s.T * s.k / DW_ROWS + s.E;   // at most; the count is on the device
   if (tiles > 16384) tiles = 16384;

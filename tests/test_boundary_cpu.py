@@ -3,6 +3,7 @@ declares, sizes its workspace sensibly and rejects bad arguments before touching
 import ctypes
 import os
 import re
+import subprocess
 
 import pytest
 import torch
@@ -217,6 +218,30 @@ def test_every_tensor_memory_load_is_waited_for_by_name():
                 pending -= set(wait.group(1).replace(" ", "").split(","))
             elif code and not code.startswith(("#pragma", "for (int t = 1; t < 3")):
                 assert not pending, f"{fn}: {pending} used before a wait that names them: {code}"
+
+
+def test_gate_gradient_finds_its_slot_at_the_largest_shapes(tmp_path):
+    """The lanes of a token are k rounded up to a power of two, so an accepted shape (T k < 2^31) has up to nearly 2^32 of them.  The lines of
+    the kernel that turn a thread into its token and slot, compiled for the CPU, at the ends of the first, a middle and the last token."""
+    text = open(os.path.join(ROOT, "paper_2605_05607_b200", "csrc", "gate_bwd.cu")).read()
+    body = text[text.index("gate_route_bwd_kernel("):]
+    lines = re.search(r"grid_dependency_sync\(\);\n(.*?)\n  const bool slot = ([^;]*);", body, re.S)
+    scale = re.search(r"int (shift|width)\) \{", body).group(1)           # what the kernel is told of the lanes per token
+    src = tmp_path / "slot.cpp"
+    src.write_text("struct Dim { unsigned x; };\n"
+                   f"extern \"C\" int slot_of(unsigned block, unsigned threads, unsigned thread, int T, int k, int {scale}, long long* out) {{\n"
+                   "  const Dim blockIdx{block}, blockDim{threads}, threadIdx{thread};\n"
+                   f"{lines.group(1)}\n  out[0] = t;\n  out[1] = j;\n  return {lines.group(2)};\n}}\n")
+    subprocess.run(["g++", "-shared", "-fPIC", "-fwrapv", "-o", str(tmp_path / "slot.so"), str(src)], check=True)
+    fn = ctypes.CDLL(str(tmp_path / "slot.so")).slot_of
+    out = (ctypes.c_longlong * 2)()
+    for k in (1, 2, 3, 8, 9, 16, 17, 31, 32):
+        T, shift = (2 ** 31 - 1) // k, (k - 1).bit_length()
+        for t in (0, T // 2, T - 1, T):
+            for j in (0, k - 1, (1 << shift) - 1):
+                block, thread = divmod((t << shift) + j, 256)
+                inside = fn(block, 256, thread, T, k, shift if scale == "shift" else 1 << shift, out)
+                assert tuple(out) == (t, j) and bool(inside) == (t < T and j < k), (T, k, t, j, tuple(out))
 
 
 def enclosing_blocks(text, at):
