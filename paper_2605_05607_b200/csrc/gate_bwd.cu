@@ -143,8 +143,12 @@ __global__ void __launch_bounds__(256) gate_finish_kernel(const float* __restric
   }
 }
 
-// dx[t, :] += sum_j dkey[t, j] * wgt[e_j, :]; a warp per token, four columns per lane and step, four slots in flight (8192 tokens top-8 of
-// d = 4096 145 -> 124 us)
+// dx[t, :] += sum_j dkey[t, j] * wgt[e_j, :]; a warp per token, four columns per lane and step.  Few tokens are bound by the latency of the
+// reads: FOUR has the rows of four slots in flight (48 registers per thread).  Many tokens hide it by their number: the plain loop
+// takes 32 registers, so that the SM is full of warps.  Whole gate gradient, us, plain / four in flight: 320 tokens top-4 of d = 1896 52.7 /
+// 45.6, 1000 top-8 of d = 4096 124 / 97, 1000 top-1 of d = 2048 44.0 / 44.3, 3001 top-4 of d = 2880 93 / 84, 4096 top-2 of d = 4096 100 / 96,
+// 8192 top-8 of d = 2048 111 / 121, of d = 4096 240 / 237, 16384 top-4 of d = 1024 85 / 96.  Same sums, same order.
+template <bool FOUR>
 __global__ void __launch_bounds__(256) gate_dx_kernel(const int32_t* __restrict__ topk_idx, const float* __restrict__ dkey,
                                                       const float* __restrict__ wgt, __nv_bfloat16* dx, int T, int E,
                                                       int k, int d) {
@@ -164,14 +168,27 @@ __global__ void __launch_bounds__(256) gate_dx_kernel(const int32_t* __restrict_
     __nv_bfloat16* row = dx + (size_t)t * d;
     for (int c = lane * 4; c < d; c += 128) {
       float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
-#pragma unroll 4
-      for (int j = 0; j < k; ++j) {
+      auto row_of = [&](int j) { return __ldg(reinterpret_cast<const float4*>(wgt + (size_t)s_e[wid][j] * d + c)); };
+      auto add = [&](int j, const float4& wv) {
         const float g = s_g[wid][j];
-        const float4 wv = __ldg(reinterpret_cast<const float4*>(wgt + (size_t)s_e[wid][j] * d + c));
         acc.x = fmaf(g, wv.x, acc.x);
         acc.y = fmaf(g, wv.y, acc.y);
         acc.z = fmaf(g, wv.z, acc.z);
         acc.w = fmaf(g, wv.w, acc.w);
+      };
+      if (FOUR) {
+        for (int j = 0; j < k; j += 4) {
+          float4 wv[4];
+#pragma unroll
+          for (int q = 0; q < 4; ++q)
+            if (j + q < k) wv[q] = row_of(j + q);
+#pragma unroll
+          for (int q = 0; q < 4; ++q)
+            if (j + q < k) add(j + q, wv[q]);
+        }
+      } else {
+#pragma unroll 4
+        for (int j = 0; j < k; ++j) add(j, row_of(j));
       }
       uint2 raw = *reinterpret_cast<const uint2*>(row + c);
       __nv_bfloat162* p2 = reinterpret_cast<__nv_bfloat162*>(&raw);
@@ -212,8 +229,10 @@ cudaError_t launch_gate_backward(const Shape& s, const GateBwdArgs& a, cudaStrea
                         static_cast<const float*>(a.part), a.mt_prefix, a.dw_gate, a.w_gate, a.wgt, s.d, s.E)) != cudaSuccess)
     return err;
   blocks = (s.T + 7) / 8;
+  // five blocks of the form with more registers fit an SM: it is taken while all of its blocks are resident
+  const auto dx = blocks <= 5 * sm_count() ? gate_dx_kernel<true> : gate_dx_kernel<false>;
   if (blocks > cap) blocks = cap;
-  return launch_pdl(gate_dx_kernel, blocks, 256, 0, st, a.topk_idx, static_cast<const float*>(a.dkey),
+  return launch_pdl(dx, blocks, 256, 0, st, a.topk_idx, static_cast<const float*>(a.dkey),
                     static_cast<const float*>(a.wgt), static_cast<__nv_bfloat16*>(a.dx), s.T, s.E, s.k, s.d);
 }
 

@@ -387,6 +387,51 @@ def test_gradients_of_ragged_rows_take_no_longer():
     assert us <= 1.3 * other
 
 
+def gate_gradient(cfg):
+    """The gate gradient of a batch whose expert gradients are there; the call, and dx as the experts left it."""
+    bw = Backward(cfg)
+    bw()
+    r = bw.run
+    dx, dw_gate = bw.dx.clone(), torch.empty(cfg.d, cfg.E, device="cuda")
+    return bw, dx, lambda: B.moe_gate_backward(r.shape, r.logits, r.t["bias"], r.idx, r.w, r.lay, r.t["w_gate"], bw.dx, dw_gate, bw.ws)
+
+
+@pytest.mark.parametrize("k", [1, 3, 4, 6, 9])
+def test_gate_gradient_of_few_and_many_tokens_gives_the_same_bits(k):
+    """Up to five blocks of eight tokens per SM the rows of four slots are in flight, beyond that one after the other."""
+    T = 5 * torch.cuda.get_device_properties(0).multi_processor_count * 8
+    out = []
+    for n in (T + 1, T):
+        bw = Backward(synth.MoEConfig("dx", T=n, d=136, f=16, E=16, k=k, G=1, seed=k))
+        t = bw.run.t
+        if out:
+            t["x"].copy_(first.run.t["x"][:n])
+            bw.dy.copy_(first.dy[:n])
+            for name in ("w_gate", "w1", "w3", "w2"):
+                t[name].copy_(first.run.t[name])
+            bw.run.route()
+            bw.run.dispatch()
+        else:
+            first = bw
+        bw()
+        before = bw.dx.clone()
+        r = bw.run
+        B.moe_gate_backward(r.shape, r.logits, t["bias"], r.idx, r.w, r.lay, t["w_gate"], bw.dx, torch.empty(136, 16, device="cuda"), bw.ws)
+        assert k == 1 or not torch.equal(bw.dx, before)      # a single slot's weight is constant
+        out.append(bw.dx[:T])
+    assert torch.equal(*out)
+
+
+def test_gate_gradient_of_few_tokens_is_no_chain_of_reads():
+    """An eighth of the tokens leave the GPU mostly idle; the rows of their slots have to be in flight together."""
+    def call(T):
+        return gate_gradient(synth.MoEConfig("dx", T=T, d=4096, f=256, E=64, k=8, G=1))[2]
+
+    # measured, taking turns: 0.40; with the slots one after the other 0.52.  The line lies in the middle.
+    us, other = H.device_us(call(1000), call(8000))
+    assert us <= 0.46 * other
+
+
 @pytest.mark.parametrize("d,f", [(16, 144), (256, 512), (272, 528), (400, 1040)])
 def test_weight_gradients_leave_alike_by_tma_and_by_the_warps(d, f):
     """An average of fewer than 192 rows per expert decides how the tiles of the gradients are stored.  One expert with 191 tokens, and with a
