@@ -242,7 +242,7 @@ ffn_gemm2_kernel(const __grid_constant__ CUtensorMap map_b0, const __grid_consta
         // Whether a warp's wait ended with the tile or with an abort is a race, and the barriers of the tile want all eight: one vote.
         // Each of them gets here in bounded time, and those that go on leave the tile's second barrier together.
         if (threadIdx.x == 0) ptx::bulk_wait_read();   // the stores of the last tile have read theirs
-        go = ptx::named_barrier_all(1, EPI_WARPS * 32, go && !*abort_flag);
+        go = ptx::named_barrier_all(1, EPI_WARPS * 32, go);
       }
       if (!go) break;
       ptx::tc_fence_after();
