@@ -77,7 +77,8 @@ constexpr uint32_t HINT = 4000;   // try_wait suspend-time hint (ns), see ptx::m
 //                 256 x 256 tile of one expert's gradient (p.K = its row count M, p.N its columns), the K walk runs over
 //                 the expert's rows in blocks of 64, both operands are MN-major boxes of 64 columns x 64 rows; CTA `rank`
 //                 holds rows m0 + 128 * rank of the tile and columns n0 + 128 * rank of B
-//                 TILE_OUT: the tile goes through shared memory and leaves by TMA (map_b1: dW), instead of warp by warp.
+//                 OUT > 0: the tile goes through shared memory, in the last OUT stages of the ring, and leaves by TMA (map_b1: dW), instead
+//                 of warp by warp.
 //   PAIR_KSPLIT   acc = A0 . B0 + A1 . B1 (dX = dA1 . W1^T + dA3 . W3^T): the first p.k_split k-blocks come from
 //                 (rows.a0, map_b0), the rest from (rows.a1, map_b1); plain epilogue
 // BKMAJ: the bf16 weight operand is read K-major (one box of 128 columns x 64 K per CTA and stage), which is how
@@ -90,15 +91,16 @@ enum { PAIR_PLAIN = 0, PAIR_GLU = 1, PAIR_GLU_BWD = 2, PAIR_KSPLIT = 3, PAIR_WGR
 // the padded UMMAs themselves are the bound.
 struct RowMaps { CUtensorMap a0[4], a1[4]; };
 
-template <bool RED, bool FP8, int MODE, bool BKMAJ, bool TILE_OUT>
+template <bool RED, bool FP8, int MODE, bool BKMAJ, int OUT>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(THREADS, 1)
 ffn_gemm2_kernel(const __grid_constant__ CUtensorMap map_b0, const __grid_constant__ CUtensorMap map_b1,
                  const __grid_constant__ RowMaps rows, const GemmParams p) {
   constexpr bool GLU = MODE == PAIR_GLU || MODE == PAIR_GLU_BWD;
   constexpr bool KMAJ = FP8 || BKMAJ;   // the weight operand is K-major in shared memory
-  constexpr int NST = TILE_OUT ? NSTAGE - 2 : NSTAGE;   // the last two stages hold the tile on its way out
+  constexpr bool TILE_OUT = OUT > 0;
+  constexpr int NST = NSTAGE - OUT;
   static_assert(!TILE_OUT || MODE == PAIR_WGRAD, "whole tiles leave by TMA in the weight gradients only");
-  static_assert(4 * BOX_BYTES <= 2 * STAGE_BYTES, "the CTA's part of a tile");
+  static_assert(2 * BOX_BYTES == STAGE_BYTES && OUT <= 2, "four boxes are the CTA's part of a tile");
   static_assert(!(MODE != PAIR_PLAIN && (RED || FP8)), "only the plain form has the reducing / FP8 variants");
   constexpr int BN_OUT = GLU ? 128 : 256;
   extern __shared__ uint8_t smem_raw[];
@@ -213,7 +215,11 @@ ffn_gemm2_kernel(const __grid_constant__ CUtensorMap map_b0, const __grid_consta
       ptx::st_shared_v4(stage + lane * 64 + ((v ^ ((lane >> 1) & 3)) << 4), q0, q1, q2, q3);
     };
     int tl = 0;
-    // (TILE_OUT: the eight warps meet in every tile, so they leave the loop together, by the vote below and not one by one)
+    // TILE_OUT: all eight warps (OUT = 2) or the four of a column half meet in every tile, so they leave the loop together, by the vote below
+    // and not one by one.
+    constexpr int MEET = EPI_WARPS * 32 / (OUT == 1 ? 2 : 1);
+    const int meet_id = 1 + threadIdx.x / MEET;
+    const bool leader = threadIdx.x % MEET == 0;
     for (int w = cluster_id; w < total && (TILE_OUT || !*abort_flag); w += num_clusters, ++tl) {
       const Tile t = tile_of(w);
       const int buf = tl & 1;
@@ -239,10 +245,10 @@ ffn_gemm2_kernel(const __grid_constant__ CUtensorMap map_b0, const __grid_consta
       bool go = ptx::mbar_wait_warp<false, HINT>(tfull_bar(buf), (tl >> 1) & 1, abort_flag, global_abort);
       if (!go) timeout(1);
       if (TILE_OUT) {
-        // Whether a warp's wait ended with the tile or with an abort is a race, and the barriers of the tile want all eight: one vote.
-        // Each of them gets here in bounded time, and those that go on leave the tile's second barrier together.
-        if (threadIdx.x == 0) ptx::bulk_wait_read();   // the stores of the last tile have read theirs
-        go = ptx::named_barrier_all(1, EPI_WARPS * 32, go);
+        // Whether a warp's wait ended with the tile or with an abort is a race, and the barriers of the tile want all of them: one vote.
+        // Each gets here in bounded time, and those that go on leave the tile's last barrier together.
+        if (leader) ptx::bulk_wait_read();   // the stores of the last tile have read theirs
+        go = ptx::named_barrier_all(meet_id, MEET, go);
       }
       if (!go) break;
       ptx::tc_fence_after();
@@ -388,7 +394,41 @@ ffn_gemm2_kernel(const __grid_constant__ CUtensorMap map_b0, const __grid_consta
             }
           }
         }
-      } else if (TILE_OUT) {
+      } else if (OUT == 1) {
+        // As below, in boxes of 64 columns of which a column half has one place: its warps fill the second box when the store of the first has
+        // read it.
+        const uint32_t box = smem_base + NST * STAGE_BYTES + half * BOX_BYTES, dst = box + (quarter * 32 + lane) * 128;
+#pragma unroll
+        for (int c = 0; c < 2; ++c) {
+          uint32_t lo[32], hi[32];
+          ptx::tmem_ld32(taddr + c * 64, lo);
+          ptx::tmem_ld32(taddr + c * 64 + 32, hi);
+          ptx::tmem_ld_wait_on(lo, hi);
+          if (t.kb == 0) {   // an expert without rows: the accumulator was never written
+#pragma unroll
+            for (int j = 0; j < 32; ++j) lo[j] = hi[j] = 0u;
+          }
+          uint32_t q[32];
+#pragma unroll
+          for (int j = 0; j < 16; ++j) {
+            q[j] = pack2(__uint_as_float(lo[2 * j]), __uint_as_float(lo[2 * j + 1]));
+            q[16 + j] = pack2(__uint_as_float(hi[2 * j]), __uint_as_float(hi[2 * j + 1]));
+          }
+          if (c > 0) {
+            if (leader) ptx::bulk_wait_read();
+            ptx::named_barrier(meet_id, MEET);
+          }
+#pragma unroll
+          for (int v = 0; v < 8; ++v) ptx::st_shared_v4(dst + ((v ^ (lane & 7)) << 4), q[v * 4], q[v * 4 + 1], q[v * 4 + 2], q[v * 4 + 3]);
+          ptx::fence_proxy_async_smem();
+          ptx::named_barrier(meet_id, MEET);
+          const int col = t.n0 + half * 128 + c * 64;
+          if (leader && t.rows > 0 && col < p.N) {
+            ptx::tma_store_3d(&map_b1, box, col, t.out_row0 - t.e * p.K, t.e);
+            ptx::bulk_commit();
+          }
+        }
+      } else if (OUT == 2) {
         // The CTA's 128 x 256 part of the tile through shared memory, four boxes of 64 columns in the layout of a 128-byte swizzle, and
         // out by TMA, which clips at the edges of dW[e].
         const uint32_t dst = smem_base + NST * STAGE_BYTES + (quarter * 32 + lane) * 128;
@@ -411,8 +451,8 @@ ffn_gemm2_kernel(const __grid_constant__ CUtensorMap map_b0, const __grid_consta
           }
         }
         ptx::fence_proxy_async_smem();
-        ptx::named_barrier(1, EPI_WARPS * 32);
-        if (threadIdx.x == 0 && t.rows > 0) {
+        ptx::named_barrier(meet_id, MEET);
+        if (leader && t.rows > 0) {
 #pragma unroll
           for (int c = 0; c < 4; ++c)
             if (t.n0 + c * 64 < p.N)
@@ -450,7 +490,7 @@ ffn_gemm2_kernel(const __grid_constant__ CUtensorMap map_b0, const __grid_consta
       // (K = 512: 860 -> 1049 TFLOP/s with the relaxed form)
       if (lane == 0) ptx::mbar_arrive_cluster_relaxed(ptx::mapa(tempty_bar(buf), 0));
     }
-    if (TILE_OUT && threadIdx.x == 0) ptx::bulk_wait();
+    if (TILE_OUT && leader) ptx::bulk_wait();
   } else if (warp == TMA_WARP) {
     // ================================ TMA producer (both CTAs) ================================
     if (lane == 0) {
@@ -572,7 +612,7 @@ int pair_grid() {
     attr.val.clusterDim.z = 1;
     cfg.attrs = &attr;
     cfg.numAttrs = 1;
-    if (cudaOccupancyMaxActiveClusters(&clusters, ffn_gemm2_kernel<false, false, PAIR_PLAIN, false, false>, &cfg) != cudaSuccess || clusters <= 0) {
+    if (cudaOccupancyMaxActiveClusters(&clusters, ffn_gemm2_kernel<false, false, PAIR_PLAIN, false, 0>, &cfg) != cudaSuccess || clusters <= 0) {
       (void)cudaGetLastError();
       clusters = sm_count() / 2;
     }
@@ -591,16 +631,17 @@ cudaError_t set_pair_attributes() {
   const int dev = current_device();
   if (!attr_set[dev].load(std::memory_order_acquire)) {
     const auto attr = cudaFuncAttributeMaxDynamicSharedMemorySize;
-    cudaError_t e = cudaFuncSetAttribute(ffn_gemm2_kernel<false, false, PAIR_PLAIN, false, false>, attr, SMEM_BYTES);
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(ffn_gemm2_kernel<true, false, PAIR_PLAIN, false, false>, attr, SMEM_BYTES);
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(ffn_gemm2_kernel<false, true, PAIR_PLAIN, false, false>, attr, SMEM_BYTES);
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(ffn_gemm2_kernel<true, true, PAIR_PLAIN, false, false>, attr, SMEM_BYTES);
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(ffn_gemm2_kernel<false, false, PAIR_GLU, false, false>, attr, SMEM_BYTES);
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(ffn_gemm2_kernel<false, false, PAIR_PLAIN, true, false>, attr, SMEM_BYTES);
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(ffn_gemm2_kernel<false, false, PAIR_GLU_BWD, false, false>, attr, SMEM_BYTES);
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(ffn_gemm2_kernel<false, false, PAIR_KSPLIT, true, false>, attr, SMEM_BYTES);
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(ffn_gemm2_kernel<false, false, PAIR_WGRAD, false, false>, attr, SMEM_BYTES);
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(ffn_gemm2_kernel<false, false, PAIR_WGRAD, false, true>, attr, SMEM_BYTES);
+    cudaError_t e = cudaFuncSetAttribute(ffn_gemm2_kernel<false, false, PAIR_PLAIN, false, 0>, attr, SMEM_BYTES);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(ffn_gemm2_kernel<true, false, PAIR_PLAIN, false, 0>, attr, SMEM_BYTES);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(ffn_gemm2_kernel<false, true, PAIR_PLAIN, false, 0>, attr, SMEM_BYTES);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(ffn_gemm2_kernel<true, true, PAIR_PLAIN, false, 0>, attr, SMEM_BYTES);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(ffn_gemm2_kernel<false, false, PAIR_GLU, false, 0>, attr, SMEM_BYTES);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(ffn_gemm2_kernel<false, false, PAIR_PLAIN, true, 0>, attr, SMEM_BYTES);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(ffn_gemm2_kernel<false, false, PAIR_GLU_BWD, false, 0>, attr, SMEM_BYTES);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(ffn_gemm2_kernel<false, false, PAIR_KSPLIT, true, 0>, attr, SMEM_BYTES);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(ffn_gemm2_kernel<false, false, PAIR_WGRAD, false, 0>, attr, SMEM_BYTES);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(ffn_gemm2_kernel<false, false, PAIR_WGRAD, false, 1>, attr, SMEM_BYTES);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(ffn_gemm2_kernel<false, false, PAIR_WGRAD, false, 2>, attr, SMEM_BYTES);
     if (e != cudaSuccess) return e;
     attr_set[dev].store(true, std::memory_order_release);
   }
@@ -626,11 +667,11 @@ cudaError_t launch_gemm2(const GemmParams& p, const CUtensorMap& m_w2, bool fp8,
   const bool red = p.y_acc != nullptr;
   const int g = pair_grid();
   if (fp8) {
-    if (red) return launch_pdl(ffn_gemm2_kernel<true, true, PAIR_PLAIN, false, false>, g, THREADS, SMEM_BYTES, st, m_w2, m_w2, rows, p);
-    return launch_pdl(ffn_gemm2_kernel<false, true, PAIR_PLAIN, false, false>, g, THREADS, SMEM_BYTES, st, m_w2, m_w2, rows, p);
+    if (red) return launch_pdl(ffn_gemm2_kernel<true, true, PAIR_PLAIN, false, 0>, g, THREADS, SMEM_BYTES, st, m_w2, m_w2, rows, p);
+    return launch_pdl(ffn_gemm2_kernel<false, true, PAIR_PLAIN, false, 0>, g, THREADS, SMEM_BYTES, st, m_w2, m_w2, rows, p);
   }
-  if (red) return launch_pdl(ffn_gemm2_kernel<true, false, PAIR_PLAIN, false, false>, g, THREADS, SMEM_BYTES, st, m_w2, m_w2, rows, p);
-  return launch_pdl(ffn_gemm2_kernel<false, false, PAIR_PLAIN, false, false>, g, THREADS, SMEM_BYTES, st, m_w2, m_w2, rows, p);
+  if (red) return launch_pdl(ffn_gemm2_kernel<true, false, PAIR_PLAIN, false, 0>, g, THREADS, SMEM_BYTES, st, m_w2, m_w2, rows, p);
+  return launch_pdl(ffn_gemm2_kernel<false, false, PAIR_PLAIN, false, 0>, g, THREADS, SMEM_BYTES, st, m_w2, m_w2, rows, p);
 }
 
 // GEMM-1 on CTA pairs from the expert-sorted activation rows (p.a_src = xs); p.tile_prefix = the 256-row pair-tile
@@ -641,7 +682,7 @@ cudaError_t launch_gemm1_pair(const GemmParams& p, const CUtensorMap& m_w1, cons
   RowMaps rows{};
   if (!make_row_maps(&rows, p, false)) return cudaErrorInvalidValue;
   ProfileScope prof(KID_GEMM1, st);
-  return launch_pdl(ffn_gemm2_kernel<false, false, PAIR_GLU, false, false>, pair_grid(), THREADS, SMEM_BYTES, st, m_w1, m_w3, rows, p);
+  return launch_pdl(ffn_gemm2_kernel<false, false, PAIR_GLU, false, 0>, pair_grid(), THREADS, SMEM_BYTES, st, m_w1, m_w3, rows, p);
 }
 
 // Backward pass, all on CTA pairs (see bwd.cu for the sequence):
@@ -653,21 +694,21 @@ cudaError_t launch_bwd_dh(const GemmParams& p, const CUtensorMap& m_w2t, cudaStr
   if (e != cudaSuccess) return e;
   RowMaps rows{};
   if (!make_row_maps(&rows, p, false)) return cudaErrorInvalidValue;
-  return launch_pdl(ffn_gemm2_kernel<false, false, PAIR_PLAIN, true, false>, pair_grid(), THREADS, SMEM_BYTES, st, m_w2t, m_w2t, rows, p);
+  return launch_pdl(ffn_gemm2_kernel<false, false, PAIR_PLAIN, true, 0>, pair_grid(), THREADS, SMEM_BYTES, st, m_w2t, m_w2t, rows, p);
 }
 cudaError_t launch_bwd_glu(const GemmParams& p, const CUtensorMap& m_w1, const CUtensorMap& m_w3, cudaStream_t st) {
   cudaError_t e = set_pair_attributes();
   if (e != cudaSuccess) return e;
   RowMaps rows{};
   if (!make_row_maps(&rows, p, false)) return cudaErrorInvalidValue;
-  return launch_pdl(ffn_gemm2_kernel<false, false, PAIR_GLU_BWD, false, false>, pair_grid(), THREADS, SMEM_BYTES, st, m_w1, m_w3, rows, p);
+  return launch_pdl(ffn_gemm2_kernel<false, false, PAIR_GLU_BWD, false, 0>, pair_grid(), THREADS, SMEM_BYTES, st, m_w1, m_w3, rows, p);
 }
 cudaError_t launch_bwd_dx(const GemmParams& p, const CUtensorMap& m_w1t, const CUtensorMap& m_w3t, cudaStream_t st) {
   cudaError_t e = set_pair_attributes();
   if (e != cudaSuccess) return e;
   RowMaps rows{};
   if (!make_row_maps(&rows, p, false)) return cudaErrorInvalidValue;
-  return launch_pdl(ffn_gemm2_kernel<false, false, PAIR_KSPLIT, true, false>, pair_grid(), THREADS, SMEM_BYTES, st, m_w1t, m_w3t, rows, p);
+  return launch_pdl(ffn_gemm2_kernel<false, false, PAIR_KSPLIT, true, 0>, pair_grid(), THREADS, SMEM_BYTES, st, m_w1t, m_w3t, rows, p);
 }
 
 // Weight gradient on CTA pairs: dw[e] = A_e^T . B_e, A = [rows, M], B = [rows, N] in the padded row space (maps with
@@ -690,18 +731,24 @@ cudaError_t launch_wgrad_pair(const CUtensorMap& m_a, const CUtensorMap& m_b, co
   rows.a0[3] = m_a;
   ProfileScope prof(KID_WGRAD, st);
   // Experts of few rows: the gradients are bound by their stores, and by what the stores take of the board's power; whole tiles leave by
-  // TMA then.  It takes two of the ring's stages and a barrier of the epilogue warps, which costs more than it gives where the tensor
-  // cores are the bound.  Ragged rows (they start inside a 32-byte sector) leave that way at any size: in pieces of 64 bytes twice as many
-  // sectors are written in two halves.  Training step, us, warps / TMA, by rows per expert: 94 skewed (128 x 2880 x 2880) 5220 / 5074, 125 (64
-  // x 2048 x 1024) 873 / 857, 125 (16 x 4096 x 4096) 1519 / 1469, 187 skewed (128 x 2880 x 2880) 7329 / 7278, 187 (64 x 2048 x 1024) 1119 / 1123,
-  // 250 (64 x 2048 x 1024) 1196 / 1213, 375 (128 x 2048 x 1024) 3011 / 3059; ragged: 19 (64 x 2888 x 2872) 3057 / 2703, 125 (64 x 2056 x 1032)
-  // 1116 / 1085, 1024 (32 x 2056 x 1032) 2411 / 2377.
-  if (rows_total < 192ll * E || (N & 15) != 0) {
+  // TMA then.  A tile on its way out takes two of the ring's six stages, or one, whose boxes are filled one after the other: up to 80 rows
+  // per expert the stores are all that counts, but four stages do not cover the latency of a long K walk, and with skewed routing the
+  // popular experts have one at any average.  Backward pass, us, by the warps / two stages / one stage, rows per expert in brackets, even and
+  // skewed routing: 128 x 2048 x 2048 (50) 1656 / 1611 / 1711, 1317 / 1283 / 1318; 128 x 2880 x 2880 (94) 4010 / 3810 / 3750, 4117 / 3977 / 3930; 128 x
+  // 1904 x 480 (100) 608 / 596 / 596, 597 / 616 / 589; 128 x 1024 x 512 (190) 430 / 433 / 424, 530 / 558 / 529; 128 x 4096 x 1536 (190) 3830 / 3773 /
+  // 3616, 4240 / 4384 / 4223.  From 192 rows on the tensor cores are the bound and the warps store.
+  // Ragged rows (they start inside a 32-byte sector) leave by TMA at any size: in pieces of 64 bytes twice as many sectors are written in
+  // two halves.  Boxes of neighbouring columns had better leave together there, so two stages are taken for longer where the gradient is large:
+  // 128 x 2888 x 2872 (100) two 4510 / one 4910, 4783 / 5330; 64 x 1896 x 480 (190) 419 / 410, 551 / 530.
+  const bool ragged = (N & 15) != 0;
+  if (rows_total < 192ll * E || ragged) {
     CUtensorMap m_dw;
     if (!make_store_map(&m_dw, dw, E, M, N)) return cudaErrorInvalidValue;
-    return launch_pdl(ffn_gemm2_kernel<false, false, PAIR_WGRAD, false, true>, pair_grid(), THREADS, SMEM_BYTES, st, m_b, m_dw, rows, p);
+    const bool two = rows_total < 80ll * E || (ragged && rows_total < 192ll * E && (long long)M * N >= 4000000);   // stages for the tile
+    const auto kernel = two ? ffn_gemm2_kernel<false, false, PAIR_WGRAD, false, 2> : ffn_gemm2_kernel<false, false, PAIR_WGRAD, false, 1>;
+    return launch_pdl(kernel, pair_grid(), THREADS, SMEM_BYTES, st, m_b, m_dw, rows, p);
   }
-  return launch_pdl(ffn_gemm2_kernel<false, false, PAIR_WGRAD, false, false>, pair_grid(), THREADS, SMEM_BYTES, st, m_b, m_b, rows, p);
+  return launch_pdl(ffn_gemm2_kernel<false, false, PAIR_WGRAD, false, 0>, pair_grid(), THREADS, SMEM_BYTES, st, m_b, m_b, rows, p);
 }
 
 }  // namespace ffn

@@ -452,3 +452,29 @@ def test_weight_gradients_leave_alike_by_tma_and_by_the_warps(d, f):
         grads.append((bw.dw1, bw.dw3, bw.dw2))
     assert all(torch.equal(a, b) for a, b in zip(*grads))
     assert float(grads[0][0].abs().max()) > 0
+
+
+@pytest.mark.parametrize("rows,d,f", [(80, 16, 144), (80, 256, 512), (80, 528, 1040), (80, 264, 520), (80, 536, 1032), (192, 528, 1040),
+                                      (192, 536, 1032), (192, 2056, 1960)])
+def test_weight_gradients_have_the_same_bits_however_their_tiles_leave(rows, d, f):
+    """The average number of rows per expert decides what of the ring holds a tile on its way out, two stages, one or none; for ragged
+    rows the size of the gradient does too.  Every token uses every expert, so each has as many rows as there are tokens, here one less than
+    at the line and as many, the last with a zero dy: the same sums.  Several tiles per CTA pair."""
+    grads = []
+    for T in (rows, rows - 1):
+        bw = Backward(synth.MoEConfig("rows", T=T, d=d, f=f, E=16, k=16, G=1, seed=d))
+        t = bw.run.t
+        if grads:
+            t["x"].copy_(x[:T])
+            bw.dy.copy_(dy[:T])
+            for n in w:
+                t[n].copy_(w[n])
+            bw.run.route()
+            bw.run.dispatch()
+        else:
+            bw.dy[rows - 1] = 0
+            x, dy, w = t["x"], bw.dy, {n: t[n] for n in ("w_gate", "w1", "w3", "w2")}
+        bw()
+        grads.append((bw.dw1, bw.dw3, bw.dw2))
+    assert all(torch.equal(a, b) for a, b in zip(*grads))
+    assert float(grads[0][0].abs().max()) > 0
