@@ -24,12 +24,16 @@ __device__ __forceinline__ void report_error(int32_t* status, int code, int wher
 }
 
 // ---- programmatic dependent launch ------------------------------------------------------------
-// Every kernel of the library (but long runs of GEMM-1) is launched with programmatic stream serialisation and starts with
-// grid_dependency_sync(): set-up that touches no global data (barrier init, TMEM allocation,
-// tensor-map prefetch) may run while the previous kernel of the stream drains; nothing is read
-// from or written to global memory before the previous kernel has completed and flushed, so
-// results are those of plain stream order.  The call also lets the next kernel of the stream
-// begin its own set-up.
+// Every kernel of the library but long runs of GEMM-1 is launched with programmatic stream serialisation: it may start once every
+// thread block of the previous kernel has called grid_dependency_sync() or ended.  Set-up that touches no global data (barrier
+// init, TMEM allocation, tensor-map prefetch) then runs while that kernel drains; grid_dependency_sync() waits until it has completed and
+// flushed, so results are those of plain stream order, and then lets the next kernel of the stream begin its own set-up.
+//
+// A kernel calls it on every path, and before it touches global memory, with two exceptions: GEMM-2 on single CTAs reads its tables, the
+// abort word and weights earlier, Combine behind a layer's experts its tables.  What they read is older than the kernel before them: no
+// kernel lets dependents go before its own wait, so when an early reader starts, everything in front of that kernel has
+// completed, and that kernel itself (GEMM-1, the quantisation of its output, GEMM-2) writes rows only.  A kernel placed in between must
+// keep to both.
 __device__ __forceinline__ void grid_dependency_sync() {
   asm volatile("griddepcontrol.wait;" ::: "memory");
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");

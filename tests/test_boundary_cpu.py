@@ -1,6 +1,7 @@
 """CPU-side checks of the C-ABI boundary: the library loads, exports every symbol the header
 declares, sizes its workspace sensibly and rejects bad arguments before touching a device."""
 import ctypes
+import functools
 import os
 import re
 import subprocess
@@ -172,30 +173,119 @@ def test_payload_efficiency_matches_the_oracle_and_the_printed_pair(lib):
             B.moe_payload_efficiency(*bad)
 
 
+CSRC = os.path.join(ROOT, "paper_2605_05607_b200", "csrc")
+
+
+@functools.lru_cache(None)
+def source(fn):
+    return re.sub(r"//[^\n]*", "", open(os.path.join(CSRC, fn)).read())
+
+
+def body_at(text, start):
+    """The brace block that opens at or behind `start`."""
+    start = text.index("{", start)
+    depth, i = 0, start
+    while True:
+        depth += {"{": 1, "}": -1}.get(text[i], 0)
+        if depth == 0:
+            return text[start:i + 1]
+        i += 1
+
+
+def kernels():
+    for fn in sorted(os.listdir(CSRC)):
+        if fn.endswith((".cu", ".cuh")):
+            text = source(fn)
+            for m in re.finditer(r"__global__[^;{]*?\b(\w+_kernel)\(", text):
+                depth, i = 1, m.end()
+                while depth:
+                    depth += {"(": 1, ")": -1}.get(text[i], 0)
+                    i += 1
+                yield fn, m.group(1), text[m.end():i - 1], body_at(text, i)
+
+
+@functools.lru_cache(None)
+def pointer_fields(kind):
+    for fn in sorted(os.listdir(CSRC)):
+        m = re.search(rf"\bstruct {kind} \{{", source(fn)) if fn.endswith((".cu", ".cuh")) else None
+        if m:
+            return re.findall(r"\*\s*(\w+)", body_at(source(fn), m.start()))
+    return []
+
+
+WAIT = "grid_dependency_sync();"
+# The kernels that may wait later than at their start, and the condition under which the others of their forms wait there
+EARLY = {"ffn_gemm1_kernel": "if (!PLAIN)", "combine_kernel": "if (!c.early)"}
+# What GEMM-2 and Combine share with the kernel before them, or read beside it: not before the wait
+GEMM2_ROWS = r"\bp\.(a_src|a_scale|gather_idx|out|topk_w|row_pair|b_scale|b_scale2|y_acc)\b"
+COMBINE_ROWS = r"\bc\.(o|y|pg)\b"
+
+
 def test_every_kernel_waits_for_its_stream_predecessor():
-    """All kernels are launched with programmatic stream serialisation, so each must call
-    grid_dependency_sync() before it touches global memory: a kernel without it could start while the
-    previous kernel of the stream still runs, and it would also break the completion chain for the
-    kernel after it."""
-    csrc = os.path.join(ROOT, "paper_2605_05607_b200", "csrc")
+    """All kernels are launched so that they may start while the kernel before them still runs.  Each has to wait for it before it touches
+    global memory, with two exceptions that read tables and weights earlier (the tests below), and on every path: the wait also
+    completes the chain for the kernel after it."""
     seen = 0
-    for fn in sorted(os.listdir(csrc)):
-        if not fn.endswith((".cu", ".cuh")):
-            continue
-        text = open(os.path.join(csrc, fn)).read()
-        for m in re.finditer(r"__global__", text):
-            body_start = text.index("{", text.index(")", m.end()))
-            # the body runs to the matching brace
-            depth, i = 0, body_start
-            while True:
-                depth += text[i] == "{"
-                depth -= text[i] == "}"
-                if depth == 0:
-                    break
-                i += 1
-            assert "grid_dependency_sync()" in text[body_start:i], f"{fn}: kernel at offset {m.start()}"
-            seen += 1
-    assert seen >= 15
+    for fn, name, params, body in kernels():
+        pre, found, _ = body.partition(WAIT)
+        assert found, f"{fn}: {name} never waits"
+        guard = re.split(r"[;{}]", pre)[-1].strip()
+        assert guard == EARLY.get(name, ""), f"{fn}: {name} waits under {guard!r}"
+        assert pre.count("{") - pre.count("}") == 1, f"{fn}: {name} waits inside a block"
+        pointers = re.findall(r"\*\s*(?:__restrict__\s+)?(\w+)", params)
+        for used in pointers:
+            assert not re.search(rf"\b{used}\b", pre), f"{fn}: {name} uses {used} before it waits"
+        for kind, v in re.findall(r"\b([A-Z]\w+)\s+(\w+)\s*(?:,|$)", params):
+            for field in pointer_fields(kind):
+                assert not re.search(rf"\b{v}\.{field}\b", pre), f"{fn}: {name} uses {v}.{field} before it waits"
+        assert not re.search(r"__ld|atomic|tma_load|cp_async", pre), f"{fn}: {name}"
+        seen += 1
+    assert seen >= 25
+    # dependents are let go by the wait alone, behind it
+    triggers = [fn for fn in os.listdir(CSRC) if fn.endswith((".cu", ".cuh")) and "launch_dependents" in source(fn)]
+    text = source("common.cuh")
+    assert triggers == ["common.cuh"] and text.count("launch_dependents") == 1
+    assert text.index("griddepcontrol.wait") < text.index("griddepcontrol.launch_dependents") < text.index("griddepcontrol.wait") + 120
+
+
+def test_gemm2_touches_rows_only_behind_its_wait():
+    """GEMM-2 on single CTAs reads its tables, the abort word and weights beside the kernel before it.  All of them are older than that kernel,
+    as long as that kernel lets dependents go behind its own wait (the test above) and writes none of them: only GEMM-1 and
+    the quantisation of its output stand before GEMM-2."""
+    body = next(b for _, name, _, b in kernels() if name == "ffn_gemm1_kernel")
+    shared, roles = body.split("  if (warp < EPI_WARPS) {", 1)
+    assert not re.search(GEMM2_ROWS, shared)
+    epilogue, rest = roles.split("  } else if (warp == TMA_WARP) {", 1)
+    tma, rest = rest.split("  } else if (warp == MMA_WARP) {", 1)
+    mma, gather = rest.split("\n  } else {\n", 1)
+    for part in (epilogue, gather):
+        pre, found, _ = part.partition("if (PLAIN) " + WAIT)
+        assert found and not re.search(GEMM2_ROWS, pre) and "{" not in pre
+    for part in (tma, mma):
+        assert not re.search(GEMM2_ROWS, part)
+    text = source("ffn.cu")
+    for fn in ("launch_expert_ffn", "launch_expert_ffn_fp8"):
+        launches = re.findall(r"\b(launch_\w+|cudaMem\w+)\(", body_at(text, re.search(rf"cudaError_t {fn}\(", text).end()))
+        assert launches.count("launch_gemm2_single") == 1
+        before = launches[: launches.index("launch_gemm2_single")]
+        assert before[-1] == ("launch_quantize_rows" if fn.endswith("fp8") else "launch_gemm1") and "launch_gemm1" in before, before
+        assert all("launch_gemm2_single" not in source(f) for f in ("api.cu", "bwd.cu", "ep.cu", "layout.cu"))
+
+
+def test_combine_touches_rows_only_behind_its_wait():
+    """Combine orders its slots beside the GEMM that writes its rows.  The tables are older than that GEMM in one place, the layer, where
+    the experts' launches stand directly before it; there alone it is told that it may."""
+    kernel = next(b for _, name, _, b in kernels() if name == "combine_kernel")
+    assert not re.search(COMBINE_ROWS, kernel) and kernel.rstrip("} \n").endswith("if (c.early) " + WAIT[:-1] + ";")
+    token = body_at(source("combine.cuh"), source("combine.cuh").index("void combine_token("))
+    pre, found, rows = token.partition("if (!COHERENT && c.early) " + WAIT)
+    assert found and not re.search(COMBINE_ROWS, pre) and "combine_rows<" not in pre and "combine_two<" not in pre
+    calls = [(fn, m) for fn in os.listdir(CSRC) if fn.endswith(".cu")
+             for m in re.finditer(r"[^;]*;[^;]*\blaunch_combine(?:_rows)?\([^;]*, true\)\)?;", source(fn))]
+    assert [fn for fn, _ in calls] == ["api.cu"]
+    before, call = calls[0][1].group(0).split(";")[:2]
+    assert re.search(r"launch_expert_ffn_fp8\(s, a, q, st\) : launch_expert_ffn\(s, a, st\)\)$", before) and "launch_combine(" in call
+    assert "bool early = false" in source("common.cuh")
 
 
 def test_every_tensor_memory_load_is_waited_for_by_name():
@@ -210,7 +300,7 @@ def test_every_tensor_memory_load_is_waited_for_by_name():
         pending = set()
         for line in open(os.path.join(csrc, fn)):
             code = line.split("//")[0].strip()
-            load, wait = re.search(r"tmem_ld32\(.*, (\w+)\);", code), re.search(r"tmem_ld_wait_on\(([^)]*)\);", code)
+            load, wait = re.search(r"tmem_ld\d+\(.*, (\w+)\);", code), re.search(r"tmem_ld_wait_on\(([^)]*)\);", code)
             if load:
                 pending.add(load.group(1))
                 seen += 1
