@@ -134,8 +134,8 @@ __global__ void __launch_bounds__(WORD_WARPS * 32) fill_layout_kernel(const int3
 // ---- K2 in one kernel ----------------------------------------------------------------------------
 // The four passes above as one kernel of at most 8 thread blocks (a cluster), for small tables (layout_in_one): every block owns a
 // contiguous range of tokens, builds its masks and their prefixes in shared memory, reads the other blocks' row totals through
-// distributed shared memory and fills its tokens' entries.  The four launches are latency, not work: 16 us of device time and
-// three launch gaps for 256 tokens of top-2, 21 us for 3001 of top-4; in one kernel 6.2 and 9.5 us.
+// distributed shared memory and fills its tokens' entries.  The four launches are latency, not work: 12.2 us for 600 tokens of
+// top-2 in 8 groups, 10.7 us for 3001 of top-4; in one kernel 4.9 and 8.2 us.
 constexpr int ONE_THREADS = 1024, ONE_MAX_BLOCKS = 8, ONE_MAX_PAIRS = 32768, ONE_MAX_SMEM = 160 * 1024;
 struct OneShape { int blocks, tokens, words; size_t smem; };   // tokens per block (a multiple of 32) and their mask words
 OneShape one_shape(const Shape& s, bool topk) {

@@ -14,7 +14,11 @@ pytestmark = pytest.mark.gpu
 @pytest.mark.parametrize("T,E,k,G", [(1, 8, 2, 8), (31, 1024, 32, 1024), (256, 8, 8, 1), (257, 12, 3, 4), (513, 6, 1, 3),
                                      (1025, 256, 8, 8), (1100, 64, 4, 32), (4096, 64, 8, 32), (4097, 64, 8, 32),
                                      (16384, 8, 2, 4), (32768, 16, 1, 16), (8192, 128, 4, 8), (8192, 64, 4, 64),
-                                     (7000, 256, 4, 256), (12001, 64, 1, 8), (14999, 16, 1, 1)])
+                                     (7000, 256, 4, 256), (12001, 64, 1, 8), (14999, 16, 1, 1),
+                                     # dense tables with several mask words per block: the last that the one kernel takes, and beyond
+                                     (1777, 128, 4, 8), (2050, 128, 8, 8), (3001, 128, 4, 8), (4096, 64, 8, 8), (4097, 64, 8, 8),
+                                     (6441, 128, 4, 8), (6442, 128, 4, 8), (8192, 64, 1, 4), (11366, 64, 1, 4), (11367, 64, 1, 4),
+                                     (2900, 256, 4, 64), (2901, 256, 4, 64)])
 def test_layout_builders(T, E, k, G):
     rng = np.random.default_rng(T + E)
     skew = -1.5 * np.log(1 + rng.permutation(E))                      # popular and empty experts
