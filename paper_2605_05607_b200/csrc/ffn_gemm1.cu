@@ -40,9 +40,9 @@ namespace {
 constexpr int RING_BYTES = 192 * 1024;       // 4 stages of A + a 256-column B, more of narrower ones
 constexpr int MAX_STAGES = 12;            // 64 rows x 64 columns: 16 KiB
 constexpr int NUM_BARS = 2 * MAX_STAGES + 4;
-// Four epilogue warps, one per row quarter; eight for short K walks (two per quarter, half of the columns each), where a tile's epilogue
-// takes longer than its main loop (512 cycles per 128 bytes of K) or is most of a layer's last round.
-__host__ __device__ constexpr int epi_warps(bool short_k) { return short_k ? 8 : 4; }
+// Four epilogue warps, one per row quarter, or eight (two per quarter, half of the columns each) where a tile's epilogue takes longer than its
+// main loop (512 cycles per 128 bytes of K) or is most of a layer's last round: see launch_width.
+__host__ __device__ constexpr int epi_warps(bool eight) { return eight ? 8 : 4; }
 constexpr int EPI_WARPS_MAX = 8;
 constexpr int STAGE_OUT_WARP = 32 * 64;      // epilogue transpose buffer of one warp: 32 rows x 32 columns, swizzled
 constexpr int TABLE_BYTES = (2 * (MAX_E + 1) * 4 + 15) & ~15;
@@ -50,7 +50,7 @@ constexpr int COLSCALE_WARP = UMMA_N / 2 * 4;   // FP8: one warp's copy of the s
 constexpr int SMEM_BYTES =
     1024 + RING_BYTES + NUM_BARS * 8 + 64 + TABLE_BYTES + EPI_WARPS_MAX * (STAGE_OUT_WARP + COLSCALE_WARP);
 constexpr int GATHER_THREADS = 128;
-__host__ __device__ constexpr int threads(bool short_k) { return (epi_warps(short_k) + 2) * 32 + GATHER_THREADS; }
+__host__ __device__ constexpr int threads(bool eight) { return (epi_warps(eight) + 2) * 32 + GATHER_THREADS; }
 // The producers (TMA thread, 128 gather threads) wait for a free stage with a suspend-time hint: parked in hardware
 // instead of polling.  At the board's power limit the layer's time follows energy: GEMM-1 alone in a loop on the
 // DeepSeek-V3 shape 15.78 -> 15.50 ms with the hint (two alternations, same box), a single cold launch 13.41 -> 13.48.
@@ -76,8 +76,8 @@ constexpr int SWAP_ROWS = 96;   // see `swapped`
 // FEW = true (narrow tiles only): tiles of 64 rows, for layers of at most 64 rows in all.  A stage is then a third smaller and
 // the ring holds more of the weights in flight (96 KiB instead of 64 in GEMM-2), which is what bounds a CTA that streams a column
 // slab of one expert: GEMM-2 of one token, top-2 of d = 4096, f = 14336, 58 -> 46 us (4.1 -> 5.1 TB/s).
-template <bool FP8, bool PLAIN, bool NARROW, bool FEW, bool SHORT_K>
-__global__ void __launch_bounds__(threads(SHORT_K), 1)
+template <bool FP8, bool PLAIN, bool NARROW, bool FEW, bool EIGHT>
+__global__ void __launch_bounds__(threads(EIGHT), 1)
 ffn_gemm1_kernel(const __grid_constant__ CUtensorMap map_w1, const __grid_constant__ CUtensorMap map_w3,
                  const GemmParams p) {
   constexpr int BN = !NARROW ? UMMA_N : PLAIN ? 64 : 128;   // accumulator columns of a tile
@@ -85,7 +85,7 @@ ffn_gemm1_kernel(const __grid_constant__ CUtensorMap map_w1, const __grid_consta
   constexpr int HALF = BN > 64 ? BN / 2 : BN;               // columns from each of the two weight maps (BN = 64: one)
   constexpr int ROWS = FEW ? 64 : BM;                       // rows of a tile
   constexpr int WROWS = ROWS / 4;                           // rows of an epilogue warp: TMEM lanes 32 q .. 32 q + WROWS - 1
-  constexpr int EPI_WARPS = epi_warps(SHORT_K), TMA_WARP = EPI_WARPS, MMA_WARP = EPI_WARPS + 1, GATHER_WARP = EPI_WARPS + 2;
+  constexpr int EPI_WARPS = epi_warps(EIGHT), TMA_WARP = EPI_WARPS, MMA_WARP = EPI_WARPS + 1, GATHER_WARP = EPI_WARPS + 2;
   constexpr int WCOLS = BN_OUT / (EPI_WARPS / 4);           // output columns of an epilogue warp
   constexpr int SCALES = UMMA_N / (EPI_WARPS / 4);          // FP8: floats of its column scales
   static_assert(NARROW || !FEW, "64-row tiles come with narrow ones");
@@ -504,28 +504,31 @@ ffn_gemm1_kernel(const __grid_constant__ CUtensorMap map_w1, const __grid_consta
 }  // namespace
 
 namespace {
-template <bool FP8, bool PLAIN, bool NARROW, bool FEW, bool SHORT_K>
+template <bool FP8, bool PLAIN, bool NARROW, bool FEW, bool EIGHT>
 cudaError_t launch_form(const GemmParams& p, const CUtensorMap& m_a, const CUtensorMap& m_b, bool overlap, cudaStream_t st) {
   // per device; several host threads may get here at once: setting the attribute twice is harmless
   static std::atomic<bool> attr_set[MAX_DEVICES];
   const int dev = current_device();
-  const auto kernel = ffn_gemm1_kernel<FP8, PLAIN, NARROW, FEW, SHORT_K>;
+  const auto kernel = ffn_gemm1_kernel<FP8, PLAIN, NARROW, FEW, EIGHT>;
   if (!attr_set[dev].load(std::memory_order_acquire)) {
     cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_BYTES);
     if (e != cudaSuccess) return e;
     attr_set[dev].store(true, std::memory_order_release);
   }
   ProfileScope prof(PLAIN ? KID_GEMM2 : KID_GEMM1, st);
-  return launch_kernel(overlap, 0, kernel, sm_count(), threads(SHORT_K), SMEM_BYTES, st, m_a, m_b, p);
+  return launch_kernel(overlap, 0, kernel, sm_count(), threads(EIGHT), SMEM_BYTES, st, m_a, m_b, p);
 }
 
 template <bool FP8, bool PLAIN>
 cudaError_t launch_width(const GemmParams& p, const CUtensorMap& m_a, const CUtensorMap& m_b, bool narrow, bool few, bool overlap,
                          cudaStream_t st) {
-  // Layers, us, four / eight epilogue warps in the full-width tiles, K walk of GEMM-1 in brackets: 10181 tokens top-1 of 8 x 656 x 4512 in
-  // 8 bits (6) 236 / 230, 529 top-4 of 16 x 608 x 1392 (10; GEMM-2 22) 50.8 / 49.7, 4000 top-4 of 32 x 1504 x 2048 (24) 377.7 / 378.5, of 2048 x
-  // 2048 (32) 461.5 / 463.4, 16384 top-8 of 128 x 4096 x 1536 in 8 bits (32) 3099 / 3106, 32768 top-8 of 256 x 7168 x 2048 (112) 21320 / 21440;
-  // narrow tiles: 256 top-2 of 8 x 512 x 1024 29.3 / 28.6, but of 64 rows (1 token, 8 x 4096 x 14336) 143 / 145.
+  // Eight epilogue warps for full-width tiles with a K walk of up to 24 blocks, and for narrow tiles of 128 rows whatever their K: such layers
+  // have one round of tiles or two, so the epilogue is not hidden.  Layers, us, four / eight in the full-width tiles, K walk of GEMM-1 in
+  // brackets: 10181 tokens top-1 of 8 x 656 x 4512 in 8 bits (6) 236 / 230, 529 top-4 of 16 x 608 x 1392 (10; GEMM-2 22) 50.8 / 49.7, 4000 top-4 of
+  // 32 x 1504 x 2048 (24) 377.7 / 378.5, of 2048 x 2048 (32) 461.5 / 463.4, 16384 top-8 of 128 x 4096 x 1536 in 8 bits (32) 3099 / 3106, 32768 top-8 of
+  // 256 x 7168 x 2048 (112) 21320 / 21440; narrow tiles, by the K of GEMM-1 and GEMM-2: 256 top-2 of 8 (512, 1024) 28.1 / 27.2, 36 top-2 of 8
+  // (4160, 1008) 64.9 / 64.2, 200 (7168, 2048) 85.1 / 84.9, 100 (6144, 4096) 79.2 / 79.1, 90 (3072, 8192) 73.9 / 73.7, 65 (4096, 14336) 117.1 / 118.2, in
+  // 8 bits 90.1 / 91.7; but of 64 rows (1 token, 8 x 4096 x 14336) 143 / 145.
   if (!narrow && p.K * (FP8 ? 1 : 2) > 24 * 128) return launch_form<FP8, PLAIN, false, false, false>(p, m_a, m_b, overlap, st);
   if (!narrow) return launch_form<FP8, PLAIN, false, false, true>(p, m_a, m_b, overlap, st);
   return few ? launch_form<FP8, PLAIN, true, true, false>(p, m_a, m_b, overlap, st) : launch_form<FP8, PLAIN, true, false, true>(p, m_a, m_b, overlap, st);
@@ -535,12 +538,14 @@ cudaError_t launch_width(const GemmParams& p, const CUtensorMap& m_a, const CUte
 // narrow: 64 output columns per tile instead of 128 (GEMM-1) or 256 (GEMM-2); p.n_tiles is set here.  The FP8 weight maps then
 // have boxes of 64 columns (make_weight_map_fp8).  few: no expert has more than 64 rows (used by narrow tiles only).
 //
-// rows: pairs of the layer.  A long GEMM starts when the kernel before it has drained, so that its thread blocks are placed on an
-// empty GPU: neighbours, which share a weight tile, then sit in the same GPC, and the tile reaches it once.  Placed one by one as
-// SMs become free they are scattered, and the GEMM spends more of the board's power on moving operands.  Layers, overlapped / drained, us:
+// rows: pairs of the layer, the unused slots of a sparse table among them (how many are used is known on the device only).  A long GEMM
+// starts when the kernel before it has drained, so that its thread blocks are placed on an empty GPU, in order, and not one by one as SMs
+// become free.  Blocks that share a weight tile then probably sit closer together (what the times show; where a block sits was not looked
+// at), and less of the board's power goes into moving operands.  Layers, overlapped / drained, us:
 // 32768 tokens, top-8 of 256 x 7168 x 2048 22750 / 21620; 16384 skewed 12970 / 12570; 8192 top-4 of 64 x 7168 x 4096 in 8 bits
 // 3490 / 3310; 16384 top-4 of 32 x 2048 x 2048 1581 / 1563; 2048 top-4 of 32 x 4096 x 4096 (2^37 products per matrix) 1072 / 1072;
-// 4096 skewed, top-8 of 32 x 2048 x 1024 (2^36) 465 / 467.
+// 4096 skewed, top-8 of 32 x 2048 x 1024 (2^36) 465 / 467.  At the line both are alike, so a sparse table that is counted as longer than it
+// is loses nothing there; one of 16384 rows that uses 2 of 8 slots counts 4 times its products.
 cudaError_t launch_gemm1(GemmParams p, const CUtensorMap& m_w1, const CUtensorMap& m_w3, long long rows, bool fp8, bool narrow, bool few,
                          cudaStream_t st) {
   p.n_tiles = narrow ? (p.N + 63) / 64 : (p.N + 127) / 128;

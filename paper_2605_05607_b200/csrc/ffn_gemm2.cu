@@ -712,7 +712,7 @@ cudaError_t launch_bwd_dx(const GemmParams& p, const CUtensorMap& m_w1t, const C
 }
 
 // Weight gradient on CTA pairs: dw[e] = A_e^T . B_e, A = [rows, M], B = [rows, N] in the padded row space (maps with
-// boxes of 64 columns x 64 rows; rows_total of them without the padding), dw [E, M, N] bf16, fully written.
+// boxes of 64 columns x 64 rows; rows_total: pairs of the layer, unused slots of a sparse table among them), dw [E, M, N] bf16, fully written.
 cudaError_t launch_wgrad_pair(const CUtensorMap& m_a, const CUtensorMap& m_b, const int32_t* poff, long long rows_total, void* dw, int E,
                               int M, int N, int32_t* status, cudaStream_t st) {
   cudaError_t e = set_pair_attributes();

@@ -382,9 +382,10 @@ def test_gradients_of_ragged_rows_take_no_longer():
         return lambda: B.moe_layer_backward(r.shape, t["x"], bw.dy, r.idx, r.w, r.lay, t["w1"], t["w3"], t["w2"], bw.dx, bw.dw1,
                                             bw.dw3, bw.dw2, bw.ws)
 
-    # measured, taking turns: 1.13-1.18; stored sector by sector 1.42-1.44.  The line lies in the middle.
+    # measured, taking turns: 1.07 with boxes of 64 columns that leave together; one after the other, or sector by sector, 1.42-1.44.  The
+    # line lies in the middle.
     us, other = H.device_us(call(4104, 1544), call(4112, 1552), n=2)
-    assert us <= 1.3 * other
+    assert us <= 1.25 * other
 
 
 def gate_gradient(cfg):
