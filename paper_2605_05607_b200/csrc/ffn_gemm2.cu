@@ -215,11 +215,18 @@ ffn_gemm2_kernel(const __grid_constant__ CUtensorMap map_b0, const __grid_consta
       ptx::st_shared_v4(stage + lane * 64 + ((v ^ ((lane >> 1) & 3)) << 4), q0, q1, q2, q3);
     };
     int tl = 0;
-    // TILE_OUT: all eight warps (OUT = 2) or the four of a column half meet in every tile, so they leave the loop together, by the vote below
-    // and not one by one.
+    // TILE_OUT: all eight warps (OUT = 2) or the four of a column half meet at barriers in every tile.  Whether a warp's wait ends with the tile
+    // or with an abort is a race between them, so none leaves early: one that gave up walks the rest of the tiles without waiting (what they
+    // hold is undefined then, as after any abort).  Left by a vote of the warps instead, a backward pass of 7 tokens on 128 experts of 2880 x 2880
+    // took 1690 us, 1654 so.
     constexpr int MEET = EPI_WARPS * 32 / (OUT == 1 ? 2 : 1);
     const int meet_id = 1 + threadIdx.x / MEET;
     const bool leader = threadIdx.x % MEET == 0;
+    auto free_boxes = [&] {   // the stores before have read theirs
+      if (leader) ptx::bulk_wait_read();
+      ptx::named_barrier(meet_id, MEET);
+    };
+    bool go = !TILE_OUT || !*abort_flag;   // no wait has given up
     for (int w = cluster_id; w < total && (TILE_OUT || !*abort_flag); w += num_clusters, ++tl) {
       const Tile t = tile_of(w);
       const int buf = tl & 1;
@@ -242,15 +249,8 @@ ffn_gemm2_kernel(const __grid_constant__ CUtensorMap map_b0, const __grid_consta
                            : make_uint4(0u, 0u, 0u, 0u);
           }
       }
-      bool go = ptx::mbar_wait_warp<false, HINT>(tfull_bar(buf), (tl >> 1) & 1, abort_flag, global_abort);
-      if (!go) timeout(1);
-      if (TILE_OUT) {
-        // Whether a warp's wait ended with the tile or with an abort is a race, and the barriers of the tile want all of them: one vote.
-        // Each gets here in bounded time, and those that go on leave the tile's last barrier together.
-        if (leader) ptx::bulk_wait_read();   // the stores of the last tile have read theirs
-        go = ptx::named_barrier_all(meet_id, MEET, go);
-      }
-      if (!go) break;
+      if (go && !ptx::mbar_wait_warp<false, HINT>(tfull_bar(buf), (tl >> 1) & 1, abort_flag, global_abort)) { timeout(1); go = false; }
+      if (!TILE_OUT && !go) break;
       ptx::tc_fence_after();
       const int lrow = row_w + lane;
       const bool valid = lrow < t.rows;
@@ -395,11 +395,12 @@ ffn_gemm2_kernel(const __grid_constant__ CUtensorMap map_b0, const __grid_consta
           }
         }
       } else if (OUT == 1) {
-        // As below, in boxes of 64 columns of which a column half has one place: its warps fill the second box when the store of the first has
-        // read it.
+        // As below, in boxes of 64 columns of which a column half has one place: its warps fill a box when the store of the one before has read
+        // it.
         const uint32_t box = smem_base + NST * STAGE_BYTES + half * BOX_BYTES, dst = box + (quarter * 32 + lane) * 128;
 #pragma unroll
         for (int c = 0; c < 2; ++c) {
+          if (c == 0) free_boxes();
           uint32_t lo[32], hi[32];
           ptx::tmem_ld32(taddr + c * 64, lo);
           ptx::tmem_ld32(taddr + c * 64 + 32, hi);
@@ -414,16 +415,13 @@ ffn_gemm2_kernel(const __grid_constant__ CUtensorMap map_b0, const __grid_consta
             q[j] = pack2(__uint_as_float(lo[2 * j]), __uint_as_float(lo[2 * j + 1]));
             q[16 + j] = pack2(__uint_as_float(hi[2 * j]), __uint_as_float(hi[2 * j + 1]));
           }
-          if (c > 0) {
-            if (leader) ptx::bulk_wait_read();
-            ptx::named_barrier(meet_id, MEET);
-          }
+          if (c > 0) free_boxes();
 #pragma unroll
           for (int v = 0; v < 8; ++v) ptx::st_shared_v4(dst + ((v ^ (lane & 7)) << 4), q[v * 4], q[v * 4 + 1], q[v * 4 + 2], q[v * 4 + 3]);
           ptx::fence_proxy_async_smem();
           ptx::named_barrier(meet_id, MEET);
           const int col = t.n0 + half * 128 + c * 64;
-          if (leader && t.rows > 0 && col < p.N) {
+          if (leader && go && t.rows > 0 && col < p.N) {
             ptx::tma_store_3d(&map_b1, box, col, t.out_row0 - t.e * p.K, t.e);
             ptx::bulk_commit();
           }
@@ -434,6 +432,7 @@ ffn_gemm2_kernel(const __grid_constant__ CUtensorMap map_b0, const __grid_consta
         const uint32_t dst = smem_base + NST * STAGE_BYTES + (quarter * 32 + lane) * 128;
 #pragma unroll
         for (int c = 0; c < 2; ++c) {
+          if (c == 0) free_boxes();
           uint32_t lo[32], hi[32];
           ptx::tmem_ld32(taddr + c * 64, lo);
           ptx::tmem_ld32(taddr + c * 64 + 32, hi);
@@ -452,7 +451,7 @@ ffn_gemm2_kernel(const __grid_constant__ CUtensorMap map_b0, const __grid_consta
         }
         ptx::fence_proxy_async_smem();
         ptx::named_barrier(meet_id, MEET);
-        if (leader && t.rows > 0) {
+        if (leader && go && t.rows > 0) {
 #pragma unroll
           for (int c = 0; c < 4; ++c)
             if (t.n0 + c * 64 < p.N)

@@ -479,3 +479,20 @@ def test_weight_gradients_have_the_same_bits_however_their_tiles_leave(rows, d, 
         grads.append((bw.dw1, bw.dw3, bw.dw2))
     assert all(torch.equal(a, b) for a, b in zip(*grads))
     assert float(grads[0][0].abs().max()) > 0
+
+
+@pytest.mark.parametrize("rows", [20, 100, 200])
+def test_a_pass_on_an_aborted_workspace_ends(rows):
+    """The abort word of a wait that gave up makes the kernels skip their work, whichever way the gradients' tiles leave; once it is reset the
+    pass gives the same bits as before."""
+    bw = Backward(synth.MoEConfig("abort", T=rows, d=272, f=528, E=32, k=32, G=1, seed=rows))
+    bw()
+    want = [t.clone() for t in (bw.dx, bw.dw1, bw.dw3, bw.dw2)]
+    B.moe_selftest_wait_timeout(bw.ws, 300_000)
+    with pytest.raises(AssertionError, match="device status"):
+        bw()
+    st = B.moe_status(bw.ws)
+    assert st[0] == B.MOE_DEV_TIMEOUT and st[1] == 9 and st[4] == 1, st
+    B.moe_status_reset(bw.ws)
+    bw()
+    assert all(torch.equal(a, b) for a, b in zip(want, (bw.dx, bw.dw1, bw.dw3, bw.dw2)))
