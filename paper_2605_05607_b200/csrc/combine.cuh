@@ -119,26 +119,30 @@ __device__ __forceinline__ void combine_two(const CombineArgs& c, int t, int lan
 // with loads that see what other thread blocks of the SAME kernel wrote (the tracker-paced kernel); otherwise
 // streaming loads.  BATCH (2, 4 or 8): rows loaded at a time; 2 is for k <= 2 only, 4 and 8 are correct for any k, the one that matches
 // k wastes no issue slots on absent slots (a top-2 layer through the 8-row form runs at a third of the bandwidth).
-template <bool COHERENT, int BATCH, int COLS = 4>
+// EARLY: the tables are read before the wait for the kernel that writes o, through L2 (an L1 line may be from before that wait); a form of its
+// own, since the wait in the token's code costs the others 1 to 8 % (16 tokens top-16 of d = 1024 10.9 -> 11.7 us, 3000 top-2 of 2880 8.6 -> 9.5, 8192
+// top-8 of 4096 106.8 -> 108.5).
+template <bool COHERENT, int BATCH, int COLS = 4, bool EARLY = false>
 __device__ __forceinline__ void combine_token(const CombineArgs& c, int t, int lane, int* s_row, int* s_dst, float* s_w,
                                               int v_begin = 0, int v_end = 0x7FFFFFFF) {
   const int k = c.k;
+  auto table = [](const auto* p) { return EARLY ? __ldcg(p) : __ldg(p); };
   // lane j < k owns slot j; order slots by (group, slot)
   int my_g = 0x7FFFFFFF, my_row = 0, my_dst = 0;
   float my_w = 1.f;
   if (lane < k) {
-    const int e = __ldcg(c.topk_idx + (size_t)t * k + lane);
+    const int e = table(c.topk_idx + (size_t)t * k + lane);
     // e < 0: unused slot of a sparse top-k table, sorts behind every real slot and is not read.  An expert
     // index or a row outside its table (the layout builder reported it and wrote row -1) is skipped the
     // same way, so no table entry is ever used as an address unchecked.
     if (e >= 0 && e < c.E) {
-      const int r = __ldcg(c.pair_row + (size_t)t * k + lane);
-      const int a = __ldcg(c.al + (size_t)(e / c.m) * c.T + t);
+      const int r = table(c.pair_row + (size_t)t * k + lane);
+      const int a = table(c.al + (size_t)(e / c.m) * c.T + t);
       if (r >= 0 && r < c.n_rows && a >= 0) {
         my_g = e / c.m;
         my_row = r;
-        my_dst = __ldcg(c.group_offsets + my_g) + a;
-        if (c.weighted) my_w = __ldcg(c.topk_w + (size_t)t * k + lane);
+        my_dst = table(c.group_offsets + my_g) + a;
+        if (c.weighted) my_w = table(c.topk_w + (size_t)t * k + lane);
       } else {
         report_error(c.status, DEV_INDEX_OUT_OF_RANGE, KID_COMBINE, t, r);
       }
@@ -155,7 +159,7 @@ __device__ __forceinline__ void combine_token(const CombineArgs& c, int t, int l
   __syncwarp();
   if (lane < k) { s_row[my_pos] = my_row; s_dst[my_pos] = my_dst; s_w[my_pos] = my_w; }
   __syncwarp();
-  if (!COHERENT && c.early) grid_dependency_sync();   // (again for each token of the warp: returns at once)
+  if (EARLY) grid_dependency_sync();   // (again for each token of the warp: returns at once)
   if (BATCH == 2) combine_two<COHERENT, COLS>(c, t, lane, kv, s_row, s_dst, s_w, v_begin, v_end);
   else combine_rows<COHERENT, BATCH>(c, t, lane, kv, s_row, s_dst, s_w, v_begin, v_end);
   __syncwarp();

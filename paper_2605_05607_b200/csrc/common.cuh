@@ -123,7 +123,6 @@ struct CombineArgs {
   const int32_t* group_offsets;   // [G + 1]
   int T, E, k, m, vec_per_row, weighted, n_rows;
   int32_t* status;
-  int early;                      // the tables were complete before the kernel that writes o started: they are read before the wait for it
 };
 
 // Scratch tables of the layout builder (inside the workspace).

@@ -489,9 +489,9 @@ cudaError_t launch_permute_rows(const Shape& s, const void* src, int src_rows, c
 // One warp per (token, column part); the per-token work is combine_token() (combine.cuh).  With few tokens a row
 // is split over `parts` warps so that enough loads are in flight to reach the memory bandwidth (one warp per token
 // leaves a 4096-token batch at a third of it).
-template <int BATCH, int COLS = 4>
+template <int BATCH, int COLS, bool EARLY>
 __global__ void __launch_bounds__(256, 3) combine_kernel(const CombineArgs c, int parts, int vec_per_part) {
-  if (!c.early) grid_dependency_sync();
+  if (!EARLY) grid_dependency_sync();
   __shared__ int s_row[8][32];   // per warp: expert-sorted row of the slot at sorted position p
   __shared__ int s_dst[8][32];   // dispatched row (t, g) of that slot's group
   __shared__ float s_w[8][32];
@@ -500,10 +500,10 @@ __global__ void __launch_bounds__(256, 3) combine_kernel(const CombineArgs c, in
   const long long units = (long long)c.T * parts;
   for (long long u = (long long)blockIdx.x * wpb + wid; u < units; u += (long long)gridDim.x * wpb) {
     const int t = (int)(u / parts), part = (int)(u % parts);
-    combine_token<false, BATCH, COLS>(c, t, lane, s_row[wid], s_dst[wid], s_w[wid], part * vec_per_part,
+    combine_token<false, BATCH, COLS, EARLY>(c, t, lane, s_row[wid], s_dst[wid], s_w[wid], part * vec_per_part,
                                 (part + 1) * vec_per_part);
   }
-  if (c.early) grid_dependency_sync();   // warps without a token
+  if (EARLY) grid_dependency_sync();   // warps without a token
 }
 
 // parts of a row so that about 32 warps per SM exist even for small batches (at most 8, at least 4 vectors per lane)
@@ -533,14 +533,16 @@ cudaError_t launch_combine_rows(const Shape& s, const void* o, const Layout& L, 
   ProfileScope prof(KID_COMBINE, st);
   CombineArgs c{static_cast<const uint4*>(o), static_cast<uint4*>(y), static_cast<uint4*>(pg), topk_idx, topk_w,
                 L.pair_row, L.al, L.group_offsets, s.T, s.E, s.k, s.E / s.G, vec, (s.flags & 1) ? 1 : 0,
-                n_rows, status, early ? 1 : 0};
+                n_rows, status};
   // parts that are no multiple of four warp strides: two columns at a time, so that the last step is not half empty (2050 tokens of
   // d = 2880 with group sums, 192 columns each: 11.8 -> 10.4 us, 10.7 with single columns)
-  if (s.k <= 2 && vec_per_part % 128 != 0)
-    return launch_pdl(combine_kernel<2, 2>, (unsigned)blocks, 256, 0, st, c, parts, vec_per_part);
-  if (s.k <= 2) return launch_pdl(combine_kernel<2>, (unsigned)blocks, 256, 0, st, c, parts, vec_per_part);
-  if (s.k <= 4) return launch_pdl(combine_kernel<4>, (unsigned)blocks, 256, 0, st, c, parts, vec_per_part);
-  return launch_pdl(combine_kernel<8>, (unsigned)blocks, 256, 0, st, c, parts, vec_per_part);
+  auto launch = [&](auto plain, auto before_wait) {
+    return launch_pdl(early ? before_wait : plain, (unsigned)blocks, 256, 0, st, c, parts, vec_per_part);
+  };
+  if (s.k <= 2 && vec_per_part % 128 != 0) return launch(combine_kernel<2, 2, false>, combine_kernel<2, 2, true>);
+  if (s.k <= 2) return launch(combine_kernel<2, 4, false>, combine_kernel<2, 4, true>);
+  if (s.k <= 4) return launch(combine_kernel<4, 4, false>, combine_kernel<4, 4, true>);
+  return launch(combine_kernel<8, 4, false>, combine_kernel<8, 4, true>);
 }
 
 // Last step of the layer when Combine ran inside GEMM-2's epilogue: the fp32 token accumulators

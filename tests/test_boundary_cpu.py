@@ -215,7 +215,7 @@ def pointer_fields(kind):
 
 WAIT = "grid_dependency_sync();"
 # The kernels that may wait later than at their start, and the condition under which the others of their forms wait there
-EARLY = {"ffn_gemm1_kernel": "if (!PLAIN)", "combine_kernel": "if (!c.early)"}
+EARLY = {"ffn_gemm1_kernel": "if (!PLAIN)", "combine_kernel": "if (!EARLY)"}
 # What GEMM-2 and Combine share with the kernel before them, or read beside it: not before the wait
 GEMM2_ROWS = r"\bp\.(a_src|a_scale|gather_idx|out|topk_w|row_pair|b_scale|b_scale2|y_acc)\b"
 COMBINE_ROWS = r"\bc\.(o|y|pg)\b"
@@ -276,9 +276,9 @@ def test_combine_touches_rows_only_behind_its_wait():
     """Combine orders its slots beside the GEMM that writes its rows.  The tables are older than that GEMM in one place, the layer, where
     the experts' launches stand directly before it; there alone it is told that it may."""
     kernel = next(b for _, name, _, b in kernels() if name == "combine_kernel")
-    assert not re.search(COMBINE_ROWS, kernel) and kernel.rstrip("} \n").endswith("if (c.early) " + WAIT[:-1] + ";")
+    assert not re.search(COMBINE_ROWS, kernel) and kernel.rstrip("} \n").endswith("if (EARLY) " + WAIT)
     token = body_at(source("combine.cuh"), source("combine.cuh").index("void combine_token("))
-    pre, found, rows = token.partition("if (!COHERENT && c.early) " + WAIT)
+    pre, found, rows = token.partition("if (EARLY) " + WAIT)
     assert found and not re.search(COMBINE_ROWS, pre) and "combine_rows<" not in pre and "combine_two<" not in pre
     calls = [(fn, m) for fn in os.listdir(CSRC) if fn.endswith(".cu")
              for m in re.finditer(r"[^;]*;[^;]*\blaunch_combine(?:_rows)?\([^;]*, true\)\)?;", source(fn))]
