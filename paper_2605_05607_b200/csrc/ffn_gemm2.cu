@@ -226,7 +226,7 @@ ffn_gemm2_kernel(const __grid_constant__ CUtensorMap map_b0, const __grid_consta
       if (leader) ptx::bulk_wait_read();
       ptx::named_barrier(meet_id, MEET);
     };
-    bool go = !TILE_OUT || !*abort_flag;   // no wait has given up
+    bool go = !TILE_OUT || __all_sync(0xFFFFFFFFu, !*abort_flag);   // no wait has given up (the same in all lanes)
     for (int w = cluster_id; w < total && (TILE_OUT || !*abort_flag); w += num_clusters, ++tl) {
       const Tile t = tile_of(w);
       const int buf = tl & 1;
