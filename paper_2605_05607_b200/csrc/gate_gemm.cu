@@ -353,7 +353,9 @@ __global__ void __launch_bounds__(256) split_gate_kernel(const float* __restrict
 // 315 -> 291 and 98 -> 91 in a replayed graph since ragged rows of logits leave whole).
 // Up to 128 experts tiles of 16 columns where the SMs take them in as many rounds: a block has half the weight to split and less to
 // move through shared memory per k-block, moe_route of (T, d, E), us, 32 / 16 columns: 64, 4096, 128 23.5 / 20.6; 300, 4096, 65 30.2 / 24.5;
-// 872, 6832, 16 35.8 / 27.8; 1669, 3520, 64 23.9 / 19.4; 200, 256, 64 7.0 / 6.3.
+// 872, 6832, 16 35.8 / 27.8; 1669, 3520, 64 23.9 / 19.4; 200, 256, 64 7.0 / 6.3.  With more than 64 experts a hundred blocks of them get in each
+// other's way, 2.4 us whatever K (1659, 256, 128: 9.8 / 10.0, 1915 tokens 9.8 / 12.1; of d = 1024 13.7 / 13.9, 13.8 / 16.0, of d = 4096 28.8 / 24.3,
+// 28.7 / 26.7).
 struct GatePlan { int gn, bm, m_sub; bool pre; };
 GatePlan plan_gate(int T, int d, int E) {
   struct Cost { double start, kb, kb_ragged; };
@@ -376,7 +378,8 @@ GatePlan plan_gate(int T, int d, int E) {
     const int rows = f.form.m_sub * f.form.bm, sms = sm_count();
     const long long tasks = (long long)((T + rows - 1) / rows) * ((E + f.form.gn - 1) / f.form.gn);
     const double round = c.start + ((d + BK - 1) / BK) * (E % 4 == 0 ? c.kb : c.kb_ragged);
-    const double us = (double)((tasks + sms - 1) / sms) * round + (f.form.pre ? PRE_US : 0.0);
+    const double crowd = f.form.gn == 16 && E > 64 && tasks > 100 ? 2.4 : 0.0;
+    const double us = (double)((tasks + sms - 1) / sms) * round + (f.form.pre ? PRE_US : 0.0) + crowd;
     if (us < best_us) { best_us = us; best = f.form; }
   }
   return best;

@@ -25,6 +25,7 @@ def test_form_cases_reach_every_form():
     text = open(os.path.join(os.path.dirname(B.__file__), "csrc", "gate_gemm.cu")).read()
     pre_min = int(re.search(r"PRE_MIN_TOKENS = (\d+);", text).group(1))
     pre_us = float(re.search(r"PRE_US = ([\d.]+);", text).group(1))
+    crowd = re.search(r"form\.gn == (\d+) && E > (\d+) && tasks > (\d+) \? ([\d.]+)", text).groups()
     cost = lambda t: None if t == "NO" else tuple(float(v) for v in t.strip("{}").split(","))
     table = [((int(gn), int(bm), int(m), pre == "true"), cost(run), cost(apart)) for gn, bm, m, pre, run, apart in
              re.findall(r"\{\{(\d+), (\d+), (\d+), (true|false)\}, (NO|\{[^}]*\}), (NO|\{[^}]*\})\}", text)]
@@ -38,6 +39,8 @@ def test_form_cases_reach_every_form():
                 continue
             rounds = -(-(-(-T // (f[1] * f[2])) * -(-E // f[0])) // 148)
             us = rounds * (c[0] + -(-d // 64) * c[1 if E % 4 == 0 else 2]) + (pre_us if f[3] else 0.0)
+            if f[0] == int(crowd[0]) and E > int(crowd[1]) and -(-T // (f[1] * f[2])) * -(-E // f[0]) > int(crowd[2]):
+                us += float(crowd[3])
             best = min(best, (us, f), key=lambda b: b[0])
         return best[1]
 
@@ -99,3 +102,20 @@ def test_fewer_experts_take_no_longer(T, d, E, wider):
     # with logits stored by the element where E is no multiple of 4 1.45, 1.38 (the last two)
     us, other = H.device_us(call(E), call(wider))
     assert us <= 1.23 * other
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("d,E", [(256, 128), (1024, 104)])
+def test_a_few_more_row_tiles_take_no_longer(d, E):
+    """13 and 16 row tiles of 128 tokens, both at one task per SM: the second call takes what the first does, the top-k of 384 tokens more aside."""
+    def call(T):
+        x = torch.randn(T, d, device="cuda").to(torch.bfloat16)
+        w = torch.randn(d, E, device="cuda") * 0.02
+        shape = B.MoEShape(T, d, 64, E, 1, 1, 0, 0)
+        ws = B.alloc_workspace(shape)
+        out = torch.empty(T, E, device="cuda"), torch.empty(T, dtype=torch.int32, device="cuda"), torch.empty(T, device="cuda")
+        return lambda: B.moe_route(shape, x, w, None, *out, ws)
+
+    # measured, taking turns: 1.02, 1.05; in 128 and 112 blocks of 16 columns 1.13, 1.12.  The line lies in the middle.
+    us, other = H.device_us(call(2048), call(1664))
+    assert us <= 1.08 * other
